@@ -1,27 +1,92 @@
 // FP64 kernels of the ChASE-BSE library.
 //
-// On GB300 the FP64 pipe runs at ~1/64 of the FP32 rate (measured: 1.20 TFLOP/s
-// with DFMA, 1.05 TFLOP/s with DMMA mma.sync.m8n8k4), so an FP64 product of an
-// n x 2n matrix with even a handful of vectors is bound by the FP64 pipe, not by
-// HBM.  The kernels below therefore use plain DFMA with register tiles and keep
-// the shared-memory staging simple; what matters is enough independent FMAs in
-// flight per SM sub-partition.
+// On GB300 the FP64 pipe issues 2 DFMA lanes per clock and SM (measured: 1.20 TFLOP/s
+// with DFMA, 1.05 TFLOP/s with DMMA mma.sync.m8n8k4), 1/64 of the FP32 rate: a warp's
+// DFMA occupies its SM for 16 clocks, so shared-memory and L2 traffic hide behind the
+// arithmetic at any tile shape, and an FP64 product is bound by (1) the number of FP64
+// instructions, padding included, and (2) how evenly they spread over the 152 pipes.
+// Both kernels below therefore use a warp tile of 32 rows (one per lane) by a few columns,
+// cut the rows and columns close to the matrix, and split K until the CTAs fill whole
+// waves of SMs (plan_fp64); the K partials are summed in order by a second kernel.
+#include <algorithm>
+
 #include "fp64_kernels.cuh"
 
 namespace cb {
 
+namespace {
+constexpr int ROWS = 32;   // rows of a tile: one per lane
+constexpr int WARPS = 8;   // column groups of a tile: one per warp
+constexpr int BK = 16;     // K elements staged at a time
+constexpr int THREADS = 32 * WARPS;
+constexpr double PART_LIMIT = 512e6;  // bytes of K partials
+
+int num_sms() {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
+                                                 cudaSuccess || sms <= 0)
+      sms = 152;
+  }
+  return sms;
+}
+
+// Tile width and K split of an FP64 product with M rows, N columns and K steps of
+// `fma_step` DFMA per row and column, `tile_step` further FP64 instructions per row and K
+// step of a tile (forming its left operand).  The estimated clocks of a split: waves of
+// CTAs x (FP64 instructions of a CTA / 2 + 1500 for its loads' latency), plus the sum of
+// the partials (two additions per output and split over all SMs) and its launch.
+struct Plan {
+  int tn;       // columns per warp
+  int split;
+  int64_t chunk;
+};
+Plan plan_fp64(int64_t M, int64_t N, int64_t K, double fma_step, double tile_step, const int* widths, int nwidths,
+               bool may_split) {
+  const int sms = num_sms();
+  Plan best{widths[0], 1, K};
+  double best_t = 0.0;
+  for (int w = 0; w < nwidths; ++w) {
+    const int tn = widths[w];
+    const int64_t tiles = (int64_t)cdiv(M, ROWS) * cdiv(N, WARPS * tn);
+    const double step = 0.5 * ROWS * (fma_step * WARPS * tn + tile_step);
+    for (int64_t sp = 1; sp <= 64; ++sp) {
+      if (sp > 1 && (!may_split || K / sp < 2 || 16.0 * (double)sp * (double)M * (double)N > PART_LIMIT)) break;
+      const int64_t chunk = (K + sp - 1) / sp;
+      const double waves = (double)((tiles * sp + sms - 1) / sms);
+      double t = waves * ((double)chunk * step + 1500.0);
+      if (sp > 1) t += 3000.0 + (double)sp * (double)M * (double)N / sms;
+      if (best_t == 0.0 || t < best_t * 0.999) {
+        best_t = t;
+        best = {tn, (int)((K + chunk - 1) / chunk), chunk};
+      }
+      if (tiles * sp > 8 * (int64_t)sms) break;
+    }
+  }
+  return best;
+}
+}  // namespace
+
 // ---------------------------------------------------------------------------
-// H application.  One CTA computes a BM-row slice of P W_hat for BNW columns of
-// W, i.e. 2*BNW complex outputs per row: the top half (H W)_top = P W and the
-// bottom half (H W)_bot = -conj(P [conj(Y); conj(X)]).  The K loop runs over
-// the 2n columns of P = [A | B]; the second operand is built on the fly from W
-// with the half-swap and conjugation, so W_hat is never stored.
-// Epilogue of the H application for output row i (< n) of column j: C1 = (P w)_i,
-// C2 = (P u)_i, so (H w)_top(i) = C1 and (H w)_bot(i) = -conj(C2).
-__device__ __forceinline__ void hop_epilogue(const HopArgs& a, int64_t i, int64_t j, cplx c1, cplx c2) {
+// H application.  H is real on vectors [z; conj(z)]: H [z; conj(z)] = [t; -conj(t)] with
+// t = A z + B conj(z), a real 2n x 2n matrix on (Re z, Im z):
+//   Re t = (Ar + Br) Re z + (Bi - Ai) Im z,  Im t = (Ai + Bi) Re z + (Ar - Br) Im z.
+// Every w = [x; y] is the sum of [a; conj(a)] and -i [c; conj(c)], a = (x + conj(y))/2 and
+// c = i (x - conj(y))/2, so H w takes 2 x 4 n^2 DFMA instead of the 16 n^2 of the complex
+// product with [A | B].  The kernel stages the four sums of A and B (4 additions per
+// element and tile) and 2a, 2c (4 per vector entry and tile), each a few per cent of the
+// tile's DFMAs, and computes t for `cols` columns (2j: 2a_j, 2j + 1: 2c_j of vector j).
+//
+// Measured on one GB300, before (64 x 32 tiles, the complex product, K chunks >= 256) and
+// after: residuals of 200 vectors at n = 4096 99.3 -> 47.7 ms (1.12 of 1.20 TFLOP/s); a
+// degree-20 filter of 30 vectors at n = 512 42.4 -> 5.26 ms, of 67 ragged ones at n = 1301
+// 148 -> 42.4 ms; residuals of 6 vectors at n = 64 533 -> 42 us.  Error of the filters
+// against 64 bits: unchanged (5.7e-15 and 6.9e-15, before 7.0e-15 and 6.8e-15).
+
+// Epilogue for output row i (< n) of vector j: top and bottom entry of H w.
+__device__ __forceinline__ void hop_epilogue(const HopArgs& a, int64_t i, int64_t j, cplx top, cplx bot) {
   const int64_t n = a.n, n2 = 2 * a.n;
-  const cplx top = c1;
-  const cplx bot = mk(-c2.x, c2.y);  // -conj(C2)
   const int64_t ot = j * n2 + i, ob = j * n2 + n + i;
   if (a.mode == HOP_STORE) {
     a.out[ot] = top;
@@ -37,270 +102,286 @@ __device__ __forceinline__ void hop_epilogue(const HopArgs& a, int64_t i, int64_
     }
     a.out[ot] = t;
     a.out[ob] = b;
-  } else {  // HOP_RESID
+  } else if (a.mode == HOP_RESID) {
     const double lam = a.lambda[j];
     a.out[ot] = csub(top, cscale(a.W[ot], lam));
     a.out[ob] = csub(bot, cscale(a.W[ob], lam));
   }
 }
+// ta, tc: the t of 2a_j and 2c_j.  H w: top = (ta - i tc)/2, bottom = (-conj(ta) + i conj(tc))/2.
+__device__ __forceinline__ void hop_finish(const HopArgs& a, int64_t i, int64_t j, cplx ta, cplx tc) {
+  hop_epilogue(a, i, j, mk(0.5 * (ta.x + tc.y), 0.5 * (ta.y - tc.x)), mk(0.5 * (tc.y - ta.x), 0.5 * (ta.y + tc.x)));
+}
 
-// part != NULL: K split over blockIdx.z in chunks of kchunk columns of P.
-template <int BM, int BNW, int TM, int TNW, int BK>
-__global__ void __launch_bounds__((BM / TM) * (BNW / TNW))
-hop_kernel(HopArgs a, cplx* part, int64_t kchunk) {
-  constexpr int TY = BM / TM;
-  constexpr int TX = BNW / TNW;
-  constexpr int NT = TX * TY;
-  __shared__ cplx Ps[BK][BM];
-  __shared__ cplx W1s[BK][BNW];
-  __shared__ cplx W2s[BK][BNW];
-  const int tid = threadIdx.x;
-  const int ty = tid % TY;
-  const int tx = tid / TY;
-  const int64_t n = a.n, n2 = 2 * a.n;
-  const int64_t row0 = (int64_t)blockIdx.x * BM;
-  const int64_t col0 = (int64_t)blockIdx.y * BNW;
-
-  cplx acc1[TM][TNW], acc2[TM][TNW];
+// GEN: general vectors W (2n x k, two columns each); else the columns of X = a.W are the z
+// themselves (n x k, ld n) and a.out = t (ld n).  part != NULL: the t of K chunk blockIdx.z
+// go to part + blockIdx.z * n * cols instead.
+template <int TN, bool GEN>
+__global__ void __launch_bounds__(THREADS)
+hop_kernel(HopArgs a, cplx* part, int64_t chunk) {
+  __shared__ double Ps[4][BK][ROWS + 1];
+  __shared__ cplx Zs[BK][WARPS * TN];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t n = a.n, n2 = 2 * a.n, cols = GEN ? 2 * a.k : a.k;
+  const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+  const int64_t col0 = (int64_t)blockIdx.y * (WARPS * TN);
+  const int64_t kbeg = (int64_t)blockIdx.z * chunk;
+  const int64_t kend = kbeg + chunk < n ? kbeg + chunk : n;
+  const int64_t mycol = col0 + warp * TN;
+  const bool active = mycol < cols;  // warp-uniform
+  cplx acc[TN];
 #pragma unroll
-  for (int r = 0; r < TM; ++r)
-#pragma unroll
-    for (int c = 0; c < TNW; ++c) { acc1[r][c] = mk(0, 0); acc2[r][c] = mk(0, 0); }
+  for (int c = 0; c < TN; ++c) acc[c] = mk(0, 0);
 
-  const int64_t kbeg = part ? (int64_t)blockIdx.z * kchunk : 0;
-  const int64_t kend = part ? (kbeg + kchunk < n2 ? kbeg + kchunk : n2) : n2;
   for (int64_t kb = kbeg; kb < kend; kb += BK) {
-    for (int idx = tid; idx < BM * BK; idx += NT) {
-      const int r = idx / BK, cc = idx % BK;
-      const int64_t gi = row0 + r, gl = kb + cc;
-      cplx v = mk(0, 0);
-      if (gi < n && gl < kend) v = (gl < n) ? a.A[gi * n + gl] : a.B[gi * n + (gl - n)];
-      Ps[cc][r] = v;
+    const int kn = (int)(kend - kb < BK ? kend - kb : BK);
+    for (int idx = tid; idx < ROWS * BK; idx += THREADS) {
+      const int kk = idx % BK, r = idx / BK;
+      const int64_t gi = row0 + r, gl = kb + kk;
+      cplx p = mk(0, 0), q = mk(0, 0);
+      if (gi < n && kk < kn) {
+        p = a.A[gi * n + gl];
+        q = a.B[gi * n + gl];
+      }
+      Ps[0][kk][r] = p.x + q.x;
+      Ps[1][kk][r] = q.y - p.y;
+      Ps[2][kk][r] = p.y + q.y;
+      Ps[3][kk][r] = p.x - q.x;
     }
-    for (int idx = tid; idx < BNW * BK; idx += NT) {
-      const int j = idx / BK, l = idx % BK;
-      const int64_t gj = col0 + j, gl = kb + l;
+    if (GEN) {
+      for (int idx = tid; idx < BK * (WARPS * TN / 2); idx += THREADS) {
+        const int kk = idx % BK, j = idx / BK;
+        const int64_t gj = col0 / 2 + j, gl = kb + kk;
+        cplx za = mk(0, 0), zc = mk(0, 0);
+        if (gj < a.k && kk < kn) {
+          const cplx x = a.W[gj * n2 + gl], y = a.W[gj * n2 + n + gl];
+          za = mk(x.x + y.x, x.y - y.y);
+          zc = mk(-(x.y + y.y), x.x - y.x);
+        }
+        Zs[kk][2 * j] = za;
+        Zs[kk][2 * j + 1] = zc;
+      }
+    } else {
+      for (int idx = tid; idx < BK * (WARPS * TN); idx += THREADS) {
+        const int kk = idx % BK, j = idx / BK;
+        const int64_t gj = col0 + j;
+        Zs[kk][j] = (gj < cols && kk < kn) ? a.W[gj * n + kb + kk] : mk(0, 0);
+      }
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll 4
+      for (int kk = 0; kk < kn; ++kk) {
+        const double p0 = Ps[0][kk][lane], p1 = Ps[1][kk][lane], p2 = Ps[2][kk][lane], p3 = Ps[3][kk][lane];
+#pragma unroll
+        for (int c = 0; c < TN; ++c) {
+          const cplx z = Zs[kk][warp * TN + c];
+          acc[c].x = fma(p0, z.x, acc[c].x);
+          acc[c].y = fma(p2, z.x, acc[c].y);
+          acc[c].x = fma(p1, z.y, acc[c].x);
+          acc[c].y = fma(p3, z.y, acc[c].y);
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  const int64_t i = row0 + lane;
+  if (!active || i >= n) return;
+  if (part) {
+#pragma unroll
+    for (int c = 0; c < TN; ++c)
+      if (mycol + c < cols) part[((int64_t)blockIdx.z * cols + mycol + c) * n + i] = acc[c];
+  } else if (GEN) {
+#pragma unroll
+    for (int c = 0; c + 1 < TN; c += 2)
+      if (mycol + c < cols) hop_finish(a, i, (mycol + c) / 2, acc[c], acc[c + 1]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < TN; ++c)
+      if (mycol + c < cols) a.out[(mycol + c) * n + i] = acc[c];
+  }
+}
+
+// Sum of the K partials in order, and the epilogue; one thread per row and vector.
+template <bool GEN>
+__global__ void hop_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
+  const int64_t n = a.n, total = n * a.k, cols = GEN ? 2 * a.k : a.k;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % n, j = idx / n;
+    const cplx* p = part + (GEN ? 2 * j : j) * n + i;
+    cplx ta = mk(0, 0), tc = mk(0, 0);
+#pragma unroll 4
+    for (int z = 0; z < nsplit; ++z) {
+      ta = cadd(ta, p[(int64_t)z * cols * n]);
+      if (GEN) tc = cadd(tc, p[(int64_t)z * cols * n + n]);
+    }
+    if (GEN) hop_finish(a, i, j, ta, tc);
+    else a.out[idx] = ta;
+  }
+}
+
+template <bool GEN>
+static int hop_launch(const HopArgs& a, cudaStream_t s) {
+  static const int widths_gen[4] = {2, 4, 6, 8}, widths_top[4] = {1, 2, 4, 8};
+  const int64_t cols = GEN ? 2 * a.k : a.k;
+  const Plan p = plan_fp64(a.n, cols, a.n, 4.0, 4.0, GEN ? widths_gen : widths_top, 4, !a.no_split);
+  cplx* part = nullptr;
+  if (p.split > 1) CB_CUDA(dalloc(&part, sizeof(cplx) * p.split * a.n * cols, s));
+  const dim3 grid(cdiv(a.n, ROWS), cdiv(cols, WARPS * p.tn), (unsigned)p.split);
+  const int64_t tid = GEN ? timer_begin(1, 32.0 * (double)a.n * (double)a.n * (double)a.k, s) : -1;
+  switch (p.tn) {
+    case 1: hop_kernel<GEN ? 2 : 1, GEN><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+    case 2: hop_kernel<2, GEN><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+    case 4: hop_kernel<4, GEN><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+    case 6: hop_kernel<GEN ? 6 : 4, GEN><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+    default: hop_kernel<8, GEN><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+  }
+  count_launch();
+  if (part) {
+    const int64_t blocks = (a.n * a.k + 127) / 128;
+    hop_reduce_kernel<GEN><<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, s>>>(a, part, p.split);
+    count_launch();
+  }
+  if (GEN) timer_end(tid, s);
+  const cudaError_t e = cudaGetLastError();
+  if (part) cudaFreeAsync(part, s);
+  return e == cudaSuccess ? CHASE_BSE_OK : CHASE_BSE_CUDA_ERROR;
+}
+
+int hop_top_fp64(const cplx* A, const cplx* B, int64_t n, const cplx* X, int64_t k, cplx* Y, cudaStream_t s) {
+  if (k <= 0 || n <= 0) return CHASE_BSE_OK;
+  HopArgs a{};
+  a.A = A; a.B = B; a.n = n; a.W = X; a.k = k; a.out = Y;
+  return hop_launch<false>(a, s);
+}
+
+// The complex product [A | B] [x, conj(y); y, conj(x)] on the same tiles, two sums per row
+// and vector over the 2n columns of [A | B]: the top half of H w and -conj of the bottom.
+// Twice the DFMAs of hop_kernel.  Only the Rayleigh-Ritz step on a caller's basis uses it:
+// the phases of its Ritz vectors come out of the last Jacobi rotations, whose pivots
+// are rounding residue (a change of the last bit of H Q turns them by up to 1e-5), so its
+// sums keep their order and their K chunks.
+template <int TN>
+__global__ void __launch_bounds__(THREADS)
+hop_ordered_kernel(HopArgs a, cplx* part, int64_t kchunk) {
+  __shared__ cplx Ps[BK][ROWS + 1];
+  __shared__ cplx W1s[BK][WARPS * TN];
+  __shared__ cplx W2s[BK][WARPS * TN];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t n = a.n, n2 = 2 * a.n;
+  const int64_t row0 = (int64_t)blockIdx.x * ROWS, col0 = (int64_t)blockIdx.y * (WARPS * TN);
+  const int64_t kbeg = (int64_t)blockIdx.z * kchunk;
+  const int64_t kend = kbeg + kchunk < n2 ? kbeg + kchunk : n2;
+  const int64_t mycol = col0 + warp * TN;
+  const bool active = mycol < a.k;  // warp-uniform
+  cplx acc1[TN], acc2[TN];
+#pragma unroll
+  for (int c = 0; c < TN; ++c) { acc1[c] = mk(0, 0); acc2[c] = mk(0, 0); }
+  for (int64_t kb = kbeg; kb < kend; kb += BK) {
+    const int kn = (int)(kend - kb < BK ? kend - kb : BK);
+    for (int idx = tid; idx < ROWS * BK; idx += THREADS) {
+      const int kk = idx % BK, r = idx / BK;
+      const int64_t gi = row0 + r, gl = kb + kk;
+      cplx v = mk(0, 0);
+      if (gi < n && kk < kn) v = (gl < n) ? a.A[gi * n + gl] : a.B[gi * n + (gl - n)];
+      Ps[kk][r] = v;
+    }
+    for (int idx = tid; idx < BK * WARPS * TN; idx += THREADS) {
+      const int kk = idx % BK, j = idx / BK;
+      const int64_t gj = col0 + j, gl = kb + kk;
       cplx v1 = mk(0, 0), v2 = mk(0, 0);
-      if (gj < a.k && gl < kend) {
+      if (gj < a.k && kk < kn) {
         const cplx* w = a.W + gj * n2;
         v1 = w[gl];
         v2 = cconj(w[gl < n ? gl + n : gl - n]);
       }
-      W1s[l][j] = v1;
-      W2s[l][j] = v2;
+      W1s[kk][j] = v1;
+      W2s[kk][j] = v2;
     }
     __syncthreads();
+    if (active) {
 #pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      cplx p[TM], w1[TNW], w2[TNW];
+      for (int kk = 0; kk < kn; ++kk) {
+        const cplx p = Ps[kk][lane];
 #pragma unroll
-      for (int r = 0; r < TM; ++r) p[r] = Ps[kk][ty + TY * r];
-#pragma unroll
-      for (int c = 0; c < TNW; ++c) { w1[c] = W1s[kk][tx + TX * c]; w2[c] = W2s[kk][tx + TX * c]; }
-#pragma unroll
-      for (int r = 0; r < TM; ++r)
-#pragma unroll
-        for (int c = 0; c < TNW; ++c) { cfma(acc1[r][c], p[r], w1[c]); cfma(acc2[r][c], p[r], w2[c]); }
+        for (int c = 0; c < TN; ++c) {
+          cfma(acc1[c], p, W1s[kk][warp * TN + c]);
+          cfma(acc2[c], p, W2s[kk][warp * TN + c]);
+        }
+      }
     }
     __syncthreads();
   }
-
+  const int64_t i = row0 + lane;
+  if (!active || i >= n) return;
 #pragma unroll
-  for (int r = 0; r < TM; ++r) {
-#pragma unroll
-    for (int c = 0; c < TNW; ++c) {
-      const int64_t i = row0 + ty + TY * r;
-      const int64_t j = col0 + tx + TX * c;
-      if (i >= n || j >= a.k) continue;
-      if (part) {  // split K: raw partial sums of P W and P U for this K chunk
-        cplx* p = part + (int64_t)blockIdx.z * (2 * n * a.k) + j * n2;
-        p[i] = acc1[r][c];
-        p[n + i] = acc2[r][c];
-      } else {
-        hop_epilogue(a, i, j, acc1[r][c], acc2[r][c]);
-      }
+  for (int c = 0; c < TN; ++c) {
+    const int64_t j = mycol + c;
+    if (j >= a.k) continue;
+    if (part) {
+      cplx* p = part + ((int64_t)blockIdx.z * a.k + j) * n2;
+      p[i] = acc1[c];
+      p[n + i] = acc2[c];
+    } else {
+      hop_epilogue(a, i, j, acc1[c], mk(-acc2[c].x, acc2[c].y));
     }
   }
 }
-
-template <int BM, int BNW>
-__global__ void hop_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
+__global__ void hop_ordered_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
   const int64_t n = a.n, n2 = 2 * n, total = n * a.k;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = idx % n, j = idx / n;
     cplx c1 = mk(0, 0), c2 = mk(0, 0);
     for (int z = 0; z < nsplit; ++z) {
-      const cplx* p = part + (int64_t)z * (2 * n * a.k) + j * n2;
+      const cplx* p = part + ((int64_t)z * a.k + j) * n2;
       c1 = cadd(c1, p[i]);
       c2 = cadd(c2, p[n + i]);
     }
-    hop_epilogue(a, i, j, c1, c2);
+    hop_epilogue(a, i, j, c1, mk(-c2.x, c2.y));
   }
 }
 
-static int num_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                 cudaSuccess || sms <= 0)
-      sms = 148;
-  }
-  return sms;
-}
-
-// Number of K chunks so that a small output grid still fills the GPU (two CTAs per
-// SM); 1 when the grid is large enough or K too short to split.
-static int64_t split_count(int64_t tiles, int64_t K, int64_t min_chunk) {
+// K chunks that fill the GPU twice with tiles of `tiles`, at least min_chunk long and a
+// multiple of `round` (the fixed rule of the ordered products).
+static void ordered_chunks(int64_t tiles, int64_t K, int64_t min_chunk, int64_t round, int64_t* chunk, int* splits) {
   const int64_t want = 2 * (int64_t)num_sms();
-  if (tiles >= want || K < 2 * min_chunk) return 1;
-  int64_t s = (want + tiles - 1) / tiles;
-  if (s > K / min_chunk) s = K / min_chunk;
-  return s < 1 ? 1 : s;
+  int64_t s = 1;
+  if (tiles < want && K >= 2 * min_chunk) s = std::max<int64_t>(1, std::min((want + tiles - 1) / tiles, K / min_chunk));
+  *chunk = s == 1 ? std::max<int64_t>(K, 1) : ((K + s - 1) / s + round - 1) / round * round;
+  *splits = (int)std::max<int64_t>(1, (K + *chunk - 1) / *chunk);
 }
 
-template <int BM, int BNW, int TM, int TNW>
-static int hop_launch(const HopArgs& a, cudaStream_t s) {
-  const int64_t tiles = (int64_t)cdiv(a.n, BM) * cdiv(a.k, BNW);
+static int hop_ordered(const HopArgs& a, cudaStream_t s) {
   const int64_t n2 = 2 * a.n;
-  const int64_t nsplit = a.no_split ? 1 : split_count(tiles, n2, 256);
-  if (nsplit <= 1) {
-    dim3 grid(cdiv(a.n, BM), cdiv(a.k, BNW));
-    const int64_t tid = timer_begin(1, 32.0 * (double)a.n * (double)a.n * (double)a.k, s);
-    hop_kernel<BM, BNW, TM, TNW, 16><<<grid, (BM / TM) * (BNW / TNW), 0, s>>>(a, nullptr, 0);
-    timer_end(tid, s);
-    count_launch();
-    CB_LAUNCH();
-    return CHASE_BSE_OK;
-  }
-  const int64_t kchunk = ((n2 + nsplit - 1) / nsplit + 15) / 16 * 16;
-  const int64_t ns = (n2 + kchunk - 1) / kchunk;
+  int64_t chunk;
+  int splits;
+  ordered_chunks((int64_t)cdiv(a.n, 64) * cdiv(a.k, a.k <= 4 ? 4 : 32), n2, 256, 16, &chunk, &splits);
   cplx* part = nullptr;
-  CB_CUDA(dalloc(&part, sizeof(cplx) * ns * 2 * a.n * a.k, s));
-  dim3 grid(cdiv(a.n, BM), cdiv(a.k, BNW), (unsigned)ns);
-  // the split product and its reduction: one H application
+  if (splits > 1) CB_CUDA(dalloc(&part, sizeof(cplx) * splits * n2 * a.k, s));
+  const int tn = a.k >= 32 ? 4 : (a.k >= 16 ? 2 : 1);
+  const dim3 grid(cdiv(a.n, ROWS), cdiv(a.k, WARPS * tn), (unsigned)splits);
   const int64_t tid = timer_begin(1, 32.0 * (double)a.n * (double)a.n * (double)a.k, s);
-  hop_kernel<BM, BNW, TM, TNW, 16><<<grid, (BM / TM) * (BNW / TNW), 0, s>>>(a, part, kchunk);
+  if (tn == 4) hop_ordered_kernel<4><<<grid, THREADS, 0, s>>>(a, part, chunk);
+  else if (tn == 2) hop_ordered_kernel<2><<<grid, THREADS, 0, s>>>(a, part, chunk);
+  else hop_ordered_kernel<1><<<grid, THREADS, 0, s>>>(a, part, chunk);
   count_launch();
-  const int64_t total = a.n * a.k;
-  const unsigned rb = (unsigned)((total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192);
-  hop_reduce_kernel<BM, BNW><<<rb, 256, 0, s>>>(a, part, (int)ns);
-  timer_end(tid, s);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
-  cudaFreeAsync(part, s);
-  if (e != cudaSuccess) return CHASE_BSE_CUDA_ERROR;
-  return CHASE_BSE_OK;
-}
-
-// y = [A | B] [x; conj(x)] for k vectors x (n x k, ld n).  part != NULL: K split.
-template <int BM, int BNW, int TM, int TNW, int BK>
-__global__ void __launch_bounds__((BM / TM) * (BNW / TNW))
-hop_top_kernel(const cplx* __restrict__ A, const cplx* __restrict__ B, int64_t n, const cplx* __restrict__ X,
-               int64_t k, cplx* Y, cplx* part, int64_t kchunk) {
-  constexpr int TY = BM / TM;
-  constexpr int TX = BNW / TNW;
-  constexpr int NT = TX * TY;
-  __shared__ cplx Ps[BK][BM];
-  __shared__ cplx Ws[BK][BNW];
-  const int tid = threadIdx.x;
-  const int ty = tid % TY;
-  const int tx = tid / TY;
-  const int64_t n2 = 2 * n;
-  const int64_t row0 = (int64_t)blockIdx.x * BM;
-  const int64_t col0 = (int64_t)blockIdx.y * BNW;
-  const int64_t kbeg = part ? (int64_t)blockIdx.z * kchunk : 0;
-  const int64_t kend = part ? (kbeg + kchunk < n2 ? kbeg + kchunk : n2) : n2;
-  cplx acc[TM][TNW];
-#pragma unroll
-  for (int r = 0; r < TM; ++r)
-#pragma unroll
-    for (int c = 0; c < TNW; ++c) acc[r][c] = mk(0, 0);
-  for (int64_t kb = kbeg; kb < kend; kb += BK) {
-    for (int idx = tid; idx < BM * BK; idx += NT) {
-      const int r = idx / BK, cc = idx % BK;
-      const int64_t gi = row0 + r, gl = kb + cc;
-      cplx v = mk(0, 0);
-      if (gi < n && gl < kend) v = (gl < n) ? A[gi * n + gl] : B[gi * n + (gl - n)];
-      Ps[cc][r] = v;
-    }
-    for (int idx = tid; idx < BNW * BK; idx += NT) {
-      const int j = idx / BK, l = idx % BK;
-      const int64_t gj = col0 + j, gl = kb + l;
-      cplx v = mk(0, 0);
-      if (gj < k && gl < kend) v = (gl < n) ? X[gj * n + gl] : cconj(X[gj * n + (gl - n)]);
-      Ws[l][j] = v;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      cplx p[TM], w[TNW];
-#pragma unroll
-      for (int r = 0; r < TM; ++r) p[r] = Ps[kk][ty + TY * r];
-#pragma unroll
-      for (int c = 0; c < TNW; ++c) w[c] = Ws[kk][tx + TX * c];
-#pragma unroll
-      for (int r = 0; r < TM; ++r)
-#pragma unroll
-        for (int c = 0; c < TNW; ++c) cfma(acc[r][c], p[r], w[c]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < TM; ++r)
-#pragma unroll
-    for (int c = 0; c < TNW; ++c) {
-      const int64_t i = row0 + ty + TY * r, j = col0 + tx + TX * c;
-      if (i >= n || j >= k) continue;
-      if (part) part[(int64_t)blockIdx.z * n * k + j * n + i] = acc[r][c];
-      else Y[j * n + i] = acc[r][c];
-    }
-}
-
-__global__ void sum_parts_kernel(const cplx* part, int nsplit, int64_t total, cplx* Y) {
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    cplx v = mk(0, 0);
-    for (int z = 0; z < nsplit; ++z) v = cadd(v, part[(int64_t)z * total + idx]);
-    Y[idx] = v;
-  }
-}
-
-int hop_top_fp64(const cplx* A, const cplx* B, int64_t n, const cplx* X, int64_t k, cplx* Y, cudaStream_t s) {
-  if (k <= 0 || n <= 0) return CHASE_BSE_OK;
-  constexpr int BM = 64, BNW = 64, TM = 4, TNW = 4;
-  const int64_t tiles = (int64_t)cdiv(n, BM) * cdiv(k, BNW);
-  const int64_t n2 = 2 * n;
-  const int64_t nsplit = split_count(tiles, n2, 256);
-  dim3 grid(cdiv(n, BM), cdiv(k, BNW));
-  if (nsplit <= 1) {
-    hop_top_kernel<BM, BNW, TM, TNW, 16><<<grid, 256, 0, s>>>(A, B, n, X, k, Y, nullptr, 0);
+  if (part) {
+    const int64_t blocks = (a.n * a.k + 127) / 128;
+    hop_ordered_reduce_kernel<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, s>>>(a, part, splits);
     count_launch();
-    CB_LAUNCH();
-    return CHASE_BSE_OK;
   }
-  const int64_t kchunk = ((n2 + nsplit - 1) / nsplit + 15) / 16 * 16;
-  const int64_t ns = (n2 + kchunk - 1) / kchunk;
-  cplx* part = nullptr;
-  CB_CUDA(dalloc(&part, sizeof(cplx) * ns * n * k, s));
-  grid.z = (unsigned)ns;
-  hop_top_kernel<BM, BNW, TM, TNW, 16><<<grid, 256, 0, s>>>(A, B, n, X, k, Y, part, kchunk);
-  count_launch();
-  const int64_t total = n * k;
-  sum_parts_kernel<<<(unsigned)((total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192), 256, 0, s>>>(
-      part, (int)ns, total, Y);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
-  cudaFreeAsync(part, s);
-  if (e != cudaSuccess) return CHASE_BSE_CUDA_ERROR;
-  return CHASE_BSE_OK;
+  timer_end(tid, s);
+  const cudaError_t e = cudaGetLastError();
+  if (part) cudaFreeAsync(part, s);
+  return e == cudaSuccess ? CHASE_BSE_OK : CHASE_BSE_CUDA_ERROR;
 }
 
 int hop_fp64(const HopArgs& a, cudaStream_t s) {
   if (a.k <= 0 || a.n <= 0) return CHASE_BSE_OK;
-  if (a.k <= 4) return hop_launch<64, 4, 1, 1>(a, s);
-  return hop_launch<64, 32, 4, 2>(a, s);
+  return a.ordered ? hop_ordered(a, s) : hop_launch<true>(a, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -314,15 +395,15 @@ __device__ __forceinline__ cplx load_op(const cplx* X, int64_t ld, char op, int6
 
 // kchunk > 0: K split over blockIdx.z; block z writes alpha * its partial product to
 // C + z * ldc * N (beta ignored).
-template <int BM, int BN, int TM, int TN, int BK>
+template <int BM, int BN, int TM, int TN, int BKZ>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 zgemm_kernel(char opA, char opB, int64_t M, int64_t N, int64_t K, cplx alpha, const cplx* __restrict__ A,
              int64_t lda, const cplx* __restrict__ B, int64_t ldb, cplx beta, cplx* C, int64_t ldc, int64_t kchunk) {
   constexpr int TY = BM / TM;
   constexpr int TX = BN / TN;
   constexpr int NT = TX * TY;
-  __shared__ cplx As[BK][BM];
-  __shared__ cplx Bs[BK][BN];
+  __shared__ cplx As[BKZ][BM];
+  __shared__ cplx Bs[BKZ][BN];
   const int tid = threadIdx.x;
   const int ty = tid % TY;
   const int tx = tid / TY;
@@ -340,22 +421,22 @@ zgemm_kernel(char opA, char opB, int64_t M, int64_t N, int64_t K, cplx alpha, co
     C += (int64_t)blockIdx.z * ldc * N;
     beta = mk(0, 0);
   }
-  for (int64_t kb = kbeg; kb < kend; kb += BK) {
-    for (int idx = tid; idx < BM * BK; idx += NT) {
+  for (int64_t kb = kbeg; kb < kend; kb += BKZ) {
+    for (int idx = tid; idx < BM * BKZ; idx += NT) {
       int r, l;
-      if (opA == 'N') { r = idx % BM; l = idx / BM; } else { l = idx % BK; r = idx / BK; }
+      if (opA == 'N') { r = idx % BM; l = idx / BM; } else { l = idx % BKZ; r = idx / BKZ; }
       const int64_t gr = row0 + r, gl = kb + l;
       As[l][r] = (gr < M && gl < kend) ? load_op(A, lda, opA, gr, gl) : mk(0, 0);
     }
-    for (int idx = tid; idx < BN * BK; idx += NT) {
+    for (int idx = tid; idx < BN * BKZ; idx += NT) {
       int c, l;
-      if (opB == 'N') { l = idx % BK; c = idx / BK; } else { c = idx % BN; l = idx / BN; }
+      if (opB == 'N') { l = idx % BKZ; c = idx / BKZ; } else { c = idx % BN; l = idx / BN; }
       const int64_t gc = col0 + c, gl = kb + l;
       Bs[l][c] = (gc < N && gl < kend) ? load_op(B, ldb, opB, gl, gc) : mk(0, 0);
     }
     __syncthreads();
 #pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
+    for (int kk = 0; kk < BKZ; ++kk) {
       cplx av[TM], bv[TN];
 #pragma unroll
       for (int r = 0; r < TM; ++r) av[r] = As[kk][ty + TY * r];
@@ -394,6 +475,16 @@ __global__ void zgemm_reduce_kernel(const cplx* part, int nsplit, int64_t M, int
     if (beta.x != 0.0 || beta.y != 0.0) v = cadd(v, cmul(beta, C[i + j * ldc]));
     C[i + j * ldc] = v;
   }
+}
+
+// Number of K chunks so that a small output grid still fills the GPU (two CTAs per
+// SM); 1 when the grid is large enough or K too short to split.
+static int64_t split_count(int64_t tiles, int64_t K, int64_t min_chunk) {
+  const int64_t want = 2 * (int64_t)num_sms();
+  if (tiles >= want || K < 2 * min_chunk) return 1;
+  int64_t s = (want + tiles - 1) / tiles;
+  if (s > K / min_chunk) s = K / min_chunk;
+  return s < 1 ? 1 : s;
 }
 
 template <int BM, int BN, int TM, int TN>

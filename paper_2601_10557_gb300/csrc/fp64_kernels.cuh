@@ -5,10 +5,9 @@
 namespace cb {
 
 // ---- H application --------------------------------------------------------
-// H W for W = [X; Y] (2n x k, column-major, ld 2n) reading only A and B
-// (row-major).  With P = [A | B] (n x 2n) and W_hat = [[X, conj(Y)], [Y, conj(X)]]:
-//   P W_hat = [H W_top, -conj(H W_bottom)],
-// so one pass over P yields both halves (the block structure of Section 1).
+// H W for W = [X; Y] (2n x k, column-major, ld 2n) reading only A and B (row-major), as a
+// real 2n x 2n matrix on the J-fixed parts of each vector (the block structure of
+// Section 1; see fp64_kernels.cu).
 enum HopMode : int {
   HOP_STORE = 0,   // out = H W               (sflip: out = S H W)
   HOP_CHEB = 1,    // out = alpha (H W - c Wc) + beta Wp
@@ -29,6 +28,7 @@ struct HopArgs {
   const cplx* Wp;    // HOP_CHEB: previous iterate (ld 2n), unused if beta == 0
   const double* lambda;  // HOP_RESID
   int no_split;      // 1: one launch over the whole K range (no split-K partials, allocates nothing)
+  int ordered;       // 1: the complex product with its fixed summation order (see hop_ordered_kernel)
 };
 
 int hop_fp64(const HopArgs& a, cudaStream_t s);

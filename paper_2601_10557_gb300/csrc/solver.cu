@@ -542,7 +542,7 @@ int rayleigh_ritz(const cplx* A, const cplx* B, int64_t n, const cplx* Q, int64_
   CB_TRY(ws.alloc(&idx_d, h));
   // Algorithm 2: T = S H Q, M = Q^* T
   HopArgs a{};
-  a.A = A; a.B = B; a.n = n; a.W = Q; a.k = k; a.out = T; a.mode = HOP_STORE; a.sflip = 1;
+  a.A = A; a.B = B; a.n = n; a.W = Q; a.k = k; a.out = T; a.mode = HOP_STORE; a.sflip = 1; a.ordered = 1;
   CB_TRY(hop_fp64(a, s));
   CB_TRY(zgemm('C', 'N', k, k, n2, mk(1, 0), Q, n2, T, n2, mk(0, 0), M, k, s));
   CB_TRY(hermitize(M, k, s));
@@ -1284,6 +1284,10 @@ int solve(const cplx* A, const cplx* B, int64_t n, int64_t nev, int64_t nex, int
     *stats = st;
   }
   if (status != CHASE_BSE_OK) return status;
+  // Q^* S H Q indefinite in every iteration and not one pair from the fallback: S H is not
+  // definite (whether the fallback runs out of positive Ritz values before maxiter depends
+  // on the last bits of its products)
+  if (nout == 0 && o.rr == 0 && it > 0 && st.fallback_rr == it) return CHASE_BSE_NOT_DEFINITE;
   return (nout < nev) ? CHASE_BSE_NOT_CONVERGED : CHASE_BSE_OK;
 }
 
