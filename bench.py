@@ -477,8 +477,10 @@ def main():
     e2e_val = whole_job_tflops(dist, efl, e2e_ms, dev)
     del hA, hB, out_gA, out_gB
 
-    # ---- roofline of the dominant kernel, the filter GEMM: the algorithmic flops of its
-    # launches in the timed steps (32 n^2 k for k vectors) over their summed device time
+    # ---- roofline of the dominant kernel, the filter GEMM: the operations its launches in
+    # the timed steps execute (16 n^2 k for k vectors: H as a real 2n x 2n matrix on two real
+    # columns per vector, half of the 32 n^2 k of the complex form that `value` and the
+    # library's record count) over their summed device time
     # (a CUDA event pair around each launch, recorded by the library on the launch's
     # stream).  Cross-check on full-width launches: two filter calls over all nev + nex
     # columns that differ only in the degree (d1 and d2 H^2 steps: 2 (d2 - d1) more
@@ -504,9 +506,10 @@ def main():
     rl = (pkg.launch_count() - rl0) // 4
     gemm_launches = 2 * (d2 - d1)
     full_launch_ms = (t2 - t1) / gemm_launches
-    full_flops = 32.0 * n * n * nevex
+    full_flops = 16.0 * n * n * nevex
     full_achieved = full_flops / (full_launch_ms / 1e3) / 1e12
     per_launch_ms = g_ms / max(g_n, 1)
+    g_flops *= 0.5
     flops_per_launch = g_flops / max(g_n, 1)
     achieved = g_flops / (g_ms / 1e3) / 1e12 if g_ms > 0 else 0.0
     # launches timed inside steps of several seconds or more (the sustained peak was
@@ -541,7 +544,7 @@ def main():
             "kernel": "hop_kernel (FP64 DFMA)" if precision == "fp64" else "tc_hop_kernel (tcgen05 filter GEMM)",
             "peak_source": peak_note, "launch_ms": per_launch_ms, "launches": g_n,
             "flops_per_launch": flops_per_launch,
-            "method": "sum of 32 n^2 k over the filter GEMM launches of the timed steps / their summed "
+            "method": "sum of 16 n^2 k over the filter GEMM launches of the timed steps / their summed "
                       "device time (a CUDA event pair around each launch on its stream)",
             "full_width_check": {
                 "achieved": full_achieved, "frac": full_achieved / peak_burst, "peak": peak_burst,

@@ -1,13 +1,16 @@
 // Mixed-precision Chebyshev filter on H^2 with tcgen05 tensor cores (sm_103a).
 //
-// One application of H is one real GEMM on 5th-generation tensor cores:
-//   C (n x 4k, FP32 in TMEM) = Pr (n x 4n) * Bop^T,   Bop: 4k x 4n,
-// where Pr holds the rows of P = [A | B] with re/im interleaved along K, and
-// every input vector w_j (2n complex) contributes four K-major rows of Bop:
-//   4j+0: (Re w, -Im w)   4j+1: (Im w, Re w)            -> P w
-//   4j+2: (Re u, -Im u)   4j+3: (Im u, Re u),  u = [conj(w_bot); conj(w_top)] -> P u
-// so that (H w)_top = P w and (H w)_bot = -conj(P u) land in four adjacent
-// accumulator columns of the same TMEM lane (row i of the tile).
+// A vector w = [x; y] is the sum [a; conj a] - i [c; conj c] of two vectors fixed by
+// J = K conj, a = (x + conj y) / 2 and c = i (x - conj y) / 2, and H maps
+// [z; conj z] to i [z'; conj z'] with z' = -i (A z + B conj z), a real-linear map of the
+// real 2n-vector (Re z, Im z):
+//   M = [[Ai + Bi, Ar - Br], [-(Ar + Br), Ai - Bi]]   (2n x 2n),   H^2: z -> -M M z.
+// So the whole recurrence runs on two real columns per vector, and one application of H is
+// one real GEMM on 5th-generation tensor cores,
+//   C (2n x 2k, FP32 in TMEM) = M (2n x 2n) * Z (2n x 2k),
+// 16 n^2 k operations, half of [A | B] against the vectors [[x, conj y], [y, conj x]]
+// (n x 4n times 4n x 4k), and a quarter of that form's operand bytes to write per step.
+// Rows of M and entries of a column are interleaved: 2i is Re, 2i + 1 is Im.
 //
 // Split products on 16-bit tensor cores: an operand x is written as a sum of
 // pieces x = x0 + x1 (+ x2), x0 = rn(x), x1 = rn(x - x0), ..., and the product
@@ -16,28 +19,33 @@
 //   BF16x3: 2 BF16 pieces each (8 + 8 bits), same products             (~2^-16)
 //   BF16x6: 3 BF16 pieces each, adds x0 y2 + x1 y1 + x2 y0             (~2^-24)
 // (FP16 pieces of this kind: Ootomo and Yokota, Int. J. HPC Appl. 2022.)  FP16 has
-// a 5-bit exponent, so every operand row is scaled by a power of two: row r of P
-// by 2^prow[r] (its largest entry in [2^12, 2^13)), vector v by 2^vexp[v], chosen
+// a 5-bit exponent, so every operand row is scaled by a power of two: row r of M
+// by 2^prow[r] (its largest entry in [2^12, 2^13)), column v by 2^vexp[v], chosen
 // from an upper bound of its entries below 2^13: the bound of an output of H is
 // L * max|input| with L the largest absolute row sum of P, and that of the
 // recurrence combines the maxima of its terms; every epilogue records the true
-// maximum of each output vector (one atomic max per warp and vector) for the
+// maximum of each output column (one atomic max per warp and column) for the
 // next bound.  The epilogue divides the accumulator by 2^(prow + vexp).  Entries
 // far below the bound only lose precision relative to the bound, which keeps the
 // product's error below that of an FP32 GEMM (|dy| <~ 2^-22 L max|w|).  The
 // BF16 schemes use the same scaling (harmless: BF16 has FP32's exponent range).
 //
-// Kernel structure (one K range of one 128 x 128 output tile per CTA, 384 threads):
-//   warp 0   TMA producer: the A pieces and the B pieces of 64 K-elements (128B
-//            swizzle) into a 3-stage (two pieces) or 2-stage (three pieces)
-//            shared-memory ring
-//   warp 1   allocates all 512 TMEM columns (two alternating x0*y0 buffers and two
-//            for the cross products); one lane issues the tcgen05.mma of a K block
-//   warps 4-11 drain the partial sums of every FLUSH K blocks (tcgen05.ld) into FP32
-//            registers while the next group accumulates in the other buffer,
-//            because the tensor core's FP32 accumulation truncates; then (with a K
-//            split) write a partial tile, the last writer of a tile summing them,
-//            and either
+// Kernel structure: persistent CTA pairs (cta_group::2, one pair per two SMs, 512 threads
+// a CTA), each working through 256 x BN output tiles (BN <= 256, chosen per launch); CTA r
+// of a pair holds rows 128 r .. 128 r + 127 of the tile, its A rows and half of the B rows.
+//   warp 0   TMA producer: the A pieces and the B half's pieces of 64 K-elements (128B
+//            swizzle) into the shared-memory ring; both CTAs' bytes count on CTA 0's barrier
+//   warp 1   allocates all 512 TMEM columns (x0*y0 and the cross products); one lane
+//            of CTA 0 issues the tcgen05.mma of a K block, x0*y0 first
+//   warps 4-11 drain x0*y0 after every FLUSH K blocks (tcgen05.ld) into FP32 registers,
+//            because the tensor core's FP32 accumulation truncates, while the block's
+//            cross products (2/3 of its MMA time) run (and, in tiles of up to 160 columns,
+//            the next blocks' x0*y0 in a second buffer); at the end of a tile they add the
+//            cross products, write the FP32 tile to a workspace that stays in L2 and go on
+//            to the next tile
+//   warps 12-15 finish a tile behind the next one's MMAs (the drain warps help with a pair's
+//            last tile, and where several pairs hold K ranges of a tile the last writer sums
+//            them): either
 //            (mode 0) store the next GEMM's B-operand pieces, or
 //            (mode 1) the fused three-term recurrence in FP32 plus the pieces, or
 //            (mode 2) Z = H X + gamma_col * X (no pieces).
@@ -62,13 +70,14 @@ namespace cb {
 namespace tc {
 
 constexpr int BM = 128;
-constexpr int KPAD = 64;              // K (4n) is padded to a multiple of this
-constexpr uint32_t TMEM_COLS = 512;   // two accumulator buffers (+ the cross products for 128-wide tiles)
+constexpr int KPAD = 64;              // K (2n) is padded to a multiple of this
+constexpr int BNMAX = 256;            // widest output tile
+constexpr uint32_t TMEM_COLS = 512;   // one or two x0*y0 buffers and the cross products
 constexpr int VEXP_MAX = 100;         // |operand exponents| are clamped to this
-// instruction descriptor, kind::f16: D = F32, A = B = BF16 (bf16) or FP16, both K-major, 128 x n
+// instruction descriptor, kind::f16: D = F32, A = B = BF16 (bf16) or FP16, both K-major, 256 x n
 __device__ __forceinline__ uint32_t make_idesc(int n, bool bf16) {
   return (1u << 4) | (bf16 ? ((1u << 7) | (1u << 10)) : 0u) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(BM >> 4) << 24);
+         ((uint32_t)(2 * BM >> 4) << 24);
 }
 
 // 16-bit piece types
@@ -98,79 +107,77 @@ struct Scheme;
 template <>
 struct Scheme<SCH_BF16X3> {
   using T = __nv_bfloat16;
-  // FLUSH: K blocks per drained partial sum of x0 * y0 (16 truncating MMA additions
-  // stay far below the 2^-16 error of the BF16 pieces; measured unchanged from 8)
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3, STAGES = 3, FLUSH = 4;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_FP16X3> {
   using T = __half;
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3, STAGES = 3, FLUSH = 4;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_BF16X6> {
   using T = __nv_bfloat16;
-  static constexpr int NPA = 3, NPW = 3, NPROD = 6, STAGES = 2, FLUSH = 2;
+  static constexpr int NPA = 3, NPW = 3, NPROD = 6;
   // (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : (i == 4 ? 1 : (i == 5 ? 2 : 0)); }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : (i == 3 ? 2 : (i == 4 ? 1 : 0)); }
 };
-// Tile geometry for BNT-wide output tiles.  128-wide: K blocks of 64 (128-byte swizzle);
-// the x0 * y0 product drains from two alternating TMEM buffers and the cross products
-// accumulate over all of K in two more (odd-numbered products in one, even in the other:
-// no two consecutive MMAs of a K step then write the same accumulator, 3-6 % faster than
-// a single cross buffer behind three rotating x0 * y0 buffers); 8 drain warps of 64 columns (two per TMEM lane
-// quarter: half the drain latency of 4 warps of 128 columns, and 135 registers a thread
-// instead of 228).  256-wide (two pieces only): K blocks of 32 (64-byte swizzle) in a
-// 4-stage ring of 48 KB stages; each SM takes in 48 KB per 768 MMA cycles instead of
-// 64 KB (the shared-memory fill per MMA cycle bounds the 128-wide tiles); all products
-// share the two alternating buffers, drained after every K block, and each block issues
-// its cross products (2^-11 of the result) before x0 * y0, so the truncating
-// accumulator adds only two MMAs at full magnitude per drain (as the 128-wide x0 * y0
-// buffer per 32 K elements); 16 drain warps of 64 columns keep the FP32 partial sums in
-// registers.
-template <int SCH, int BNT, int FL>
-struct Geo {
-  static constexpr int BK = (BNT == 256) ? 32 : 64;
-  static constexpr int SWZ = BK * 2;                       // swizzle span (bytes) = one row of a tile
-  static constexpr int STAGES = (BNT == 256) ? 4 : Scheme<SCH>::STAGES;
-  static constexpr int FLUSH = FL;
-  static constexpr bool CROSS = (BNT == 128);             // separate cross-product buffers
-  static constexpr int NB = 2;                             // alternating x0 * y0 (or all-product) buffers
-  static constexpr int NCROSS = CROSS ? 2 : 0;             // cross-product buffers
-  static constexpr int A_BYTES = BM * BK * 2;
-  static constexpr int B_BYTES = BNT * BK * 2;
-  static constexpr int STAGE_BYTES = Scheme<SCH>::NPA * A_BYTES + Scheme<SCH>::NPW * B_BYTES;
-  static constexpr int NBAR = 2 * STAGES + 2 * NB + 1;  // full, empty, acc_full[NB], acc_empty[NB], done
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-  static constexpr int DCOLS = 64;                         // columns per drain warp
-  static constexpr int DRAIN_WARPS = 4 * (BNT / DCOLS);
-  static constexpr int THREADS = 128 + 32 * DRAIN_WARPS;
-  static_assert(STAGE_BYTES * STAGES + 1280 <= 232448, "shared memory");
-  static_assert((NB + NCROSS) * BNT <= (int)TMEM_COLS, "TMEM columns");
-};
+// Geometry.  A K block is 64 K-elements (128-byte swizzle); a stage of the ring holds the
+// pieces of 128 A rows and of BN / 2 B rows, so a pair takes in 64 KB per CTA and 1536 MMA
+// cycles at BN = 256 where one CTA per 128 x 128 tile takes 64 KB per 768: shared-memory
+// traffic (operand reads of the MMAs plus the fill) bounds the smaller tile.  Of x0 * y0
+// 16 truncating MMA additions go into a drained sum, as many as the 22-bit pieces' error
+// allows; 8 cost 2-8 %.  K blocks of 32 in twice the stages lost 10-25 % (64-byte rows).
+//
+// Measured on one GB300, FP16x3, time of one launch of a degree's two, before (one CTA per
+// 128 x 128 tile, [A | B] against four columns per vector) and after: n = 16384, k = 1300
+// 28.0 -> 11.6 ms (three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained);
+// n = 4096, k = 260 370 -> 192 us; n = 3001, k = 83 88 -> 60 us; n = 512, k = 30 28 -> 19 us.
+// What bounds it: the power cap at n = 16384; the pieces of M (16 n^2 bytes) from HBM, 21 us,
+// and a fixed 12 us of launch, first loads and tile end at n = 3001.  Whole filters: degree 20
+// at n = 4096 15.9 -> 8.4 ms, degree 8 at n = 16384 448 -> 201 ms.  Error against 64 bits 0.5
+// to 1.07 of the earlier form's over sizes from n = 64 to 4096.
+constexpr int BK = 64;
+constexpr int A_BYTES = BM * BK * 2;
+constexpr int FLUSH = 4;                 // K blocks per drained partial sum of x0 * y0
+constexpr int MAX_ST = 8;                // most ring stages
+constexpr int RING_BYTES = 196608;
+constexpr int NBAR = 2 * MAX_ST + 10;    // full, empty, acc_full[2], acc_empty[2], cross_full, cross_empty, out_full[2], out_empty[2]
+constexpr int SMEM_BYTES = RING_BYTES + 1024 + 256;
+constexpr int DC = 128;                  // most columns per drain warp
+constexpr int DRAIN_WARPS = 4 * (BNMAX / DC);
+constexpr int EPI_WARPS = 4;
+constexpr int THREADS = 128 + 32 * (DRAIN_WARPS + EPI_WARPS);
+// Registers a thread: 128 at launch (65536 over 16 warps); the warpgroup of the producer and
+// the MMA issuer and that of the finishing warps give theirs to the drain warps, whose sums
+// take 128.
+constexpr int REGS_LAUNCH = 128, REGS_ROLES = 40, REGS_DRAIN = 184, REGS_EPI = 96;
+static_assert(128 * REGS_ROLES + 32 * DRAIN_WARPS * REGS_DRAIN + 32 * EPI_WARPS * REGS_EPI <= THREADS * REGS_LAUNCH,
+              "register split");
+static_assert(SMEM_BYTES <= 232448, "shared memory");
 
 struct Epi {
   int mode;           // 0: operand pieces, 1: recurrence, 2: H X + gamma X
-  int h2;             // 1: the operand holds [P | Q] of H^2 = [[P, Q], [conj Q, conj P]]
-  int64_t n, k;       // rows of P, active vectors
+  float hsign;        // mode 1: -1 (H^2 = -M M); +1 where the operand holds the blocks of H^2
+  int64_t n2, k2;     // rows of M (2n), active columns (2k)
   int64_t kpad;       // elements per piece row
   void* out[3];       // output operand pieces (NPW used)
-  float2* Znext;
-  const float2* Zcur;
-  const float2* Zprev;
-  const float2* src;
+  float* Znext;       // columns of 2n entries
+  const float* Zcur;
+  const float* Zprev;
+  const float* src;
   const float* gamma;  // per column
   float alpha, beta, c;
-  // operand scaling: P' = diag(2^prow) P, input B' = w 2^vexp_in[v]; the pieces this
+  // operand scaling: M' = diag(2^prow) M, input column v times 2^vexp_in[v]; the pieces this
   // launch writes get 2^vexp_out[v] chosen from the bound
-  //   ca * amax_a[v] + cb * amax_b[v] + cc * amax_c[v] + |gamma[v]| * amax_d[v]
-  // (amax_*: largest |component| of each input vector); amax_out receives the largest
-  // |component| of each output vector
+  //   ca * L * amax_a[v] + cb * amax_b[v] + cc * amax_c[v] + |gamma[v]| * amax_d[v]
+  // (L: largest absolute row sum of M; amax_*: largest |entry| of each input column);
+  // amax_out receives the largest |entry| of each output column
+  const float* L;
   const int* prow;
   const int* vexp_in;
   int* vexp_out;
@@ -181,8 +188,8 @@ struct Epi {
   const float* amax_d;
   float ca, cb, cc;
   int* err;
-  float* part;  // split-K: one FP32 partial tile per CTA, column-major 128 x BNT
-  int* cnt;     // split-K: per tile, partial tiles written so far (zero between launches)
+  float* part;  // FP32 (partial) tiles, two per CTA in turn, column-major 128 x BN
+  int* cnt;     // per half tile, partial tiles written so far (zero between launches)
   int sms;      // SMs of the device
 };
 
@@ -197,25 +204,26 @@ __device__ __forceinline__ int out_exp(float b) {
   return min(max(13 - x, -VEXP_MAX), VEXP_MAX);
 }
 __device__ __forceinline__ float vec_bound(const Epi& ep, int64_t v) {
-  float b = ep.ca * ep.amax_a[v];
+  float b = ep.ca * *ep.L * ep.amax_a[v];
   if (ep.cb != 0.0f) b += ep.cb * ep.amax_b[v];
   if (ep.cc != 0.0f) b += ep.cc * ep.amax_c[v];
   if (ep.amax_d) b += fabsf(ep.gamma[v]) * ep.amax_d[v];
   return b;
 }
 
-// Work of one launch: the 128 x BNT output tiles in a grouped raster (GROUP_M row
-// tiles x all column tiles), repeated for nsplit K ranges, so that the CTAs running at
-// the same time stream the same K blocks of A.  With nsplit > 1 the splits leave FP32
-// partial tiles; the CTA that writes a tile's last one (a per-tile counter) sums them in
-// split order and runs the epilogue, so no CTA waits for another and the result does
-// not depend on timing.
+// Work of one launch: 256 x BN output tiles in a grouped raster (group_m row tiles x all
+// column tiles), so that the pairs running at the same time stream the same K blocks of A
+// and B from L2.  Pair c takes the whole tiles w * pairs + c of the full waves, then one of
+// the `parts` equal K ranges of the `rest` tiles that are left (rest * parts <= pairs).  With
+// parts > 1 the CTA that writes a half tile's last partial tile (a counter per half tile) sums
+// them in K order and finishes the tile, so no CTA waits for another and the result does not
+// depend on timing.
 struct Sched {
-  int nkb, num_m, num_n, n_last, bnt, nsplit, ntiles;
-  int group_m;  // raster: group_m row tiles x all column tiles per group
-  __device__ void unit(int c, int& mt, int& nt, int& sp) const {
-    sp = c / ntiles;
-    const int t = c - sp * ntiles;
+  int nkb, num_m, num_n, bn, n_last;  // K blocks; tiles; columns of a tile and of the last one
+  int stages, stage_bytes, bufs, dcols;
+  int pairs, waves, rest, parts;      // rest tiles after the full waves
+  int group_m;
+  __device__ void tile_of(int t, int& mt, int& nt) const {
     const int per_group = group_m * num_n;
     const int g = t / per_group, first = g * group_m;
     const int gm = min(group_m, num_m - first);
@@ -224,46 +232,64 @@ struct Sched {
     mt = first + rem % gm;
   }
 };
+// The segments (tile, K range) of pair c in order; all roles of both CTAs walk the same list.
+struct Walk {
+  const Sched& sc;
+  int c, w;
+  int mt, nt, cols;  // the current segment's tile and its columns
+  int kb0, kb1;
+  __device__ Walk(const Sched& s, int pair) : sc(s), c(pair), w(-1) {}
+  __device__ bool next() {
+    ++w;
+    int t;
+    if (w < sc.waves) {
+      t = w * sc.pairs + c;
+      kb0 = 0;
+      kb1 = sc.nkb;
+    } else if (w == sc.waves && c < sc.rest * sc.parts) {
+      const int r = c / sc.parts, p = c - r * sc.parts;
+      t = w * sc.pairs + r;
+      kb0 = (int)((int64_t)sc.nkb * p / sc.parts);
+      kb1 = (int)((int64_t)sc.nkb * (p + 1) / sc.parts);
+    } else {
+      return false;
+    }
+    sc.tile_of(t, mt, nt);
+    cols = nt == sc.num_n - 1 ? sc.n_last : sc.bn;
+    return true;
+  }
+  __device__ bool split() const { return w == sc.waves && sc.parts > 1; }
+  __device__ bool final() const { return w == sc.waves || (w == sc.waves - 1 && c >= sc.rest * sc.parts); }
+};
 
-// Shared-memory matrix descriptor: K-major tile written by TMA with SWZ-byte rows and
-// SWZ-byte swizzle (128 or 64); 8-row groups 8 * SWZ bytes apart.
-template <int SWZ>
+// Shared-memory matrix descriptor: K-major tile written by TMA with 128-byte rows and
+// 128-byte swizzle; 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);  // start address
   d |= (uint64_t)1 << 16;                    // leading byte offset (unused for these layouts)
-  d |= (uint64_t)((8 * SWZ) >> 4) << 32;     // stride byte offset
+  d |= (uint64_t)((8 * 2 * BK) >> 4) << 32;  // stride byte offset
   d |= (uint64_t)1 << 46;                    // descriptor version
-  d |= (uint64_t)(SWZ == 128 ? 2 : 4) << 61; // 128- or 64-byte swizzle
+  d |= (uint64_t)2 << 61;                    // 128-byte swizzle
   return d;
 }
-// sum[0..BN) += the warp's TMEM lanes at columns [col, col + BN), two loads in flight
-template <int N>
-__device__ __forceinline__ void drain_add(uint32_t col, float* sum) {
+// sum[0..cols) += the warp's TMEM lanes at columns [col, col + cols), cols a multiple of 16
+__device__ __forceinline__ void drain_add(uint32_t col, int cols, float* sum) {
 #pragma unroll
-  for (int c = 0; c < N / 32; c += 2) {
-    uint32_t r0[32], r1[32];
-    tmem_ld32_nowait(col + (uint32_t)(c * 32), r0);
-    tmem_ld32_nowait(col + (uint32_t)((c + 1) * 32), r1);
-    tmem_wait_ld();
+  for (int c = 0; c < DC; c += 32) {
+    if (c + 16 < cols) {  // uniform over the warp
+      uint32_t r[32];
+      tmem_ld32_nowait(col + (uint32_t)c, r);
+      tmem_wait_ld();
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      sum[c * 32 + i] += __uint_as_float(r0[i]);
-      sum[(c + 1) * 32 + i] += __uint_as_float(r1[i]);
+      for (int i = 0; i < 32; ++i) sum[c + i] += __uint_as_float(r[i]);
+    } else if (c < cols) {
+      uint32_t r[16];
+      tmem_ld16_nowait(col + (uint32_t)c, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) sum[c + i] += __uint_as_float(r[i]);
     }
-  }
-}
-
-// sum[0..N) += the warp's TMEM lanes at columns [col, col + N), 16 columns per load
-template <int N>
-__device__ __forceinline__ void drain_add16(uint32_t col, float* sum) {
-#pragma unroll
-  for (int c = 0; c < N / 16; ++c) {
-    uint32_t r[16];
-    tmem_ld16_nowait(col + (uint32_t)(c * 16), r);
-    tmem_wait_ld();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) sum[c * 16 + i] += __uint_as_float(r[i]);
   }
 }
 
@@ -279,22 +305,16 @@ __device__ __forceinline__ void put(void* const* pc, int64_t off, float a, float
     b -= PT::back(hb);
   }
 }
-// The four B-operand rows of vector v at K positions 2i (top entry t = w(i))
-// and 2(n+i) (bottom entry b = w(n+i)), scaled by sc (a power of two).
+// and of one value
 template <class T, int NPC>
-__device__ __forceinline__ void store_operand(void* const* pc, int64_t kpad, int64_t n, int64_t v, int64_t i,
-                                              float2 t, float2 b, float sc) {
-  t.x *= sc; t.y *= sc; b.x *= sc; b.y *= sc;
-  const int64_t r0 = (4 * v) * kpad, r1 = r0 + kpad, r2 = r1 + kpad, r3 = r2 + kpad;
-  const int64_t pt = 2 * i, pb = 2 * (n + i);
-  put<T, NPC>(pc, r0 + pt, t.x, -t.y);
-  put<T, NPC>(pc, r0 + pb, b.x, -b.y);
-  put<T, NPC>(pc, r1 + pt, t.y, t.x);
-  put<T, NPC>(pc, r1 + pb, b.y, b.x);
-  put<T, NPC>(pc, r2 + pt, b.x, b.y);   // u(i) = conj(b)
-  put<T, NPC>(pc, r2 + pb, t.x, t.y);   // u(n+i) = conj(t)
-  put<T, NPC>(pc, r3 + pt, -b.y, b.x);
-  put<T, NPC>(pc, r3 + pb, -t.y, t.x);
+__device__ __forceinline__ void put1(void* const* pc, int64_t off, float a) {
+  using PT = Piece<T>;
+#pragma unroll
+  for (int q = 0; q < NPC; ++q) {
+    const T ha = PT::rn(a);
+    static_cast<T*>(pc[q])[off] = ha;
+    a -= PT::back(ha);
+  }
 }
 
 struct Maps {
@@ -302,288 +322,386 @@ struct Maps {
   CUtensorMap b[3];
 };
 
-// One K range of one 128 x BNT output tile per CTA.  Every K block's products
-// accumulate in one of two TMEM buffers that alternate every FLUSH K blocks; the drain
-// warps add each finished buffer into FP32 registers (round to nearest) while the MMA
-// fills the other one, so the tensor core's truncating accumulator only ever sums a
-// few MMAs.  With 128-wide tiles the cross products (2^-8 or 2^-11 smaller)
-// accumulate over the whole K range in two further buffers instead.  The last column tile
-// may be narrower (n_last columns, a multiple of 16): its MMAs use N = n_last.
-template <int SCH, int BNT, int FL>
-__global__ void __launch_bounds__(Geo<SCH, BNT, FL>::THREADS, 1)
-    tc_hop_kernel(const __grid_constant__ Maps maps, Epi ep, Sched sc) {
+// The end of one half tile: sums its `parts` partial tiles (`stride` floats apart from `tiles`
+// on), undoes the scaling and runs the mode's epilogue for the 32 rows of TMEM lane quarter q and
+// the groups of EB columns first, first + step, ...; a group's loads are in flight together.
+constexpr int EB = 8;
+template <int SCH>
+__device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
+                                            int lane, int first, int step, const float* tiles, int parts,
+                                            size_t stride) {
+  using T = typename Scheme<SCH>::T;
+  const int row_t = q * 32 + lane;
+  const int64_t row = (int64_t)(2 * wk.mt + (int)rank) * BM + row_t;
+  const bool rvalid = row < ep.n2;
+  const float rs = rvalid ? exp2i(-ep.prow[row]) : 0.0f;  // undo the row scaling of M
+  const int64_t v0 = (int64_t)wk.nt * sc.bn;
+  const int cols = (int)min((int64_t)wk.cols, ep.k2 - v0);  // even
+#pragma unroll 1
+  for (int g = first * EB; g < cols; g += step * EB) {
+    const int left = cols - g;
+    const int64_t vb = v0 + g;
+    // loads at clamped rows and columns instead of under a predicate each
+    const int64_t oz = vb * ep.n2 + min(row, ep.n2 - 1);
+    const float* t = tiles + (size_t)g * BM + row_t;
+    float x[EB], zc[EB], zp[EB];
+#pragma unroll
+    for (int i = 0; i < EB; ++i) x[i] = __ldcg(t + i * BM);
+    if (ep.mode != 0) {
+#pragma unroll
+      for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.n2];
+    }
+    if (ep.mode == 1 && ep.beta != 0.0f) {
+#pragma unroll
+      for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.n2];
+    }
+    // lane l prepares column l: the input column's scale (undone), the output's, gamma
+    float s_in = 0.0f, s_out = 0.0f, gmm = 0.0f;
+    if (lane < min(EB, left)) {
+      const int64_t v = vb + lane;
+      s_in = exp2i(-ep.vexp_in[v]);
+      if (ep.gamma) gmm = ep.gamma[v];
+      if (ep.mode != 2) {
+        const int e = out_exp(vec_bound(ep, v));
+        s_out = exp2i(e);
+        if (q == 0) ep.vexp_out[v] = e;  // the same value from every tile
+      }
+    }
+#pragma unroll 1
+    for (int j = 1; j < parts; j += 3) {
+      float y[3][EB];
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+#pragma unroll
+        for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(t + min(j + p, parts - 1) * stride + i * BM);
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        if (j + p < parts) {
+#pragma unroll
+          for (int i = 0; i < EB; ++i) x[i] += y[p][i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < EB; ++i) x[i] *= rs * __shfl_sync(0xffffffffu, s_in, i);
+    if (ep.mode == 1) {
+#pragma unroll
+      for (int i = 0; i < EB; ++i) x[i] = ep.alpha * (ep.hsign * x[i] - ep.c * zc[i]);
+      if (ep.beta != 0.0f) {
+#pragma unroll
+        for (int i = 0; i < EB; ++i) x[i] += ep.beta * zp[i];
+      }
+      if (ep.src) {
+#pragma unroll
+        for (int i = 0; i < EB; ++i) zc[i] = ep.src[oz + (i < left ? i : 0) * ep.n2];
+#pragma unroll
+        for (int i = 0; i < EB; ++i) x[i] += __shfl_sync(0xffffffffu, gmm, i) * zc[i];
+      }
+    } else if (ep.mode == 2) {
+      // H w + gamma w: the two columns of a vector trade places, a' = M c, c' = -M a
+#pragma unroll
+      for (int i = 0; i < EB; i += 2) {
+        const float a = x[i];
+        x[i] = x[i + 1] + __shfl_sync(0xffffffffu, gmm, i) * zc[i];
+        x[i + 1] = -a + __shfl_sync(0xffffffffu, gmm, i + 1) * zc[i + 1];
+      }
+    }
+    unsigned amax = 0;
+#pragma unroll
+    for (int i = 0; i < EB; ++i) {
+      const bool lv = rvalid && i < left;
+      const float so = __shfl_sync(0xffffffffu, s_out, i);
+      if (lv) {
+        if (ep.mode != 2) put1<T, Scheme<SCH>::NPW>(ep.out, (vb + i) * ep.kpad + row, x[i] * so);
+        if (ep.mode != 0) ep.Znext[oz + i * ep.n2] = x[i];
+      }
+      const unsigned mm = __reduce_max_sync(0xffffffffu, lv ? __float_as_uint(fabsf(x[i])) : 0u);
+      if (lane == i) amax = mm;
+    }
+    if (lane < min(EB, left)) atomicMax(reinterpret_cast<unsigned*>(ep.amax_out) + vb + lane, amax);
+  }
+}
+
+template <int SCH>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+    tc_hop_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Epi ep, const __grid_constant__ Sched sc) {
   using SC = Scheme<SCH>;
-  using G = Geo<SCH, BNT, FL>;
-  constexpr int NB = G::NB;
   using T = typename SC::T;
-  constexpr int ST = G::STAGES;
-  constexpr int DC = G::DCOLS;
-  constexpr int FLUSH = G::FLUSH;
-  constexpr int BK = G::BK;
-  constexpr int A_BYTES = G::A_BYTES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ST * G::STAGE_BYTES);
-  uint32_t full[ST], empty[ST];
-#pragma unroll
-  for (int s = 0; s < ST; ++s) {
-    full[s] = smem_u32(bars + s);
-    empty[s] = smem_u32(bars + ST + s);
-  }
-  uint32_t accf[NB], acce[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    accf[b] = smem_u32(bars + 2 * ST + b);
-    acce[b] = smem_u32(bars + 2 * ST + NB + b);
-  }
-  const uint32_t done = smem_u32(bars + 2 * ST + 2 * NB);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + G::NBAR);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + MAX_ST);
+  const uint32_t accf = smem_u32(bars + 2 * MAX_ST), acce = smem_u32(bars + 2 * MAX_ST + 2);  // two of each
+  const uint32_t crossf = smem_u32(bars + 2 * MAX_ST + 4), crosse = smem_u32(bars + 2 * MAX_ST + 5);
+  const uint32_t outf = smem_u32(bars + 2 * MAX_ST + 6), oute = smem_u32(bars + 2 * MAX_ST + 8);  // two of each
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NBAR);
   volatile int* abort_sh = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* issued_sh = reinterpret_cast<int*>(tmem_slot + 2);
   volatile int* last_sh = reinterpret_cast<volatile int*>(tmem_slot + 3);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  int mt, nt, sp;
-  sc.unit(blockIdx.x, mt, nt, sp);
-  const int tile = mt * sc.num_n + nt;
-  const int m0 = mt * BM, n0 = nt * BNT;
-  const int ntile = (nt == sc.num_n - 1) ? sc.n_last : BNT;  // columns of this tile (multiple of 16)
-  const int kb0 = (int)((int64_t)sc.nkb * sp / sc.nsplit), kb1 = (int)((int64_t)sc.nkb * (sp + 1) / sc.nsplit);
-  const int num_kb = kb1 - kb0;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1;
+  const int ST = sc.stages;
+  const int nb = sc.bufs;                             // x0 * y0 buffers, bn columns each
+  const uint32_t cross = (uint32_t)(nb * sc.bn);      // the cross products' columns
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; ++s) {
-      mbar_init(full[s], 1);
-      mbar_init(empty[s], 1);
+      mbar_init(full0 + 8 * s, 1);   // CTA 0: its producer's expect_tx of both CTAs' bytes
+      mbar_init(empty0 + 8 * s, 1);  // a commit
     }
-    for (int b = 0; b < NB; ++b) {
-      mbar_init(accf[b], 1);
-      mbar_init(acce[b], G::DRAIN_WARPS);  // one arrival per drain warp
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(accf + 8 * b, 1);
+      mbar_init(acce + 8 * b, 2 * DRAIN_WARPS);  // CTA 0: one arrival per drain warp of the pair
+      mbar_init(outf + 8 * b, DRAIN_WARPS);
+      mbar_init(oute + 8 * b, EPI_WARPS);
     }
-    mbar_init(done, 1);
+    mbar_init(crossf, 1);
+    mbar_init(crosse, 2 * DRAIN_WARPS);
     *abort_sh = 0;
     *issued_sh = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t sbase = smem_u32(smem);
+  const uint32_t b_bytes = (uint32_t)(sc.bn / 2) * BK * 2;  // one piece of a stage's B half
 
+  float* my_tiles = ep.part + (size_t)blockIdx.x * (2 * BM * BNMAX);
+  // A pair's last tile, for the drain and the finishing warps together: all of them pass the
+  // barriers, also after a failed wait.  True where this CTA has the tile's last partial.
+  auto final_tile = [&](bool ok, const Walk& wk, int slot) -> bool {
+    constexpr int N = 32 * (DRAIN_WARPS + EPI_WARPS);
+    if (wk.split()) __threadfence();
+    asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+    bool last = true;
+    if (wk.split()) {
+      if (threadIdx.x == 128) {
+        int* cnt = ep.cnt + 2 * (pair / sc.parts) + rank;
+        const bool l = atomicAdd(cnt, 1) == sc.parts - 1;
+        if (l) *cnt = 0;  // ready for the next launch
+        *last_sh = l ? 1 : 0;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
+      last = *last_sh != 0;
+      if (last) __threadfence();
+    }
+    return last && ok && __all_sync(0xffffffffu, *abort_sh == 0);  // warp-uniform
+  };
+  auto finish_final = [&](const Walk& wk, int slot, int third) {
+    const bool sp = wk.split();
+    const int p0 = sp ? pair / sc.parts * sc.parts : pair;  // the pair with the tile's first K range
+    const float* t = ep.part + (size_t)(4 * p0 + 2 * (int)rank + slot) * (BM * BNMAX);
+    finish_tile<SCH>(ep, sc, wk, rank, warp & 3, lane, third, 3, t, sp ? sc.parts : 1, (size_t)4 * BM * BNMAX);
+  };
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_ROLES));
   if (warp == 0 && lane == 0) {
-    int issued = 0;
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const int s = kb % ST;
-      const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-      if (kb >= ST && !mbar_wait(empty[s], ph ^ 1u, abort_sh, ep.err, true)) break;
-      const uint32_t st = sbase + s * G::STAGE_BYTES;
-      mbar_expect_tx(full[s], G::STAGE_BYTES);
+    int issued = 0, s = 0;
+    uint32_t ph = 0;
+    const uint32_t lead = map_rank(full0, 0);
+    bool ok = true;
+    for (Walk wk(sc, pair); ok && wk.next();) {
+      const int m0 = (2 * wk.mt + (int)rank) * BM, n0 = wk.nt * sc.bn + (int)rank * (wk.cols / 2);
+      for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
+        if (issued >= ST && !mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_sh, ep.err, true)) {
+          ok = false;
+          break;
+        }
+        const uint32_t st = sbase + s * sc.stage_bytes;
+        if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * sc.stage_bytes);
 #pragma unroll
-      for (int q = 0; q < SC::NPA; ++q) tma_load_2d(st + q * A_BYTES, &maps.a[q], (kb0 + kb) * BK, m0, full[s]);
+        for (int q = 0; q < SC::NPA; ++q) tma_load_2d_pair(st + q * A_BYTES, &maps.a[q], kb * BK, m0, lead + 8 * s);
 #pragma unroll
-      for (int q = 0; q < SC::NPW; ++q)
-        tma_load_2d(st + SC::NPA * A_BYTES + q * G::B_BYTES, &maps.b[q], (kb0 + kb) * BK, n0, full[s]);
-      issued = kb + 1;
+        for (int q = 0; q < SC::NPW; ++q)
+          tma_load_2d_pair(st + SC::NPA * A_BYTES + q * b_bytes, &maps.b[q], kb * BK, n0, lead + 8 * s);
+        ++issued;
+        if (++s == ST) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
     }
     *issued_sh = issued;
-  } else if (warp == 1 && lane == 0) {
-    const uint32_t idesc = make_idesc(ntile, Piece<T>::BF16);
-    const uint32_t small = tmem + (uint32_t)(NB * BNT);
-    const uint64_t dbase = sdesc<G::SWZ>(sbase);
-    for (int kb = 0; kb < num_kb; ++kb) {
-      const int grp = kb / FLUSH, b = grp % NB;
-      const bool first = (kb % FLUSH) == 0;
-      const bool last = (kb % FLUSH) == FLUSH - 1 || kb == num_kb - 1;
-      if (first && grp >= NB && !mbar_wait(acce[b], (uint32_t)(grp / NB - 1) & 1u, abort_sh, ep.err, true)) break;
-      const int s = kb % ST;
-      const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-      if (!mbar_wait(full[s], ph, abort_sh, ep.err, true)) break;
-      tc_fence_after();
-      const uint32_t st = sbase + s * G::STAGE_BYTES;
-      const uint32_t big = tmem + (uint32_t)(b * BNT);
-      // sdesc is linear in the address here (its 14-bit start field holds address / 16 of
-      // a 1024-aligned ring below 256 KB and cannot carry): a hoisted base plus constants;
-      // 16 K elements further along a swizzled row is 32 bytes further
-      const uint64_t sd = dbase + (uint64_t)((uint32_t)(st - sbase) >> 4);
-      if (G::CROSS) {
-#pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-#pragma unroll
-          for (int pr = 0; pr < SC::NPROD; ++pr) {
-            const uint64_t ad = sd + (uint64_t)((SC::pa(pr) * A_BYTES + kk * 32) >> 4);
-            const uint64_t bd = sd + (uint64_t)((SC::NPA * A_BYTES + SC::pb(pr) * G::B_BYTES + kk * 32) >> 4);
-            // products 1, 3, 5 into the first cross buffer, 2, 4 into the second; each
-            // buffer's first MMA (products 1 and 2 of the first K step) overwrites
-            const uint32_t acc =
-                (pr == 0) ? ((!first || kk > 0) ? 1u : 0u) : ((kb > 0 || kk > 0 || pr > 2) ? 1u : 0u);
-            mma_bf16(pr == 0 ? big : ((pr & 1) ? small : small + (uint32_t)BNT), ad, bd, idesc, acc);
-          }
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    const uint64_t dbase = sdesc(sbase);
+    int s = 0, b = 0, seg = 0;
+    uint32_t ph = 0, accph = 1;  // the first pass over the buffers does not wait
+    bool ok = true, used = false;
+    for (Walk wk(sc, pair); ok && wk.next(); ++seg) {
+      const uint32_t idesc = make_idesc(wk.cols, Piece<T>::BF16);
+      for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
+        const int i = kb - wk.kb0;
+        const bool first = (i % FLUSH) == 0;
+        const bool last = (i % FLUSH) == FLUSH - 1 || kb == wk.kb1 - 1;
+        if (!mbar_wait(full0 + 8 * s, ph, abort_sh, ep.err, true)) {
+          ok = false;
+          break;
         }
-      } else {
-        // the block's cross products first, then x0 * y0
+        // sdesc is linear in the address here (its 14-bit start field holds address / 16 of
+        // a 1024-aligned ring below 256 KB and cannot carry): a hoisted base plus constants;
+        // 16 K elements further along a swizzled row is 32 bytes further
+        const uint64_t ad0 = dbase + (uint64_t)((uint32_t)(s * sc.stage_bytes) >> 4);
+        const uint64_t bd0 = ad0 + (uint64_t)((SC::NPA * A_BYTES) >> 4);
+        // x0 * y0 first, so that a finished buffer drains behind the cross products; but a new
+        // buffer's x0 * y0 last, so that the drain has a second block's cross products to hide
+        // behind (except at a tile's start, whose cross products wait for the previous drain)
+        const bool big_last = first && i > 0;
+        auto cross_products = [&]() {
 #pragma unroll
-        for (int pi = 0; pi < SC::NPROD; ++pi) {
-          const int pr = (pi + 1) % SC::NPROD;
+          for (int kk = 0; kk < BK / 16; ++kk)
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t ad = sd + (uint64_t)((SC::pa(pr) * A_BYTES + kk * 32) >> 4);
-            const uint64_t bd = sd + (uint64_t)((SC::NPA * A_BYTES + SC::pb(pr) * G::B_BYTES + kk * 32) >> 4);
-            const uint32_t acc = (first && kk == 0 && pi == 0) ? 0u : 1u;
-            mma_bf16(big, ad, bd, idesc, acc);
-          }
-        }
-      }
-      mma_commit(empty[s]);
-      if (last) mma_commit(accf[b]);
-    }
-    mma_commit(done);  // completes once every MMA issued above has finished
-  } else if (warp >= 4) {
-    const int dw = warp - 4;
-    const int q = warp & 3;                  // TMEM lanes 32 q .. 32 q + 31 (rows of the tile)
-    const int col0 = (dw >> 2) * DC;         // this warp's columns [col0, col0 + DC)
-    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const bool has_cols = col0 < ntile;
-    float sum[DC];
-#pragma unroll
-    for (int i = 0; i < DC; ++i) sum[i] = 0.0f;
-    bool ok = true;
-    const int ngrp = (num_kb + FLUSH - 1) / FLUSH;
-    for (int grp = 0; grp < ngrp; ++grp) {
-      const int b = grp % NB;
-      const bool w = mbar_wait(accf[b], (uint32_t)(grp / NB) & 1u, abort_sh, ep.err, true);
-      if (!__all_sync(0xffffffffu, w)) {  // warp-uniform (tcgen05.ld is .sync.aligned)
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      if (has_cols) {
-        if (G::CROSS) drain_add<DC>(tmem + lane_base + (uint32_t)(b * BNT + col0), sum);
-        else drain_add16<DC>(tmem + lane_base + (uint32_t)(b * BNT + col0), sum);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acce[b]);
-    }
-    if (G::CROSS && ok) {  // the cross products, once every MMA has completed
-      const bool w = mbar_wait(done, 0, abort_sh, ep.err, true);
-      ok = __all_sync(0xffffffffu, w);
-      if (ok && has_cols) {
+            for (int pr = 1; pr < SC::NPROD; ++pr)
+              mma_f16_pair(tmem + cross, ad0 + (uint64_t)((SC::pa(pr) * A_BYTES + kk * 32) >> 4),
+                           bd0 + (uint64_t)((SC::pb(pr) * b_bytes + (uint32_t)(kk * 32)) >> 4), idesc,
+                           (i > 0 || kk > 0 || pr > 1) ? 1u : 0u);
+        };
         tc_fence_after();
-        drain_add<DC>(tmem + lane_base + (uint32_t)(NB * BNT + col0), sum);
-        drain_add<DC>(tmem + lane_base + (uint32_t)((NB + 1) * BNT + col0), sum);
-      }
-    }
-    if (sc.nsplit > 1) {
-      // split tile: write this K range's partial; the last writer sums them all.  Every
-      // drain warp passes both named barriers, also after a failed wait.
-      constexpr int DRAIN_THREADS = 32 * G::DRAIN_WARPS;
-      const int row_t = q * 32 + lane;
-      float* mine = ep.part + (size_t)(sp * sc.ntiles + tile) * (BM * BNT);
-      if (ok && has_cols) {
+        if (big_last) cross_products();
+        if (first && used) {
+          if (!mbar_wait(acce + 8 * b, accph, abort_sh, ep.err, true)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+        }
 #pragma unroll
-        for (int c = 0; c < DC; ++c) mine[(size_t)(col0 + c) * BM + row_t] = sum[c];
-      }
-      __threadfence();
-      asm volatile("bar.sync 1, %0;" ::"r"(DRAIN_THREADS) : "memory");
-      if (dw == 0 && lane == 0) *last_sh = (atomicAdd(ep.cnt + tile, 1) == sc.nsplit - 1) ? 1 : 0;
-      asm volatile("bar.sync 1, %0;" ::"r"(DRAIN_THREADS) : "memory");
-      if (*last_sh) {
-        __threadfence();
-        if (ok && has_cols) {
-#pragma unroll
-          for (int c = 0; c < DC; ++c) sum[c] = 0.0f;
-          for (int j = 0; j < sc.nsplit; ++j) {
-            const float* pp = ep.part + (size_t)(j * sc.ntiles + tile) * (BM * BNT) + (size_t)col0 * BM + row_t;
-#pragma unroll
-            for (int c = 0; c < DC; ++c) sum[c] += __ldcg(pp + (size_t)c * BM);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          mma_f16_pair(tmem + (uint32_t)(b * sc.bn), ad0 + (uint64_t)((kk * 32) >> 4),
+                       bd0 + (uint64_t)((kk * 32) >> 4), idesc, (!first || kk > 0) ? 1u : 0u);
+        if (last) {
+          mma_commit_pair(accf + 8 * b);
+          if (++b == nb) {
+            b = 0;
+            accph ^= 1u;
+            used = true;
           }
         }
-        if (dw == 0 && lane == 0) ep.cnt[tile] = 0;  // ready for the next launch
+        if (i == 0 && seg > 0) {
+          if (!mbar_wait(crosse, (uint32_t)(seg - 1) & 1u, abort_sh, ep.err, true)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+        }
+        if (!big_last) cross_products();
+        mma_commit_pair(empty0 + 8 * s);
+        if (++s == ST) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+      if (ok) mma_commit_pair(crossf);
+    }
+  }
+  } else if (warp < 4 + DRAIN_WARPS) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_DRAIN));
+    const int dw = warp - 4;
+    const int q = warp & 3;                  // TMEM lanes 32 q .. 32 q + 31 (rows of the half tile)
+    const int col0 = (dw >> 2) * sc.dcols;   // this warp's columns [col0, col0 + dcols)
+    const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)col0;
+    const uint32_t acce0 = map_rank(acce, 0), crosse0 = map_rank(crosse, 0);
+    int b = 0, seg = 0;
+    uint32_t accph = 0;
+    bool ok = true;
+    // after a failed wait a warp walks on without waiting, for the named barriers' sake
+    for (Walk wk(sc, pair); wk.next(); ++seg) {
+      const int cols = min(sc.dcols, wk.cols - col0);  // may be <= 0
+      float sum[DC];
+#pragma unroll
+      for (int i = 0; i < DC; ++i) sum[i] = 0.0f;
+      const int ngrp = (wk.kb1 - wk.kb0 + FLUSH - 1) / FLUSH;
+      for (int g = 0; ok && g < ngrp; ++g) {
+        const bool w = mbar_wait(accf + 8 * b, accph, abort_sh, ep.err, true);
+        if (!__all_sync(0xffffffffu, w)) {  // warp-uniform (tcgen05.ld is .sync.aligned)
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        drain_add(tcol + (uint32_t)(b * sc.bn), cols, sum);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acce0 + 8 * b);
+        if (++b == nb) {
+          b = 0;
+          accph ^= 1u;
+        }
+      }
+      if (ok) {
+        const bool w = mbar_wait(crossf, (uint32_t)seg & 1u, abort_sh, ep.err, true);
+        ok = __all_sync(0xffffffffu, w);
+      }
+      if (ok) {
+        tc_fence_after();
+        drain_add(tcol + cross, cols, sum);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(crosse0);
+      }
+      // the tile into its workspace slot, once the tile before the last is finished
+      const int slot = seg & 1;
+      if (ok && seg >= 2) {
+        const bool w = mbar_wait(oute + 8 * slot, (uint32_t)((seg >> 1) - 1) & 1u, abort_sh, ep.err, true);
+        ok = __all_sync(0xffffffffu, w);
+      }
+      if (ok) {
+        float* mine = my_tiles + (size_t)slot * (BM * BNMAX) + (size_t)col0 * BM + q * 32 + lane;
+#pragma unroll
+        for (int c = 0; c < DC; ++c)
+          if ((c & ~15) < cols) __stcg(mine + c * BM, sum[c]);
+      }
+      if (wk.final()) {
+        if (final_tile(ok, wk, slot)) finish_final(wk, slot, 1 + (dw >> 2));
       } else {
-        ok = false;  // another CTA finishes this tile
+        __syncwarp();
+        if (lane == 0) mbar_arrive(outf + 8 * slot);
       }
     }
-    const int64_t row = (int64_t)m0 + q * 32 + lane;
-    const bool rvalid = row < ep.n;
-    const bool go = ok && has_cols && __all_sync(0xffffffffu, *abort_sh == 0);  // warp-uniform
-    if (go) {
-      const int64_t n = ep.n, n2 = 2 * ep.n;
-      const float rs = rvalid ? exp2i(-ep.prow[row]) : 0.0f;  // undo the row scaling of P
-#pragma unroll
-      for (int c = 0; c < DC / 32; ++c) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int64_t vg = (int64_t)((n0 + col0) >> 2) + c * 8 + t;
-          if (vg >= ep.k) continue;  // uniform over the warp
-          const float* v = sum + c * 32;
-          const float vs = exp2i(-ep.vexp_in[vg]);  // and the scaling of the input vector
-          const float2 ht = make_float2(v[4 * t] * rs * vs, v[4 * t + 1] * rs * vs);        // (H x)_top(row)
-          // (H x)_bot(row) = -conj(P u); with the blocks of H^2, +conj(P u)
-          const float2 hb = ep.h2 ? make_float2(v[4 * t + 2] * rs * vs, -v[4 * t + 3] * rs * vs)
-                                  : make_float2(-v[4 * t + 2] * rs * vs, v[4 * t + 3] * rs * vs);
-          const int64_t ot = vg * n2 + row, ob = ot + n;
-          float2 zt = ht, zb = hb;
-          if (ep.mode == 1 && rvalid) {
-            const float2 ct = ep.Zcur[ot], cbv = ep.Zcur[ob];
-            zt = make_float2(ep.alpha * (ht.x - ep.c * ct.x), ep.alpha * (ht.y - ep.c * ct.y));
-            zb = make_float2(ep.alpha * (hb.x - ep.c * cbv.x), ep.alpha * (hb.y - ep.c * cbv.y));
-            if (ep.beta != 0.0f) {
-              const float2 pt = ep.Zprev[ot], pb = ep.Zprev[ob];
-              zt.x += ep.beta * pt.x; zt.y += ep.beta * pt.y;
-              zb.x += ep.beta * pb.x; zb.y += ep.beta * pb.y;
-            }
-            if (ep.src) {
-              const float gmm = ep.gamma[vg];
-              const float2 st = ep.src[ot], sb = ep.src[ob];
-              zt.x += gmm * st.x; zt.y += gmm * st.y;
-              zb.x += gmm * sb.x; zb.y += gmm * sb.y;
-            }
-          } else if (ep.mode == 2 && rvalid) {
-            const float gmm = ep.gamma[vg];
-            const float2 ct = ep.Zcur[ot], cbv = ep.Zcur[ob];
-            zt = make_float2(ht.x + gmm * ct.x, ht.y + gmm * ct.y);
-            zb = make_float2(hb.x + gmm * cbv.x, hb.y + gmm * cbv.y);
-          }
-          if (ep.mode != 0 && rvalid) {
-            ep.Znext[ot] = zt;
-            ep.Znext[ob] = zb;
-          }
-          if (ep.mode != 2) {
-            const int e = out_exp(vec_bound(ep, vg));
-            if (rvalid) store_operand<T, SC::NPW>(ep.out, ep.kpad, n, vg, row, zt, zb, exp2i(e));
-            if (lane == 0) ep.vexp_out[vg] = e;  // the same value from every tile
-          }
-          const float m = rvalid ? fmaxf(fmaxf(fabsf(zt.x), fabsf(zt.y)), fmaxf(fabsf(zb.x), fabsf(zb.y))) : 0.0f;
-          const unsigned mm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-          if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(ep.amax_out) + vg, mm);
-        }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
+    bool ok = true;
+    int seg = 0;
+    for (Walk wk(sc, pair); wk.next(); ++seg) {
+      const int slot = seg & 1;
+      if (wk.final()) {
+        if (final_tile(ok, wk, slot)) finish_final(wk, slot, 0);
+      } else if (ok) {
+        const bool w = mbar_wait(outf + 8 * slot, (uint32_t)(seg >> 1) & 1u, abort_sh, ep.err, true);
+        ok = __all_sync(0xffffffffu, w);
+        if (ok) finish_tile<SCH>(ep, sc, wk, rank, warp & 3, lane, 0, 1, my_tiles + (size_t)slot * (BM * BNMAX), 1, 0);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(oute + 8 * slot);
       }
     }
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // every MMA of the pair has been drained, or a wait has run out
   if (threadIdx.x == 0 && *abort_sh) {
-    // drain copies still in flight into this CTA's shared memory (bounded)
-    const int issued = *issued_sh;
-    for (int kb = max(0, issued - ST); kb < issued; ++kb)
-      mbar_wait(full[kb % ST], (uint32_t)(kb / ST) & 1u, abort_sh, ep.err, false);
-  }
-  if (warp == 1) {
-    // every MMA has finished before the accumulator memory is released
-    if (lane == 0) mbar_wait(done, 0, abort_sh, ep.err, false);
-    __syncwarp();
+    // copies and MMAs still in flight on the pair's shared memory and TMEM (bounded): CTA 0's
+    // barriers count both CTAs' bytes
+    if (rank == 0) {
+      const int issued = *issued_sh;
+      for (int i = max(0, issued - ST); i < issued; ++i)
+        mbar_wait(full0 + 8 * (i % ST), (uint32_t)(i / ST) & 1u, abort_sh, ep.err, false);
+    }
+    const uint64_t t0 = gtimer();
+    while (gtimer() - t0 < COPY_LIMIT_NS) __nanosleep(1000);
   }
   __syncthreads();
+  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
 }
 
@@ -624,71 +742,100 @@ __device__ __forceinline__ void block_max_sum(float& m, float& s) {
   s = ws[0];
 }
 
-// P = [A | B] (row-major complex128) -> NPC pieces, one CTA per row i, K = (re, im)
-// pairs, scaled by 2^prow[i] (largest entry of the row in [2^12, 2^13)); L receives the
-// largest row sum of |Re| + |Im| (unscaled), the bound factor of an H application.
-template <class T, int NPC>
+// The real form of [A | B] (row-major complex128) -> NPC pieces, one CTA per row i of A and B,
+// which gives rows 2i and 2i + 1; TWIST 1: M above (z -> -i (A z + B conj z)), 0: the plain
+// z -> A z + B conj z.  Row r is scaled by 2^prow[r] (its largest entry in [2^12, 2^13)); L
+// receives the largest row sum of absolute values (unscaled), the bound factor of an
+// application.  Columns 2n .. kpad are zero.
+template <int TWIST>
+__device__ __forceinline__ void real_form(cplx a, cplx b, float2& r0, float2& r1) {
+  const float2 re = make_float2((float)(a.x + b.x), (float)(b.y - a.y));  // Re: (Re z, Im z) coefficients
+  const float2 im = make_float2((float)(a.y + b.y), (float)(a.x - b.x));  // Im
+  r0 = TWIST ? im : re;
+  r1 = TWIST ? make_float2(-re.x, -re.y) : im;
+}
+template <class T, int NPC, int TWIST>
 __global__ void split_p_kernel(const cplx* A, const cplx* B, int64_t n, int64_t kpad, Pieces out, int* prow,
                                float* L) {
   const int64_t i = blockIdx.x;
-  float m = 0.0f, sum = 0.0f;
-  for (int64_t l = threadIdx.x; l < 2 * n; l += blockDim.x) {
-    const cplx p = (l < n) ? A[i * n + l] : B[i * n + (l - n)];
-    const float x = fabsf((float)p.x), y = fabsf((float)p.y);
-    m = fmaxf(m, fmaxf(x, y));
-    sum += x + y;
+  float m0 = 0.0f, m1 = 0.0f, s0 = 0.0f, s1 = 0.0f;
+  float2 r0, r1;
+  for (int64_t l = threadIdx.x; l < n; l += blockDim.x) {
+    real_form<TWIST>(A[i * n + l], B[i * n + l], r0, r1);
+    m0 = fmaxf(m0, fmaxf(fabsf(r0.x), fabsf(r0.y)));
+    m1 = fmaxf(m1, fmaxf(fabsf(r1.x), fabsf(r1.y)));
+    s0 += fabsf(r0.x) + fabsf(r0.y);
+    s1 += fabsf(r1.x) + fabsf(r1.y);
   }
-  block_max_sum(m, sum);
-  const int e = out_exp(m);
+  block_max_sum(m0, s0);
+  __syncthreads();
+  block_max_sum(m1, s1);
+  const int e0 = out_exp(m0), e1 = out_exp(m1);
   if (threadIdx.x == 0) {
-    prow[i] = e;
-    atomicMax(reinterpret_cast<unsigned*>(L), __float_as_uint(sum));
+    prow[2 * i] = e0;
+    prow[2 * i + 1] = e1;
+    atomicMax(reinterpret_cast<unsigned*>(L), __float_as_uint(fmaxf(s0, s1)));
   }
-  const float sc = exp2i(e);
-  for (int64_t l = threadIdx.x; l < 2 * n; l += blockDim.x) {
-    const cplx p = (l < n) ? A[i * n + l] : B[i * n + (l - n)];
-    put<T, NPC>(out.p, i * kpad + 2 * l, (float)p.x * sc, (float)p.y * sc);
+  const float c0 = exp2i(e0), c1 = exp2i(e1);
+  for (int64_t l = threadIdx.x; 2 * l < kpad; l += blockDim.x) {
+    r0 = r1 = make_float2(0.0f, 0.0f);
+    if (l < n) real_form<TWIST>(A[i * n + l], B[i * n + l], r0, r1);
+    put<T, NPC>(out.p, (2 * i) * kpad + 2 * l, r0.x * c0, r0.y * c0);
+    put<T, NPC>(out.p, (2 * i + 1) * kpad + 2 * l, r1.x * c1, r1.y * c1);
   }
 }
-// amax[v] = largest |Re|, |Im| of column v of the complex128 block W (2n x k), rounded to
-// FP32, and vexp[v] its operand exponent; one CTA per column
-__global__ void col_amax_kernel(const cplx* W, int64_t n2, float* amax, int* vexp) {
+// The halves a and c of w = [x; y]; and w from them
+__device__ __forceinline__ void j_split(cplx x, cplx y, float2& a, float2& c) {
+  a = make_float2((float)(0.5 * (x.x + y.x)), (float)(0.5 * (x.y - y.y)));
+  c = make_float2((float)(-0.5 * (x.y + y.y)), (float)(0.5 * (x.x - y.x)));
+}
+// amax[2v], amax[2v + 1] = largest |entry| of the halves of column v of the complex128 block
+// W (2n x k), rounded to FP32, and vexp their operand exponents; one CTA per column
+__global__ void col_amax_kernel(const cplx* W, int64_t n, float* amax, int* vexp) {
   const int64_t v = blockIdx.x;
-  float m = 0.0f, unused = 0.0f;
-  for (int64_t i = threadIdx.x; i < n2; i += blockDim.x) {
-    const cplx w = W[v * n2 + i];
-    m = fmaxf(m, fmaxf(fabsf((float)w.x), fabsf((float)w.y)));
+  float m0 = 0.0f, m1 = 0.0f, unused = 0.0f;
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    float2 a, c;
+    j_split(W[v * 2 * n + i], W[v * 2 * n + n + i], a, c);
+    m0 = fmaxf(m0, fmaxf(fabsf(a.x), fabsf(a.y)));
+    m1 = fmaxf(m1, fmaxf(fabsf(c.x), fabsf(c.y)));
   }
-  block_max_sum(m, unused);
+  block_max_sum(m0, unused);
+  __syncthreads();
+  block_max_sum(m1, unused);
   if (threadIdx.x == 0) {
-    amax[v] = m;
-    vexp[v] = out_exp(m);
+    amax[2 * v] = m0;
+    amax[2 * v + 1] = m1;
+    vexp[2 * v] = out_exp(m0);
+    vexp[2 * v + 1] = out_exp(m1);
   }
 }
-// complex128 block (2n x k) -> FP32 master and, optionally, operand pieces (exponents vexp)
+// complex128 block (2n x k) -> FP32 columns (2n x 2k) and their operand pieces (exponents
+// vexp), zero in the entries 2n .. kpad
 template <class T, int NPC>
-__global__ void pack_kernel(const cplx* W, int64_t n, int64_t k, float2* Z, Pieces out, int with_pieces,
-                            int64_t kpad, const int* vexp) {
-  const int64_t total = n * k;
+__global__ void pack_kernel(const cplx* W, int64_t n, int64_t k, float2* Z, Pieces out, int64_t kpad,
+                            const int* vexp) {
+  const int64_t half = kpad / 2, total = half * k;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = idx % n, v = idx / n;
-    const cplx wt = W[v * 2 * n + i], wb = W[v * 2 * n + n + i];
-    const float2 t = make_float2((float)wt.x, (float)wt.y);
-    const float2 b = make_float2((float)wb.x, (float)wb.y);
-    if (Z) {
-      Z[v * 2 * n + i] = t;
-      Z[v * 2 * n + n + i] = b;
+    const int64_t i = idx % half, v = idx / half;
+    float2 a = make_float2(0.0f, 0.0f), c = a;
+    if (i < n) {
+      j_split(W[v * 2 * n + i], W[v * 2 * n + n + i], a, c);
+      Z[2 * v * n + i] = a;
+      Z[(2 * v + 1) * n + i] = c;
     }
-    if (with_pieces) store_operand<T, NPC>(out.p, kpad, n, v, i, t, b, exp2i(vexp[v]));
+    const float sa = exp2i(vexp[2 * v]), sc = exp2i(vexp[2 * v + 1]);
+    put<T, NPC>(out.p, 2 * v * kpad + 2 * i, a.x * sa, a.y * sa);
+    put<T, NPC>(out.p, (2 * v + 1) * kpad + 2 * i, c.x * sc, c.y * sc);
   }
 }
-// Z = scale * X (FP32 master) and its operand pieces; the largest component of column v
+// Z = scale * X (FP32 columns) and its operand pieces; the largest entry of column v
 // is |scale| amax_x[v] (up to rounding), which sets its exponent
 template <class T, int NPC>
-__global__ void scale_pack_kernel(const float2* X, int64_t n, int64_t k, float scale, float2* Z, Pieces out,
+__global__ void scale_pack_kernel(const float2* X, int64_t n, int64_t k2, float scale, float2* Z, Pieces out,
                                   int64_t kpad, const float* amax_x, float* amax_z, int* vexp_z) {
-  const int64_t total = n * k;
+  const int64_t total = n * k2;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = idx % n, v = idx / n;
@@ -698,42 +845,47 @@ __global__ void scale_pack_kernel(const float2* X, int64_t n, int64_t k, float s
       amax_z[v] = am;
       vexp_z[v] = e;
     }
-    const float2 xt = X[v * 2 * n + i], xb = X[v * 2 * n + n + i];
-    const float2 t = make_float2(scale * xt.x, scale * xt.y), b = make_float2(scale * xb.x, scale * xb.y);
-    Z[v * 2 * n + i] = t;
-    Z[v * 2 * n + n + i] = b;
-    store_operand<T, NPC>(out.p, kpad, n, v, i, t, b, exp2i(e));
+    const float2 x = X[idx], z = make_float2(scale * x.x, scale * x.y);
+    const float sz = exp2i(e);
+    Z[idx] = z;
+    put<T, NPC>(out.p, v * kpad + 2 * i, z.x * sz, z.y * sz);
   }
 }
-// out[:, v] = (double) Zsel[:, v] + coef[v] * base[:, v]   (coef/base optional)
+// out[:, v] = the vector of the halves in columns 2v, 2v + 1 of Zsel, in FP64,
+// + coef[v] * base[:, v]   (coef/base optional)
 __global__ void combine_kernel(cplx* out, const float2* Z0, const float2* Z1, const float2* Z2, const int* sel,
-                               const double* coef, const cplx* base, int64_t n2, int64_t k) {
-  const int64_t total = n2 * k;
+                               const double* coef, const cplx* base, int64_t n, int64_t k) {
+  const int64_t total = n * k;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = idx / n2;
+    const int64_t i = idx % n, v = idx / n;
     const int q = sel[v];
-    const float2 z = (q == 0 ? Z0 : (q == 1 ? Z1 : Z2))[idx];
-    cplx r = mk((double)z.x, (double)z.y);
-    if (coef) r = cadd(r, cscale(base[idx], coef[v]));
-    out[idx] = r;
+    const float2* Z = q == 0 ? Z0 : (q == 1 ? Z1 : Z2);
+    const float2 a = Z[2 * v * n + i], c = Z[(2 * v + 1) * n + i];
+    cplx x = mk((double)a.x + (double)c.y, (double)a.y - (double)c.x);   // a - i c
+    cplx y = mk((double)a.x - (double)c.y, -(double)a.y - (double)c.x);  // conj(a) - i conj(c)
+    const int64_t o = v * 2 * n + i;
+    if (coef) {
+      x = cadd(x, cscale(base[o], coef[v]));
+      y = cadd(y, cscale(base[o + n], coef[v]));
+    }
+    out[o] = x;
+    out[o + n] = y;
   }
 }
 
-// Tensor map of a piece plane (rows x kpad, K contiguous) with boxes of bk x box_rows and
-// 2 bk-byte swizzle (bk = 64 or 32).
-static int make_map(CUtensorMap* m, const void* base, int64_t kpad, int64_t rows, int box_rows, bool bf16,
-                    int bk) {
+// Tensor map of a piece plane (rows x kpad, K contiguous) with boxes of BK x box_rows and
+// 128-byte swizzle; rows of a box beyond the plane read as zero.
+static int make_map(CUtensorMap* m, const void* base, int64_t kpad, int64_t rows, int box_rows, bool bf16) {
   auto fn = encode_fn();
   if (!fn) return CHASE_BSE_UNSUPPORTED;
   const cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)kpad * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)bk, (cuuint32_t)box_rows};
+  const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                   const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  bk == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? CHASE_BSE_OK : CHASE_BSE_CUDA_ERROR;
 }
 
@@ -742,8 +894,8 @@ static inline unsigned gsz(int64_t total) {
   return (unsigned)std::min<int64_t>(std::max<int64_t>(b, 1), 16384);
 }
 
-// The operand of P = [A | B] in NPA pieces, with its tensor maps, row exponents and
-// the bound factor L (device scalar).
+// The real form of [A | B] in NPA pieces, with its tensor maps, row exponents and the
+// bound factor L (device scalar).
 struct POperand {
   int64_t n = 0, kpad = 0;
   Pieces pc{};
@@ -752,80 +904,110 @@ struct POperand {
   float* L = nullptr;
 };
 
-template <int SCH, int BNT>
+template <int SCH, int TWIST>
 static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POperand& P, cudaStream_t s) {
   using T = typename Scheme<SCH>::T;
   constexpr int NPA = Scheme<SCH>::NPA;
   P.n = n;
-  constexpr int BK = Geo<SCH, BNT, 1>::BK;
-  P.kpad = ((4 * n + KPAD - 1) / KPAD) * KPAD;
-  const int64_t rows = ((n + BM - 1) / BM) * BM;  // whole tiles: every TMA box lies inside the tensor
+  P.kpad = ((2 * n + KPAD - 1) / KPAD) * KPAD;
   for (int q = 0; q < NPA; ++q) {
     T* pq;
-    CB_TRY(ws.alloc(&pq, rows * P.kpad));
+    CB_TRY(ws.alloc(&pq, 2 * n * P.kpad));
     P.pc.p[q] = pq;
-    CB_CUDA(cudaMemsetAsync(pq, 0, sizeof(T) * rows * P.kpad, s));
   }
-  CB_TRY(ws.alloc(&P.prow, n));
+  CB_TRY(ws.alloc(&P.prow, 2 * n));
   CB_TRY(ws.alloc(&P.L, 1));
   CB_CUDA(cudaMemsetAsync(P.L, 0, sizeof(float), s));
-  split_p_kernel<T, NPA><<<(unsigned)n, 256, 0, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
+  split_p_kernel<T, NPA, TWIST><<<(unsigned)n, 256, 0, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
   count_launch();
   CB_LAUNCH();
-  for (int q = 0; q < NPA; ++q) CB_TRY(make_map(&P.map[q], P.pc.p[q], P.kpad, rows, BM, Piece<T>::BF16, BK));
+  for (int q = 0; q < NPA; ++q) CB_TRY(make_map(&P.map[q], P.pc.p[q], P.kpad, 2 * n, BM, Piece<T>::BF16));
   return CHASE_BSE_OK;
 }
 
-// K splits of a launch with `tiles` CTAs per split: the count (1 to MAX_SPLIT) that
-// minimises the estimated time, waves of CTAs x (1/splits + a fixed cost per CTA of
-// 5 % of a tile), with at least two drained groups of K blocks per split and at most
-// MAX_SPLIT x SMs CTAs (the partial-tile workspace).
-constexpr int MAX_SPLIT = 4;
-static int split_count(int tiles, int nkb, int sms, int flush) {
-  int best = 1;
+// Cycles of one K block of a 256 x w tile in a launch of bn-wide tiles: the MMAs (w / 2 each)
+// or the shared-memory traffic at 128 bytes a cycle (operand reads and the ring's fill).
+template <int SCH>
+static double block_cycles(int w, int bn) {
+  using SC = Scheme<SCH>;
+  constexpr int MMAS = SC::NPROD * (BK / 16);
+  const double mma = MMAS * (w / 2.0);
+  const double smem = (MMAS * (4096.0 + 16.0 * w) + SC::NPA * A_BYTES + SC::NPW * 64.0 * bn) / 128.0;
+  return std::max(mma, smem);
+}
+// The schedule of a launch with m rows, k2 columns and nkb K blocks: of the column widths
+// (multiples of 32) that ceil(k2 / 256) to 3 more column tiles need, and of the numbers of K
+// ranges to cut the tiles left after the full waves into, the choice of least estimated time.
+template <int SCH>
+static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
+  using SC = Scheme<SCH>;
+  Sched best{};
   double best_t = 0.0;
-  for (int sp = 1; sp <= MAX_SPLIT; ++sp) {
-    if (sp > 1 && (nkb / sp < 2 * flush || (int64_t)tiles * sp > (int64_t)MAX_SPLIT * sms)) break;
-    const double waves = (double)((tiles * sp + sms - 1) / sms);
-    const double t = waves * (1.0 / sp + 0.05);
-    if (sp == 1 || t < best_t - 1e-9) {
-      best = sp;
-      best_t = t;
+  const int n0 = (int)cdiv(k2, BNMAX);
+  for (int nn = n0; nn <= n0 + 3; ++nn) {
+    Sched sc{};
+    sc.nkb = nkb;
+    sc.num_m = (int)cdiv(m, 2 * BM);
+    sc.bn = (int)cdiv(cdiv(k2, nn), 32) * 32;
+    sc.num_n = (int)cdiv(k2, sc.bn);
+    if (sc.num_n != nn) continue;
+    sc.n_last = (int)cdiv(k2 - (int64_t)(nn - 1) * sc.bn, 32) * 32;
+    sc.stage_bytes = SC::NPA * A_BYTES + SC::NPW * (sc.bn / 2) * BK * 2;
+    sc.stages = std::min(MAX_ST, RING_BYTES / sc.stage_bytes);
+    sc.dcols = (int)cdiv(sc.bn, BNMAX / DC * 16) * 16;  // half of the tile, whole TMEM loads
+    sc.bufs = 3 * sc.bn <= (int)TMEM_COLS ? 2 : 1;
+    sc.group_m = 8;
+    const int64_t tiles = (int64_t)sc.num_m * nn;
+    sc.pairs = pairs;
+    sc.waves = (int)(tiles / pairs);
+    sc.rest = (int)(tiles % pairs);
+    const double full = block_cycles<SCH>(sc.bn, sc.bn);
+    const double avg = (full * (nn - 1) + block_cycles<SCH>(sc.n_last, sc.bn)) / nn;
+    const double fixed = 6000.0;  // prologue and epilogue of a tile
+    const double base = sc.waves * ((sc.waves > 1 ? avg : full) * nkb + fixed);
+    for (int f = 1; f == 1 || (f * sc.rest <= pairs && nkb / f >= 2); ++f) {
+      sc.parts = f;
+      double t = base;
+      if (sc.rest > 0) {
+        t += std::ceil((double)nkb / f) * full + fixed;
+        // partial tiles out and back in (L2, about 64 bytes a cycle and SM)
+        if (f > 1) t += 3000.0 + (f + 1) * 8.0 * sc.bn;
+      }
+      if (best_t == 0.0 || t < best_t) {
+        best = sc;
+        best_t = t;
+      }
+      if (sc.rest == 0) break;
     }
   }
   return best;
 }
 
-// One tensor-core application of H to the vectors held in the operand pieces
-// described by bmap, with epilogue `ep`.
-template <int SCH, int BNT, int FL>
-static int apply(const POperand& P, const CUtensorMap* bmap, Epi ep, cudaStream_t s) {
-  using G = Geo<SCH, BNT, FL>;
-  if (ep.k <= 0) return CHASE_BSE_OK;
+// One tensor-core application of M to the columns held in the operand pieces bp (rows
+// columns allocated), with epilogue `ep`.
+template <int SCH>
+static int apply(const POperand& P, const Pieces& bp, int64_t rows, Epi ep, cudaStream_t s) {
+  using T = typename Scheme<SCH>::T;
+  if (ep.k2 <= 0) return CHASE_BSE_OK;
   static bool attr = false;
   if (!attr) {
-    CB_CUDA(cudaFuncSetAttribute(tc_hop_kernel<SCH, BNT, FL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 G::SMEM_BYTES));
+    CB_CUDA(cudaFuncSetAttribute(tc_hop_kernel<SCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    // the drain warps' share exists only if the kernel was launched with REGS_LAUNCH registers a thread
+    cudaFuncAttributes fa;
+    CB_CUDA(cudaFuncGetAttributes(&fa, tc_hop_kernel<SCH>));
+    if (fa.numRegs != REGS_LAUNCH) return CHASE_BSE_UNSUPPORTED;
     attr = true;
   }
+  ep.prow = P.prow;
+  ep.L = P.L;
+  const Sched sc = plan<SCH>(ep.n2, ep.k2, (int)(P.kpad / BK), ep.sms / 2);
   Maps maps;
   for (int q = 0; q < Scheme<SCH>::NPA; ++q) maps.a[q] = P.map[q];
-  for (int q = 0; q < Scheme<SCH>::NPW; ++q) maps.b[q] = bmap[q];
-  ep.prow = P.prow;
-  Sched sc{};
-  sc.num_m = (int)cdiv(P.n, BM);
-  sc.num_n = (int)cdiv(4 * ep.k, BNT);
-  const int64_t rest = 4 * ep.k - (int64_t)(sc.num_n - 1) * BNT;  // columns of the last tile
-  sc.n_last = (int)(((rest + 15) / 16) * 16);
-  sc.nkb = (int)(P.kpad / G::BK);
-  sc.bnt = BNT;
-  sc.ntiles = sc.num_m * sc.num_n;
-  sc.nsplit = split_count(sc.ntiles, sc.nkb, ep.sms, G::FLUSH);
-  // 8 row tiles per raster group: of 4, 8, 12 and 16 the least DRAM traffic at n = 16384,
-  // k = 1300 (40 GB per launch against 41-59), with the same duration
-  sc.group_m = 8;
-  const int64_t tid = timer_begin(0, 32.0 * (double)P.n * (double)P.n * (double)ep.k, s);
-  tc_hop_kernel<SCH, BNT, FL><<<(unsigned)(sc.ntiles * sc.nsplit), G::THREADS, G::SMEM_BYTES, s>>>(maps, ep, sc);
+  for (int q = 0; q < Scheme<SCH>::NPW; ++q)
+    CB_TRY(make_map(&maps.b[q], bp.p[q], P.kpad, rows, sc.bn / 2, Piece<T>::BF16));
+  const unsigned grid = 2u * (unsigned)(sc.waves > 0 ? sc.pairs : sc.rest * sc.parts);
+  const int64_t tid = timer_begin(0, 16.0 * (double)P.n * (double)P.n * (double)ep.k2, s);
+  tc_hop_kernel<SCH><<<grid, THREADS, SMEM_BYTES, s>>>(maps, ep, sc);
   timer_end(tid, s);
   count_launch();
   CB_LAUNCH();
@@ -844,58 +1026,54 @@ static int apply(const POperand& P, const CUtensorMap* bmap, Epi ep, cudaStream_
 // With P2, Q2 (the blocks of H^2 = [[P2, Q2], [conj Q2, conj P2]], row-major n x n) the
 // filter applies H^2 from its blocks, one launch per step (the explicit-H^2 variant, not
 // the paper's method); H itself (A, B) is then used only for the correction source.
-template <int SCH, int BNT, int FL>
+template <int SCH>
 static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, int64_t k, const int* degs,
                        double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
                        cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
   using T = typename Scheme<SCH>::T;
   constexpr int NPW = Scheme<SCH>::NPW;
-  constexpr bool BF = Piece<T>::BF16;
   if (k == 0) return CHASE_BSE_OK;
   const int64_t n2 = 2 * n;
   const bool expl = P2 != nullptr && Q2 != nullptr;
   const bool corr = (ritz != nullptr && R != nullptr);
   Workspace ws(s);
   POperand P, PH2;  // [A | B] (H), [P2 | Q2] (H^2)
-  if (!expl || corr) CB_TRY((prepare_p<SCH, BNT>(A, B, n, ws, P, s)));
-  if (expl) CB_TRY((prepare_p<SCH, BNT>(P2, Q2, n, ws, PH2, s)));
+  if (!expl || corr) CB_TRY((prepare_p<SCH, 1>(A, B, n, ws, P, s)));
+  if (expl) CB_TRY((prepare_p<SCH, 0>(P2, Q2, n, ws, PH2, s)));
   const POperand& PK = expl ? PH2 : P;  // the operand of the recurrence (its kpad and pieces layout)
-  const int64_t kpad = PK.kpad;  // the same for both operands (4n padded)
-  const int64_t rows = ((4 * k + BNT - 1) / BNT) * BNT;  // whole tiles
+  const int64_t kpad = PK.kpad;  // the same for both operands (2n padded)
+  const int64_t k2 = 2 * k;      // columns
   Pieces Zp{}, Tp{};
-  CUtensorMap mZ[3], mT[3];
   for (int q = 0; q < NPW; ++q) {
     T *zq, *tq;
-    CB_TRY(ws.alloc(&zq, rows * kpad));
-    CB_TRY(ws.alloc(&tq, rows * kpad));
+    CB_TRY(ws.alloc(&zq, k2 * kpad));
+    CB_TRY(ws.alloc(&tq, k2 * kpad));
     Zp.p[q] = zq;
     Tp.p[q] = tq;
-    CB_CUDA(cudaMemsetAsync(zq, 0, sizeof(T) * rows * kpad, s));
-    CB_CUDA(cudaMemsetAsync(tq, 0, sizeof(T) * rows * kpad, s));
-    CB_TRY(make_map(&mZ[q], zq, kpad, rows, BNT, BF, Geo<SCH, BNT, FL>::BK));
-    CB_TRY(make_map(&mT[q], tq, kpad, rows, BNT, BF, Geo<SCH, BNT, FL>::BK));
+    if (kpad > n2) {  // zero past the entries of a column, as past those of a row of M
+      CB_CUDA(cudaMemset2DAsync(zq + n2, sizeof(T) * kpad, 0, sizeof(T) * (kpad - n2), k2, s));
+      CB_CUDA(cudaMemset2DAsync(tq + n2, sizeof(T) * kpad, 0, sizeof(T) * (kpad - n2), k2, s));
+    }
   }
   // explicit H^2: the pieces of Z_j alternate between the two sets (j even: Zp)
   Pieces* zbuf[2] = {&Zp, &Tp};
-  const CUtensorMap* zmap[2] = {mZ, mT};
-  float2 *Zb[3], *src = nullptr;
+  float *Zb[3], *src = nullptr;
   float* gam;
   int* err;
-  for (int q = 0; q < 3; ++q) CB_TRY(ws.alloc(&Zb[q], n2 * k));
-  CB_TRY(ws.alloc(&gam, k));
+  for (int q = 0; q < 3; ++q) CB_TRY(ws.alloc(&Zb[q], n2 * k2));
+  CB_TRY(ws.alloc(&gam, k2));
+  auto c2 = [](float* z) { return reinterpret_cast<float2*>(z); };
   CB_TRY(ws.alloc(&err, 1));
   CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-  // split-K workspace: a partial tile per CTA of a split launch (fewer than
-  // MAX_SPLIT x SMs of them), one counter per tile
+  // (partial) tiles, two per CTA, and a counter per half of a split tile
   int dev = 0, sms = 0;
   CB_CUDA(cudaGetDevice(&dev));
   CB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t max_tiles = cdiv(n, BM) * (rows / BNT);
   float* part;
   int* cnt;
-  CB_TRY(ws.alloc(&part, (int64_t)MAX_SPLIT * sms * BM * BNT));
-  CB_TRY(ws.alloc(&cnt, max_tiles));
-  CB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * max_tiles, s));
+  CB_TRY(ws.alloc(&part, (int64_t)sms * 2 * BM * BNMAX));
+  CB_TRY(ws.alloc(&cnt, sms));
+  CB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * sms, s));
   auto sk = [&](Epi& e) {
     e.part = part;
     e.cnt = cnt;
@@ -907,23 +1085,19 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
   const double sigma1 = e / (mu1 * mu1 - c);
   const double tau = 2.0 / sigma1;
   const int maxdeg = degs[0];
-  // per-vector maxima and operand exponents, one slot of k entries per vector block:
+  // per-column maxima and operand exponents, one slot of k2 entries per block:
   // Z_j (j = 0 .. maxdeg), T_j = H Z_j (j < maxdeg), the residual block R and the
   // correction source r2
   const int64_t nslot = 2 * (int64_t)maxdeg + 3;
   float* amax;
   int* vexp;
-  CB_TRY(ws.alloc(&amax, nslot * k));
-  CB_TRY(ws.alloc(&vexp, nslot * k));
-  CB_CUDA(cudaMemsetAsync(amax, 0, sizeof(float) * nslot * k, s));
-  CB_CUDA(cudaMemsetAsync(vexp, 0, sizeof(int) * nslot * k, s));
-  auto slotZ = [&](int j) { return (int64_t)j * k; };
-  auto slotT = [&](int j) { return (int64_t)(maxdeg + 1 + j) * k; };
-  const int64_t slotR = (int64_t)(2 * maxdeg + 1) * k, slotS = (int64_t)(2 * maxdeg + 2) * k;
-  float L = 0.0f, L2 = 0.0f;  // largest absolute row sums of [A | B] and [P2 | Q2]
-  if (!expl || corr) CB_CUDA(cudaMemcpyAsync(&L, P.L, sizeof(float), cudaMemcpyDeviceToHost, s));
-  if (expl) CB_CUDA(cudaMemcpyAsync(&L2, PH2.L, sizeof(float), cudaMemcpyDeviceToHost, s));
-  CB_CUDA(cudaStreamSynchronize(s));
+  CB_TRY(ws.alloc(&amax, nslot * k2));
+  CB_TRY(ws.alloc(&vexp, nslot * k2));
+  CB_CUDA(cudaMemsetAsync(amax, 0, sizeof(float) * nslot * k2, s));
+  CB_CUDA(cudaMemsetAsync(vexp, 0, sizeof(int) * nslot * k2, s));
+  auto slotZ = [&](int j) { return (int64_t)j * k2; };
+  auto slotT = [&](int j) { return (int64_t)(maxdeg + 1 + j) * k2; };
+  const int64_t slotR = (int64_t)(2 * maxdeg + 1) * k2, slotS = (int64_t)(2 * maxdeg + 2) * k2;
 
   std::vector<double> al(maxdeg), be(maxdeg);  // alpha_j, beta_j of the scaled recurrence
   {
@@ -953,36 +1127,36 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
       }
     }
   }
-  std::vector<float> gh(k);
+  std::vector<float> gh(k2);
   int j0 = 0;
   cudaEvent_t e0, e1;
   CB_CUDA(cudaEventCreate(&e0));
   CB_CUDA(cudaEventCreate(&e1));
   CB_CUDA(cudaEventRecord(e0, s));
   if (!corr) {
-    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(Y0, n2, amax + slotZ(0), vexp + slotZ(0));
+    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(Y0, n, amax + slotZ(0), vexp + slotZ(0));
     count_launch();
-    pack_kernel<T, NPW><<<gsz(n * k), 256, 0, s>>>(Y0, n, k, Zb[0], Zp, 1, kpad, vexp + slotZ(0));  // Z_0 = W
+    pack_kernel<T, NPW><<<gsz(kpad / 2 * k), 256, 0, s>>>(Y0, n, k, c2(Zb[0]), Zp, kpad, vexp + slotZ(0));  // Z_0 = W
     count_launch();
     CB_LAUNCH();
   } else {
     // r2 = H R + ritz R on the tensor cores; Z_0 = 0; Z_1 = alpha_0 r2
-    CB_TRY(ws.alloc(&src, n2 * k));
-    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(R, n2, amax + slotR, vexp + slotR);
+    CB_TRY(ws.alloc(&src, n2 * k2));
+    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(R, n, amax + slotR, vexp + slotR);
     count_launch();
-    pack_kernel<T, NPW><<<gsz(n * k), 256, 0, s>>>(R, n, k, Zb[2], Zp, 1, kpad, vexp + slotR);
+    pack_kernel<T, NPW><<<gsz(kpad / 2 * k), 256, 0, s>>>(R, n, k, c2(Zb[2]), Zp, kpad, vexp + slotR);
     count_launch();
-    for (int64_t i = 0; i < k; ++i) gh[i] = (float)ritz[i];
-    CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * k, cudaMemcpyHostToDevice, s));
+    for (int64_t i = 0; i < k; ++i) gh[2 * i] = gh[2 * i + 1] = (float)ritz[i];
+    CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * k2, cudaMemcpyHostToDevice, s));
     Epi ep{};
-    ep.mode = 2; ep.n = n; ep.k = k; ep.kpad = kpad; ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam; ep.err = err;
+    ep.mode = 2; ep.n2 = n2; ep.k2 = k2; ep.kpad = kpad; ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam; ep.err = err;
     ep.vexp_in = vexp + slotR;
     ep.amax_out = amax + slotS;
     sk(ep);
-    CB_TRY((apply<SCH, BNT, FL>)(P, mZ, ep, s));
-    CB_CUDA(cudaMemsetAsync(Zb[0], 0, sizeof(float2) * n2 * k, s));
-    scale_pack_kernel<T, NPW><<<gsz(n * k), 256, 0, s>>>(src, n, k, (float)al[0], Zb[1], expl ? Tp : Zp, kpad,
-                                                          amax + slotS, amax + slotZ(1), vexp + slotZ(1));
+    CB_TRY(apply<SCH>(P, Zp, k2, ep, s));
+    CB_CUDA(cudaMemsetAsync(Zb[0], 0, sizeof(float) * n2 * k2, s));
+    scale_pack_kernel<T, NPW><<<gsz(n * k2), 256, 0, s>>>(c2(src), n, k2, (float)al[0], c2(Zb[1]), expl ? Tp : Zp,
+                                                           kpad, amax + slotS, amax + slotZ(1), vexp + slotZ(1));
     count_launch();
     CB_LAUNCH();
     j0 = 1;
@@ -996,7 +1170,7 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     int64_t kj = 0;
     while (kj < k && degs[kj] >= j + 1) ++kj;
     Epi ep{};
-    ep.mode = 1; ep.h2 = 1; ep.n = n; ep.k = kj; ep.kpad = kpad; ep.err = err;
+    ep.mode = 1; ep.hsign = 1.0f; ep.n2 = n2; ep.k2 = 2 * kj; ep.kpad = kpad; ep.err = err;
     sk(ep);
     for (int q = 0; q < NPW; ++q) ep.out[q] = zbuf[(j + 1) % 2]->p[q];
     ep.Znext = Zb[(j + 1) % 3]; ep.Zcur = Zb[j % 3]; ep.Zprev = Zb[(j + 2) % 3];
@@ -1007,17 +1181,17 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     ep.amax_a = amax + slotZ(j);
     ep.amax_b = amax + slotZ(j);
     ep.amax_c = amax + slotZ(j > 0 ? j - 1 : 0);
-    ep.ca = (float)(std::fabs(al[j]) * L2);
+    ep.ca = (float)std::fabs(al[j]);
     ep.cb = (float)std::fabs(al[j] * c);
     ep.cc = (float)std::fabs(be[j]);
     if (corr) {
-      for (int64_t i = 0; i < kj; ++i) gh[i] = (float)(al[j] * pj[(size_t)j * k + i]);
-      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * kj, cudaMemcpyHostToDevice, s));
+      for (int64_t i = 0; i < kj; ++i) gh[2 * i] = gh[2 * i + 1] = (float)(al[j] * pj[(size_t)j * k + i]);
+      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * 2 * kj, cudaMemcpyHostToDevice, s));
       ep.src = src;
       ep.gamma = gam;
       ep.amax_d = amax + slotS;
     }
-    CB_TRY((apply<SCH, BNT, FL>)(PH2, zmap[j % 2], ep, s));
+    CB_TRY(apply<SCH>(PH2, *zbuf[j % 2], k2, ep, s));
     if (fs) {
       fs->flops += 32.0 * (double)n * (double)n * (double)kj;  // the product with the blocks of H^2
       fs->launches += 1;
@@ -1027,17 +1201,17 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     int64_t kj = 0;
     while (kj < k && degs[kj] >= j + 1) ++kj;
     Epi e1p{};
-    e1p.mode = 0; e1p.n = n; e1p.k = kj; e1p.kpad = P.kpad; e1p.err = err;
+    e1p.mode = 0; e1p.n2 = n2; e1p.k2 = 2 * kj; e1p.kpad = P.kpad; e1p.err = err;
     sk(e1p);
     for (int q = 0; q < NPW; ++q) e1p.out[q] = Tp.p[q];
     e1p.vexp_in = vexp + slotZ(j);
     e1p.vexp_out = vexp + slotT(j);
     e1p.amax_out = amax + slotT(j);
     e1p.amax_a = amax + slotZ(j);
-    e1p.ca = L;
-    CB_TRY((apply<SCH, BNT, FL>)(P, mZ, e1p, s));  // T = H Z_j
+    e1p.ca = 1.0f;
+    CB_TRY(apply<SCH>(P, Zp, k2, e1p, s));  // T = M Z_j
     Epi e2p{};
-    e2p.mode = 1; e2p.n = n; e2p.k = kj; e2p.kpad = P.kpad; e2p.err = err;
+    e2p.mode = 1; e2p.hsign = -1.0f; e2p.n2 = n2; e2p.k2 = 2 * kj; e2p.kpad = P.kpad; e2p.err = err;
     sk(e2p);
     for (int q = 0; q < NPW; ++q) e2p.out[q] = Zp.p[q];
     e2p.Znext = Zb[(j + 1) % 3]; e2p.Zcur = Zb[j % 3]; e2p.Zprev = Zb[(j + 2) % 3];
@@ -1048,17 +1222,17 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     e2p.amax_a = amax + slotT(j);
     e2p.amax_b = amax + slotZ(j);
     e2p.amax_c = amax + slotZ(j > 0 ? j - 1 : 0);
-    e2p.ca = (float)(std::fabs(al[j]) * L);
+    e2p.ca = (float)std::fabs(al[j]);
     e2p.cb = (float)std::fabs(al[j] * c);
     e2p.cc = (float)std::fabs(be[j]);
     if (corr) {
-      for (int64_t i = 0; i < kj; ++i) gh[i] = (float)(al[j] * pj[(size_t)j * k + i]);
-      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * kj, cudaMemcpyHostToDevice, s));
+      for (int64_t i = 0; i < kj; ++i) gh[2 * i] = gh[2 * i + 1] = (float)(al[j] * pj[(size_t)j * k + i]);
+      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * 2 * kj, cudaMemcpyHostToDevice, s));
       e2p.src = src;
       e2p.gamma = gam;
       e2p.amax_d = amax + slotS;
     }
-    CB_TRY((apply<SCH, BNT, FL>)(P, mT, e2p, s));  // Z_{j+1} = alpha (H T - c Z_j) + beta Z_{j-1} (+ source)
+    CB_TRY(apply<SCH>(P, Tp, k2, e2p, s));  // Z_{j+1} = alpha (-M T - c Z_j) + beta Z_{j-1} (+ source)
     if (fs) {
       fs->flops += 64.0 * (double)n * (double)n * (double)kj;
       fs->launches += 2;
@@ -1077,7 +1251,8 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
   CB_TRY(ws.alloc(&dcoef, k));
   CB_CUDA(cudaMemcpyAsync(dsel, sel.data(), sizeof(int) * k, cudaMemcpyHostToDevice, s));
   CB_CUDA(cudaMemcpyAsync(dcoef, coef.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
-  combine_kernel<<<gsz(n2 * k), 256, 0, s>>>(out, Zb[0], Zb[1], Zb[2], dsel, corr ? dcoef : nullptr, Y0, n2, k);
+  combine_kernel<<<gsz(n * k), 256, 0, s>>>(out, c2(Zb[0]), c2(Zb[1]), c2(Zb[2]), dsel, corr ? dcoef : nullptr, Y0, n,
+                                           k);
   count_launch();
   CB_LAUNCH();
   int herr = 0;
@@ -1106,32 +1281,16 @@ bool mixed_available() {
   return major == 10 && minor == 3 && tc::encode_fn() != nullptr;
 }
 
-// Output tiles of 128 columns.  (Measured alternatives, degree-20 calls at n = 4096,
-// k = 260 and degree-4 calls at n = 16384, k = 1300: 256-wide tiles with K blocks of 32
-// in a 4-stage ring and all products in two alternating buffers drained every 4 K
-// blocks ran 9 % faster at n = 16384 but missed the 1e-5 filter gate (1.3e-5 at
-// n = 4096); drained after every K block they ran 10-17 % slower.  Draining the 128-wide
-// x0 * y0 buffers every 1 or 2 K blocks instead of 4 cost 4-8 % and did not lower the
-// error, which the 22-bit pieces and the recurrence set: 8.9e-6 at n = 4096 and
-// 7.6e-6 at n = 16384 against the FP64 oracle.)
-template <int SCH>
-static int filter_dispatch(const cplx* A, const cplx* B, int64_t n, cplx* V, int64_t k, const int* degs,
-                           double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
-                           cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
-  return tc::filter_impl<SCH, 128, tc::Scheme<SCH>::FLUSH>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R,
-                                                            s, fs, P2, Q2);
-}
-
 static int filter_scheme(int scheme, const cplx* A, const cplx* B, int64_t n, cplx* V, int64_t k, const int* degs,
                          double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
                          cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
   switch (scheme) {
     case SCHEME_BF16X3:
-      return filter_dispatch<tc::SCH_BF16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return tc::filter_impl<tc::SCH_BF16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
     case SCHEME_BF16X6:
-      return filter_dispatch<tc::SCH_BF16X6>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return tc::filter_impl<tc::SCH_BF16X6>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
     case SCHEME_FP16X3:
-      return filter_dispatch<tc::SCH_FP16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return tc::filter_impl<tc::SCH_FP16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
     default:
       return CHASE_BSE_BAD_ARG;
   }
