@@ -190,13 +190,13 @@ bool verbose() {
 }
 
 // ------------------------------------------------------------------- filter
-// nxt = alpha (HT - c cur) + beta prev over `total` entries (the recurrence step of the
-// FP64 filter whose H applications ran as sliced tensor-core GEMMs)
-__global__ void cheb_combine_kernel(cplx* nxt, const cplx* HT, const cplx* cur, const cplx* prev, double alpha,
+// nxt = alpha (H^2 cur - c cur) + beta prev over `total` entries of the J-fixed halves, from
+// U = P'(-i P'cur): H^2 z = i U (the recurrence step of the filter on sliced products)
+__global__ void cheb_combine_kernel(cplx* nxt, const cplx* U, const cplx* cur, const cplx* prev, double alpha,
                                     double beta, double c, int64_t total) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const cplx h = HT[i], y = cur[i];
-    cplx z = mk(alpha * (h.x - c * y.x), alpha * (h.y - c * y.y));
+    const cplx u = U[i], y = cur[i];
+    cplx z = mk(alpha * (-u.y - c * y.x), alpha * (u.x - c * y.y));
     if (beta != 0.0) {
       const cplx p = prev[i];
       z.x = fma(beta, p.x, z.x);
@@ -209,19 +209,39 @@ __global__ void cheb_combine_kernel(cplx* nxt, const cplx* HT, const cplx* cur, 
 // FP64 three-term recurrence on H^2 over columns sorted by descending degree:
 // at step j only the prefix of columns with deg >= j+1 is active.  Y_j lives in
 // buffer j mod 3; a finished column keeps its last iterate in buffer deg mod 3.
-// With ph (the sliced operand of slice_hamiltonian) both H applications of a step run
-// as FP64-accurate sliced GEMMs on the tensor cores, else on the FP64 pipe (the second
-// one with the recurrence fused).
+// With ph (the sliced operand P' of slice_hamiltonian) both H applications of a step run
+// as FP64-accurate sliced GEMMs on the tensor cores, and the whole recurrence on the J-fixed
+// halves z of the vectors (two columns each): H [z; conj z] = i [z'; conj z'] with
+// z' = -i P'z, so the second product takes the first one's result as pairs (b, -a) and no
+// step leaves that form.  Else on the FP64 pipe (the second one with the recurrence fused).
 static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0, int64_t k, const int* degs,
                               double mu1, double mu_nevex, double muN, cplx* out, Workspace& ws, cudaStream_t s,
                               FilterStats* fs, const SlicedOp* ph) {
   const int64_t n2 = 2 * n;
-  cplx *Y1, *Y2, *T, *HT = nullptr;
+  cplx *Y1, *Y2, *T, *U = nullptr;
+  int* err = nullptr;
+  SlicedOp sz;
   CB_TRY(ws.alloc(&Y1, n2 * k));
   CB_TRY(ws.alloc(&Y2, n2 * k));
   CB_TRY(ws.alloc(&T, n2 * k));
-  if (ph) CB_TRY(ws.alloc(&HT, n2 * k));
   cplx* Yb[3] = {Y0, Y1, Y2};
+  if (ph) {
+    CB_TRY(ws.alloc(&U, n2 * k));
+    CB_TRY(ws.alloc(&Yb[0], n2 * k));
+    CB_TRY(ws.alloc(&err, 1));
+    CB_TRY(sliced_alloc(ws, sz, 2 * k, n2, s));
+    CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+    CB_TRY(jsplit(Y0, n, k, Yb[0], s));
+  }
+  // out (complex n x 2 kj) = P' in, the pairs of `in` taken by mode
+  auto product = [&](const cplx* in, int mode, cplx* o, int64_t kj) -> int {
+    const int64_t tid = timer_begin(2, 32.0 * (double)n * (double)n * (double)kj, s);
+    sz.rows = 2 * kj;
+    CB_TRY(slice_rows(reinterpret_cast<const double*>(in), n2, mode, sz, s));
+    CB_TRY(sliced_gemm(*ph, sz, 1.0, reinterpret_cast<double*>(o), 1, n2, false, s, err));
+    timer_end(tid, s);
+    return CHASE_BSE_OK;
+  };
   const double a = mu_nevex * mu_nevex, b = muN * muN;
   const double c = 0.5 * (a + b), e = 0.5 * (b - a);
   const double sigma1 = e / (mu1 * mu1 - c);
@@ -239,7 +259,7 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
     cplx* nxt = Yb[(j + 1) % 3];
     cplx* prev = Yb[(j + 2) % 3];
     if (ph) {
-      CB_TRY(hop_sliced(*ph, cur, n, kj, T, s));
+      CB_TRY(product(cur, 0, T, kj));
     } else {
       HopArgs h{};
       h.A = A; h.B = B; h.n = n; h.W = cur; h.k = kj; h.out = T; h.mode = HOP_STORE;
@@ -256,10 +276,10 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
       sigma = sn;
     }
     if (ph) {
-      CB_TRY(hop_sliced(*ph, T, n, kj, HT, s));
+      CB_TRY(product(T, 1, U, kj));
       const int64_t total = n2 * kj;
       const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, 8192);
-      cheb_combine_kernel<<<blocks, 256, 0, s>>>(nxt, HT, cur, prev, alpha, beta, c, total);
+      cheb_combine_kernel<<<blocks, 256, 0, s>>>(nxt, U, cur, prev, alpha, beta, c, total);
       count_launch();
       CB_LAUNCH();
     } else {
@@ -280,7 +300,19 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
   int* dsel;
   CB_TRY(ws.alloc(&dsel, k));
   CB_CUDA(cudaMemcpyAsync(dsel, sel.data(), sizeof(int) * k, cudaMemcpyHostToDevice, s));
-  CB_TRY(collect_cols(out, Yb[0], Yb[1], Yb[2], dsel, n2, k, s));
+  if (ph) {
+    CB_TRY(jmerge(out, Yb[0], Yb[1], Yb[2], dsel, n, k, s));
+    int herr = 0;
+    CB_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CB_CUDA(cudaStreamSynchronize(s));
+    if (herr) {
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      return CHASE_BSE_DEVICE_TIMEOUT;
+    }
+  } else {
+    CB_TRY(collect_cols(out, Yb[0], Yb[1], Yb[2], dsel, n2, k, s));
+  }
   if (fs) {
     CB_CUDA(cudaEventSynchronize(e1));
     float ms = 0;
@@ -865,6 +897,29 @@ int residuals(const cplx* A, const cplx* B, int64_t n, const cplx* W, const doub
   return CHASE_BSE_OK;
 }
 
+// The residual check of a caller's pairs.  FP64 products run at 1/64 of the FP32 rate, so H W is
+// a sliced product (error against 64 bits no larger) where it is faster: the pipe takes
+// 1.43e-5 us n^2 k + 45 us, the sliced path 3.6e-5 us n^2 for H's digits + 120 us.  A workspace that
+// cannot be had also leaves it to the pipe.  Measured on one GB300: n = 4096, k = 200
+// 47.8 -> 1.72 ms; k = 8 2.03 -> 0.71 ms; n = 1024, k = 16 0.29 -> 0.15 ms; n = 512, k = 50
+// 0.27 -> 0.13 ms.
+static bool residual_sliced_faster(int64_t n, int64_t k) {
+  const double n2 = (double)n * (double)n;
+  return 1.43e-5 * n2 * (double)k > 4.0e-5 * n2 + 100.0;
+}
+int residuals_check(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k,
+                    double* res, cudaStream_t s) {
+  if (k > 0 && residual_sliced_faster(n, k) && mixed_available()) {
+    Workspace ws(s);
+    cplx* R;
+    int st = ws.alloc(&R, 2 * n * k);
+    if (st == CHASE_BSE_OK) st = residual_sliced(A, B, n, W, lambda, k, R, ws, s);
+    if (st == CHASE_BSE_OK) return col_norms(R, 2 * n, k, res, s);
+    if (st != CHASE_BSE_OOM) return st;
+  }
+  return residuals(A, B, n, W, lambda, k, res, s);
+}
+
 int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, cplx* gB, cudaStream_t s) {
   Workspace ws(s);
   cplx *Uc, *U2, *Ub, *U3;
@@ -882,13 +937,20 @@ int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, c
     double* tmp;
     CB_TRY(sliced_alloc(ws, sa, 2 * n, 4 * nev, s));
     CB_TRY(sliced_alloc(ws, sb, n, 4 * nev, s));
+    int* err;
     CB_TRY(ws.alloc(&tmp, 8 * n * nev));
+    CB_TRY(ws.alloc(&err, 1));
+    CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     CB_TRY(slice_complex_rows(Uc, n, n, 2 * nev, tmp, sa, s));
     CB_TRY(slice_plain_rows(U2, n, sb, s));
-    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gA), 1, 2 * n, false, s));
+    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gA), 1, 2 * n, false, s, err));
     CB_TRY(slice_complex_rows(Ub, n, n, 2 * nev, tmp, sa, s));
     CB_TRY(slice_plain_rows(U3, n, sb, s));
-    return sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gB), 1, 2 * n, false, s);
+    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gB), 1, 2 * n, false, s, err));
+    int herr = 0;
+    CB_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CB_CUDA(cudaStreamSynchronize(s));
+    return herr ? CHASE_BSE_DEVICE_TIMEOUT : CHASE_BSE_OK;
   }
   CB_TRY(zgemm('N', 'T', n, n, 2 * nev, mk(1, 0), Uc, n, U2, n, mk(0, 0), gA, n, s));
   CB_TRY(zgemm('N', 'T', n, n, 2 * nev, mk(1, 0), Ub, n, U3, n, mk(0, 0), gB, n, s));

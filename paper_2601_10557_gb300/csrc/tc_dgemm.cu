@@ -1,6 +1,7 @@
 // FP64-accurate sliced GEMM on tcgen05 tensor cores (see tc_dgemm.cuh).
 //
-// Kernel (one CTA per 128 x 32 output tile and K split, 384 threads):
+// Kernel (persistent CTAs of 384 threads, each working through 128 x 32 output tiles, or K
+// splits of them; the ring and the two accumulator buffers run on from one tile to the next):
 //   warp 0    TMA producer: per 32-long K block, all 7 digit planes of the A tile
 //             (one 3-D box of 32 x 128 x 7) and of the B tile (32 x 32 x 7), 64-byte
 //             swizzle, into a 3-stage ring (70 KB per stage)
@@ -12,10 +13,16 @@
 //   warps 4-11 drain each finished buffer (warps 4-7 columns 0-15, warps 8-11
 //             columns 16-31 of every group): the exact integer group sums of
 //             weights 2^0 .. 2^-24 into one 64-bit integer per output, those of
-//             2^-32 .. 2^-48 into a second one; at the end they write both to a
-//             per-split partial tile
-// A second kernel sums the splits in order, applies the row and column exponents
-// and writes the FP64 result with arbitrary strides.
+//             2^-32 .. 2^-48 into a second one; at the end they round their exact sum
+//             to FP64, apply the row and column exponents and write the result with
+//             arbitrary strides, while the next tile's MMAs run (with a K split: both
+//             integers to a partial tile, and a second kernel sums the splits)
+// Bound: shared memory.  A K step of 16 reads 56 KB of operand digits in 448 MMA cycles
+// (128 bytes a cycle) while the ring takes in 78 bytes a cycle.  Measured on one GB300,
+// before (one CTA per tile, int64 partial tiles of every product) and after: the two
+// products of the gradient at n = 8192 (16384 x 8192, K = 400) 11.7 -> 6.35 ms; the FP64_TC
+// filter of 130 vectors at n = 2048 (24 products 4096 x 260, K = 4096, their slices and the
+// recurrence) 8.1 -> 5.1 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -61,18 +68,57 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
   return d;
 }
 
+// Exponent of an operand row with an infinity or a NaN: its products are NaN.
+constexpr int EXP_NONFINITE = 1 << 20;
+
 struct Args {
   int num_m, num_n, kb_total, kb_per_split;
+  int items;           // tiles x splits
   int n_fast;          // raster: the CTAs of one A tile (1) or of one B tile (0) run together
   int64_t mp;          // rows of a partial tile column (A rows_pad)
   int64_t np;          // columns per split (B rows_pad)
-  long long* hi;       // [split][col][row]
+  long long* hi;       // [split][col][row]; NULL: one split, the tiles go to out
   long long* lo;
+  const int* ea;       // row and column exponents
+  const int* eb;
+  int64_t M, N;
+  double alpha;
+  double* out;
+  int64_t rs, cs;
+  int neg_odd;
   int* err;
 };
 
+// (h 2^24 + l) 2^(e - 62) rounded once to FP64 (to nearest, ties to even): the sum and the
+// rounding in integers, whose pipe is 32 times as wide as the FP64 one
+__device__ __forceinline__ double fold(long long h, long long l, int e) {
+  const __int128 sum = ((__int128)h << 24) + l;
+  if (sum == 0) return 0.0;
+  unsigned __int128 a = sum < 0 ? (unsigned __int128)(-sum) : (unsigned __int128)sum;
+  const unsigned long long up = (unsigned long long)(a >> 64);
+  const int lz = up ? __clzll((long long)up) : 64 + __clzll((long long)(unsigned long long)a);
+  a <<= lz;
+  const unsigned long long top = (unsigned long long)(a >> 64), low = (unsigned long long)a;
+  unsigned long long m = top >> 11;  // 53 bits, the leading one among them
+  const unsigned long long rem = top & 0x7ff;
+  m += (rem > 0x400 || (rem == 0x400 && (low != 0 || (m & 1)))) ? 1 : 0;
+  // the leading bit weighs 2^(127 - lz); a carry out of m raises the exponent by itself
+  const int x = 127 - lz - 48, x1 = x + e - 14;
+  const unsigned long long sign = sum < 0 ? 1ull << 63 : 0ull;
+  if (x1 > -1022 && x1 < 1023) return __longlong_as_double((long long)(sign | (((unsigned long long)(x1 + 1022) << 52) + m)));
+  return ldexp(__longlong_as_double((long long)(sign | (((unsigned long long)(x + 1022) << 52) + m))), e - 14);
+}
+__device__ __forceinline__ void put_out(const Args& g, int64_t r, int64_t c, long long h, long long l) {
+  const int ea = g.ea[r], eb = g.eb[c];
+  double y = max(ea, eb) >= EXP_NONFINITE ? nan("") : fold(h, l, ea + eb);
+  if (g.alpha != 1.0) y *= g.alpha;
+  if (g.neg_odd && (r & 1)) y = -y;
+  g.out[r * g.rs + c * g.cs] = y;
+}
+
 __global__ void __launch_bounds__(THREADS, 1)
-    sliced_gemm_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, Args g) {
+    sliced_gemm_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
+                       const __grid_constant__ Args g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ST * STAGE_BYTES);
@@ -92,12 +138,14 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   // the CTAs sharing a tile of the larger operand run together, so that it is read
   // from DRAM once and the other operand's tiles come from L2
-  const int bid = blockIdx.x;
-  const int mt = g.n_fast ? (bid / g.num_n) % g.num_m : bid % g.num_m;
-  const int nt = g.n_fast ? bid % g.num_n : (bid / g.num_m) % g.num_n;
-  const int sp = bid / (g.num_m * g.num_n);
-  const int kb0 = sp * g.kb_per_split;
-  const int nkb = min(g.kb_per_split, g.kb_total - kb0);
+  auto item = [&](int id, int& mt, int& nt, int& sp, int& kb0, int& nkb) {
+    mt = g.n_fast ? (id / g.num_n) % g.num_m : id % g.num_m;
+    nt = g.n_fast ? id % g.num_n : (id / g.num_m) % g.num_n;
+    sp = id / (g.num_m * g.num_n);
+    kb0 = sp * g.kb_per_split;
+    nkb = min(g.kb_per_split, g.kb_total - kb0);
+  };
+  int mt, nt, sp, kb0, nkb;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; ++s) {
@@ -126,28 +174,44 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t sbase = smem_u32(smem);
 
   if (warp == 0 && lane == 0) {
-    int issued = 0;
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % ST;
-      const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-      if (kb >= ST && !mbar_wait(empty[s], ph ^ 1u, abort_sh, g.err, true)) break;
-      const uint32_t st = sbase + s * STAGE_BYTES;
-      mbar_expect_tx(full[s], STAGE_BYTES);
-      tma_load_3d(st, &ma, (kb0 + kb) * BK, mt * BM, 0, full[s]);
-      tma_load_3d(st + S * A_SLICE, &mb, (kb0 + kb) * BK, nt * BNS, 0, full[s]);
-      issued = kb + 1;
+    int issued = 0, s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int id = blockIdx.x; ok && id < g.items; id += gridDim.x) {
+      item(id, mt, nt, sp, kb0, nkb);
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (issued >= ST && !mbar_wait(empty[0] + 8 * s, ph ^ 1u, abort_sh, g.err, true)) {
+          ok = false;
+          break;
+        }
+        const uint32_t st = sbase + s * STAGE_BYTES;
+        mbar_expect_tx(full[0] + 8 * s, STAGE_BYTES);
+        tma_load_3d(st, &ma, (kb0 + kb) * BK, mt * BM, 0, full[0] + 8 * s);
+        tma_load_3d(st + S * A_SLICE, &mb, (kb0 + kb) * BK, nt * BNS, 0, full[0] + 8 * s);
+        ++issued;
+        if (++s == ST) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
     }
     *issued_sh = issued;
   } else if (warp == 1 && lane == 0) {
     const uint64_t dbase = sdesc64(sbase);
+    int s = 0, grp = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int id = blockIdx.x; ok && id < g.items; id += gridDim.x) {
+    item(id, mt, nt, sp, kb0, nkb);
     for (int kb = 0; kb < nkb; ++kb) {
-      const int grp = kb / CHUNK, b = grp & 1;
+      const int b = grp & 1;
       const bool first = (kb % CHUNK) == 0;
       const bool last = (kb % CHUNK) == CHUNK - 1 || kb == nkb - 1;
-      if (first && grp >= 2 && !mbar_wait(acce[b], (uint32_t)((grp >> 1) - 1) & 1u, abort_sh, g.err, true)) break;
-      const int s = kb % ST;
-      const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-      if (!mbar_wait(full[s], ph, abort_sh, g.err, true)) break;
+      if ((first && grp >= 2 && !mbar_wait(acce[b], (uint32_t)((grp >> 1) - 1) & 1u, abort_sh, g.err, true)) ||
+          !mbar_wait(full[0] + 8 * s, ph, abort_sh, g.err, true)) {
+        ok = false;
+        break;
+      }
       tc_fence_after();
       const uint32_t st = sbase + s * STAGE_BYTES;
       const uint32_t buf = tmem + (uint32_t)(b * GCOLS);
@@ -164,8 +228,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           mma_bf16(buf + (uint32_t)(t * BNS), ad, bd, idesc_n((S - t) * BNS), acc);
         }
       }
-      mma_commit(empty[s]);
-      if (last) mma_commit(accf[b]);
+      mma_commit(empty[0] + 8 * s);
+      if (last) {
+        mma_commit(accf[b]);
+        ++grp;
+      }
+      if (++s == ST) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
     }
     mma_commit(done);
   } else if (warp >= 4) {
@@ -173,15 +245,18 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int q = warp & 3, half = (warp - 4) >> 2;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     constexpr int NC = BNS / 2;
+    bool ok = true;
+    int grp0 = 0;
+    for (int id = blockIdx.x; ok && id < g.items; id += gridDim.x) {
+    item(id, mt, nt, sp, kb0, nkb);
     long long hi[NC], lo[NC];
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
       hi[i] = 0;
       lo[i] = 0;
     }
-    bool ok = true;
     const int ngrp = (nkb + CHUNK - 1) / CHUNK;
-    for (int grp = 0; grp < ngrp; ++grp) {
+    for (int grp = grp0; grp < grp0 + ngrp; ++grp) {
       const int b = grp & 1;
       const bool w = mbar_wait(accf[b], (uint32_t)(grp >> 1) & 1u, abort_sh, g.err, true);
       if (!__all_sync(0xffffffffu, w)) {
@@ -224,14 +299,23 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(acce[b]);
     }
+    grp0 += ngrp;
     if (ok && !*abort_sh) {
       const int64_t row = (int64_t)mt * BM + q * 32 + lane;  // < mp: rows are padded to whole tiles
-      const int64_t base = ((int64_t)sp * g.np + (int64_t)nt * BNS + half * NC) * g.mp + row;
+      const int64_t col = (int64_t)nt * BNS + half * NC;
+      if (g.hi) {
+        const int64_t base = ((int64_t)sp * g.np + col) * g.mp + row;
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        g.hi[base + (int64_t)i * g.mp] = hi[i];
-        g.lo[base + (int64_t)i * g.mp] = lo[i];
+        for (int i = 0; i < NC; ++i) {
+          g.hi[base + (int64_t)i * g.mp] = hi[i];
+          g.lo[base + (int64_t)i * g.mp] = lo[i];
+        }
+      } else if (row < g.M) {
+#pragma unroll
+        for (int i = 0; i < NC; ++i)
+          if (col + i < g.N) put_out(g, row, col + i, hi[i], lo[i]);
       }
+    }
     }
   }
   tc_fence_before();
@@ -252,24 +336,19 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-__global__ void sliced_finalize_kernel(const long long* hi, const long long* lo, int splits, int64_t mp, int64_t np,
-                                       const int* ea, const int* eb, int64_t M, int64_t N, double alpha,
-                                       double* out, int64_t rs, int64_t cs, int neg_odd) {
-  const int64_t total = M * N;
+// The sum of the splits' integers
+__global__ void sliced_finalize_kernel(const __grid_constant__ Args g, int splits) {
+  const int64_t total = g.M * g.N;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = idx % M, c = idx / M;
+    const int64_t r = idx % g.M, c = idx / g.M;
     long long h = 0, l = 0;
     for (int sp = 0; sp < splits; ++sp) {
-      const int64_t o = ((int64_t)sp * np + c) * mp + r;
-      h += hi[o];
-      l += lo[o];
+      const int64_t o = ((int64_t)sp * g.np + c) * g.mp + r;
+      h += g.hi[o];
+      l += g.lo[o];
     }
-    // exact when |h|, |l| < 2^53; one rounding for the sum
-    const double v = fma((double)l, 0x1p-48, (double)h * 0x1p-24);
-    double y = alpha * ldexp(v, ea[r] + eb[c] - 14);
-    if (neg_odd && (r & 1)) y = -y;
-    out[r * rs + c * cs] = y;
+    put_out(g, r, c, h, l);
   }
 }
 
@@ -305,37 +384,79 @@ __device__ __forceinline__ void int_digits(double x, int e, int* d) {
 __device__ __forceinline__ int row_exponent(unsigned long long mbits) {
   if (mbits == 0) return 0;
   const int ef = (int)(mbits >> 52);
+  if (ef == 0x7ff) return EXP_NONFINITE;
   if (ef) return ef - 1022;
   return (64 - __clzll((long long)mbits)) - 1074;  // subnormal
 }
-template <class Src>
-__global__ void slice_kernel(Src src, int64_t rows, int64_t K, int64_t kpad, int64_t plane, __nv_bfloat16* planes,
-                             int* exps) {
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (r >= rows) return;
-  unsigned long long m = 0;
-  for (int64_t p = lane; 2 * p < K; p += 32) {
-    const double2 v = src.pair(r, p);
-    const unsigned long long a0 = (unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull;
-    const unsigned long long a1 = (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull;
-    m = max(m, max(a0, a1));
-  }
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const int e = row_exponent(m);
-  __nv_bfloat16* row = planes + r * kpad;
-  for (int64_t p = lane; 2 * p < kpad; p += 32) {
-    double2 v = make_double2(0.0, 0.0);
-    if (2 * p < K) v = src.pair(r, p);
-    int d0[S], d1[S];
-    int_digits(v.x, e, d0);
-    int_digits(v.y, e, d1);
+__device__ __forceinline__ unsigned long long abs_bits(double2 v) {
+  const unsigned long long a0 = (unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull;
+  const unsigned long long a1 = (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull;
+  return max(a0, a1);
+}
+__device__ __forceinline__ void put_digits(double2 v, int e, __nv_bfloat16* p, int64_t plane) {
+  int d0[S], d1[S];
+  int_digits(v.x, e, d0);
+  int_digits(v.y, e, d1);
 #pragma unroll
-    for (int t = 0; t < S; ++t)
-      *reinterpret_cast<__nv_bfloat162*>(row + t * plane + 2 * p) =
-          __halves2bfloat162(__int2bfloat16_rn(d0[t]), __int2bfloat16_rn(d1[t]));
+  for (int t = 0; t < S; ++t)
+    *reinterpret_cast<__nv_bfloat162*>(p + t * plane) =
+        __halves2bfloat162(__int2bfloat16_rn(d0[t]), __int2bfloat16_rn(d1[t]));
+}
+// max over the CTA of one value per thread (blockDim.x a multiple of 32)
+__device__ __forceinline__ unsigned long long cta_max(unsigned long long m) {
+  __shared__ unsigned long long w[32];
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = m;
+  __syncthreads();
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = max(m, w[i]);
+  __syncthreads();
+  return m;
+}
+// One CTA per row (32 to 256 threads by its length: a block of vectors has too few rows to
+// occupy the GPU with one warp each).
+template <class Src>
+__global__ void slice_kernel(Src src, int64_t K, int64_t kpad, int64_t plane, __nv_bfloat16* planes, int* exps) {
+  const int64_t r = blockIdx.x;
+  unsigned long long m = 0;
+  for (int64_t p = threadIdx.x; 2 * p < K; p += blockDim.x) m = max(m, abs_bits(src.pair(r, p)));
+  const int e = row_exponent(cta_max(m));
+  __nv_bfloat16* row = planes + r * kpad;
+  for (int64_t p = threadIdx.x; 2 * p < kpad; p += blockDim.x)
+    put_digits(2 * p < K ? src.pair(r, p) : make_double2(0.0, 0.0), e, row + 2 * p, plane);
+  if (threadIdx.x == 0) exps[r] = e;
+}
+// The real form P' of rows i0 .. of H, one CTA per row i, which gives rows 2i and 2i + 1 from
+// one read of A and B each pass: y = A x + B conj(x) in (re, im) interleaved form,
+// Re y: (Ar + Br, Bi - Ai), Im y: (Ai + Bi, Ar - Br).  The FP64 additions (4 per entry and pass)
+// take as long as the memory traffic.  The residual check of 8 vectors at n = 4096, most of it
+// these digits, 1.11 -> 0.71 ms against one warp per row of P'.
+__global__ void slice_ham_kernel(const cplx* A, const cplx* B, int64_t n, int64_t kpad, int64_t plane,
+                                 __nv_bfloat16* planes, int* exps) {
+  const int64_t i = blockIdx.x;
+  const cplx *Ai = A + i * n, *Bi = B + i * n;
+  unsigned long long m0 = 0, m1 = 0;
+#pragma unroll 2
+  for (int64_t l = threadIdx.x; l < n; l += blockDim.x) {
+    const cplx a = Ai[l], b = Bi[l];
+    m0 = max(m0, abs_bits(make_double2(a.x + b.x, b.y - a.y)));
+    m1 = max(m1, abs_bits(make_double2(a.y + b.y, a.x - b.x)));
   }
-  if (lane == 0) exps[r] = e;
+  const int e0 = row_exponent(cta_max(m0)), e1 = row_exponent(cta_max(m1));
+  __nv_bfloat16* row = planes + 2 * i * kpad;
+  for (int64_t l = threadIdx.x; 2 * l < kpad; l += blockDim.x) {
+    double2 v0 = make_double2(0.0, 0.0), v1 = v0;
+    if (l < n) {
+      const cplx a = Ai[l], b = Bi[l];
+      v0 = make_double2(a.x + b.x, b.y - a.y);
+      v1 = make_double2(a.y + b.y, a.x - b.x);
+    }
+    put_digits(v0, e0, row + 2 * l, plane);
+    put_digits(v1, e1, row + kpad + 2 * l, plane);
+  }
+  if (threadIdx.x == 0) {
+    exps[2 * i] = e0;
+    exps[2 * i + 1] = e1;
+  }
 }
 
 struct RowsSrc {  // row r at p + r * ld, pairs transformed by mode
@@ -360,18 +481,6 @@ struct RowsSrcUnaligned {  // same, for an odd ld or offset
     return make_double2(a, b);
   }
 };
-struct HamSrc {  // rows of P': y = A x + B conj(x) in (re, im) interleaved form
-  const cplx* A;
-  const cplx* B;
-  int64_t n;
-  __device__ double2 pair(int64_t r, int64_t l) const {
-    const int64_t i = r >> 1;
-    const cplx a = A[i * n + l], b = B[i * n + l];
-    if ((r & 1) == 0) return make_double2(a.x + b.x, b.y - a.y);  // Re y: (Re x, Im x) coefficients
-    return make_double2(a.y + b.y, a.x - b.x);                    // Im y
-  }
-};
-
 // The blocks of H^2 as C = [A | -B] R, R = [[A, B], [conj B, conj A]], computed as
 // C^T = R^T [A | -B]^T so that the result lands row-major: the A operand holds the
 // real-form rows of the columns j0 + r/2 of R's left (part 0: P2) or right (part 1: Q2)
@@ -465,6 +574,34 @@ __global__ void jcombine_kernel(const cplx* T, int64_t n, int64_t k, cplx* out) 
   }
 }
 
+// W (2n x k) from the halves in the columns 2v, 2v + 1 of the block Zsel[v]
+__global__ void jmerge_kernel(cplx* W, const cplx* Z0, const cplx* Z1, const cplx* Z2, const int* sel, int64_t n,
+                              int64_t k) {
+  const int64_t total = n * k;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % n, j = idx / n;
+    const cplx* Z = sel[j] == 0 ? Z0 : (sel[j] == 1 ? Z1 : Z2);
+    const cplx a = Z[2 * j * n + i], c = Z[(2 * j + 1) * n + i];
+    W[j * 2 * n + i] = mk(a.x + c.y, a.y - c.x);       // a - i c
+    W[j * 2 * n + n + i] = mk(a.x - c.y, -a.y - c.x);  // conj(a) - i conj(c)
+  }
+}
+// R = H W - W diag(lambda) from T = [P'a_j, P'c_j]; NaN where a wait of the products ran out
+__global__ void jresidual_kernel(const cplx* T, const cplx* W, const double* lambda, int64_t n, int64_t k, cplx* R,
+                                 const int* err) {
+  const int64_t total = n * k;
+  const double bad = *err ? nan("") : 0.0;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % n, j = idx / n, o = j * 2 * n + i;
+    const cplx ta = T[(2 * j) * n + i], tc = T[(2 * j + 1) * n + i], x = W[o], y = W[o + n];
+    const double lam = lambda[j];
+    R[o] = mk(fma(-lam, x.x, ta.x + tc.y) + bad, fma(-lam, x.y, ta.y - tc.x) + bad);
+    R[o + n] = mk(fma(-lam, y.x, tc.y - ta.x), fma(-lam, y.y, ta.y + tc.x));
+  }
+}
+
 static unsigned gsz(int64_t total) {
   const int64_t b = (total + 255) / 256;
   return (unsigned)std::min<int64_t>(std::max<int64_t>(b, 1), 16384);
@@ -485,9 +622,16 @@ static int make_map3(CUtensorMap* m, const void* base, int64_t kpad, int64_t row
 
 template <class Src>
 static int run_slice(const Src& src, SlicedOp& op, cudaStream_t s) {
-  const int64_t warps = op.rows;
-  slice_kernel<Src><<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(src, op.rows, op.K, op.kpad,
-                                                                          op.rows_pad * op.kpad, op.planes, op.exps);
+  const int threads = op.K >= 4096 ? 256 : (op.K >= 512 ? 128 : 32);
+  slice_kernel<Src><<<(unsigned)op.rows, threads, 0, s>>>(src, op.K, op.kpad, op.rows_pad * op.kpad, op.planes,
+                                                          op.exps);
+  count_launch();
+  CB_LAUNCH();
+  return CHASE_BSE_OK;
+}
+// rows of H -> op.rows / 2 row pairs of P'
+static int run_slice_ham(const cplx* A, const cplx* B, int64_t n, SlicedOp& op, cudaStream_t s) {
+  slice_ham_kernel<<<(unsigned)(op.rows / 2), 256, 0, s>>>(A, B, n, op.kpad, op.rows_pad * op.kpad, op.planes, op.exps);
   count_launch();
   CB_LAUNCH();
   return CHASE_BSE_OK;
@@ -589,11 +733,52 @@ int form_h2(const cplx* A, const cplx* B, int64_t n, cplx* P2, cplx* Q2, cudaStr
 
 int slice_hamiltonian(const cplx* A, const cplx* B, int64_t n, SlicedOp& op, cudaStream_t s) {
   if (op.rows != 2 * n || op.K != 2 * n) return CHASE_BSE_BAD_ARG;
-  return tcd::run_slice(tcd::HamSrc{A, B, n}, op, s);
+  return tcd::run_slice_ham(A, B, n, op, s);
+}
+
+int jsplit(const cplx* W, int64_t n, int64_t k, cplx* Z, cudaStream_t s) {
+  tcd::jsplit_kernel<<<tcd::gsz(n * k), 256, 0, s>>>(W, n, k, Z);
+  count_launch();
+  CB_LAUNCH();
+  return CHASE_BSE_OK;
+}
+int jmerge(cplx* W, const cplx* Z0, const cplx* Z1, const cplx* Z2, const int* sel, int64_t n, int64_t k,
+           cudaStream_t s) {
+  tcd::jmerge_kernel<<<tcd::gsz(n * k), 256, 0, s>>>(W, Z0, Z1, Z2, sel, n, k);
+  count_launch();
+  CB_LAUNCH();
+  return CHASE_BSE_OK;
+}
+
+int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k, cplx* R,
+                    Workspace& ws, cudaStream_t s) {
+  // H in blocks of rows whose digits take at most 2 GB
+  int64_t m = std::max<int64_t>(64, (int64_t)(2.0e9 / (56.0 * (double)n)) / 64 * 64);
+  m = std::min(m, n);
+  cplx *Z, *T;
+  int* err;
+  SlicedOp sz, ph;
+  CB_TRY(ws.alloc(&Z, n * 2 * k));
+  CB_TRY(ws.alloc(&T, n * 2 * k));
+  CB_TRY(ws.alloc(&err, 1));
+  CB_TRY(sliced_alloc(ws, sz, 2 * k, 2 * n, s));
+  CB_TRY(sliced_alloc(ws, ph, 2 * m, 2 * n, s));
+  CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+  CB_TRY(jsplit(W, n, k, Z, s));
+  CB_TRY(slice_rows(reinterpret_cast<const double*>(Z), 2 * n, 0, sz, s));
+  for (int64_t i0 = 0; i0 < n; i0 += m) {
+    ph.rows = 2 * std::min(m, n - i0);  // a shorter last block leaves the previous one's digits behind its rows
+    CB_TRY(tcd::run_slice_ham(A + i0 * n, B + i0 * n, n, ph, s));
+    CB_TRY(sliced_gemm(ph, sz, 1.0, reinterpret_cast<double*>(T + i0), 1, 2 * n, false, s, err));
+  }
+  tcd::jresidual_kernel<<<tcd::gsz(n * k), 256, 0, s>>>(T, W, lambda, n, k, R, err);
+  count_launch();
+  CB_LAUNCH();
+  return CHASE_BSE_OK;
 }
 
 int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out, int64_t rs, int64_t cs,
-                bool neg_odd, cudaStream_t s) {
+                bool neg_odd, cudaStream_t s, int* err) {
   using namespace tcd;
   if (a.K != b.K || a.kpad != b.kpad) return CHASE_BSE_BAD_ARG;
   static bool attr = false;
@@ -607,34 +792,63 @@ int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out,
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // split K until about two CTAs per SM, keeping whole 128-long chunks per split
+  // K splits (whole 128-long chunks): the number of least estimated time, in K blocks (about
+  // 0.75 us each): waves of CTAs x (blocks of a split + 2 for the tile's end), and with a split
+  // the partial tiles' traffic (32 bytes an output and split, about 5 TB/s) and a second launch
   const int64_t tiles = (int64_t)num_m * num_n;
-  const int max_split = std::max(1, kb_total / CHUNK);
-  int splits = (int)std::min<int64_t>(max_split, std::max<int64_t>(1, (2 * sms + tiles - 1) / tiles));
-  int kb_per = (kb_total + splits - 1) / splits;
-  kb_per = ((kb_per + CHUNK - 1) / CHUNK) * CHUNK;
-  splits = (kb_total + kb_per - 1) / kb_per;
-  Workspace ws(s);
   const int64_t np = (int64_t)num_n * BNS, mp = a.rows_pad;
+  int splits = 1, kb_per = ((kb_total + CHUNK - 1) / CHUNK) * CHUNK;
+  double best = 0.0;
+  for (int want = 1; want <= std::max(1, kb_total / CHUNK) && want <= 64; ++want) {
+    const int per = ((kb_total + want - 1) / want + CHUNK - 1) / CHUNK * CHUNK;
+    const int sp = (kb_total + per - 1) / per;
+    const double waves = (double)((tiles * sp + sms - 1) / sms);
+    double t = waves * (std::min(per, kb_total) + 2.0);
+    if (sp > 1) t += 8.0 + (double)sp * (double)np * (double)mp * 32.0 / 3.75e6;
+    if (best == 0.0 || t < best * 0.98) {
+      best = t;
+      splits = sp;
+      kb_per = per;
+    }
+    if (tiles * sp > 4 * (int64_t)sms) break;
+  }
+  Workspace ws(s);
   Args g{};
   g.num_m = num_m;
   g.num_n = num_n;
   g.n_fast = a.rows_pad >= b.rows_pad ? 1 : 0;
   g.kb_total = kb_total;
   g.kb_per_split = kb_per;
+  g.items = (int)(tiles * splits);
   g.mp = mp;
   g.np = np;
-  CB_TRY(ws.alloc(&g.hi, (size_t)splits * np * mp));
-  CB_TRY(ws.alloc(&g.lo, (size_t)splits * np * mp));
-  CB_TRY(ws.alloc(&g.err, 1));
-  CB_CUDA(cudaMemsetAsync(g.err, 0, sizeof(int), s));
-  sliced_gemm_kernel<<<(unsigned)(tiles * splits), THREADS, SMEM_BYTES, s>>>(a.map_a, b.map_b, g);
+  g.ea = a.exps;
+  g.eb = b.exps;
+  g.M = a.rows;
+  g.N = b.rows;
+  g.alpha = alpha;
+  g.out = out;
+  g.rs = rs;
+  g.cs = cs;
+  g.neg_odd = neg_odd ? 1 : 0;
+  g.err = err;
+  if (splits > 1) {
+    CB_TRY(ws.alloc(&g.hi, (size_t)splits * np * mp));
+    CB_TRY(ws.alloc(&g.lo, (size_t)splits * np * mp));
+  }
+  if (!err) {
+    CB_TRY(ws.alloc(&g.err, 1));
+    CB_CUDA(cudaMemsetAsync(g.err, 0, sizeof(int), s));
+  }
+  sliced_gemm_kernel<<<(unsigned)std::min<int64_t>(g.items, sms), THREADS, SMEM_BYTES, s>>>(a.map_a, b.map_b, g);
   count_launch();
   CB_LAUNCH();
-  sliced_finalize_kernel<<<gsz(a.rows * b.rows), 256, 0, s>>>(g.hi, g.lo, splits, mp, np, a.exps, b.exps, a.rows,
-                                                              b.rows, alpha, out, rs, cs, neg_odd ? 1 : 0);
-  count_launch();
-  CB_LAUNCH();
+  if (splits > 1) {
+    sliced_finalize_kernel<<<gsz(a.rows * b.rows), 256, 0, s>>>(g, splits);
+    count_launch();
+    CB_LAUNCH();
+  }
+  if (err) return CHASE_BSE_OK;
   int herr = 0;
   CB_CUDA(cudaMemcpyAsync(&herr, g.err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CB_CUDA(cudaStreamSynchronize(s));

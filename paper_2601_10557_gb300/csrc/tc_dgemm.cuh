@@ -62,11 +62,22 @@ int slice_hamiltonian(const cplx* A, const cplx* B, int64_t n, SlicedOp& op, cud
 // [a; conj(a)] and -i [c; conj(c)], a = (x + conj(y))/2, c = i (x - conj(y))/2,
 // and H [z; conj(z)] = [P'z; -conj(P'z)].
 int hop_sliced(const SlicedOp& ph, const cplx* W, int64_t n, int64_t k, cplx* out, cudaStream_t s);
+// The halves a_j, c_j of W (2n x k) as the columns 2j, 2j + 1 of Z (n x 2k), and W from the
+// halves in the block Z0, Z1 or Z2 that sel[j] (device) names.
+int jsplit(const cplx* W, int64_t n, int64_t k, cplx* Z, cudaStream_t s);
+int jmerge(cplx* W, const cplx* Z0, const cplx* Z1, const cplx* Z2, const int* sel, int64_t n, int64_t k,
+           cudaStream_t s);
+// R = H W - W diag(lambda) (2n x k) by a sliced product with blocks of rows of H, without a
+// host synchronisation (NaN where a wait of the products ran out).
+int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k, cplx* R,
+                    Workspace& ws, cudaStream_t s);
 
 // C[r][c] = alpha * sum_k a[r][k] b[c][k] for r < a.rows, c < b.rows, written to
 // out[r * rs + c * cs]; with neg_odd the rows r odd are negated (complex
-// conjugate of a real-form result).
+// conjugate of a real-form result).  Waits for the product and returns its status; with err
+// (a zeroed device word that a wait running out sets) it only launches, and the caller
+// reads err once behind a chain of products.
 int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out, int64_t rs, int64_t cs,
-                bool neg_odd, cudaStream_t s);
+                bool neg_odd, cudaStream_t s, int* err = nullptr);
 
 }  // namespace cb
