@@ -482,17 +482,26 @@ __global__ void jacobi_apply_kernel(cplx* G, cplx* V, int64_t k, int r, const cp
   }
 }
 
-__global__ void offdiag_norm_kernel(const cplx* G, int64_t k, double* red) {
+// part[2b], part[2b + 1]: block b's share of sum |g_ij|^2, i != j, and over all entries (one
+// block alone is bound by its SM's FP64 pipe: 224 us at k = 520)
+__global__ void offdiag_norm_kernel(const cplx* G, int64_t k, double* part) {
   __shared__ double sh[32];
   double off = 0.0, tot = 0.0;
-  for (int64_t i = threadIdx.x; i < k * k; i += blockDim.x) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k * k; i += (int64_t)gridDim.x * blockDim.x) {
     const double v = cabs2(G[i]);
     tot += v;
     if (i % k != i / k) off += v;
   }
   off = block_sum(off, sh);
   tot = block_sum(tot, sh);
-  if (threadIdx.x == 0) { red[0] = off; red[1] = tot; }
+  if (threadIdx.x == 0) { part[2 * blockIdx.x] = off; part[2 * blockIdx.x + 1] = tot; }
+}
+__global__ void offdiag_sum_kernel(const double* part, int nblk, double* red) {
+  if (threadIdx.x < 2) {
+    double v = 0.0;
+    for (int b = 0; b < nblk; ++b) v += part[2 * b + threadIdx.x];
+    red[threadIdx.x] = v;
+  }
 }
 
 // ---- Jacobi sweeps with one grid barrier per round ------------------------
@@ -578,15 +587,20 @@ __device__ __forceinline__ void rot_block(const Rot& A, const Rot& B, const cplx
   z[2] = mk(B.c * y10.x - B.s * u1.x, B.c * y10.y - B.s * u1.y);
   z[3] = mk(B.s * y10.x + B.c * u1.x, B.s * y10.y + B.c * u1.y);
 }
-// Diagonal entry i (0: p, 1: q) of J^* X J for the hermitian diagonal block X of (p, q):
-// c^2 x_pp + s^2 x_qq -+ 2 c s Re(e x_pq).
-__device__ __forceinline__ double rot_diag(const Rot& A, const cplx* G, int k, int p, int q, int i) {
-  const double xpp = __ldcg(G + p + (int64_t)p * k).x, xqq = __ldcg(G + q + (int64_t)q * k).x;
-  if (A.s == 0.0) return i == 0 ? xpp : xqq;
-  const cplx xpq = __ldcg(G + p + (int64_t)q * k);
-  const double re = A.er * xpq.x - A.ei * xpq.y;  // Re(e x_pq)
+// Diagonal entry i (0: p, 1: q) of J^* X J for the hermitian diagonal block X = (x_pp, x_qq,
+// x_pq) of a pair: c^2 x_pp + s^2 x_qq -+ 2 c s Re(e x_pq).
+struct DiagBlock {
+  double pp, qq;
+  cplx pq;
+};
+__device__ __forceinline__ DiagBlock load_diag(const cplx* G, int k, int p, int q) {
+  return DiagBlock{__ldcg(G + p + (int64_t)p * k).x, __ldcg(G + q + (int64_t)q * k).x, __ldcg(G + p + (int64_t)q * k)};
+}
+__device__ __forceinline__ double rot_diag(const Rot& A, const DiagBlock& X, int i) {
+  if (A.s == 0.0) return i == 0 ? X.pp : X.qq;
+  const double re = A.er * X.pq.x - A.ei * X.pq.y;  // Re(e x_pq)
   const double cc = A.c * A.c, ss = A.s * A.s, cs2 = 2.0 * A.c * A.s;
-  return i == 0 ? fma(cc, xpp, fma(ss, xqq, -cs2 * re)) : fma(ss, xpp, fma(cc, xqq, cs2 * re));
+  return i == 0 ? fma(cc, X.pp, fma(ss, X.qq, -cs2 * re)) : fma(ss, X.pp, fma(cc, X.qq, cs2 * re));
 }
 __device__ __forceinline__ void load_block(const cplx* G, int k, int p0, int q0, int p1, int q1, cplx x[4]) {
   x[0] = __ldcg(G + p0 + (int64_t)p1 * k);
@@ -633,6 +647,23 @@ __global__ void jacobi_sweep_kernel(cplx* Ga, cplx* Gb, int k, Rot* rots, const 
       const Rot A = ld_rot(R + a), B = ld_rot(R + b);
       cplx x[4], z[4];
       load_block(Gi, k, pa, qa, pb, qb, x);
+      // the pivots of round r + 1 in this block (partner yi[ix] of row ix); what their new
+      // diagonal entries need is loaded with the block
+      int pos[2], yi[2];
+      bool pivot = false;
+      if (a != b && r + 1 < k - 1) {
+#pragma unroll
+        for (int ix = 0; ix < 2; ++ix) {
+          pos[ix] = jpos(ix == 0 ? pa : qa, r + 1, k);
+          yi[ix] = jat(k - 1 - pos[ix], r + 1, k);
+          pivot |= yi[ix] == pb || yi[ix] == qb;
+        }
+      }
+      DiagBlock da{}, db{};
+      if (pivot) {
+        da = load_diag(Gi, k, pa, qa);
+        db = load_diag(Gi, k, pb, qb);
+      }
       if (A.s == 0.0 && B.s == 0.0) {
         z[0] = x[0]; z[1] = x[1]; z[2] = x[2]; z[3] = x[3];
       } else {
@@ -647,19 +678,17 @@ __global__ void jacobi_sweep_kernel(cplx* Ga, cplx* Gb, int k, Rot* rots, const 
       Go[qb + (int64_t)pa * k] = cconj(z[1]);
       Go[pb + (int64_t)qa * k] = cconj(z[2]);
       Go[qb + (int64_t)qa * k] = cconj(z[3]);
-      if (r + 1 >= k - 1) continue;
+      if (!pivot) continue;
 #pragma unroll
       for (int ix = 0; ix < 2; ++ix) {
+        if (yi[ix] != pb && yi[ix] != qb) continue;
         const int xi = ix == 0 ? pa : qa;
-        const int pos = jpos(xi, r + 1, k);
-        const int yi = jat(k - 1 - pos, r + 1, k);
-        if (yi != pb && yi != qb) continue;
-        const int iy = (yi == pb) ? 0 : 1;
+        const int iy = (yi[ix] == pb) ? 0 : 1;
         const cplx zxy = z[2 * ix + iy];
-        const double dx = rot_diag(A, Gi, k, pa, qa, ix), dy = rot_diag(B, Gi, k, pb, qb, iy);
-        const int slot = pos < k - 1 - pos ? pos : k - 1 - pos;
+        const double dx = rot_diag(A, da, ix), dy = rot_diag(B, db, iy);
+        const int slot = pos[ix] < k - 1 - pos[ix] ? pos[ix] : k - 1 - pos[ix];
         rots[(int64_t)(r + 1) * half + slot] =
-            xi < yi ? jacobi_rotation(dx, dy, zxy, sn, n2s, t2a, t2b, applied)
+            xi < yi[ix] ? jacobi_rotation(dx, dy, zxy, sn, n2s, t2a, t2b, applied)
                     : jacobi_rotation(dy, dx, cconj(zxy), sn, n2s, t2a, t2b, applied);
       }
     }
@@ -770,8 +799,14 @@ static cudaStream_t jacobi_stream() {
 }
 
 int offdiag_norms(const cplx* G, int64_t k, double* red, cudaStream_t s) {
-  offdiag_norm_kernel<<<1, 1024, 0, s>>>(G, k, red);
+  const int nblk = (int)std::min<int64_t>(std::max<int64_t>(k * k / 4096, 1), 128);
+  double* part = nullptr;
+  CB_CUDA(dalloc(&part, sizeof(double) * 2 * nblk, s));
+  offdiag_norm_kernel<<<nblk, 256, 0, s>>>(G, k, part);
   count_launch();
+  offdiag_sum_kernel<<<1, 32, 0, s>>>(part, nblk, red);
+  count_launch();
+  cudaFreeAsync(part, s);
   CB_LAUNCH();
   return CHASE_BSE_OK;
 }
@@ -789,8 +824,7 @@ int jacobi_eigh(cplx* G, int64_t k, cplx* V, double* theta, cplx* rot, double* r
   double hred[2] = {0, 0};
   int* applied = nullptr;
   CB_CUDA(dalloc(&applied, sizeof(int), s));
-  offdiag_norm_kernel<<<1, 1024, 0, s>>>(G, k, red);  // red[1] = ||G||_F^2 (invariant)
-  count_launch();
+  CB_TRY(offdiag_norms(G, k, red, s));  // red[1] = ||G||_F^2 (invariant)
   // Preferred: one cooperative launch per sweep (one grid barrier per round),
   // then the V pass over the stored rotations.
   {
@@ -807,6 +841,10 @@ int jacobi_eigh(cplx* G, int64_t k, cplx* V, double* theta, cplx* rot, double* r
       static bool attr = false;
       if (!attr) {
         CB_CUDA(cudaFuncSetAttribute(jacobi_vpass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        CB_CUDA(cudaFuncSetAttribute(jacobi_vpass_staged_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     200 * 1024));
+        CB_CUDA(cudaFuncSetAttribute(jacobi_vpass_staged_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     200 * 1024));
         CB_CUDA(cudaFuncSetAttribute(jacobi_vpass_staged_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      200 * 1024));
         attr = true;
@@ -843,7 +881,12 @@ int jacobi_eigh(cplx* G, int64_t k, cplx* V, double* theta, cplx* rot, double* r
           break;
         }
         count_launch();
-        if (staged_smem <= 200 * 1024)
+        // the FP64 work of V's rows over as many SMs as there are rows
+        if (staged_smem <= 200 * 1024 && k <= sms)
+          jacobi_vpass_staged_kernel<1><<<(unsigned)k, 32, staged_smem, s>>>(V, ki, rots);
+        else if (staged_smem <= 200 * 1024 && k <= 2 * sms)
+          jacobi_vpass_staged_kernel<2><<<(unsigned)((k + 1) / 2), 64, staged_smem, s>>>(V, ki, rots);
+        else if (staged_smem <= 200 * 1024)
           jacobi_vpass_staged_kernel<4><<<(unsigned)((k + 3) / 4), 128, staged_smem, s>>>(V, ki, rots);
         else
           jacobi_vpass_kernel<<<(unsigned)((k + VROWS - 1) / VROWS), 32 * VROWS, vsmem, s>>>(V, ki, rots);

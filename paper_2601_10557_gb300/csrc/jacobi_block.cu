@@ -31,18 +31,22 @@ namespace bj {
 
 constexpr int BS = 32;        // indices per block
 constexpr int PS = 2 * BS;    // indices of a block pair
-constexpr int THREADS = 256;
+// Threads of a CTA: a block pair's inner sweep is 63 rounds of 32 rotations in one CTA, one
+// round's 1024 2 x 2 blocks of S and 2048 row pairs of U between two barriers, so the FP32
+// kernel takes 512; in FP64 the registers of the 64 x 64 products allow 256.
 
 template <class R>
 struct Cx;
 template <>
 struct Cx<float> {
   using T = float2;
+  static constexpr int TPB = 512;
   __device__ static T mk(float r, float i) { return make_float2(r, i); }
 };
 template <>
 struct Cx<double> {
   using T = double2;
+  static constexpr int TPB = 256;
   __device__ static T mk(double r, double i) { return make_double2(r, i); }
 };
 
@@ -95,7 +99,7 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
   jpair32(g, r, P.nb, I, J);
   const int tid = threadIdx.x;
   constexpr int LD = PS + 1;
-  for (int e = tid; e < PS * PS; e += THREADS) {
+  for (int e = tid; e < PS * PS; e += Cx<R>::TPB) {
     const int i = e % PS, j = e / PS;
     S[i + j * LD] = __ldcg(P.G + gidx(i, I, J) + (int64_t)gidx(j, I, J) * P.kp);
     Uu[i + j * LD] = Cx<R>::mk(i == j ? R(1) : R(0), R(0));
@@ -103,6 +107,22 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
   __shared__ int any;
   if (tid == 0) any = 0;
   __syncthreads();
+  // A sub-problem without an entry above the thresholds keeps the identity (no rotation of the
+  // sweep would change an entry): late sweeps rotate 1 to 40 of 153 pairs at k = 520.
+  bool above = false;
+  for (int e = tid; e < PS * PS; e += Cx<R>::TPB) {
+    const int i = e % PS, j = e / PS;
+    const C x = S[i + j * LD];
+    const R r2 = x.x * x.x + x.y * x.y;
+    above |= i < j && r2 > P.t2 * fabs(S[i + i * LD].x * S[j + j * LD].x) && r2 > P.f2 && r2 > R(0);
+  }
+  if (!__syncthreads_or(above)) {
+    if (tid == 0) P.rotated[g] = 0;
+    C* Ug = P.U + (int64_t)g * PS * PS;
+    for (int e = tid; e < PS * PS; e += Cx<R>::TPB) Ug[e] = Uu[(e % PS) + (e / PS) * LD];
+    __syncthreads();
+    return;
+  }
   for (int ir = 0; ir < PS - 1; ++ir) {
     if (tid < BS) {
       int p, q;
@@ -111,9 +131,9 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
       rot[tid] = rotation<R>(S[p + p * LD].x, S[q + q * LD].x, x.x, x.y, P.t2, P.f2);
       if (rot[tid].s != R(0)) any = 1;
     }
-    __syncthreads();
+    if (!__syncthreads_or(tid < BS && rot[tid].s != R(0))) continue;
     // S <- J^* S J on every 2 x 2 block (slots a, b)
-    for (int item = tid; item < BS * BS; item += THREADS) {
+    for (int item = tid; item < BS * BS; item += Cx<R>::TPB) {
       const int a = item / BS, b = item % BS;
       const BRot<R> A = rot[a], B = rot[b];
       if (A.s == R(0) && B.s == R(0)) continue;
@@ -139,7 +159,7 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
       S[qa + qb * LD] = Cx<R>::mk(B.s * y2.x + B.c * u3.x, B.s * y2.y + B.c * u3.y);
     }
     // Uu <- Uu J (rows independent)
-    for (int item = tid; item < PS * BS; item += THREADS) {
+    for (int item = tid; item < PS * BS; item += Cx<R>::TPB) {
       const int i = item / BS, sl = item % BS;
       const BRot<R> B = rot[sl];
       if (B.s == R(0)) continue;
@@ -156,7 +176,7 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
   // tiles of pairs that both kept the identity (a tile with one rotated pair still reads
   // this U)
   C* Ug = P.U + (int64_t)g * PS * PS;
-  for (int e = tid; e < PS * PS; e += THREADS) Ug[e] = Uu[(e % PS) + (e / PS) * LD];
+  for (int e = tid; e < PS * PS; e += Cx<R>::TPB) Ug[e] = Uu[(e % PS) + (e / PS) * LD];
   if (tid == 0) {
     P.rotated[g] = any;
     if (any) atomicAdd(P.nrot, 1);
@@ -165,19 +185,19 @@ __device__ void solve_pair(const Params<R>& P, int r, int g, typename Cx<R>::T* 
 }
 
 // out (64 x 64, ld LD) = op(X) * Y with X, Y 64 x 64 (ld LD) in shared memory;
-// op(X) = X (conjx = false) or X^* (conjx = true).  Each thread owns a 4 x 4 tile.
+// op(X) = X (conjx = false) or X^* (conjx = true).  Each thread owns a 4 x NJ tile.
 template <class R>
 __device__ __forceinline__ void mm64(const typename Cx<R>::T* X, const typename Cx<R>::T* Y, bool conjx,
-                                     typename Cx<R>::T acc[4][4]) {
+                                     typename Cx<R>::T acc[4][1024 / Cx<R>::TPB]) {
   using C = typename Cx<R>::T;
-  constexpr int LD = PS + 1;
-  const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;  // rows tr + 16 i, columns tc + 16 j
+  constexpr int LD = PS + 1, NJ = 1024 / Cx<R>::TPB, CS = PS / NJ;
+  const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;  // rows tr + 16 i, columns tc + CS j
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = Cx<R>::mk(R(0), R(0));
+    for (int j = 0; j < NJ; ++j) acc[i][j] = Cx<R>::mk(R(0), R(0));
   for (int l = 0; l < PS; ++l) {
-    C xa[4], yb[4];
+    C xa[4], yb[NJ];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int row = tr + 16 * i;
@@ -189,11 +209,11 @@ __device__ __forceinline__ void mm64(const typename Cx<R>::T* X, const typename 
       }
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) yb[j] = Y[l + (tc + 16 * j) * LD];
+    for (int j = 0; j < NJ; ++j) yb[j] = Y[l + (tc + CS * j) * LD];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < NJ; ++j) {
         acc[i][j].x = fma(xa[i].x, yb[j].x, acc[i][j].x);
         acc[i][j].x = fma(-xa[i].y, yb[j].y, acc[i][j].x);
         acc[i][j].y = fma(xa[i].x, yb[j].y, acc[i][j].y);
@@ -206,7 +226,7 @@ template <class R>
 __device__ void load_u(const Params<R>& P, int g, typename Cx<R>::T* Us) {
   constexpr int LD = PS + 1;
   const typename Cx<R>::T* Ug = P.U + (int64_t)g * PS * PS;
-  for (int e = threadIdx.x; e < PS * PS; e += THREADS) Us[(e % PS) + (e / PS) * LD] = __ldcg(Ug + e);
+  for (int e = threadIdx.x; e < PS * PS; e += Cx<R>::TPB) Us[(e % PS) + (e / PS) * LD] = __ldcg(Ug + e);
 }
 
 // Phase B, G tile (g, h), g <= h: G[P_g, P_h] <- U_g^* G[P_g, P_h] U_h (and the mirror).
@@ -214,39 +234,39 @@ template <class R>
 __device__ void update_tile(const Params<R>& P, int r, int g, int h, typename Cx<R>::T* T, typename Cx<R>::T* Ua,
                             typename Cx<R>::T* Ub) {
   using C = typename Cx<R>::T;
-  constexpr int LD = PS + 1;
+  constexpr int LD = PS + 1, NJ = 1024 / Cx<R>::TPB, CS = PS / NJ;
   int Ig, Jg, Ih, Jh;
   jpair32(g, r, P.nb, Ig, Jg);
   jpair32(h, r, P.nb, Ih, Jh);
-  for (int e = threadIdx.x; e < PS * PS; e += THREADS) {
+  for (int e = threadIdx.x; e < PS * PS; e += Cx<R>::TPB) {
     const int i = e % PS, j = e / PS;
     T[i + j * LD] = __ldcg(P.G + gidx(i, Ig, Jg) + (int64_t)gidx(j, Ih, Jh) * P.kp);
   }
   load_u<R>(P, g, Ua);
   load_u<R>(P, h, Ub);
   __syncthreads();
-  C acc[4][4];
+  C acc[4][NJ];
   mm64<R>(T, Ub, false, acc);  // W = T U_h
   __syncthreads();
   const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) T[(tr + 16 * i) + (tc + 16 * j) * LD] = acc[i][j];
+    for (int j = 0; j < NJ; ++j) T[(tr + 16 * i) + (tc + CS * j) * LD] = acc[i][j];
   __syncthreads();
   mm64<R>(Ua, T, true, acc);  // U_g^* W
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) T[(tr + 16 * i) + (tc + 16 * j) * LD] = acc[i][j];
+    for (int j = 0; j < NJ; ++j) T[(tr + 16 * i) + (tc + CS * j) * LD] = acc[i][j];
   __syncthreads();
-  for (int e = threadIdx.x; e < PS * PS; e += THREADS) {
+  for (int e = threadIdx.x; e < PS * PS; e += Cx<R>::TPB) {
     const int i = e % PS, j = e / PS;
     P.G[gidx(i, Ig, Jg) + (int64_t)gidx(j, Ih, Jh) * P.kp] = T[i + j * LD];
   }
   if (g != h) {
-    for (int e = threadIdx.x; e < PS * PS; e += THREADS) {
+    for (int e = threadIdx.x; e < PS * PS; e += Cx<R>::TPB) {
       const int j = e % PS, i = e / PS;  // element (j of P_h, i of P_g) = conj(T[i, j])
       const C v = T[i + j * LD];
       P.G[gidx(j, Ih, Jh) + (int64_t)gidx(i, Ig, Jg) * P.kp] = Cx<R>::mk(v.x, -v.y);
@@ -259,28 +279,28 @@ __device__ void update_tile(const Params<R>& P, int r, int g, int h, typename Cx
 template <class R>
 __device__ void update_v(const Params<R>& P, int r, int c, int g, typename Cx<R>::T* T, typename Cx<R>::T* Ua) {
   using C = typename Cx<R>::T;
-  constexpr int LD = PS + 1;
+  constexpr int LD = PS + 1, NJ = 1024 / Cx<R>::TPB, CS = PS / NJ;
   int Ig, Jg;
   jpair32(g, r, P.nb, Ig, Jg);
-  for (int e = threadIdx.x; e < PS * PS; e += THREADS) {
+  for (int e = threadIdx.x; e < PS * PS; e += Cx<R>::TPB) {
     const int i = e % PS, j = e / PS;
     T[i + j * LD] = __ldcg(P.V + (int64_t)PS * c + i + (int64_t)gidx(j, Ig, Jg) * P.kp);
   }
   load_u<R>(P, g, Ua);
   __syncthreads();
-  C acc[4][4];
+  C acc[4][NJ];
   mm64<R>(T, Ua, false, acc);
   const int tr = threadIdx.x % 16, tc = threadIdx.x / 16;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      P.V[(int64_t)PS * c + tr + 16 * i + (int64_t)gidx(tc + 16 * j, Ig, Jg) * P.kp] = acc[i][j];
+    for (int j = 0; j < NJ; ++j)
+      P.V[(int64_t)PS * c + tr + 16 * i + (int64_t)gidx(tc + CS * j, Ig, Jg) * P.kp] = acc[i][j];
   __syncthreads();
 }
 
 template <class R>
-__global__ void __launch_bounds__(THREADS, 1) bj_sweep_kernel(Params<R> P) {
+__global__ void __launch_bounds__(Cx<R>::TPB, 1) bj_sweep_kernel(Params<R> P) {
   using C = typename Cx<R>::T;
   constexpr int LD = PS + 1;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -383,7 +403,7 @@ static int run(const cplx* G, int64_t k, cplx* V, double* theta, double t, doubl
     attr = true;
   }
   int per_sm = 0;
-  CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bj_sweep_kernel<R>, THREADS, smem));
+  CB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bj_sweep_kernel<R>, Cx<R>::TPB, smem));
   if (per_sm < 1) return CHASE_BSE_UNSUPPORTED;
   Workspace ws(s);
   C *Gp, *Vp, *U;
@@ -435,7 +455,7 @@ static int run(const cplx* G, int64_t k, cplx* V, double* theta, double t, doubl
     CB_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int), s));
     CB_CUDA(cudaMemsetAsync(nrot, 0, sizeof(int), s));
     void* args[] = {&P};
-    if (cudaLaunchCooperativeKernel((const void*)bj_sweep_kernel<R>, dim3(grid), dim3(THREADS), args, smem, s) !=
+    if (cudaLaunchCooperativeKernel((const void*)bj_sweep_kernel<R>, dim3(grid), dim3(Cx<R>::TPB), args, smem, s) !=
         cudaSuccess) {
       cudaGetLastError();
       return CHASE_BSE_CUDA_ERROR;
@@ -466,7 +486,7 @@ static int run(const cplx* G, int64_t k, cplx* V, double* theta, double t, doubl
 // coupled), one CTA per set: cyclic Jacobi sweeps in shared memory (zero padding is
 // decoupled) until a sweep applies no rotation, at most 40 sweeps.  Writes the set's
 // rows and columns of V2 (preset to the identity) and its entries of theta.
-__global__ void __launch_bounds__(THREADS) cluster_eig_kernel(const cplx* G, int64_t k, const int* idx,
+__global__ void __launch_bounds__(Cx<double>::TPB) cluster_eig_kernel(const cplx* G, int64_t k, const int* idx,
                                                                const int* off, double t2, double f2, cplx* V2,
                                                                double* theta) {
   using R = double;
@@ -480,7 +500,7 @@ __global__ void __launch_bounds__(THREADS) cluster_eig_kernel(const cplx* G, int
   const int j = blockIdx.x;
   const int o = off[j], c = off[j + 1] - o;
   const int tid = threadIdx.x;
-  for (int e = tid; e < PS * PS; e += THREADS) {
+  for (int e = tid; e < PS * PS; e += Cx<R>::TPB) {
     const int a = e % PS, b = e / PS;
     S[a + b * LD] = (a < c && b < c) ? G[idx[o + a] + (int64_t)idx[o + b] * k] : make_double2(0.0, 0.0);
     Uu[a + b * LD] = make_double2(a == b ? 1.0 : 0.0, 0.0);
@@ -498,7 +518,7 @@ __global__ void __launch_bounds__(THREADS) cluster_eig_kernel(const cplx* G, int
         if (rot[tid].s != 0.0) atomicAdd(&applied, 1);
       }
       __syncthreads();
-      for (int item = tid; item < BS * BS; item += THREADS) {
+      for (int item = tid; item < BS * BS; item += Cx<R>::TPB) {
         const int a = item / BS, b = item % BS;
         const BRot<R> A = rot[a], B = rot[b];
         if (A.s == 0.0 && B.s == 0.0) continue;
@@ -521,7 +541,7 @@ __global__ void __launch_bounds__(THREADS) cluster_eig_kernel(const cplx* G, int
         S[qa + pb * LD] = make_double2(B.c * y2.x - B.s * u3.x, B.c * y2.y - B.s * u3.y);
         S[qa + qb * LD] = make_double2(B.s * y2.x + B.c * u3.x, B.s * y2.y + B.c * u3.y);
       }
-      for (int item = tid; item < PS * BS; item += THREADS) {
+      for (int item = tid; item < PS * BS; item += Cx<R>::TPB) {
         const int i = item / BS, sl = item % BS;
         const BRot<R> B = rot[sl];
         if (B.s == 0.0) continue;
@@ -537,11 +557,11 @@ __global__ void __launch_bounds__(THREADS) cluster_eig_kernel(const cplx* G, int
     if (applied == 0) break;
     __syncthreads();
   }
-  for (int e = tid; e < c * c; e += THREADS) {
+  for (int e = tid; e < c * c; e += Cx<R>::TPB) {
     const int a = e % c, b = e / c;
     V2[idx[o + a] + (int64_t)idx[o + b] * k] = Uu[a + b * LD];
   }
-  for (int a = tid; a < c; a += THREADS) theta[idx[o + a]] = S[a + a * LD].x;
+  for (int a = tid; a < c; a += Cx<R>::TPB) theta[idx[o + a]] = S[a + a * LD].x;
 }
 
 // Pairs i < j with |g_ij|^2 > t2 |g_ii g_jj| and > f2, appended to pairs (at most cap of
@@ -606,7 +626,7 @@ int cluster_eig(const cplx* G, int64_t k, const std::vector<int>& idx, const std
     CB_CUDA(cudaFuncSetAttribute(bj::cluster_eig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr = true;
   }
-  bj::cluster_eig_kernel<<<(unsigned)ncl, bj::THREADS, smem, s>>>(G, k, di, doff, thr * thr, floor_abs * floor_abs,
+  bj::cluster_eig_kernel<<<(unsigned)ncl, bj::Cx<double>::TPB, smem, s>>>(G, k, di, doff, thr * thr, floor_abs * floor_abs,
                                                                   V2, theta);
   count_launch();
   CB_LAUNCH();
