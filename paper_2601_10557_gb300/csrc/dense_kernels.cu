@@ -122,108 +122,128 @@ __device__ __forceinline__ cplx scale_re(cplx a, double s) {
   return REAL ? mk(a.x * s, 0.0) : cscale(a, s);
 }
 
+// Block columns of CB = 16: the diagonal block is a serial chain on one CTA (a square root and a
+// division a column, about 1 us), a panel row a serial chain of CB^2 / 2 updates, and a trailing
+// tile one SM's FP64 work, so narrow blocks shorten all three between two grid barriers.  CTA 0
+// takes the trailing tile that is the next diagonal block and factors it while the others
+// finish theirs: two barriers a block column.  Each element's operations are in column order for
+// any block width, so the factor does not change a bit.  Measured on one GB300, before (CB = 32,
+// three barriers) and after: k = 520 complex 2.64 -> 1.35 ms, real 1.21 -> 0.84 ms.
+constexpr int CB = 16;
+template <bool REAL>
+__device__ __forceinline__ void chol_diag(cplx (*a)[CB + 1], double* dinv, int jb, int64_t j0, int* info) {
+  const int t = threadIdx.x;
+  for (int c = 0; c < jb; ++c) {
+    if (t == 0) {
+      double d = a[c][c].x;
+      if (!(d > 0.0)) {
+        atomicCAS(info, 0, (int)(j0 + c + 1));
+        d = 1.0;
+      }
+      const double sd = sqrt(d);
+      a[c][c] = mk(sd, 0.0);
+      dinv[c] = 1.0 / sd;
+    }
+    __syncthreads();
+    const double inv = dinv[c];
+    for (int r = c + 1 + t; r < jb; r += blockDim.x) a[r][c] = scale_re<REAL>(a[r][c], inv);
+    __syncthreads();
+    const int m = jb - c - 1;
+    for (int idx = t; idx < m * m; idx += blockDim.x) {
+      const int r = c + 1 + idx % m, q = c + 1 + idx / m;
+      if (q <= r) a[r][q] = msub_conj<REAL>(a[r][q], a[r][c], a[q][c]);
+    }
+    __syncthreads();
+  }
+}
+
 template <bool REAL>
 __global__ void chol_coop_kernel(cplx* G, int64_t k, int* info, GridSync* gsync, int* err) {
-  __shared__ cplx buf[2][NB][NB + 1];
-  auto& a = buf[0];   // diagonal block (phases 1, 2)
-  auto& pi = buf[0];  // panel rows of tile row I (phase 3)
-  auto& pk = buf[1];  // panel rows of tile column K (phase 3)
-  __shared__ double dinv[NB];
+  __shared__ cplx buf[2][CB][CB + 1];
+  auto& a = buf[0];   // diagonal block
+  auto& pi = buf[0];  // panel rows of tile row I
+  auto& pk = buf[1];  // panel rows of tile column K
+  __shared__ double dinv[CB];
   const int t = threadIdx.x;
-  const int64_t nb = (k + NB - 1) / NB;
+  const int64_t nb = (k + CB - 1) / CB;
+  if (blockIdx.x == 0) {
+    const int jb = (int)(k < CB ? k : CB);
+    for (int idx = t; idx < jb * jb; idx += blockDim.x) a[idx % jb][idx / jb] = __ldcg(G + idx % jb + (idx / jb) * k);
+    __syncthreads();
+    chol_diag<REAL>(a, dinv, jb, 0, info);
+    for (int idx = t; idx < jb * jb; idx += blockDim.x) {
+      const int r = idx % jb, c = idx / jb;
+      G[r + c * k] = (r >= c) ? a[r][c] : mk(0, 0);
+    }
+  }
+  if (!grid_barrier(gsync, err)) return;
   for (int64_t J = 0; J < nb; ++J) {
-    const int64_t j0 = J * NB;
-    const int jb = (int)((k - j0) < NB ? (k - j0) : NB);
-    if (blockIdx.x == 0) {
-      for (int idx = t; idx < jb * jb; idx += blockDim.x) {
-        const int r = idx % jb, c = idx / jb;
-        a[r][c] = __ldcg(G + (j0 + r) + (j0 + c) * k);
-      }
-      __syncthreads();
-      for (int c = 0; c < jb; ++c) {
-        if (t == 0) {
-          double d = a[c][c].x;
-          if (!(d > 0.0)) {
-            atomicCAS(info, 0, (int)(j0 + c + 1));
-            d = 1.0;
-          }
-          const double sd = sqrt(d);
-          a[c][c] = mk(sd, 0.0);
-          dinv[c] = 1.0 / sd;
+    const int64_t j0 = J * CB;
+    const int jb = (int)((k - j0) < CB ? (k - j0) : CB);
+    const int64_t rest = k - j0 - jb;
+    if (rest <= 0) return;
+    // panel: rows i >= j0 + jb solve x L_JJ^* = a_i (forward substitution)
+    for (int idx = t; idx < jb * jb; idx += blockDim.x) {
+      const int r = idx % jb, c = idx / jb;
+      a[r][c] = __ldcg(G + (j0 + r) + (j0 + c) * k);
+    }
+    __syncthreads();
+    if (t < jb) dinv[t] = 1.0 / a[t][t].x;
+    __syncthreads();
+    // consecutive rows on consecutive CTAs: the FP64 work spreads over all SMs
+    for (int64_t i = j0 + jb + blockIdx.x + (int64_t)gridDim.x * t; i < k; i += (int64_t)gridDim.x * blockDim.x) {
+      cplx x[CB];
+#pragma unroll
+      for (int c = 0; c < CB; ++c) x[c] = (c < jb) ? __ldcg(G + i + (j0 + c) * k) : mk(0, 0);
+#pragma unroll
+      for (int c = 0; c < CB; ++c) {
+        if (c < jb) {
+          cplx v = x[c];
+#pragma unroll
+          for (int q = 0; q < CB; ++q)
+            if (q < c) v = msub_conj<REAL>(v, x[q], a[c][q]);
+          x[c] = scale_re<REAL>(v, dinv[c]);
         }
-        __syncthreads();
-        const double inv = dinv[c];
-        for (int r = c + 1 + t; r < jb; r += blockDim.x) a[r][c] = scale_re<REAL>(a[r][c], inv);
-        __syncthreads();
-        const int m = jb - c - 1;
-        for (int idx = t; idx < m * m; idx += blockDim.x) {
-          const int r = c + 1 + idx % m, q = c + 1 + idx / m;
-          if (q <= r) a[r][q] = msub_conj<REAL>(a[r][q], a[r][c], a[q][c]);
-        }
-        __syncthreads();
       }
-      for (int idx = t; idx < jb * jb; idx += blockDim.x) {
-        const int r = idx % jb, c = idx / jb;
-        G[(j0 + r) + (j0 + c) * k] = (r >= c) ? a[r][c] : mk(0, 0);
-      }
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+        if (c < jb) G[i + (j0 + c) * k] = x[c];
     }
     if (!grid_barrier(gsync, err)) return;
-    const int64_t rest = k - j0 - jb;
-    if (rest > 0) {
-      // panel: rows i >= j0 + jb solve x L_JJ^* = a_i (forward substitution)
-      for (int idx = t; idx < jb * jb; idx += blockDim.x) {
-        const int r = idx % jb, c = idx / jb;
-        a[r][c] = __ldcg(G + (j0 + r) + (j0 + c) * k);
+    // trailing update, CB x CB tiles (I, K) with K <= I over the lower triangle, one entry per
+    // thread; tile 0, the next diagonal block, and its factorisation are CTA 0's
+    const int64_t T = (rest + CB - 1) / CB, ntile = T * (T + 1) / 2;
+    const int64_t others = gridDim.x > 1 ? gridDim.x - 1 : 1;
+    for (int64_t tile = blockIdx.x; tile < ntile; tile += (tile == 0 && gridDim.x > 1) ? ntile : others) {
+      int64_t I = (int64_t)((sqrtf(8.0f * (float)tile + 1.0f) - 1.0f) * 0.5f);
+      while (I * (I + 1) / 2 > tile) --I;
+      while ((I + 1) * (I + 2) / 2 <= tile) ++I;
+      const int64_t K = tile - I * (I + 1) / 2;
+      const int64_t i0 = j0 + jb + I * CB, c0 = j0 + jb + K * CB;
+      const int ib = (int)((k - i0) < CB ? (k - i0) : CB), cbk = (int)((k - c0) < CB ? (k - c0) : CB);
+      __syncthreads();
+      for (int idx = t; idx < CB * jb; idx += blockDim.x) {
+        const int r = idx % CB, q = idx / CB;
+        pi[r][q] = (r < ib) ? __ldcg(G + (i0 + r) + (j0 + q) * k) : mk(0, 0);
+        pk[r][q] = (r < cbk) ? __ldcg(G + (c0 + r) + (j0 + q) * k) : mk(0, 0);
+      }
+      const int r = t % CB, c = t / CB;  // blockDim.x = CB * CB
+      const bool mine = r < ib && c < cbk && !(I == K && c > r);
+      cplx acc = mine ? __ldcg(G + (i0 + r) + (c0 + c) * k) : mk(0, 0);
+      __syncthreads();
+      if (mine)
+        for (int q = 0; q < jb; ++q) acc = msub_conj<REAL>(acc, pi[r][q], pk[c][q]);
+      if (tile > 0) {
+        if (mine) G[(i0 + r) + (c0 + c) * k] = acc;
+        continue;
       }
       __syncthreads();
-      if (t < jb) dinv[t] = 1.0 / a[t][t].x;
+      if (r < ib && c < cbk) a[r][c] = mine ? acc : mk(0, 0);
       __syncthreads();
-      // consecutive rows on consecutive CTAs: the FP64 work spreads over all SMs
-      for (int64_t i = j0 + jb + blockIdx.x + (int64_t)gridDim.x * t; i < k; i += (int64_t)gridDim.x * blockDim.x) {
-        cplx x[NB];
-#pragma unroll
-        for (int c = 0; c < NB; ++c) x[c] = (c < jb) ? __ldcg(G + i + (j0 + c) * k) : mk(0, 0);
-#pragma unroll
-        for (int c = 0; c < NB; ++c) {
-          if (c < jb) {
-            cplx v = x[c];
-#pragma unroll
-            for (int q = 0; q < NB; ++q)
-              if (q < c) v = msub_conj<REAL>(v, x[q], a[c][q]);
-            x[c] = scale_re<REAL>(v, dinv[c]);
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < NB; ++c)
-          if (c < jb) G[i + (j0 + c) * k] = x[c];
-      }
-      if (!grid_barrier(gsync, err)) return;
-      // trailing update, NB x NB tiles (I, K) with K <= I over the lower triangle
-      const int64_t T = (rest + NB - 1) / NB;
-      for (int64_t tile = blockIdx.x; tile < T * (T + 1) / 2; tile += gridDim.x) {
-        int64_t I = (int64_t)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
-        while (I * (I + 1) / 2 > tile) --I;
-        while ((I + 1) * (I + 2) / 2 <= tile) ++I;
-        const int64_t K = tile - I * (I + 1) / 2;
-        const int64_t i0 = j0 + jb + I * NB, c0 = j0 + jb + K * NB;
-        const int ib = (int)((k - i0) < NB ? (k - i0) : NB), cbk = (int)((k - c0) < NB ? (k - c0) : NB);
-        __syncthreads();
-        for (int idx = t; idx < NB * jb; idx += blockDim.x) {
-          const int r = idx % NB, q = idx / NB;
-          pi[r][q] = (r < ib) ? __ldcg(G + (i0 + r) + (j0 + q) * k) : mk(0, 0);
-          pk[r][q] = (r < cbk) ? __ldcg(G + (c0 + r) + (j0 + q) * k) : mk(0, 0);
-        }
-        __syncthreads();
-        for (int idx = t; idx < ib * cbk; idx += blockDim.x) {
-          const int r = idx % ib, c = idx / ib;
-          if (I == K && c > r) continue;
-          cplx acc = __ldcg(G + (i0 + r) + (c0 + c) * k);
-          for (int q = 0; q < jb; ++q) acc = msub_conj<REAL>(acc, pi[r][q], pk[c][q]);
-          G[(i0 + r) + (c0 + c) * k] = acc;
-        }
-      }
-      if (!grid_barrier(gsync, err)) return;
+      chol_diag<REAL>(a, dinv, ib, i0, info);
+      if (r < ib && c < cbk) G[(i0 + r) + (c0 + c) * k] = mine ? a[r][c] : mk(0, 0);
     }
+    if (!grid_barrier(gsync, err)) return;
   }
 }
 
@@ -242,7 +262,7 @@ int cholesky(cplx* G, int64_t k, int* info_dev, int* info_host, cudaStream_t s, 
   CB_CUDA(cudaMemsetAsync(info_dev, 0, sizeof(int), s));
   int grid = 0;
   const void* kern = real ? (const void*)chol_coop_kernel<true> : (const void*)chol_coop_kernel<false>;
-  if (coop_grid(kern, 256, &grid)) {
+  if (coop_grid(kern, CB * CB, &grid)) {
     GridSync* gsync = nullptr;
     int* err = nullptr;
     CB_CUDA(dalloc(&gsync, sizeof(GridSync), s));
@@ -251,7 +271,7 @@ int cholesky(cplx* G, int64_t k, int* info_dev, int* info_host, cudaStream_t s, 
     CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     int64_t kk = k;
     void* args[] = {&G, &kk, &info_dev, &gsync, &err};
-    const cudaError_t le = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(256), args, 0, s);
+    const cudaError_t le = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(CB * CB), args, 0, s);
     if (le != cudaSuccess) cudaGetLastError();
     count_launch();
     zero_upper_kernel<<<cdiv(k * k, 256) < 4096 ? cdiv(k * k, 256) : 4096, 256, 0, s>>>(G, k);
@@ -289,6 +309,7 @@ int cholesky(cplx* G, int64_t k, int* info_dev, int* info_host, cudaStream_t s, 
 }
 
 // ------------------------------------------------------ triangular inverse
+// Inverses of the NB x NB diagonal blocks, one warp and one column per lane.
 __global__ void inv_diag_blocks_kernel(const cplx* L, int64_t k, cplx* X) {
   __shared__ cplx a[NB][NB + 1];
   const int64_t j0 = (int64_t)blockIdx.x * NB;
@@ -315,6 +336,51 @@ __global__ void inv_diag_blocks_kernel(const cplx* L, int64_t k, cplx* X) {
 #pragma unroll
   for (int r = 0; r < NB; ++r)
     if (r < nb) X[(j0 + r) + (j0 + c) * k] = x[r];
+}
+
+// The same for a real factor, one CTA of 256 threads each: thread (c, g) holds rows
+// g, g + 8, g + 16, g + 24 of column c and takes each finished row off them, so a row costs one
+// update and a barrier instead of a chain over all rows before it (147 -> 38 us).
+// A complex factor keeps the chain above: the contraction of its products into FMAs shows in the
+// phases of the Rayleigh-Ritz vectors.
+__global__ void __launch_bounds__(256) inv_diag_real_kernel(const cplx* L, int64_t k, cplx* X) {
+  constexpr int G = 8;
+  __shared__ double a[NB][NB + 1];
+  __shared__ double xr[2][NB];
+  __shared__ double inv[NB];
+  const int64_t j0 = (int64_t)blockIdx.x * NB;
+  const int nb = (int)((k - j0) < NB ? (k - j0) : NB);
+  for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) {
+    const int r = idx % nb, c = idx / nb;
+    a[r][c] = L[(j0 + r) + (j0 + c) * k].x;
+  }
+  __syncthreads();
+  if (threadIdx.x < nb) inv[threadIdx.x] = 1.0 / a[threadIdx.x][threadIdx.x];
+  __syncthreads();
+  const int c = threadIdx.x & (NB - 1), g = threadIdx.x / NB;
+  double v[NB / G];
+#pragma unroll
+  for (int i = 0; i < NB / G; ++i) v[i] = (g + G * i == c) ? 1.0 : 0.0;
+#pragma unroll
+  for (int r = 0; r < NB; ++r) {
+    if (r < nb) {  // uniform
+      if (g == r % G) {
+        const double x = (r >= c) ? v[r / G] * inv[r] : 0.0;
+        v[r / G] = x;
+        xr[r & 1][c] = x;
+      }
+      __syncthreads();
+      const double x = xr[r & 1][c];
+#pragma unroll
+      for (int i = 0; i < NB / G; ++i) {
+        const int q = g + G * i;
+        if (q > r && q < nb && r >= c) v[i] = fma(-a[q][r], x, v[i]);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NB / G; ++i)
+    if (g + G * i < nb && c < nb) X[(j0 + g + G * i) + (j0 + c) * k] = mk(v[i], 0.0);
 }
 
 // X = L^{-1} by block forward substitution on TCB columns per CTA:
@@ -348,9 +414,11 @@ __global__ void trinv_cols_kernel(const cplx* __restrict__ L, int64_t k, cplx* X
       const cplx* Lr = L + i0 + r;
       if (REAL) {
         double a = 0.0;
+#pragma unroll 16
         for (int64_t l = from; l < to; ++l) a = fma(Lr[l * k].x, xs[l * TCB + c].x, a);
         acc = mk(a, 0.0);
       } else {
+#pragma unroll 8
         for (int64_t l = from; l < to; ++l) acc = cadd(acc, cmul(Lr[l * k], xs[l * TCB + c]));
       }
     }
@@ -375,7 +443,8 @@ __global__ void trinv_cols_kernel(const cplx* __restrict__ L, int64_t k, cplx* X
 int tri_inverse(const cplx* L, int64_t k, cplx* X, cplx* T, cudaStream_t s, bool real) {
   CB_CUDA(cudaMemsetAsync(X, 0, sizeof(cplx) * k * k, s));
   const int64_t nblk = (k + NB - 1) / NB;
-  inv_diag_blocks_kernel<<<(unsigned)nblk, NB, 0, s>>>(L, k, X);
+  if (real) inv_diag_real_kernel<<<(unsigned)nblk, 256, 0, s>>>(L, k, X);
+  else inv_diag_blocks_kernel<<<(unsigned)nblk, NB, 0, s>>>(L, k, X);
   count_launch();
   CB_LAUNCH();
   const size_t smem = sizeof(cplx) * (size_t)k * TCB;
