@@ -943,10 +943,10 @@ int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, c
     CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     CB_TRY(slice_complex_rows(Uc, n, n, 2 * nev, tmp, sa, s));
     CB_TRY(slice_plain_rows(U2, n, sb, s));
-    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gA), 1, 2 * n, false, s, err));
+    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gA), 1, 2 * n, false, s, err, 1));
     CB_TRY(slice_complex_rows(Ub, n, n, 2 * nev, tmp, sa, s));
     CB_TRY(slice_plain_rows(U3, n, sb, s));
-    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gB), 1, 2 * n, false, s, err));
+    CB_TRY(sliced_gemm(sa, sb, 1.0, reinterpret_cast<double*>(gB), 1, 2 * n, false, s, err, 2));
     int herr = 0;
     CB_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     CB_CUDA(cudaStreamSynchronize(s));

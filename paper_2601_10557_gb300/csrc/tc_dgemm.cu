@@ -20,7 +20,8 @@
 // Bound: shared memory.  A K step of 16 reads 56 KB of operand digits in 448 MMA cycles
 // (128 bytes a cycle) while the ring takes in 78 bytes a cycle.  Measured on one GB300,
 // before (one CTA per tile, int64 partial tiles of every product) and after: the two
-// products of the gradient at n = 8192 (16384 x 8192, K = 400) 11.7 -> 6.35 ms; the FP64_TC
+// products of the gradient at n = 8192 (16384 x 8192, K = 400) 11.7 -> 6.35 ms, 3.67 ms
+// with only the lower triangle computed; the FP64_TC
 // filter of 130 vectors at n = 2048 (24 products 4096 x 260, K = 4096, their slices and the
 // recurrence) 8.1 -> 5.1 ms.
 #include <cuda_bf16.h>
@@ -86,6 +87,7 @@ struct Args {
   double* out;
   int64_t rs, cs;
   int neg_odd;
+  int sym;             // 1 hermitian, 2 symmetric: only the lower triangle is computed (see sliced_gemm)
   int* err;
 };
 
@@ -108,12 +110,41 @@ __device__ __forceinline__ double fold(long long h, long long l, int e) {
   if (x1 > -1022 && x1 < 1023) return __longlong_as_double((long long)(sign | (((unsigned long long)(x1 + 1022) << 52) + m)));
   return ldexp(__longlong_as_double((long long)(sign | (((unsigned long long)(x + 1022) << 52) + m))), e - 14);
 }
-__device__ __forceinline__ void put_out(const Args& g, int64_t r, int64_t c, long long h, long long l) {
+__device__ __forceinline__ double result(const Args& g, int64_t r, int64_t c, long long h, long long l) {
   const int ea = g.ea[r], eb = g.eb[c];
   double y = max(ea, eb) >= EXP_NONFINITE ? nan("") : fold(h, l, ea + eb);
   if (g.alpha != 1.0) y *= g.alpha;
-  if (g.neg_odd && (r & 1)) y = -y;
-  g.out[r * g.rs + c * g.cs] = y;
+  return g.neg_odd && (r & 1) ? -y : y;
+}
+__device__ __forceinline__ void put_out(const Args& g, int64_t r, int64_t c, long long h, long long l) {
+  g.out[r * g.rs + c * g.cs] = result(g, r, c, h, l);
+}
+// The 16 columns from col on of row `row` (lanes: consecutive rows from an even one) of a
+// hermitian or symmetric complex result: entries (i, j), i = row / 2 >= j, and their mirrors.  Of
+// a lane pair, which holds Re and Im of the same entries, one lane writes the mirrors of the
+// first eight columns and one those of the other eight, 128 contiguous bytes each.
+template <int NC>
+__device__ __forceinline__ void put_sym(const Args& g, int64_t row, int64_t col, const long long* hi,
+                                        const long long* lo) {
+  const bool rv = row < g.M, odd = row & 1;
+  const int64_t i = row >> 1;
+  double y[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    y[c] = 0.0;
+    if (rv && col + c < g.N && i >= col + c) {
+      y[c] = result(g, row, col + c, hi[c], lo[c]);
+      g.out[row + (col + c) * g.cs] = y[c];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC / 2; ++c) {
+    const double got = __shfl_xor_sync(0xffffffffu, odd ? y[c] : y[c + NC / 2], 1);
+    const double re = odd ? got : y[c], im = odd ? y[c + NC / 2] : got;
+    const int64_t j = col + c + (odd ? NC / 2 : 0);
+    if (rv && j < g.N && i > j)
+      *reinterpret_cast<double2*>(g.out + i * g.cs + 2 * j) = make_double2(re, g.sym == 1 ? -im : im);
+  }
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -139,6 +170,15 @@ __global__ void __launch_bounds__(THREADS, 1)
   // the CTAs sharing a tile of the larger operand run together, so that it is read
   // from DRAM once and the other operand's tiles come from L2
   auto item = [&](int id, int& mt, int& nt, int& sp, int& kb0, int& nkb) {
+    if (g.sym) {  // the 2 mt + 2 column tiles of row tile mt that reach the lower triangle
+      mt = (int)((sqrtf(4.0f * (float)id + 1.0f) - 1.0f) * 0.5f);
+      while (mt * (mt + 1) > id) --mt;
+      while ((mt + 1) * (mt + 2) <= id) ++mt;
+      nt = id - mt * (mt + 1);
+      sp = kb0 = 0;
+      nkb = g.kb_total;
+      return;
+    }
     mt = g.n_fast ? (id / g.num_n) % g.num_m : id % g.num_m;
     nt = g.n_fast ? id % g.num_n : (id / g.num_m) % g.num_n;
     sp = id / (g.num_m * g.num_n);
@@ -310,6 +350,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           g.hi[base + (int64_t)i * g.mp] = hi[i];
           g.lo[base + (int64_t)i * g.mp] = lo[i];
         }
+      } else if (g.sym) {
+        put_sym<NC>(g, row, col, hi, lo);
       } else if (row < g.M) {
 #pragma unroll
         for (int i = 0; i < NC; ++i)
@@ -778,7 +820,7 @@ int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, cons
 }
 
 int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out, int64_t rs, int64_t cs,
-                bool neg_odd, cudaStream_t s, int* err) {
+                bool neg_odd, cudaStream_t s, int* err, int sym) {
   using namespace tcd;
   if (a.K != b.K || a.kpad != b.kpad) return CHASE_BSE_BAD_ARG;
   static bool attr = false;
@@ -812,14 +854,19 @@ int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out,
     }
     if (tiles * sp > 4 * (int64_t)sms) break;
   }
+  // a triangle's tiles, where they alone keep the SMs busy and need no K split
+  const int64_t tri = (int64_t)num_m * (num_m + 1);
+  const bool half = sym != 0 && rs == 1 && a.rows == 2 * b.rows && cs == a.rows && tri >= 2 * (int64_t)sms;
+  if (half) splits = 1, kb_per = kb_total;
   Workspace ws(s);
   Args g{};
+  g.sym = half ? sym : 0;
   g.num_m = num_m;
   g.num_n = num_n;
   g.n_fast = a.rows_pad >= b.rows_pad ? 1 : 0;
   g.kb_total = kb_total;
   g.kb_per_split = kb_per;
-  g.items = (int)(tiles * splits);
+  g.items = (int)(half ? tri : tiles * splits);
   g.mp = mp;
   g.np = np;
   g.ea = a.exps;

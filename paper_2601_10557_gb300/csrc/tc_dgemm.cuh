@@ -77,7 +77,11 @@ int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, cons
 // conjugate of a real-form result).  Waits for the product and returns its status; with err
 // (a zeroed device word that a wait running out sets) it only launches, and the caller
 // reads err once behind a chain of products.
+// sym 1 (2): C is the real form, rows 2i, 2i + 1 = Re, Im of row i, of a square complex
+// matrix that is hermitian (symmetric) but for rounding, out its row-major storage's
+// transpose (rs = 1, cs = a.rows = 2 b.rows): only the entries i >= j are computed (where
+// there are tiles enough), the others mirrored.
 int sliced_gemm(const SlicedOp& a, const SlicedOp& b, double alpha, double* out, int64_t rs, int64_t cs,
-                bool neg_odd, cudaStream_t s, int* err = nullptr);
+                bool neg_odd, cudaStream_t s, int* err = nullptr, int sym = 0);
 
 }  // namespace cb
