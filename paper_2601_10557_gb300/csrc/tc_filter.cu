@@ -145,7 +145,7 @@ constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int FLUSH = 4;                 // K blocks per drained partial sum of x0 * y0
 constexpr int MAX_ST = 8;                // most ring stages
-constexpr int RING_BYTES = 196608;
+constexpr int RING_BYTES = 196608;       // (all 227 KB, 4 stages at BN = 192, ran 2-5 % slower)
 constexpr int NBAR = 2 * MAX_ST + 10;    // full, empty, acc_full[2], acc_empty[2], cross_full, cross_empty, out_full[2], out_empty[2]
 constexpr int SMEM_BYTES = RING_BYTES + 1024 + 256;
 constexpr int DC = 128;                  // most columns per drain warp
@@ -324,7 +324,8 @@ struct Maps {
 
 // The end of one half tile: sums its `parts` partial tiles (`stride` floats apart from `tiles`
 // on), undoes the scaling and runs the mode's epilogue for the 32 rows of TMEM lane quarter q and
-// the groups of EB columns first, first + step, ...; a group's loads are in flight together.
+// the groups of EB columns first, first + step, ...  It is a chain of L2 latencies, so the scales of
+// four groups are prepared at a time and all loads of a group are in flight together.
 constexpr int EB = 8;
 template <int SCH>
 __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
@@ -338,86 +339,94 @@ __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, cons
   const int64_t v0 = (int64_t)wk.nt * sc.bn;
   const int cols = (int)min((int64_t)wk.cols, ep.k2 - v0);  // even
 #pragma unroll 1
-  for (int g = first * EB; g < cols; g += step * EB) {
-    const int left = cols - g;
-    const int64_t vb = v0 + g;
-    // loads at clamped rows and columns instead of under a predicate each
-    const int64_t oz = vb * ep.n2 + min(row, ep.n2 - 1);
-    const float* t = tiles + (size_t)g * BM + row_t;
-    float x[EB], zc[EB], zp[EB];
-#pragma unroll
-    for (int i = 0; i < EB; ++i) x[i] = __ldcg(t + i * BM);
-    if (ep.mode != 0) {
-#pragma unroll
-      for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.n2];
-    }
-    if (ep.mode == 1 && ep.beta != 0.0f) {
-#pragma unroll
-      for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.n2];
-    }
-    // lane l prepares column l: the input column's scale (undone), the output's, gamma
+  for (int g0 = first; g0 * EB < cols; g0 += 4 * step) {
+    // lane l prepares column l % 8 of group l / 8: the input column's scale (undone), the
+    // output's, gamma
+    const int pc = (g0 + (lane >> 3) * step) * EB + (lane & 7);
     float s_in = 0.0f, s_out = 0.0f, gmm = 0.0f;
-    if (lane < min(EB, left)) {
-      const int64_t v = vb + lane;
-      s_in = exp2i(-ep.vexp_in[v]);
+    if (pc < cols) {
+      const int64_t v = v0 + pc;
+      const int ein = ep.vexp_in[v];
       if (ep.gamma) gmm = ep.gamma[v];
       if (ep.mode != 2) {
         const int e = out_exp(vec_bound(ep, v));
         s_out = exp2i(e);
         if (q == 0) ep.vexp_out[v] = e;  // the same value from every tile
       }
-    }
-#pragma unroll 1
-    for (int j = 1; j < parts; j += 3) {
-      float y[3][EB];
-#pragma unroll
-      for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(t + min(j + p, parts - 1) * stride + i * BM);
-#pragma unroll
-      for (int p = 0; p < 3; ++p)
-        if (j + p < parts) {
-#pragma unroll
-          for (int i = 0; i < EB; ++i) x[i] += y[p][i];
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < EB; ++i) x[i] *= rs * __shfl_sync(0xffffffffu, s_in, i);
-    if (ep.mode == 1) {
-#pragma unroll
-      for (int i = 0; i < EB; ++i) x[i] = ep.alpha * (ep.hsign * x[i] - ep.c * zc[i]);
-      if (ep.beta != 0.0f) {
-#pragma unroll
-        for (int i = 0; i < EB; ++i) x[i] += ep.beta * zp[i];
-      }
-      if (ep.src) {
-#pragma unroll
-        for (int i = 0; i < EB; ++i) zc[i] = ep.src[oz + (i < left ? i : 0) * ep.n2];
-#pragma unroll
-        for (int i = 0; i < EB; ++i) x[i] += __shfl_sync(0xffffffffu, gmm, i) * zc[i];
-      }
-    } else if (ep.mode == 2) {
-      // H w + gamma w: the two columns of a vector trade places, a' = M c, c' = -M a
-#pragma unroll
-      for (int i = 0; i < EB; i += 2) {
-        const float a = x[i];
-        x[i] = x[i + 1] + __shfl_sync(0xffffffffu, gmm, i) * zc[i];
-        x[i + 1] = -a + __shfl_sync(0xffffffffu, gmm, i + 1) * zc[i + 1];
-      }
+      s_in = exp2i(-ein);
     }
     unsigned amax = 0;
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+      const int g = (g0 + t * step) * EB;
+      if (g >= cols) break;
+      const int left = cols - g;
+      const int64_t vb = v0 + g;
+      // loads at clamped rows and columns instead of under a predicate each
+      const int64_t oz = vb * ep.n2 + min(row, ep.n2 - 1);
+      const float* tp = tiles + (size_t)g * BM + row_t;
+      float x[EB], zc[EB], zp[EB];
 #pragma unroll
-    for (int i = 0; i < EB; ++i) {
-      const bool lv = rvalid && i < left;
-      const float so = __shfl_sync(0xffffffffu, s_out, i);
-      if (lv) {
-        if (ep.mode != 2) put1<T, Scheme<SCH>::NPW>(ep.out, (vb + i) * ep.kpad + row, x[i] * so);
-        if (ep.mode != 0) ep.Znext[oz + i * ep.n2] = x[i];
+      for (int i = 0; i < EB; ++i) x[i] = __ldcg(tp + i * BM);
+      if (ep.mode != 0) {
+#pragma unroll
+        for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.n2];
       }
-      const unsigned mm = __reduce_max_sync(0xffffffffu, lv ? __float_as_uint(fabsf(x[i])) : 0u);
-      if (lane == i) amax = mm;
+      if (ep.mode == 1 && ep.beta != 0.0f) {
+#pragma unroll
+        for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.n2];
+      }
+#pragma unroll 1
+      for (int j = 1; j < parts; j += 3) {
+        float y[3][EB];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(tp + min(j + p, parts - 1) * stride + i * BM);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          if (j + p < parts) {
+#pragma unroll
+            for (int i = 0; i < EB; ++i) x[i] += y[p][i];
+          }
+      }
+#pragma unroll
+      for (int i = 0; i < EB; ++i) x[i] *= rs * __shfl_sync(0xffffffffu, s_in, t * EB + i);
+      if (ep.mode == 1) {
+#pragma unroll
+        for (int i = 0; i < EB; ++i) x[i] = ep.alpha * (ep.hsign * x[i] - ep.c * zc[i]);
+        if (ep.beta != 0.0f) {
+#pragma unroll
+          for (int i = 0; i < EB; ++i) x[i] += ep.beta * zp[i];
+        }
+        if (ep.src) {
+#pragma unroll
+          for (int i = 0; i < EB; ++i) zc[i] = ep.src[oz + (i < left ? i : 0) * ep.n2];
+#pragma unroll
+          for (int i = 0; i < EB; ++i) x[i] += __shfl_sync(0xffffffffu, gmm, t * EB + i) * zc[i];
+        }
+      } else if (ep.mode == 2) {
+        // H w + gamma w: the two columns of a vector trade places, a' = M c, c' = -M a
+#pragma unroll
+        for (int i = 0; i < EB; i += 2) {
+          const float a = x[i];
+          x[i] = x[i + 1] + __shfl_sync(0xffffffffu, gmm, t * EB + i) * zc[i];
+          x[i + 1] = -a + __shfl_sync(0xffffffffu, gmm, t * EB + i + 1) * zc[i + 1];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < EB; ++i) {
+        const bool lv = rvalid && i < left;
+        const float so = __shfl_sync(0xffffffffu, s_out, t * EB + i);
+        if (lv) {
+          if (ep.mode != 2) put1<T, Scheme<SCH>::NPW>(ep.out, (vb + i) * ep.kpad + row, x[i] * so);
+          if (ep.mode != 0) ep.Znext[oz + i * ep.n2] = x[i];
+        }
+        const unsigned mm = __reduce_max_sync(0xffffffffu, lv ? __float_as_uint(fabsf(x[i])) : 0u);
+        if (lane == t * EB + i) amax = mm;
+      }
     }
-    if (lane < min(EB, left)) atomicMax(reinterpret_cast<unsigned*>(ep.amax_out) + vb + lane, amax);
+    if (pc < cols) atomicMax(reinterpret_cast<unsigned*>(ep.amax_out) + v0 + pc, amax);
   }
 }
 
@@ -925,15 +934,19 @@ static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POp
   return CHASE_BSE_OK;
 }
 
-// Cycles of one K block of a 256 x w tile in a launch of bn-wide tiles: the MMAs (w / 2 each)
-// or the shared-memory traffic at 128 bytes a cycle (operand reads and the ring's fill).
+// Cycles of one K block of a 256 x w tile in a launch of bn-wide tiles with a share `active` of the
+// pairs at work: the MMAs (w / 2 each), the shared-memory traffic at 128 bytes a cycle (operand
+// reads and the ring's fill), or the stage's way from L2, which gives the 152 SMs about 10 TB/s in
+// all (measured 0.8-0.85 us a K block for tiles of 160 and of 192 columns at n = 4096, whose MMAs
+// take 0.5 and 0.6).  That favours wide tiles: n = 6000, k = 100 225 -> 182 us a launch, n = 8192,
+// k = 300 786 -> 720 us against a choice by the other two terms.
 template <int SCH>
-static double block_cycles(int w, int bn) {
+static double block_cycles(int w, int bn, double active) {
   using SC = Scheme<SCH>;
   constexpr int MMAS = SC::NPROD * (BK / 16);
-  const double mma = MMAS * (w / 2.0);
-  const double smem = (MMAS * (4096.0 + 16.0 * w) + SC::NPA * A_BYTES + SC::NPW * 64.0 * bn) / 128.0;
-  return std::max(mma, smem);
+  const double mma = MMAS * (w / 2.0), stage = SC::NPA * A_BYTES + SC::NPW * 64.0 * bn;
+  const double smem = (MMAS * (4096.0 + 16.0 * w) + stage) / 128.0;
+  return std::max(std::max(mma, smem), 0.027 * stage * std::max(active, 0.5));
 }
 // The schedule of a launch with m rows, k2 columns and nkb K blocks: of the column widths
 // (multiples of 32) that ceil(k2 / 256) to 3 more column tiles need, and of the numbers of K
@@ -961,15 +974,15 @@ static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
     sc.pairs = pairs;
     sc.waves = (int)(tiles / pairs);
     sc.rest = (int)(tiles % pairs);
-    const double full = block_cycles<SCH>(sc.bn, sc.bn);
-    const double avg = (full * (nn - 1) + block_cycles<SCH>(sc.n_last, sc.bn)) / nn;
+    const double full = block_cycles<SCH>(sc.bn, sc.bn, 1.0);
+    const double avg = (full * (nn - 1) + block_cycles<SCH>(sc.n_last, sc.bn, 1.0)) / nn;
     const double fixed = 6000.0;  // prologue and epilogue of a tile
     const double base = sc.waves * ((sc.waves > 1 ? avg : full) * nkb + fixed);
     for (int f = 1; f == 1 || (f * sc.rest <= pairs && nkb / f >= 2); ++f) {
       sc.parts = f;
       double t = base;
       if (sc.rest > 0) {
-        t += std::ceil((double)nkb / f) * full + fixed;
+        t += std::ceil((double)nkb / f) * block_cycles<SCH>(sc.bn, sc.bn, (double)(f * sc.rest) / pairs) + fixed;
         // partial tiles out and back in (L2, about 64 bytes a cycle and SM)
         if (f > 1) t += 3000.0 + (f + 1) * 8.0 * sc.bn;
       }
