@@ -100,28 +100,29 @@ struct Piece<__half> {
   __device__ static T2 pair(__half a, __half b) { return __halves2half2(a, b); }
 };
 
-// Scheme: piece type, pieces of A (NPA) and B (NPW), product list (product 0 is x0 * y0).
+// Scheme: piece type, pieces of A (NPA) and B (NPW), product list (product 0 is x0 * y0), K blocks
+// per drained partial sum of x0 * y0 (FLUSH).
 enum : int { SCH_BF16X3 = 1, SCH_BF16X6 = 2, SCH_FP16X3 = 3 };
 template <int SCH>
 struct Scheme;
 template <>
 struct Scheme<SCH_BF16X3> {
   using T = __nv_bfloat16;
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_FP16X3> {
   using T = __half;
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_BF16X6> {
   using T = __nv_bfloat16;
-  static constexpr int NPA = 3, NPW = 3, NPROD = 6;
+  static constexpr int NPA = 3, NPW = 3, NPROD = 6, FLUSH = 2;
   // (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : (i == 4 ? 1 : (i == 5 ? 2 : 0)); }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : (i == 3 ? 2 : (i == 4 ? 1 : 0)); }
@@ -130,20 +131,19 @@ struct Scheme<SCH_BF16X6> {
 // pieces of 128 A rows and of BN / 2 B rows, so a pair takes in 64 KB per CTA and 1536 MMA
 // cycles at BN = 256 where one CTA per 128 x 128 tile takes 64 KB per 768: shared-memory
 // traffic (operand reads of the MMAs plus the fill) bounds the smaller tile.  Of x0 * y0
-// 16 truncating MMA additions go into a drained sum, as many as the 22-bit pieces' error
-// allows; 8 cost 2-8 %.  K blocks of 32 in twice the stages lost 10-25 % (64-byte rows).
+// 16 truncating MMA additions go into a drained sum with two pieces (8 cost 2-8 %), 8 with
+// three, whose 24 bits the truncation of 16 would show (1.9 times the error).  K blocks of 32 in twice the stages lost 10-25 % (64-byte rows).
 //
 // Measured on one GB300, FP16x3, time of one launch of a degree's two, before (one CTA per
 // 128 x 128 tile, [A | B] against four columns per vector) and after: n = 16384, k = 1300
-// 28.0 -> 11.6 ms (three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained);
-// n = 4096, k = 260 370 -> 192 us; n = 3001, k = 83 88 -> 60 us; n = 512, k = 30 28 -> 19 us.
-// What bounds it: the power cap at n = 16384; the pieces of M (16 n^2 bytes) from HBM, 21 us,
+// 28.0 -> 11.7 ms (three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained);
+// n = 4096, k = 260 370 -> 185 us; n = 3001, k = 83 88 -> 58 us; n = 512, k = 30 28 -> 17 us.
+// What bounds it: the power cap, which holds the clock near 1.45 of 2.07 GHz, from n = 4096 on; the pieces of M (16 n^2 bytes) from HBM, 21 us,
 // and a fixed 12 us of launch, first loads and tile end at n = 3001.  Whole filters: degree 20
-// at n = 4096 15.9 -> 8.4 ms, degree 8 at n = 16384 448 -> 201 ms.  Error against 64 bits 0.5
-// to 1.07 of the earlier form's over sizes from n = 64 to 4096.
+// at n = 4096 15.9 -> 8.2 ms, degree 8 at n = 16384 448 -> 201 ms.  Error against 64 bits 0.46
+// to 1.03 of the earlier form's over 36 drawn cases of n = 64 to 2600, 0.95 at n = 4096.
 constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int FLUSH = 4;                 // K blocks per drained partial sum of x0 * y0
 constexpr int MAX_ST = 8;                // most ring stages
 constexpr int RING_BYTES = 196608;       // (all 227 KB, 4 stages at BN = 192, ran 2-5 % slower)
 constexpr int NBAR = 2 * MAX_ST + 10;    // full, empty, acc_full[2], acc_empty[2], cross_full, cross_empty, out_full[2], out_empty[2]
@@ -435,6 +435,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     tc_hop_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Epi ep, const __grid_constant__ Sched sc) {
   using SC = Scheme<SCH>;
   using T = typename SC::T;
+  constexpr int FLUSH = SC::FLUSH;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
@@ -936,10 +937,12 @@ static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POp
 
 // Cycles of one K block of a 256 x w tile in a launch of bn-wide tiles with a share `active` of the
 // pairs at work: the MMAs (w / 2 each), the shared-memory traffic at 128 bytes a cycle (operand
-// reads and the ring's fill), or the stage's way from L2, which gives the 152 SMs about 10 TB/s in
-// all (measured 0.8-0.85 us a K block for tiles of 160 and of 192 columns at n = 4096, whose MMAs
-// take 0.5 and 0.6).  That favours wide tiles: n = 6000, k = 100 225 -> 182 us a launch, n = 8192,
-// k = 300 786 -> 720 us against a choice by the other two terms.
+// reads and the ring's fill), or 0.027 cycles a byte of a stage, a fit to what a K block was
+// measured to take with all pairs busy (0.8-0.85 us for tiles of 160 and of 192 columns at n = 4096,
+// whose MMAs take 0.5 and 0.6 at the top clock; the same with half of B's loads replaced by
+// multicasts between two pairs and with the accumulators alternating, so the clock under the
+// power cap is the likely cause).  It favours wide tiles: n = 6000, k = 100 225 -> 182 us a
+// launch, n = 8192, k = 300 786 -> 704 us against a choice by the other two terms.
 template <int SCH>
 static double block_cycles(int w, int bn, double active) {
   using SC = Scheme<SCH>;
