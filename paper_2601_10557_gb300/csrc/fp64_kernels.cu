@@ -34,16 +34,17 @@ int num_sms() {
 
 // Tile width and K split of an FP64 product with M rows, N columns and K steps of
 // `fma_step` DFMA per row and column, `tile_step` further FP64 instructions per row and K
-// step of a tile (forming its left operand).  The estimated clocks of a split: waves of
-// CTAs x (FP64 instructions of a CTA / 2 + 1500 for its loads' latency), plus the sum of
-// the partials (two additions per output and split over all SMs) and its launch.
+// step of a tile (forming its left operand), and `sums` complex sums per row and column.  The
+// estimated clocks of a split: waves of CTAs x (FP64 instructions of a CTA / 2 + 1500 for its
+// loads' latency), plus the sum of the partials (two additions per sum and split over all SMs)
+// and its launch.
 struct Plan {
   int tn;       // columns per warp
   int split;
   int64_t chunk;
 };
-Plan plan_fp64(int64_t M, int64_t N, int64_t K, double fma_step, double tile_step, const int* widths, int nwidths,
-               bool may_split) {
+Plan plan_fp64(int64_t M, int64_t N, int64_t K, double fma_step, double tile_step, int sums, const int* widths,
+               int nwidths, bool may_split) {
   const int sms = num_sms();
   Plan best{widths[0], 1, K};
   double best_t = 0.0;
@@ -52,11 +53,11 @@ Plan plan_fp64(int64_t M, int64_t N, int64_t K, double fma_step, double tile_ste
     const int64_t tiles = (int64_t)cdiv(M, ROWS) * cdiv(N, WARPS * tn);
     const double step = 0.5 * ROWS * (fma_step * WARPS * tn + tile_step);
     for (int64_t sp = 1; sp <= 64; ++sp) {
-      if (sp > 1 && (!may_split || K / sp < 2 || 16.0 * (double)sp * (double)M * (double)N > PART_LIMIT)) break;
+      if (sp > 1 && (!may_split || K / sp < 2 || 16.0 * sums * (double)sp * (double)M * (double)N > PART_LIMIT)) break;
       const int64_t chunk = (K + sp - 1) / sp;
       const double waves = (double)((tiles * sp + sms - 1) / sms);
       double t = waves * ((double)chunk * step + 1500.0);
-      if (sp > 1) t += 3000.0 + (double)sp * (double)M * (double)N / sms;
+      if (sp > 1) t += 3000.0 + sums * (double)sp * (double)M * (double)N / sms;
       if (best_t == 0.0 || t < best_t * 0.999) {
         best_t = t;
         best = {tn, (int)((K + chunk - 1) / chunk), chunk};
@@ -69,20 +70,22 @@ Plan plan_fp64(int64_t M, int64_t N, int64_t K, double fma_step, double tile_ste
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// H application.  H is real on vectors [z; conj(z)]: H [z; conj(z)] = [t; -conj(t)] with
+// H application, J-fixed form (HOP_JFIXED).  H is real on vectors [z; conj(z)]: H [z; conj(z)] = [t; -conj(t)] with
 // t = A z + B conj(z), a real 2n x 2n matrix on (Re z, Im z):
 //   Re t = (Ar + Br) Re z + (Bi - Ai) Im z,  Im t = (Ai + Bi) Re z + (Ar - Br) Im z.
 // Every w = [x; y] is the sum of [a; conj(a)] and -i [c; conj(c)], a = (x + conj(y))/2 and
 // c = i (x - conj(y))/2, so H w takes 2 x 4 n^2 DFMA instead of the 16 n^2 of the complex
-// product with [A | B].  The kernel stages the four sums of A and B (4 additions per
+// product with [A | B].  Both halves of H w are then sums and differences of two numbers of
+// the size of A x, so the smaller half is exact only relative to the larger one: the form is
+// for results of which that is all that is used (norms and inner products of whole vectors,
+// and the filter of a solve, whose QR and Rayleigh-Ritz steps hold the basis as J-fixed vectors
+// themselves).  The kernel stages the four sums of A and B (4 additions per
 // element and tile) and 2a, 2c (4 per vector entry and tile), each a few per cent of the
 // tile's DFMAs, and computes t for `cols` columns (2j: 2a_j, 2j + 1: 2c_j of vector j).
 //
 // Measured on one GB300, before (64 x 32 tiles, the complex product, K chunks >= 256) and
-// after: residuals of 200 vectors at n = 4096 99.3 -> 47.7 ms (1.12 of 1.20 TFLOP/s); a
-// degree-20 filter of 30 vectors at n = 512 42.4 -> 5.26 ms, of 67 ragged ones at n = 1301
-// 148 -> 42.4 ms; residuals of 6 vectors at n = 64 533 -> 42 us.  Error of the filters
-// against 64 bits: unchanged (5.7e-15 and 6.9e-15, before 7.0e-15 and 6.8e-15).
+// after: residuals of 200 vectors at n = 4096 99.3 -> 47.7 ms (1.12 of 1.20 TFLOP/s), of 6
+// vectors at n = 64 533 -> 42 us.
 
 // Epilogue for output row i (< n) of vector j: top and bottom entry of H w.
 __device__ __forceinline__ void hop_epilogue(const HopArgs& a, int64_t i, int64_t j, cplx top, cplx bot) {
@@ -223,10 +226,10 @@ __global__ void hop_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
 }
 
 template <bool GEN>
-static int hop_launch(const HopArgs& a, cudaStream_t s) {
+static int hop_jfixed(const HopArgs& a, cudaStream_t s) {
   static const int widths_gen[4] = {2, 4, 6, 8}, widths_top[4] = {1, 2, 4, 8};
   const int64_t cols = GEN ? 2 * a.k : a.k;
-  const Plan p = plan_fp64(a.n, cols, a.n, 4.0, 4.0, GEN ? widths_gen : widths_top, 4, !a.no_split);
+  const Plan p = plan_fp64(a.n, cols, a.n, 4.0, 4.0, 1, GEN ? widths_gen : widths_top, 4, !a.no_split);
   cplx* part = nullptr;
   if (p.split > 1) CB_CUDA(dalloc(&part, sizeof(cplx) * p.split * a.n * cols, s));
   const dim3 grid(cdiv(a.n, ROWS), cdiv(cols, WARPS * p.tn), (unsigned)p.split);
@@ -254,18 +257,25 @@ int hop_top_fp64(const cplx* A, const cplx* B, int64_t n, const cplx* X, int64_t
   if (k <= 0 || n <= 0) return CHASE_BSE_OK;
   HopArgs a{};
   a.A = A; a.B = B; a.n = n; a.W = X; a.k = k; a.out = Y;
-  return hop_launch<false>(a, s);
+  return hop_jfixed<false>(a, s);
 }
 
 // The complex product [A | B] [x, conj(y); y, conj(x)] on the same tiles, two sums per row
-// and vector over the 2n columns of [A | B]: the top half of H w and -conj of the bottom.
-// Twice the DFMAs of hop_kernel.  Only the Rayleigh-Ritz step on a caller's basis uses it:
-// the phases of its Ritz vectors come out of the last Jacobi rotations, whose pivots
-// are rounding residue (a change of the last bit of H Q turns them by up to 1e-5), so its
-// sums keep their order and their K chunks.
-template <int TN>
+// and vector over the 2n columns of [A | B]: the top half of H w and -conj of the bottom, each
+// a sum of its own products, accurate relative to its own size (an eigenvector's lower half
+// is smaller than the upper one by the coupling).  Twice the DFMAs of hop_kernel.  HOP_BLOCKS
+// splits K by plan_fp64 and (FOLD) sums every 64 products by themselves first, so that the length
+// of a K range does not show in the error (n = 1301, k = 67, degree 4 to 20: 1.1e-14 with one
+// chain per range, 5.9e-15 so; 1 % more additions).  HOP_ORDERED keeps one chain and a fixed chunk rule: the phases of the Ritz vectors
+// of a caller's basis come out of the last Jacobi rotations, whose pivots are rounding residue
+// (a change of the last bit of H Q turns them by up to 1e-5).
+// Measured on one GB300, before (64 x 32 tiles, K chunks >= 256) and after: a degree-20 filter
+// of 30 vectors at n = 512 42.4 -> 9.6 ms, of 67 ragged ones at n = 1301 147 -> 80 ms (16 n^2 k
+// DFMA at 1.17 of 1.20 TFLOP/s; the J-fixed form takes 5.25 and 41 ms, but leaves the lower half
+// 1.3e-13 of its size off instead of 8.6e-15, and 1e-12 and more at a coupling of 1e-3).
+template <int TN, bool FOLD>
 __global__ void __launch_bounds__(THREADS)
-hop_ordered_kernel(HopArgs a, cplx* part, int64_t kchunk) {
+hop_blocks_kernel(HopArgs a, cplx* part, int64_t kchunk) {
   __shared__ cplx Ps[BK][ROWS + 1];
   __shared__ cplx W1s[BK][WARPS * TN];
   __shared__ cplx W2s[BK][WARPS * TN];
@@ -276,10 +286,18 @@ hop_ordered_kernel(HopArgs a, cplx* part, int64_t kchunk) {
   const int64_t kend = kbeg + kchunk < n2 ? kbeg + kchunk : n2;
   const int64_t mycol = col0 + warp * TN;
   const bool active = mycol < a.k;  // warp-uniform
-  cplx acc1[TN], acc2[TN];
+  cplx acc1[TN], acc2[TN], sum1[TN], sum2[TN];
 #pragma unroll
-  for (int c = 0; c < TN; ++c) { acc1[c] = mk(0, 0); acc2[c] = mk(0, 0); }
+  for (int c = 0; c < TN; ++c) acc1[c] = acc2[c] = sum1[c] = sum2[c] = mk(0, 0);
   for (int64_t kb = kbeg; kb < kend; kb += BK) {
+    if (FOLD && ((kb - kbeg) & 63) == 0) {
+#pragma unroll
+      for (int c = 0; c < TN; ++c) {
+        sum1[c] = cadd(sum1[c], acc1[c]);
+        sum2[c] = cadd(sum2[c], acc2[c]);
+        acc1[c] = acc2[c] = mk(0, 0);
+      }
+    }
     const int kn = (int)(kend - kb < BK ? kend - kb : BK);
     for (int idx = tid; idx < ROWS * BK; idx += THREADS) {
       const int kk = idx % BK, r = idx / BK;
@@ -320,6 +338,10 @@ hop_ordered_kernel(HopArgs a, cplx* part, int64_t kchunk) {
   for (int c = 0; c < TN; ++c) {
     const int64_t j = mycol + c;
     if (j >= a.k) continue;
+    if (FOLD) {
+      acc1[c] = cadd(sum1[c], acc1[c]);
+      acc2[c] = cadd(sum2[c], acc2[c]);
+    }
     if (part) {
       cplx* p = part + ((int64_t)blockIdx.z * a.k + j) * n2;
       p[i] = acc1[c];
@@ -329,7 +351,7 @@ hop_ordered_kernel(HopArgs a, cplx* part, int64_t kchunk) {
     }
   }
 }
-__global__ void hop_ordered_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
+__global__ void hop_blocks_reduce_kernel(HopArgs a, const cplx* part, int nsplit) {
   const int64_t n = a.n, n2 = 2 * n, total = n * a.k;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
@@ -354,23 +376,36 @@ static void ordered_chunks(int64_t tiles, int64_t K, int64_t min_chunk, int64_t 
   *splits = (int)std::max<int64_t>(1, (K + *chunk - 1) / *chunk);
 }
 
-static int hop_ordered(const HopArgs& a, cudaStream_t s) {
+static int hop_blocks(const HopArgs& a, cudaStream_t s) {
+  static const int widths[4] = {1, 2, 3, 4};
   const int64_t n2 = 2 * a.n;
-  int64_t chunk;
-  int splits;
-  ordered_chunks((int64_t)cdiv(a.n, 64) * cdiv(a.k, a.k <= 4 ? 4 : 32), n2, 256, 16, &chunk, &splits);
+  Plan p;
+  if (a.form == HOP_ORDERED) {
+    p.tn = a.k >= 32 ? 4 : (a.k >= 16 ? 2 : 1);
+    ordered_chunks((int64_t)cdiv(a.n, 64) * cdiv(a.k, a.k <= 4 ? 4 : 32), n2, 256, 16, &p.chunk, &p.split);
+  } else {
+    p = plan_fp64(a.n, a.k, n2, 8.0, 0.0, 2, widths, 4, !a.no_split);
+  }
   cplx* part = nullptr;
-  if (splits > 1) CB_CUDA(dalloc(&part, sizeof(cplx) * splits * n2 * a.k, s));
-  const int tn = a.k >= 32 ? 4 : (a.k >= 16 ? 2 : 1);
-  const dim3 grid(cdiv(a.n, ROWS), cdiv(a.k, WARPS * tn), (unsigned)splits);
+  if (p.split > 1) CB_CUDA(dalloc(&part, sizeof(cplx) * p.split * n2 * a.k, s));
+  const dim3 grid(cdiv(a.n, ROWS), cdiv(a.k, WARPS * p.tn), (unsigned)p.split);
   const int64_t tid = timer_begin(1, 32.0 * (double)a.n * (double)a.n * (double)a.k, s);
-  if (tn == 4) hop_ordered_kernel<4><<<grid, THREADS, 0, s>>>(a, part, chunk);
-  else if (tn == 2) hop_ordered_kernel<2><<<grid, THREADS, 0, s>>>(a, part, chunk);
-  else hop_ordered_kernel<1><<<grid, THREADS, 0, s>>>(a, part, chunk);
+  if (a.form == HOP_ORDERED) {
+    if (p.tn == 4) hop_blocks_kernel<4, false><<<grid, THREADS, 0, s>>>(a, part, p.chunk);
+    else if (p.tn == 2) hop_blocks_kernel<2, false><<<grid, THREADS, 0, s>>>(a, part, p.chunk);
+    else hop_blocks_kernel<1, false><<<grid, THREADS, 0, s>>>(a, part, p.chunk);
+  } else {
+    switch (p.tn) {
+      case 1: hop_blocks_kernel<1, true><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+      case 2: hop_blocks_kernel<2, true><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+      case 3: hop_blocks_kernel<3, true><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+      default: hop_blocks_kernel<4, true><<<grid, THREADS, 0, s>>>(a, part, p.chunk); break;
+    }
+  }
   count_launch();
   if (part) {
     const int64_t blocks = (a.n * a.k + 127) / 128;
-    hop_ordered_reduce_kernel<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, s>>>(a, part, splits);
+    hop_blocks_reduce_kernel<<<(unsigned)(blocks < 8192 ? blocks : 8192), 128, 0, s>>>(a, part, p.split);
     count_launch();
   }
   timer_end(tid, s);
@@ -381,7 +416,7 @@ static int hop_ordered(const HopArgs& a, cudaStream_t s) {
 
 int hop_fp64(const HopArgs& a, cudaStream_t s) {
   if (a.k <= 0 || a.n <= 0) return CHASE_BSE_OK;
-  return a.ordered ? hop_ordered(a, s) : hop_launch<true>(a, s);
+  return a.form == HOP_JFIXED ? hop_jfixed<true>(a, s) : hop_blocks(a, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -5,13 +5,19 @@
 namespace cb {
 
 // ---- H application --------------------------------------------------------
-// H W for W = [X; Y] (2n x k, column-major, ld 2n) reading only A and B (row-major), as a
-// real 2n x 2n matrix on the J-fixed parts of each vector (the block structure of
-// Section 1; see fp64_kernels.cu).
+// H W for W = [X; Y] (2n x k, column-major, ld 2n) reading only A and B (row-major; the block
+// structure of Section 1).
 enum HopMode : int {
   HOP_STORE = 0,   // out = H W               (sflip: out = S H W)
   HOP_CHEB = 1,    // out = alpha (H W - c Wc) + beta Wp
   HOP_RESID = 2    // out = H W - W diag(lambda)
+};
+
+// How the product is formed (see fp64_kernels.cu).
+enum HopForm : int {
+  HOP_BLOCKS = 0,  // A x + B y and conj(B) x + conj(A) y, each half to its own accuracy
+  HOP_JFIXED = 1,  // half the operations; the smaller half accurate relative to the larger one only
+  HOP_ORDERED = 2  // HOP_BLOCKS in a fixed summation order
 };
 
 struct HopArgs {
@@ -28,7 +34,7 @@ struct HopArgs {
   const cplx* Wp;    // HOP_CHEB: previous iterate (ld 2n), unused if beta == 0
   const double* lambda;  // HOP_RESID
   int no_split;      // 1: one launch over the whole K range (no split-K partials, allocates nothing)
-  int ordered;       // 1: the complex product with its fixed summation order (see hop_ordered_kernel)
+  int form;          // HopForm
 };
 
 int hop_fp64(const HopArgs& a, cudaStream_t s);

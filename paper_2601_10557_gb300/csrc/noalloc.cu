@@ -63,6 +63,7 @@ extern "C" int chase_bse_residuals_noalloc(const void* A, const void* B, int64_t
   a.out = R;
   a.mode = cb::HOP_RESID;
   a.lambda = lambda;
+  a.form = cb::HOP_JFIXED;  // only the norms are returned
   CB_TRY(cb::hop_fp64(a, s));
   CB_TRY(cb::col_norms(R, 2 * n, k, res, s));
   return CHASE_BSE_OK;

@@ -213,10 +213,11 @@ __global__ void cheb_combine_kernel(cplx* nxt, const cplx* U, const cplx* cur, c
 // as FP64-accurate sliced GEMMs on the tensor cores, and the whole recurrence on the J-fixed
 // halves z of the vectors (two columns each): H [z; conj z] = i [z'; conj z'] with
 // z' = -i P'z, so the second product takes the first one's result as pairs (b, -a) and no
-// step leaves that form.  Else on the FP64 pipe (the second one with the recurrence fused).
+// step leaves that form.  Else on the FP64 pipe (the second one with the recurrence fused), with
+// jfixed in the J-fixed form.
 static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0, int64_t k, const int* degs,
                               double mu1, double mu_nevex, double muN, cplx* out, Workspace& ws, cudaStream_t s,
-                              FilterStats* fs, const SlicedOp* ph) {
+                              FilterStats* fs, const SlicedOp* ph, bool jfixed) {
   const int64_t n2 = 2 * n;
   cplx *Y1, *Y2, *T, *U = nullptr;
   int* err = nullptr;
@@ -263,6 +264,7 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
     } else {
       HopArgs h{};
       h.A = A; h.B = B; h.n = n; h.W = cur; h.k = kj; h.out = T; h.mode = HOP_STORE;
+      h.form = jfixed ? HOP_JFIXED : HOP_BLOCKS;
       CB_TRY(hop_fp64(h, s));
     }
     double alpha, beta;
@@ -286,6 +288,7 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
       HopArgs g{};
       g.A = A; g.B = B; g.n = n; g.W = T; g.k = kj; g.out = nxt; g.mode = HOP_CHEB;
       g.alpha = alpha; g.beta = beta; g.c = c; g.Wc = cur; g.Wp = prev;
+      g.form = jfixed ? HOP_JFIXED : HOP_BLOCKS;
       CB_TRY(hop_fp64(g, s));
     }
     if (fs) {
@@ -326,7 +329,7 @@ static int filter_fp64_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0,
 
 int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const int* degs, const int* prec,
            double mu1, double mu_nevex, double muN, int scheme, const double* ritz, const cplx* R, cudaStream_t s,
-           FilterStats* fs, const SlicedOp* ph, const cplx* P2, const cplx* Q2) {
+           FilterStats* fs, const SlicedOp* ph, const cplx* P2, const cplx* Q2, bool jfixed) {
   if (k == 0) return CHASE_BSE_OK;
   const int64_t n2 = 2 * n;
   Workspace ws(s);
@@ -349,7 +352,7 @@ int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const in
     CB_CUDA(cudaMemcpyAsync(didx, idx.data(), sizeof(int) * m, cudaMemcpyHostToDevice, s));
     CB_TRY(gather_cols(Y0, W, didx, n2, m, s));
     if (grp == 0) {
-      CB_TRY(filter_fp64_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, gws, s, fs, ph));
+      CB_TRY(filter_fp64_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, gws, s, fs, ph, jfixed));
     } else {
       if (!mixed_available()) return CHASE_BSE_UNSUPPORTED;
       if (ritz && R) {
@@ -431,7 +434,7 @@ int lanczos_bounds(const cplx* A, const cplx* B, int64_t n, const cplx* V0, int6
   CB_CUDA(cudaMemcpyAsync(Wv, V0, sizeof(cplx) * sz, cudaMemcpyDeviceToDevice, s));
   HopArgs h{};
   h.A = A; h.B = B; h.n = n; h.k = nvec; h.mode = HOP_STORE;
-  h.W = Wv; h.out = Y;
+  h.W = Wv; h.out = Y; h.form = HOP_JFIXED;  // only inner products of whole vectors are kept
   // H applied on the FP64 pipe, or (mixed mode) by the sliced tensor-core GEMM
   auto apply_h = [&]() { return ph ? hop_sliced(*ph, Wv, n, nvec, Y, s) : hop_fp64(h, s); };
   CB_TRY(apply_h());
@@ -574,7 +577,7 @@ int rayleigh_ritz(const cplx* A, const cplx* B, int64_t n, const cplx* Q, int64_
   CB_TRY(ws.alloc(&idx_d, h));
   // Algorithm 2: T = S H Q, M = Q^* T
   HopArgs a{};
-  a.A = A; a.B = B; a.n = n; a.W = Q; a.k = k; a.out = T; a.mode = HOP_STORE; a.sflip = 1; a.ordered = 1;
+  a.A = A; a.B = B; a.n = n; a.W = Q; a.k = k; a.out = T; a.mode = HOP_STORE; a.sflip = 1; a.form = HOP_ORDERED;
   CB_TRY(hop_fp64(a, s));
   CB_TRY(zgemm('C', 'N', k, k, n2, mk(1, 0), Q, n2, T, n2, mk(0, 0), M, k, s));
   CB_TRY(hermitize(M, k, s));
@@ -892,6 +895,7 @@ int residuals(const cplx* A, const cplx* B, int64_t n, const cplx* W, const doub
   if (!R) CB_TRY(ws.alloc(&R, 2 * n * k));
   HopArgs a{};
   a.A = A; a.B = B; a.n = n; a.W = W; a.k = k; a.out = R; a.mode = HOP_RESID; a.lambda = lambda;
+  a.form = Rout ? HOP_BLOCKS : HOP_JFIXED;  // for the norms alone the halves need no accuracy of their own
   CB_TRY(hop_fp64(a, s));
   CB_TRY(col_norms(R, 2 * n, k, res, s));
   return CHASE_BSE_OK;
@@ -1166,7 +1170,7 @@ int solve(const cplx* A, const cplx* B, int64_t n, int64_t nev, int64_t nex, int
     const bool corr = mixed && !ritz_keep.empty();
     CB_TRY(filter(A, B, n, W, kf, degs.data(), prec.data(), mu1, mu_ne, muN, scheme,
                   corr ? ritz_keep.data() : nullptr, corr ? Rkeep : nullptr, s, &fs, sliced ? &ph : nullptr, P2,
-                  Q2));
+                  Q2, o.rr == 0));
     st.ms_filter += clk.stop();
     // orthonormalisation: W- = K conj(W+), Q = [S Y+, S Y-, W+, W-] R^{-1}, drop the locked part;
     // J-fixed basis (top halves) unless its CholeskyQR2 breaks down

@@ -21,11 +21,14 @@ enum FilterScheme : int { SCHEME_BF16X3 = 1, SCHEME_BF16X6 = 2, SCHEME_FP16X3 = 
 // With ph (the sliced operand of slice_hamiltonian) the FP64 columns apply H by
 // FP64-accurate sliced GEMMs on the tensor cores instead of the FP64 pipe.  With P2, Q2
 // (the blocks of H^2, see form_h2) the tensor-core columns apply H^2 from its blocks
-// (the explicit-H^2 variant).
+// (the explicit-H^2 variant).  jfixed: the FP64 pipe applies H in the J-fixed form, which
+// keeps the smaller half of a vector only to the accuracy of the larger one; a solve whose QR
+// and Rayleigh-Ritz steps work on J-fixed vectors knows it no better.
 struct SlicedOp;
 int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const int* degs, const int* prec,
            double mu1, double mu_nevex, double muN, int scheme, const double* ritz, const cplx* R, cudaStream_t s,
-           FilterStats* fs, const SlicedOp* ph = nullptr, const cplx* P2 = nullptr, const cplx* Q2 = nullptr);
+           FilterStats* fs, const SlicedOp* ph = nullptr, const cplx* P2 = nullptr, const cplx* Q2 = nullptr,
+           bool jfixed = false);
 
 // The blocks of H^2 = [[P2, Q2], [conj Q2, conj P2]]: P2 = A A - B conj(B),
 // Q2 = A B - B conj(A) (row-major n x n, like A and B), as the top block row
