@@ -207,8 +207,6 @@ int chase_bse_rr(const void* A, const void* B, int64_t n, const void* Q, int64_t
                  double* ritz, void* Wpos, void* stream);
 
 /* Residual norms ||H w_j - lambda_j w_j||_2 (Section 4.5).
- * On compute capability 10.3 H W is an FP64-accurate sliced tensor-core product where
- * that is faster than the FP64 pipe (see chase_bse_dgemm_sliced), else FP64 DFMA.
  *   W      device, 2n x k; lambda device, k doubles; res device, k doubles. */
 int chase_bse_residuals(const void* A, const void* B, int64_t n, const void* W,
                         const double* lambda, int64_t k, double* res, void* stream);
@@ -222,9 +220,8 @@ int chase_bse_residuals(const void* A, const void* B, int64_t n, const void* W,
  * CHASE_BSE_NOALLOC_MAX_ENTRIES complex128 entries (8 MiB) that every device
  * using the library holds until the process exits, and the call performs no
  * allocation or free: its H product runs as one launch over the whole K range,
- * without the split-K partial sums of chase_bse_residuals and without the
- * FP64-accurate sliced tensor-core product that larger problems take there (slower;
- * results equal to FP64 rounding).
+ * without the split-K partial sums of chase_bse_residuals (slower when 2n * k is
+ * small, identical results up to the order of the FP64 sums).
  *   - 2n * k > CHASE_BSE_NOALLOC_MAX_ENTRIES returns BAD_ARG; nothing runs.
  *   - The first call on a device looks up the array's device address (once per
  *     device, with that device current); make that first call before any stream

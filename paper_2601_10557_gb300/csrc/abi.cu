@@ -172,7 +172,7 @@ int chase_bse_residuals(const void* A, const void* B, int64_t n, const void* W, 
                         double* res, void* stream) {
   if (k == 0) return CHASE_BSE_OK;
   if (!A || !B || !W || !lambda || !res || n < 1 || k < 0) return CHASE_BSE_BAD_ARG;
-  CB_GUARD(return cb::residuals_check((const cplx*)A, (const cplx*)B, n, (const cplx*)W, lambda, k, res,
+  CB_GUARD(return cb::residuals((const cplx*)A, (const cplx*)B, n, (const cplx*)W, lambda, k, res,
                                 (cudaStream_t)stream);)
 }
 

@@ -887,6 +887,12 @@ static int rayleigh_ritz_jfixed(const cplx* A, const cplx* B, int64_t n, const c
   return CHASE_BSE_OK;
 }
 
+// On the FP64 pipe whatever the size: a converged pair's residual is a difference at the
+// rounding level of its terms, where an FP64 sum's error follows the products that occur, a sliced
+// product's the largest entries of the row and of the vector.  Refined pairs of a diagonally
+// dominant H with n = 768: sliced 9e-14, pipe 7e-17 off a residual of 6e-14; of a graded diagonal to
+// 1e7 1.8e-8 off one of 3e-11.  (The sliced product would take 1.7 of the pipe's 48 ms at
+// n = 4096, k = 200.)
 int residuals(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k, double* res,
               cudaStream_t s, cplx* Rout) {
   if (k == 0) return CHASE_BSE_OK;
@@ -899,29 +905,6 @@ int residuals(const cplx* A, const cplx* B, int64_t n, const cplx* W, const doub
   CB_TRY(hop_fp64(a, s));
   CB_TRY(col_norms(R, 2 * n, k, res, s));
   return CHASE_BSE_OK;
-}
-
-// The residual check of a caller's pairs.  FP64 products run at 1/64 of the FP32 rate, so H W is
-// a sliced product (error against 64 bits no larger) where it is faster: the pipe takes
-// 1.43e-5 us n^2 k + 45 us, the sliced path 3.6e-5 us n^2 for H's digits + 120 us.  A workspace that
-// cannot be had also leaves it to the pipe.  Measured on one GB300: n = 4096, k = 200
-// 47.8 -> 1.72 ms; k = 8 2.03 -> 0.71 ms; n = 1024, k = 16 0.29 -> 0.15 ms; n = 512, k = 50
-// 0.27 -> 0.13 ms.
-static bool residual_sliced_faster(int64_t n, int64_t k) {
-  const double n2 = (double)n * (double)n;
-  return 1.43e-5 * n2 * (double)k > 4.0e-5 * n2 + 100.0;
-}
-int residuals_check(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k,
-                    double* res, cudaStream_t s) {
-  if (k > 0 && residual_sliced_faster(n, k) && mixed_available()) {
-    Workspace ws(s);
-    cplx* R;
-    int st = ws.alloc(&R, 2 * n * k);
-    if (st == CHASE_BSE_OK) st = residual_sliced(A, B, n, W, lambda, k, R, ws, s);
-    if (st == CHASE_BSE_OK) return col_norms(R, 2 * n, k, res, s);
-    if (st != CHASE_BSE_OOM) return st;
-  }
-  return residuals(A, B, n, W, lambda, k, res, s);
 }
 
 int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, cplx* gB, cudaStream_t s) {

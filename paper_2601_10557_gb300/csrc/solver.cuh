@@ -54,9 +54,6 @@ int rayleigh_ritz(const cplx* A, const cplx* B, int64_t n, const cplx* Q, int64_
 // vectors are kept in Rout when it is not NULL (2n x k).
 int residuals(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k,
               double* res, cudaStream_t s, cplx* Rout = nullptr);
-// The norms for a caller's pairs: H W as a sliced tensor-core product where that is faster.
-int residuals_check(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k,
-                    double* res, cudaStream_t s);
 
 int solve(const cplx* A, const cplx* B, int64_t n, int64_t nev, int64_t nex, int deg, double tol,
           const chase_bse_opts* opts, double* evals, cplx* evecs, chase_bse_stats* stats);

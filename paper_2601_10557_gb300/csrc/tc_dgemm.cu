@@ -467,11 +467,10 @@ __global__ void slice_kernel(Src src, int64_t K, int64_t kpad, int64_t plane, __
     put_digits(2 * p < K ? src.pair(r, p) : make_double2(0.0, 0.0), e, row + 2 * p, plane);
   if (threadIdx.x == 0) exps[r] = e;
 }
-// The real form P' of rows i0 .. of H, one CTA per row i, which gives rows 2i and 2i + 1 from
+// The real form P' of H, one CTA per row i, which gives rows 2i and 2i + 1 from
 // one read of A and B each pass: y = A x + B conj(x) in (re, im) interleaved form,
 // Re y: (Ar + Br, Bi - Ai), Im y: (Ai + Bi, Ar - Br).  The FP64 additions (4 per entry and pass)
-// take as long as the memory traffic.  The residual check of 8 vectors at n = 4096, most of it
-// these digits, 1.11 -> 0.71 ms against one warp per row of P'.
+// take as long as the memory traffic.
 __global__ void slice_ham_kernel(const cplx* A, const cplx* B, int64_t n, int64_t kpad, int64_t plane,
                                  __nv_bfloat16* planes, int* exps) {
   const int64_t i = blockIdx.x;
@@ -629,20 +628,6 @@ __global__ void jmerge_kernel(cplx* W, const cplx* Z0, const cplx* Z1, const cpl
     W[j * 2 * n + n + i] = mk(a.x - c.y, -a.y - c.x);  // conj(a) - i conj(c)
   }
 }
-// R = H W - W diag(lambda) from T = [P'a_j, P'c_j]; NaN where a wait of the products ran out
-__global__ void jresidual_kernel(const cplx* T, const cplx* W, const double* lambda, int64_t n, int64_t k, cplx* R,
-                                 const int* err) {
-  const int64_t total = n * k;
-  const double bad = *err ? nan("") : 0.0;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = idx % n, j = idx / n, o = j * 2 * n + i;
-    const cplx ta = T[(2 * j) * n + i], tc = T[(2 * j + 1) * n + i], x = W[o], y = W[o + n];
-    const double lam = lambda[j];
-    R[o] = mk(fma(-lam, x.x, ta.x + tc.y) + bad, fma(-lam, x.y, ta.y - tc.x) + bad);
-    R[o + n] = mk(fma(-lam, y.x, tc.y - ta.x), fma(-lam, y.y, ta.y + tc.x));
-  }
-}
 
 static unsigned gsz(int64_t total) {
   const int64_t b = (total + 255) / 256;
@@ -667,13 +652,6 @@ static int run_slice(const Src& src, SlicedOp& op, cudaStream_t s) {
   const int threads = op.K >= 4096 ? 256 : (op.K >= 512 ? 128 : 32);
   slice_kernel<Src><<<(unsigned)op.rows, threads, 0, s>>>(src, op.K, op.kpad, op.rows_pad * op.kpad, op.planes,
                                                           op.exps);
-  count_launch();
-  CB_LAUNCH();
-  return CHASE_BSE_OK;
-}
-// rows of H -> op.rows / 2 row pairs of P'
-static int run_slice_ham(const cplx* A, const cplx* B, int64_t n, SlicedOp& op, cudaStream_t s) {
-  slice_ham_kernel<<<(unsigned)(op.rows / 2), 256, 0, s>>>(A, B, n, op.kpad, op.rows_pad * op.kpad, op.planes, op.exps);
   count_launch();
   CB_LAUNCH();
   return CHASE_BSE_OK;
@@ -775,7 +753,10 @@ int form_h2(const cplx* A, const cplx* B, int64_t n, cplx* P2, cplx* Q2, cudaStr
 
 int slice_hamiltonian(const cplx* A, const cplx* B, int64_t n, SlicedOp& op, cudaStream_t s) {
   if (op.rows != 2 * n || op.K != 2 * n) return CHASE_BSE_BAD_ARG;
-  return tcd::run_slice_ham(A, B, n, op, s);
+  tcd::slice_ham_kernel<<<(unsigned)n, 256, 0, s>>>(A, B, n, op.kpad, op.rows_pad * op.kpad, op.planes, op.exps);
+  count_launch();
+  CB_LAUNCH();
+  return CHASE_BSE_OK;
 }
 
 int jsplit(const cplx* W, int64_t n, int64_t k, cplx* Z, cudaStream_t s) {
@@ -787,33 +768,6 @@ int jsplit(const cplx* W, int64_t n, int64_t k, cplx* Z, cudaStream_t s) {
 int jmerge(cplx* W, const cplx* Z0, const cplx* Z1, const cplx* Z2, const int* sel, int64_t n, int64_t k,
            cudaStream_t s) {
   tcd::jmerge_kernel<<<tcd::gsz(n * k), 256, 0, s>>>(W, Z0, Z1, Z2, sel, n, k);
-  count_launch();
-  CB_LAUNCH();
-  return CHASE_BSE_OK;
-}
-
-int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k, cplx* R,
-                    Workspace& ws, cudaStream_t s) {
-  // H in blocks of rows whose digits take at most 2 GB
-  int64_t m = std::max<int64_t>(64, (int64_t)(2.0e9 / (56.0 * (double)n)) / 64 * 64);
-  m = std::min(m, n);
-  cplx *Z, *T;
-  int* err;
-  SlicedOp sz, ph;
-  CB_TRY(ws.alloc(&Z, n * 2 * k));
-  CB_TRY(ws.alloc(&T, n * 2 * k));
-  CB_TRY(ws.alloc(&err, 1));
-  CB_TRY(sliced_alloc(ws, sz, 2 * k, 2 * n, s));
-  CB_TRY(sliced_alloc(ws, ph, 2 * m, 2 * n, s));
-  CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-  CB_TRY(jsplit(W, n, k, Z, s));
-  CB_TRY(slice_rows(reinterpret_cast<const double*>(Z), 2 * n, 0, sz, s));
-  for (int64_t i0 = 0; i0 < n; i0 += m) {
-    ph.rows = 2 * std::min(m, n - i0);  // a shorter last block leaves the previous one's digits behind its rows
-    CB_TRY(tcd::run_slice_ham(A + i0 * n, B + i0 * n, n, ph, s));
-    CB_TRY(sliced_gemm(ph, sz, 1.0, reinterpret_cast<double*>(T + i0), 1, 2 * n, false, s, err));
-  }
-  tcd::jresidual_kernel<<<tcd::gsz(n * k), 256, 0, s>>>(T, W, lambda, n, k, R, err);
   count_launch();
   CB_LAUNCH();
   return CHASE_BSE_OK;

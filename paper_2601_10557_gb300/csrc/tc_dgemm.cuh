@@ -67,10 +67,6 @@ int hop_sliced(const SlicedOp& ph, const cplx* W, int64_t n, int64_t k, cplx* ou
 int jsplit(const cplx* W, int64_t n, int64_t k, cplx* Z, cudaStream_t s);
 int jmerge(cplx* W, const cplx* Z0, const cplx* Z1, const cplx* Z2, const int* sel, int64_t n, int64_t k,
            cudaStream_t s);
-// R = H W - W diag(lambda) (2n x k) by a sliced product with blocks of rows of H, without a
-// host synchronisation (NaN where a wait of the products ran out).
-int residual_sliced(const cplx* A, const cplx* B, int64_t n, const cplx* W, const double* lambda, int64_t k, cplx* R,
-                    Workspace& ws, cudaStream_t s);
 
 // C[r][c] = alpha * sum_k a[r][k] b[c][k] for r < a.rows, c < b.rows, written to
 // out[r * rs + c * cs]; with neg_odd the rows r odd are negated (complex
