@@ -478,14 +478,15 @@ def main():
     del hA, hB, out_gA, out_gB
 
     # ---- roofline of the dominant kernel, the filter GEMM: the operations its launches in
-    # the timed steps execute (16 n^2 k for k vectors: H as a real 2n x 2n matrix on two real
-    # columns per vector, half of the 32 n^2 k of the complex form that `value` and the
-    # library's record count) over their summed device time
+    # the timed steps execute (16 n^2 k for k vectors: a solve applies H as a real 2n x 2n matrix
+    # on two real columns per vector, half of the 32 n^2 k of the complex form that `value` and the
+    # library's record count; its thinnest launches, which run the complex form, are undercounted
+    # so) over their summed device time
     # (a CUDA event pair around each launch, recorded by the library on the launch's
     # stream).  Cross-check on full-width launches: two filter calls over all nev + nex
     # columns that differ only in the degree (d1 and d2 H^2 steps: 2 (d2 - d1) more
     # launches of the same shape; the split of P, the packing and the final combination,
-    # the same in both, cancel)
+    # the same in both, cancel); a filter call runs the complex form, 32 n^2 k
     d1, d2 = (2, 6) if n >= 16384 else (4, 20)
 
     def filter_ms(deg):
@@ -506,7 +507,7 @@ def main():
     rl = (pkg.launch_count() - rl0) // 4
     gemm_launches = 2 * (d2 - d1)
     full_launch_ms = (t2 - t1) / gemm_launches
-    full_flops = 16.0 * n * n * nevex
+    full_flops = 32.0 * n * n * nevex
     full_achieved = full_flops / (full_launch_ms / 1e3) / 1e12
     per_launch_ms = g_ms / max(g_n, 1)
     g_flops *= 0.5
@@ -537,8 +538,9 @@ def main():
         # captured on full-width launches (k = nev + nex); scaled to the timed launches'
         # average width by the units processed (the operand re-reads grow with the
         # number of column tiles)
-        traffic = traffic_full * flops_per_launch / full_flops
-        traffic_src += f"; full-width launch {traffic_full:.4g} B scaled by the average width {flops_per_launch / full_flops:.3f}"
+        width = 2.0 * flops_per_launch / full_flops
+        traffic = traffic_full * width
+        traffic_src += f"; full-width launch {traffic_full:.4g} B scaled by the average width {width:.3f}"
     roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic, "traffic_source": traffic_src,
             "kernel": "hop_kernel (FP64 DFMA)" if precision == "fp64" else "tc_hop_kernel (tcgen05 filter GEMM)",

@@ -355,17 +355,16 @@ int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const in
       CB_TRY(filter_fp64_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, gws, s, fs, ph, jfixed));
     } else {
       if (!mixed_available()) return CHASE_BSE_UNSUPPORTED;
-      if (ritz && R) {
-        cplx* Rs;
+      const bool corr = ritz && R;
+      cplx* Rs = nullptr;
+      std::vector<double> rs(corr ? m : 0);
+      if (corr) {
         CB_TRY(gws.alloc(&Rs, n2 * m));
         CB_TRY(gather_cols(Rs, R, didx, n2, m, s));
-        std::vector<double> rs(m);
         for (int64_t i = 0; i < m; ++i) rs[i] = ritz[idx[i]];
-        CB_TRY(filter_mixed_correction_sorted(A, B, n, Y0, m, ds.data(), rs.data(), Rs, mu1, mu_nevex, muN, out,
-                                              scheme, s, fs, P2, Q2));
-      } else {
-        CB_TRY(filter_mixed_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, scheme, s, fs, P2, Q2));
       }
+      CB_TRY(filter_mixed_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, scheme, jfixed,
+                                 corr ? rs.data() : nullptr, Rs, s, fs, P2, Q2));
     }
     CB_TRY(scatter_cols(W, out, didx, n2, m, s));
     // host vectors idx/ds must outlive the async copies: synchronise before they go

@@ -21,9 +21,9 @@ enum FilterScheme : int { SCHEME_BF16X3 = 1, SCHEME_BF16X6 = 2, SCHEME_FP16X3 = 
 // With ph (the sliced operand of slice_hamiltonian) the FP64 columns apply H by
 // FP64-accurate sliced GEMMs on the tensor cores instead of the FP64 pipe.  With P2, Q2
 // (the blocks of H^2, see form_h2) the tensor-core columns apply H^2 from its blocks
-// (the explicit-H^2 variant).  jfixed: the FP64 pipe applies H in the J-fixed form, which
-// keeps the smaller half of a vector only to the accuracy of the larger one; a solve whose QR
-// and Rayleigh-Ritz steps work on J-fixed vectors knows it no better.
+// (the explicit-H^2 variant).  jfixed: the FP64 pipe and the tensor cores apply H in the J-fixed
+// form, which keeps the smaller half of a vector only to the accuracy of the larger one; a
+// solve whose QR and Rayleigh-Ritz steps work on J-fixed vectors knows it no better.
 struct SlicedOp;
 int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const int* degs, const int* prec,
            double mu1, double mu_nevex, double muN, int scheme, const double* ritz, const cplx* R, cudaStream_t s,
@@ -79,16 +79,12 @@ int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, c
 // Mixed-precision (tcgen05) filter on a column group whose columns are sorted
 // by descending degree; defined in the tensor-core translation unit.
 // scheme: a FilterScheme.
-// With P2, Q2 (the blocks of H^2, see form_h2) the filter applies H^2 from its blocks.
-int filter_mixed_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0, int64_t k, const int* degs_sorted,
-                        double mu1, double mu_nevex, double muN, cplx* out, int scheme, cudaStream_t s,
-                        FilterStats* fs, const cplx* P2 = nullptr, const cplx* Q2 = nullptr);
-// Correction form (see tc_filter.cu): V holds Ritz vectors, ritz their values,
-// R = H V - V diag(ritz) (FP64); out = p(H^2) V.
-int filter_mixed_correction_sorted(const cplx* A, const cplx* B, int64_t n, cplx* V, int64_t k,
-                                   const int* degs_sorted, const double* ritz_sorted, const cplx* R, double mu1,
-                                   double mu_nevex, double muN, cplx* out, int scheme, cudaStream_t s,
-                                   FilterStats* fs, const cplx* P2 = nullptr, const cplx* Q2 = nullptr);
+// With ritz and R (R = H V - V diag(ritz), FP64; V = Y0 holds the Ritz vectors) in correction
+// form (see tc_filter.cu).  jfixed: the J form, half the operations.  With P2, Q2 (the blocks of
+// H^2, see form_h2) the filter applies H^2 from its blocks.
+int filter_mixed_sorted(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, int64_t k, const int* degs_sorted,
+                        double mu1, double mu_nevex, double muN, cplx* out, int scheme, bool jfixed, const double* ritz,
+                        const cplx* R, cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2);
 bool mixed_available();
 
 }  // namespace cb

@@ -1,16 +1,28 @@
 // Mixed-precision Chebyshev filter on H^2 with tcgen05 tensor cores (sm_103a).
 //
-// A vector w = [x; y] is the sum [a; conj a] - i [c; conj c] of two vectors fixed by
-// J = K conj, a = (x + conj y) / 2 and c = i (x - conj y) / 2, and H maps
-// [z; conj z] to i [z'; conj z'] with z' = -i (A z + B conj z), a real-linear map of the
-// real 2n-vector (Re z, Im z):
+// One application of H to a block of k vectors is one real GEMM on 5th-generation tensor
+// cores, FP32 in TMEM, in one of two forms:
+//
+// Blocks: C (n x 4k) = P (n x 4n) * W (4n x 4k), P the rows of [A | B] as (re, im) pairs.  A vector
+// w = [x; y] gives four columns: w and i w for the top half of H w, u = [conj y; conj x] and
+// i u for -conj of the bottom half.  32 n^2 k operations.  Each half is a sum of its own
+// products, so both keep the scheme's accuracy relative to their own size (the lower half of an
+// eigenvector is smaller than the upper one by the coupling |B| / |A|).  The filter entry points.
+//
+// J form: w is the sum [a; conj a] - i [c; conj c] of two vectors fixed by J = K conj,
+// a = (x + conj y) / 2 and c = i (x - conj y) / 2, and H maps [z; conj z] to i [z'; conj z']
+// with z' = -i (A z + B conj z), a real-linear map of the real 2n-vector (Re z, Im z):
 //   M = [[Ai + Bi, Ar - Br], [-(Ar + Br), Ai - Bi]]   (2n x 2n),   H^2: z -> -M M z.
-// So the whole recurrence runs on two real columns per vector, and one application of H is
-// one real GEMM on 5th-generation tensor cores,
-//   C (2n x 2k, FP32 in TMEM) = M (2n x 2n) * Z (2n x 2k),
-// 16 n^2 k operations, half of [A | B] against the vectors [[x, conj y], [y, conj x]]
-// (n x 4n times 4n x 4k), and a quarter of that form's operand bytes to write per step.
-// Rows of M and entries of a column are interleaved: 2i is Re, 2i + 1 is Im.
+// So the whole recurrence runs on two real columns per vector and one application is
+//   C (2n x 2k) = M (2n x 2n) * Z (2n x 2k),
+// 16 n^2 k operations and a quarter of the operand bytes to write per step; rows of M and
+// entries of a column are interleaved, 2i is Re, 2i + 1 is Im.  The smaller half of a vector
+// comes out as a difference of two numbers of the size of the larger one and is accurate relative
+// to that (lower half of a degree-20 filter at n = 512, FP16x3: coupling 0.3 1.4e-5 instead of
+// 2.0e-6, coupling 1e-3 6e-4 instead of 3e-6).  The solves: their QR and Rayleigh-Ritz steps hold
+// the basis as J-fixed vectors, the correction form below lets a filter's error shrink with
+// the residual, and the lower half y of a locked pair is off by (conj A + lambda)^{-1} times its
+// residual whatever the form (measured equal at couplings 0.3 to 1e-6 and tolerances to 1e-12).
 //
 // Split products on 16-bit tensor cores: an operand x is written as a sum of
 // pieces x = x0 + x1 (+ x2), x0 = rn(x), x1 = rn(x - x0), ..., and the product
@@ -20,11 +32,11 @@
 //   BF16x6: 3 BF16 pieces each, adds x0 y2 + x1 y1 + x2 y0             (~2^-24)
 // (FP16 pieces of this kind: Ootomo and Yokota, Int. J. HPC Appl. 2022.)  FP16 has
 // a 5-bit exponent, so every operand row is scaled by a power of two: row r of M
-// by 2^prow[r] (its largest entry in [2^12, 2^13)), column v by 2^vexp[v], chosen
+// or P by 2^prow[r] (its largest entry in [2^12, 2^13)), column (blocks: vector) v by 2^vexp[v], chosen
 // from an upper bound of its entries below 2^13: the bound of an output of H is
 // L * max|input| with L the largest absolute row sum of P, and that of the
 // recurrence combines the maxima of its terms; every epilogue records the true
-// maximum of each output column (one atomic max per warp and column) for the
+// maximum of each output column or vector (one atomic max per warp and column) for the
 // next bound.  The epilogue divides the accumulator by 2^(prow + vexp).  Entries
 // far below the bound only lose precision relative to the bound, which keeps the
 // product's error below that of an FP32 GEMM (|dy| <~ 2^-22 L max|w|).  The
@@ -48,7 +60,7 @@
 //            them): either
 //            (mode 0) store the next GEMM's B-operand pieces, or
 //            (mode 1) the fused three-term recurrence in FP32 plus the pieces, or
-//            (mode 2) Z = H X + gamma_col * X (no pieces).
+//            (mode 2) Z = H X + gamma * X (no pieces).
 // Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the kernel
 // sets an error flag, waits (bounded) for its copies in flight into its shared
 // memory, frees its TMEM and returns.
@@ -90,6 +102,7 @@ struct Piece<__nv_bfloat16> {
   __device__ static __nv_bfloat16 rn(float x) { return __float2bfloat16_rn(x); }
   __device__ static float back(__nv_bfloat16 x) { return __bfloat162float(x); }
   __device__ static T2 pair(__nv_bfloat16 a, __nv_bfloat16 b) { return __halves2bfloat162(a, b); }
+  __device__ static unsigned bits(T2 p) { return *reinterpret_cast<unsigned*>(&p); }
 };
 template <>
 struct Piece<__half> {
@@ -98,34 +111,51 @@ struct Piece<__half> {
   __device__ static __half rn(float x) { return __float2half_rn(x); }
   __device__ static float back(__half x) { return __half2float(x); }
   __device__ static T2 pair(__half a, __half b) { return __halves2half2(a, b); }
+  __device__ static unsigned bits(T2 p) { return *reinterpret_cast<unsigned*>(&p); }
 };
 
 // Scheme: piece type, pieces of A (NPA) and B (NPW), product list (product 0 is x0 * y0), K blocks
-// per drained partial sum of x0 * y0 (FLUSH).
+// per drained partial sum of x0 * y0 in the J form (FLUSH) and in the blocks form, whose sums are
+// twice as long (FLUSH_BLOCKS; against FLUSH there: FP16x3 3-5 % longer for 0.5 to 0.8 of the
+// error, BF16x6 3-5 % for 0.6 to 0.8 below n = 3500).
 enum : int { SCH_BF16X3 = 1, SCH_BF16X6 = 2, SCH_FP16X3 = 3 };
 template <int SCH>
 struct Scheme;
 template <>
 struct Scheme<SCH_BF16X3> {
   using T = __nv_bfloat16;
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4, FLUSH_BLOCKS = 4;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_FP16X3> {
   using T = __half;
-  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4;
+  static constexpr int NPA = 2, NPW = 2, NPROD = 3, FLUSH = 4, FLUSH_BLOCKS = 2;
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : 0; }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : 0; }
 };
 template <>
 struct Scheme<SCH_BF16X6> {
   using T = __nv_bfloat16;
-  static constexpr int NPA = 3, NPW = 3, NPROD = 6, FLUSH = 2;
+  static constexpr int NPA = 3, NPW = 3, NPROD = 6, FLUSH = 2, FLUSH_BLOCKS = 1;
   // (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
   __device__ static constexpr int pa(int i) { return i == 2 ? 1 : (i == 4 ? 1 : (i == 5 ? 2 : 0)); }
   __device__ static constexpr int pb(int i) { return i == 1 ? 1 : (i == 3 ? 2 : (i == 4 ? 1 : 0)); }
+};
+// Form of an application: operand rows per row of A, operand columns per vector and, of
+// those, how many differ in scale (a master, an exponent and a maximum each); K elements per
+// row of A.
+enum : int { FORM_J = 0, FORM_BLOCKS = 1 };
+template <int FORM>
+struct Form;
+template <>
+struct Form<FORM_J> {
+  static constexpr int ROWS = 2, COLS = 2, SCALES = 2, KEL = 2;
+};
+template <>
+struct Form<FORM_BLOCKS> {
+  static constexpr int ROWS = 1, COLS = 4, SCALES = 1, KEL = 4;
 };
 // Geometry.  A K block is 64 K-elements (128-byte swizzle); a stage of the ring holds the
 // pieces of 128 A rows and of BN / 2 B rows, so a pair takes in 64 KB per CTA and 1536 MMA
@@ -135,13 +165,13 @@ struct Scheme<SCH_BF16X6> {
 // three, whose 24 bits the truncation of 16 would show (1.9 times the error).  K blocks of 32 in twice the stages lost 10-25 % (64-byte rows).
 //
 // Measured on one GB300, FP16x3, time of one launch of a degree's two, before (one CTA per
-// 128 x 128 tile, [A | B] against four columns per vector) and after: n = 16384, k = 1300
-// 28.0 -> 11.7 ms (three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained);
-// n = 4096, k = 260 370 -> 185 us; n = 3001, k = 83 88 -> 58 us; n = 512, k = 30 28 -> 17 us.
-// What bounds it: the power cap, which holds the clock near 1.45 of 2.07 GHz, from n = 4096 on; the pieces of M (16 n^2 bytes) from HBM, 21 us,
-// and a fixed 12 us of launch, first loads and tile end at n = 3001.  Whole filters: degree 20
-// at n = 4096 15.9 -> 8.2 ms, degree 8 at n = 16384 448 -> 201 ms.  Error against 64 bits 0.46
-// to 1.03 of the earlier form's over 36 drawn cases of n = 64 to 2600, 0.95 at n = 4096.
+// 128 x 128 tile, blocks form) and after, blocks and J form: n = 16384, k = 1300 26.5 -> 23.2 and
+// 11.5 ms (J form: three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained); n = 8192,
+// k = 300 1717 -> 1216 and 715 us; n = 4096, k = 260 367 -> 320 and 185 us; n = 3001, k = 83 88 -> 90
+// and 60 us; n = 512, k = 30 29 -> 22 and 20 us.  Whole filters in blocks form: degree 20 at n = 4096
+// 15.1 -> 13.0 ms, degree 8 at n = 16384 431 -> 377 ms.  Errors against 64 bits, of the earlier
+// kernel's: each half in blocks form 0.5 to 1.03 (n = 128 to 16384), the whole vector in J form 0.46
+// to 1.03.
 constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int MAX_ST = 8;                // most ring stages
@@ -162,17 +192,18 @@ static_assert(SMEM_BYTES <= 232448, "shared memory");
 
 struct Epi {
   int mode;           // 0: operand pieces, 1: recurrence, 2: H X + gamma X
-  float hsign;        // mode 1: -1 (H^2 = -M M); +1 where the operand holds the blocks of H^2
-  int64_t n2, k2;     // rows of M (2n), active columns (2k)
+  int h2;             // the operand holds the blocks of H^2
+  int64_t n;          // rows of A
+  int64_t rows, cols; // rows of the operand, active columns
   int64_t kpad;       // elements per piece row
   void* out[3];       // output operand pieces (NPW used)
-  float* Znext;       // columns of 2n entries
+  float* Znext;       // masters: 2n reals per column (J form), 2n complex per vector (blocks)
   const float* Zcur;
   const float* Zprev;
   const float* src;
   const float* gamma;  // per column
   float alpha, beta, c;
-  // operand scaling: M' = diag(2^prow) M, input column v times 2^vexp_in[v]; the pieces this
+  // operand scaling: M' = diag(2^prow) M, scaled column v times 2^vexp_in[v]; the pieces this
   // launch writes get 2^vexp_out[v] chosen from the bound
   //   ca * L * amax_a[v] + cb * amax_b[v] + cc * amax_c[v] + |gamma[v]| * amax_d[v]
   // (L: largest absolute row sum of M; amax_*: largest |entry| of each input column);
@@ -220,7 +251,7 @@ __device__ __forceinline__ float vec_bound(const Epi& ep, int64_t v) {
 // depend on timing.
 struct Sched {
   int nkb, num_m, num_n, bn, n_last;  // K blocks; tiles; columns of a tile and of the last one
-  int stages, stage_bytes, bufs, dcols;
+  int stages, stage_bytes, bufs, dcols, flush;
   int pairs, waves, rest, parts;      // rest tiles after the full waves
   int group_m;
   __device__ void tile_of(int t, int& mt, int& nt) const {
@@ -317,6 +348,40 @@ __device__ __forceinline__ void put1(void* const* pc, int64_t off, float a) {
   }
 }
 
+// The four operand rows of vector v in the blocks form at K positions 2i (top entry t) and
+// 2(n + i) (bottom entry b): w, i w, u, i u as (re, -im), (im, re) pairs, u = [conj(b); conj(t)],
+// times sc.
+template <class T, int NPC>
+__device__ __forceinline__ void store_operand(void* const* pc, int64_t kpad, int64_t n, int64_t v, int64_t i, float2 t,
+                                              float2 b, float sc) {
+  using PT = Piece<T>;
+  t.x *= sc; t.y *= sc; b.x *= sc; b.y *= sc;
+#pragma unroll
+  for (int q = 0; q < NPC; ++q) {
+    // each value is rounded once; the eight pairs are its pieces swapped and negated
+    const T tx = PT::rn(t.x), ty = PT::rn(t.y), bx = PT::rn(b.x), by = PT::rn(b.y);
+    const unsigned tt = PT::bits(PT::pair(tx, ty)), bb = PT::bits(PT::pair(bx, by));
+    const unsigned ts = __byte_perm(tt, tt, 0x1032), bs = __byte_perm(bb, bb, 0x1032);
+    unsigned* r = reinterpret_cast<unsigned*>(static_cast<T*>(pc[q]) + 4 * v * kpad) + i;  // kpad even
+    const int64_t row = kpad / 2;
+    r[0] = tt ^ 0x80000000u;
+    r[n] = bb ^ 0x80000000u;
+    r += row;
+    r[0] = ts;
+    r[n] = bs;
+    r += row;
+    r[0] = bb;
+    r[n] = tt;
+    r += row;
+    r[0] = bs ^ 0x00008000u;
+    r[n] = ts ^ 0x00008000u;
+    t.x -= PT::back(tx);
+    t.y -= PT::back(ty);
+    b.x -= PT::back(bx);
+    b.y -= PT::back(by);
+  }
+}
+
 struct Maps {
   CUtensorMap a[3];
   CUtensorMap b[3];
@@ -328,16 +393,17 @@ struct Maps {
 // four groups are prepared at a time and all loads of a group are in flight together.
 constexpr int EB = 8;
 template <int SCH>
-__device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
+__device__ __forceinline__ void finish_jform(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
                                             int lane, int first, int step, const float* tiles, int parts,
                                             size_t stride) {
   using T = typename Scheme<SCH>::T;
   const int row_t = q * 32 + lane;
   const int64_t row = (int64_t)(2 * wk.mt + (int)rank) * BM + row_t;
-  const bool rvalid = row < ep.n2;
+  const bool rvalid = row < ep.rows;
   const float rs = rvalid ? exp2i(-ep.prow[row]) : 0.0f;  // undo the row scaling of M
+  const float hsign = ep.h2 ? 1.0f : -1.0f;               // H^2 = -M M
   const int64_t v0 = (int64_t)wk.nt * sc.bn;
-  const int cols = (int)min((int64_t)wk.cols, ep.k2 - v0);  // even
+  const int cols = (int)min((int64_t)wk.cols, ep.cols - v0);  // even
 #pragma unroll 1
   for (int g0 = first; g0 * EB < cols; g0 += 4 * step) {
     // lane l prepares column l % 8 of group l / 8: the input column's scale (undone), the
@@ -363,18 +429,18 @@ __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, cons
       const int left = cols - g;
       const int64_t vb = v0 + g;
       // loads at clamped rows and columns instead of under a predicate each
-      const int64_t oz = vb * ep.n2 + min(row, ep.n2 - 1);
+      const int64_t oz = vb * ep.rows + min(row, ep.rows - 1);
       const float* tp = tiles + (size_t)g * BM + row_t;
       float x[EB], zc[EB], zp[EB];
 #pragma unroll
       for (int i = 0; i < EB; ++i) x[i] = __ldcg(tp + i * BM);
       if (ep.mode != 0) {
 #pragma unroll
-        for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.n2];
+        for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.rows];
       }
       if (ep.mode == 1 && ep.beta != 0.0f) {
 #pragma unroll
-        for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.n2];
+        for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.rows];
       }
 #pragma unroll 1
       for (int j = 1; j < parts; j += 3) {
@@ -394,14 +460,14 @@ __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, cons
       for (int i = 0; i < EB; ++i) x[i] *= rs * __shfl_sync(0xffffffffu, s_in, t * EB + i);
       if (ep.mode == 1) {
 #pragma unroll
-        for (int i = 0; i < EB; ++i) x[i] = ep.alpha * (ep.hsign * x[i] - ep.c * zc[i]);
+        for (int i = 0; i < EB; ++i) x[i] = ep.alpha * (hsign * x[i] - ep.c * zc[i]);
         if (ep.beta != 0.0f) {
 #pragma unroll
           for (int i = 0; i < EB; ++i) x[i] += ep.beta * zp[i];
         }
         if (ep.src) {
 #pragma unroll
-          for (int i = 0; i < EB; ++i) zc[i] = ep.src[oz + (i < left ? i : 0) * ep.n2];
+          for (int i = 0; i < EB; ++i) zc[i] = ep.src[oz + (i < left ? i : 0) * ep.rows];
 #pragma unroll
           for (int i = 0; i < EB; ++i) x[i] += __shfl_sync(0xffffffffu, gmm, t * EB + i) * zc[i];
         }
@@ -420,7 +486,7 @@ __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, cons
         const float so = __shfl_sync(0xffffffffu, s_out, t * EB + i);
         if (lv) {
           if (ep.mode != 2) put1<T, Scheme<SCH>::NPW>(ep.out, (vb + i) * ep.kpad + row, x[i] * so);
-          if (ep.mode != 0) ep.Znext[oz + i * ep.n2] = x[i];
+          if (ep.mode != 0) ep.Znext[oz + i * ep.rows] = x[i];
         }
         const unsigned mm = __reduce_max_sync(0xffffffffu, lv ? __float_as_uint(fabsf(x[i])) : 0u);
         if (lane == t * EB + i) amax = mm;
@@ -430,12 +496,132 @@ __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, cons
   }
 }
 
+// The same for the blocks form: row i of the operand holds, per vector, top = P w (columns
+// 4v, 4v + 1) and P u (4v + 2, 4v + 3), whose -conj (with the blocks of H^2, conj) is the bottom.
+// A group of EB columns is two vectors.
 template <int SCH>
+__device__ __forceinline__ void finish_blocks(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
+                                              int lane, int first, int step, const float* tiles, int parts,
+                                              size_t stride) {
+  using T = typename Scheme<SCH>::T;
+  const int row_t = q * 32 + lane;
+  const int64_t row = (int64_t)(2 * wk.mt + (int)rank) * BM + row_t;
+  const bool rvalid = row < ep.n;
+  const float rs = rvalid ? exp2i(-ep.prow[row]) : 0.0f;  // undo the row scaling of the operand
+  const int64_t v0 = (int64_t)wk.nt * (sc.bn / 4), n2 = 2 * ep.n, rc = min(row, ep.n - 1);
+  const int vecs = (int)min((int64_t)(wk.cols / 4), ep.cols / 4 - v0);
+#pragma unroll 1
+  for (int g0 = first; 2 * g0 < vecs; g0 += 4 * step) {
+    // lane l < 8 prepares vector l % 2 of group l / 2
+    const int pv = 2 * (g0 + (lane >> 1) * step) + (lane & 1);
+    const bool mine = lane < EB && pv < vecs;
+    float s_in = 0.0f, s_out = 0.0f, gmm = 0.0f;
+    if (mine) {
+      const int64_t v = v0 + pv;
+      const int ein = ep.vexp_in[v];
+      if (ep.gamma) gmm = ep.gamma[v];
+      if (ep.mode != 2) {
+        const int e = out_exp(vec_bound(ep, v));
+        s_out = exp2i(e);
+        if (q == 0) ep.vexp_out[v] = e;  // the same value from every tile
+      }
+      s_in = exp2i(-ein);
+    }
+    unsigned amax = 0;
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+      const int vb = 2 * (g0 + t * step);
+      if (vb >= vecs) break;
+      const float* tp = tiles + (size_t)(4 * vb) * BM + row_t;
+      // masters of the group's two vectors (a missing second one reads the first)
+      const int64_t o[2] = {(v0 + vb) * n2 + rc, (v0 + (vb + 1 < vecs ? vb + 1 : vb)) * n2 + rc};
+      float x[EB];
+      float2 zc[4], zp[4];
+#pragma unroll
+      for (int i = 0; i < EB; ++i) x[i] = __ldcg(tp + i * BM);
+      if (ep.mode != 0) {
+        const float2* Z = reinterpret_cast<const float2*>(ep.Zcur);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) zc[h] = Z[o[h >> 1] + (h & 1) * ep.n];
+      }
+      if (ep.mode == 1 && ep.beta != 0.0f) {
+        const float2* Z = reinterpret_cast<const float2*>(ep.Zprev);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) zp[h] = Z[o[h >> 1] + (h & 1) * ep.n];
+      }
+#pragma unroll 1
+      for (int j = 1; j < parts; j += 3) {
+        float y[3][EB];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(tp + min(j + p, parts - 1) * stride + i * BM);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          if (j + p < parts) {
+#pragma unroll
+            for (int i = 0; i < EB; ++i) x[i] += y[p][i];
+          }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float vs = rs * __shfl_sync(0xffffffffu, s_in, 2 * t + u);
+        const float so = __shfl_sync(0xffffffffu, s_out, 2 * t + u);
+        const float gm = __shfl_sync(0xffffffffu, gmm, 2 * t + u);
+        float2 z[2] = {make_float2(x[4 * u] * vs, x[4 * u + 1] * vs),
+                       ep.h2 ? make_float2(x[4 * u + 2] * vs, -x[4 * u + 3] * vs)
+                             : make_float2(-x[4 * u + 2] * vs, x[4 * u + 3] * vs)};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 c = zc[2 * u + h];
+          if (ep.mode == 1) {
+            z[h].x = ep.alpha * (z[h].x - ep.c * c.x);
+            z[h].y = ep.alpha * (z[h].y - ep.c * c.y);
+            if (ep.beta != 0.0f) {
+              z[h].x += ep.beta * zp[2 * u + h].x;
+              z[h].y += ep.beta * zp[2 * u + h].y;
+            }
+            if (ep.src) {
+              const float2 r = reinterpret_cast<const float2*>(ep.src)[o[u] + h * ep.n];
+              z[h].x += gm * r.x;
+              z[h].y += gm * r.y;
+            }
+          } else if (ep.mode == 2) {
+            z[h].x += gm * c.x;
+            z[h].y += gm * c.y;
+          }
+        }
+        const bool lv = rvalid && vb + u < vecs;
+        if (lv) {
+          if (ep.mode != 2) store_operand<T, Scheme<SCH>::NPW>(ep.out, ep.kpad, ep.n, v0 + vb + u, row, z[0], z[1], so);
+          if (ep.mode != 0) {
+            float2* Z = reinterpret_cast<float2*>(ep.Znext);
+            Z[o[u]] = z[0];
+            Z[o[u] + ep.n] = z[1];
+          }
+        }
+        const float m = fmaxf(fmaxf(fabsf(z[0].x), fabsf(z[0].y)), fmaxf(fabsf(z[1].x), fabsf(z[1].y)));
+        const unsigned mm = __reduce_max_sync(0xffffffffu, lv ? __float_as_uint(m) : 0u);
+        if (lane == 2 * t + u) amax = mm;
+      }
+    }
+    if (mine) atomicMax(reinterpret_cast<unsigned*>(ep.amax_out) + v0 + pv, amax);
+  }
+}
+template <int SCH, int FORM>
+__device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
+                                            int lane, int first, int step, const float* tiles, int parts,
+                                            size_t stride) {
+  if (FORM == FORM_J) finish_jform<SCH>(ep, sc, wk, rank, q, lane, first, step, tiles, parts, stride);
+  else finish_blocks<SCH>(ep, sc, wk, rank, q, lane, first, step, tiles, parts, stride);
+}
+
+template <int SCH, int FORM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     tc_hop_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Epi ep, const __grid_constant__ Sched sc) {
   using SC = Scheme<SCH>;
   using T = typename SC::T;
-  constexpr int FLUSH = SC::FLUSH;
+  const int FLUSH = FORM == FORM_J ? SC::FLUSH : sc.flush;  // a power of two
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
@@ -510,7 +696,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     const bool sp = wk.split();
     const int p0 = sp ? pair / sc.parts * sc.parts : pair;  // the pair with the tile's first K range
     const float* t = ep.part + (size_t)(4 * p0 + 2 * (int)rank + slot) * (BM * BNMAX);
-    finish_tile<SCH>(ep, sc, wk, rank, warp & 3, lane, third, 3, t, sp ? sc.parts : 1, (size_t)4 * BM * BNMAX);
+    finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, third, 3, t, sp ? sc.parts : 1, (size_t)4 * BM * BNMAX);
   };
 
   if (warp < 4) {
@@ -551,8 +737,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const uint32_t idesc = make_idesc(wk.cols, Piece<T>::BF16);
       for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
         const int i = kb - wk.kb0;
-        const bool first = (i % FLUSH) == 0;
-        const bool last = (i % FLUSH) == FLUSH - 1 || kb == wk.kb1 - 1;
+        const bool first = (i & (FLUSH - 1)) == 0;
+        const bool last = (i & (FLUSH - 1)) == FLUSH - 1 || kb == wk.kb1 - 1;
         if (!mbar_wait(full0 + 8 * s, ph, abort_sh, ep.err, true)) {
           ok = false;
           break;
@@ -687,7 +873,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       } else if (ok) {
         const bool w = mbar_wait(outf + 8 * slot, (uint32_t)(seg >> 1) & 1u, abort_sh, ep.err, true);
         ok = __all_sync(0xffffffffu, w);
-        if (ok) finish_tile<SCH>(ep, sc, wk, rank, warp & 3, lane, 0, 1, my_tiles + (size_t)slot * (BM * BNMAX), 1, 0);
+        if (ok) finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, 0, 1, my_tiles + (size_t)slot * (BM * BNMAX), 1, 0);
         __syncwarp();
         if (lane == 0) mbar_arrive(oute + 8 * slot);
       }
@@ -806,6 +992,104 @@ __global__ void split_p_kernel(const cplx* A, const cplx* B, int64_t n, int64_t 
     put<T, NPC>(out.p, (2 * i + 1) * kpad + 2 * l, r1.x * c1, r1.y * c1);
   }
 }
+// The rows of [A | B] (row-major complex128) as (re, im) pairs -> NPC pieces, one CTA per row,
+// scaled by 2^prow[i] (largest entry in [2^12, 2^13)); L as above; columns 4n .. kpad are zero.
+// CACHE: the FP32 entries (16 n bytes) wait in shared memory for the row's exponent.
+template <class T, int NPC, bool CACHE>
+__global__ void split_blocks_kernel(const cplx* A, const cplx* B, int64_t n, int64_t kpad, Pieces out, int* prow,
+                                    float* L) {
+  extern __shared__ float4 row_cache[];
+  const int64_t i = blockIdx.x;
+  float m = 0.0f, sum = 0.0f;
+  auto load = [&](int64_t l) {
+    const cplx a = A[i * n + l], b = B[i * n + l];
+    return make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+  };
+#pragma unroll 4
+  for (int64_t l = threadIdx.x; l < n; l += blockDim.x) {
+    const float4 v = load(l);
+    if (CACHE) row_cache[l] = v;  // read back by this thread
+    m = fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+    sum += (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
+  }
+  block_max_sum(m, sum);
+  const int e = out_exp(m);
+  if (threadIdx.x == 0) {
+    prow[i] = e;
+    atomicMax(reinterpret_cast<unsigned*>(L), __float_as_uint(sum));
+  }
+  const float c = exp2i(e);
+  for (int64_t l = threadIdx.x; l < n; l += blockDim.x) {
+    const float4 v = CACHE ? row_cache[l] : load(l);
+    put<T, NPC>(out.p, i * kpad + 2 * l, v.x * c, v.y * c);
+    put<T, NPC>(out.p, i * kpad + 2 * (n + l), v.z * c, v.w * c);
+  }
+  for (int64_t l = 4 * n + 2 * threadIdx.x; l < kpad; l += 2 * blockDim.x) put<T, NPC>(out.p, i * kpad + l, 0.0f, 0.0f);
+}
+// amax[v] = largest |Re|, |Im| of column v of W, rounded to FP32, and its operand exponent
+__global__ void col_amax_blocks_kernel(const cplx* W, int64_t n, float* amax, int* vexp) {
+  const int64_t v = blockIdx.x;
+  float m = 0.0f, unused = 0.0f;
+  for (int64_t i = threadIdx.x; i < 2 * n; i += blockDim.x) {
+    const cplx w = W[v * 2 * n + i];
+    m = fmaxf(m, fmaxf(fabsf((float)w.x), fabsf((float)w.y)));
+  }
+  block_max_sum(m, unused);
+  if (threadIdx.x == 0) {
+    amax[v] = m;
+    vexp[v] = out_exp(m);
+  }
+}
+// complex128 block (2n x k) -> FP32 masters and operand pieces (exponents vexp)
+template <class T, int NPC>
+__global__ void pack_blocks_kernel(const cplx* W, int64_t n, int64_t k, float2* Z, Pieces out, int64_t kpad,
+                                   const int* vexp) {
+  const int64_t total = n * k;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % n, v = idx / n, o = v * 2 * n + i;
+    const cplx x = W[o], y = W[o + n];
+    const float2 t = make_float2((float)x.x, (float)x.y), b = make_float2((float)y.x, (float)y.y);
+    Z[o] = t;
+    Z[o + n] = b;
+    store_operand<T, NPC>(out.p, kpad, n, v, i, t, b, exp2i(vexp[v]));
+  }
+}
+// Z = scale * X (masters) and its operand pieces, as scale_pack_kernel
+template <class T, int NPC>
+__global__ void scale_pack_blocks_kernel(const float2* X, int64_t n, int64_t k, float scale, float2* Z, Pieces out,
+                                         int64_t kpad, const float* amax_x, float* amax_z, int* vexp_z) {
+  const int64_t total = n * k;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = idx % n, v = idx / n, o = v * 2 * n + i;
+    const float am = fabsf(scale) * amax_x[v];
+    const int e = out_exp(am);
+    if (i == 0) {
+      amax_z[v] = am;
+      vexp_z[v] = e;
+    }
+    const float2 x = X[o], y = X[o + n];
+    const float2 t = make_float2(scale * x.x, scale * x.y), b = make_float2(scale * y.x, scale * y.y);
+    Z[o] = t;
+    Z[o + n] = b;
+    store_operand<T, NPC>(out.p, kpad, n, v, i, t, b, exp2i(e));
+  }
+}
+// out[:, v] = the master of vector v in Zsel, in FP64, + coef[v] * base[:, v] (coef/base optional)
+__global__ void combine_blocks_kernel(cplx* out, const float2* Z0, const float2* Z1, const float2* Z2, const int* sel,
+                                      const double* coef, const cplx* base, int64_t n2, int64_t k) {
+  const int64_t total = n2 * k;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = idx / n2;
+    const int q = sel[v];
+    const float2 z = (q == 0 ? Z0 : (q == 1 ? Z1 : Z2))[idx];
+    cplx r = mk((double)z.x, (double)z.y);
+    if (coef) r = cadd(r, cscale(base[idx], coef[v]));
+    out[idx] = r;
+  }
+}
 // The halves a and c of w = [x; y]; and w from them
 __device__ __forceinline__ void j_split(cplx x, cplx y, float2& a, float2& c) {
   a = make_float2((float)(0.5 * (x.x + y.x)), (float)(0.5 * (x.y - y.y)));
@@ -916,47 +1200,53 @@ static inline unsigned gsz(int64_t total) {
   return (unsigned)std::min<int64_t>(std::max<int64_t>(b, 1), 16384);
 }
 
-// The real form of [A | B] in NPA pieces, with its tensor maps, row exponents and the
+// The operand of A and B in NPA pieces, with its tensor maps, row exponents and the
 // bound factor L (device scalar).
+constexpr size_t CACHE_MAX = 220 * 1024;  // shared memory for a row's FP32 entries
 struct POperand {
-  int64_t n = 0, kpad = 0;
+  int64_t n = 0, rows = 0, kpad = 0;
   Pieces pc{};
   CUtensorMap map[3];
   int* prow = nullptr;
   float* L = nullptr;
 };
 
-template <int SCH, int TWIST>
+template <int SCH, int FORM, int TWIST>
 static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POperand& P, cudaStream_t s) {
   using T = typename Scheme<SCH>::T;
   constexpr int NPA = Scheme<SCH>::NPA;
   P.n = n;
-  P.kpad = ((2 * n + KPAD - 1) / KPAD) * KPAD;
+  P.rows = Form<FORM>::ROWS * n;
+  P.kpad = ((Form<FORM>::KEL * n + KPAD - 1) / KPAD) * KPAD;
   for (int q = 0; q < NPA; ++q) {
     T* pq;
-    CB_TRY(ws.alloc(&pq, 2 * n * P.kpad));
+    CB_TRY(ws.alloc(&pq, P.rows * P.kpad));
     P.pc.p[q] = pq;
   }
-  CB_TRY(ws.alloc(&P.prow, 2 * n));
+  CB_TRY(ws.alloc(&P.prow, P.rows));
   CB_TRY(ws.alloc(&P.L, 1));
   CB_CUDA(cudaMemsetAsync(P.L, 0, sizeof(float), s));
   const size_t cache = sizeof(float4) * (size_t)n;
-  if (cache <= 220 * 1024) {
+  void (*kern)(const cplx*, const cplx*, int64_t, int64_t, Pieces, int*, float*);
+  // as many threads an SM where only one or two rows fit it
+  const int threads = cache > 72 * 1024 && cache <= CACHE_MAX ? 512 : 256;
+  if (cache <= CACHE_MAX) {
+    if (FORM == FORM_J) kern = split_p_kernel<T, NPA, TWIST, true>;
+    else kern = split_blocks_kernel<T, NPA, true>;
     static bool attr = false;
     if (!attr) {
-      CB_CUDA(cudaFuncSetAttribute(split_p_kernel<T, NPA, TWIST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   220 * 1024));
+      CB_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CACHE_MAX));
       attr = true;
     }
-    // as many threads an SM where only one or two rows fit it
-    const int threads = cache > 72 * 1024 ? 512 : 256;
-    split_p_kernel<T, NPA, TWIST, true><<<(unsigned)n, threads, cache, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
+    kern<<<(unsigned)n, threads, cache, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
   } else {
-    split_p_kernel<T, NPA, TWIST, false><<<(unsigned)n, 256, 0, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
+    if (FORM == FORM_J) kern = split_p_kernel<T, NPA, TWIST, false>;
+    else kern = split_blocks_kernel<T, NPA, false>;
+    kern<<<(unsigned)n, threads, 0, s>>>(A, B, n, P.kpad, P.pc, P.prow, P.L);
   }
   count_launch();
   CB_LAUNCH();
-  for (int q = 0; q < NPA; ++q) CB_TRY(make_map(&P.map[q], P.pc.p[q], P.kpad, 2 * n, BM, Piece<T>::BF16));
+  for (int q = 0; q < NPA; ++q) CB_TRY(make_map(&P.map[q], P.pc.p[q], P.kpad, P.rows, BM, Piece<T>::BF16));
   return CHASE_BSE_OK;
 }
 
@@ -968,18 +1258,30 @@ static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POp
 // multicasts between two pairs and with the accumulators alternating, so the clock under the
 // power cap is the likely cause).  It favours wide tiles: n = 6000, k = 100 225 -> 182 us a
 // launch, n = 8192, k = 300 786 -> 704 us against a choice by the other two terms.
-template <int SCH>
+// Blocks form: a K block takes no less than 1400 cycles however narrow the tile (n = 1301, tiles of
+// 32 to 160 columns in one K range: 78 to 88 us a launch, 82 blocks).
+template <int SCH, int FORM>
 static double block_cycles(int w, int bn, double active) {
   using SC = Scheme<SCH>;
   constexpr int MMAS = SC::NPROD * (BK / 16);
   const double mma = MMAS * (w / 2.0), stage = SC::NPA * A_BYTES + SC::NPW * 64.0 * bn;
   const double smem = (MMAS * (4096.0 + 16.0 * w) + stage) / 128.0;
-  return std::max(std::max(mma, smem), 0.027 * stage * std::max(active, 0.5));
+  const double t = std::max(std::max(mma, smem), 0.027 * stage * std::max(active, 0.5));
+  return FORM == FORM_J ? t : std::max(t, 1400.0);
+}
+// Cycles to finish a pair's last tile behind its MMAs, summing `parts` partial tiles: three sets of
+// warps take its groups of 8 columns in turn, each a chain of L2 latencies (2 us, and 0.7 us for
+// every three partial tiles more; n = 700 to 1301).  The J form's choices rest on a constant
+// fitted with the rest of its terms.
+template <int FORM>
+static double finish_cycles(int bn, int parts) {
+  if (FORM == FORM_J) return parts > 1 ? 9000.0 + (parts + 1) * 8.0 * bn : 6000.0;
+  return 10000.0 + (double)cdiv(bn, 3 * EB) * (3900.0 + 1350.0 * (double)cdiv(parts - 1, 3));
 }
 // The schedule of a launch with m rows, k2 columns and nkb K blocks: of the column widths
 // (multiples of 32) that ceil(k2 / 256) to 3 more column tiles need, and of the numbers of K
 // ranges to cut the tiles left after the full waves into, the choice of least estimated time.
-template <int SCH>
+template <int SCH, int FORM>
 static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
   using SC = Scheme<SCH>;
   Sched best{};
@@ -998,21 +1300,26 @@ static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
     sc.dcols = (int)cdiv(sc.bn, BNMAX / DC * 16) * 16;  // half of the tile, whole TMEM loads
     sc.bufs = 3 * sc.bn <= (int)TMEM_COLS ? 2 : 1;
     sc.group_m = 8;
+    // narrow tiles of an operand that streams from HBM wait for their drains (n = 16384, k = 20
+    // 833 us a launch drained every four K blocks, 901 every two)
+    const bool streamed = sc.bn <= 128 && (double)m * nkb * BK * 4.0 > 126e6;
+    // and with three pieces the FP32 additions of a long sum outweigh the truncation again (lower
+    // halves at n = 4096, k = 260 3.9e-6, drained every K block 4.8e-6)
+    sc.flush = streamed || (SC::NPA == 3 && nkb > 224) ? SC::FLUSH : SC::FLUSH_BLOCKS;
     const int64_t tiles = (int64_t)sc.num_m * nn;
     sc.pairs = pairs;
     sc.waves = (int)(tiles / pairs);
     sc.rest = (int)(tiles % pairs);
-    const double full = block_cycles<SCH>(sc.bn, sc.bn, 1.0);
-    const double avg = (full * (nn - 1) + block_cycles<SCH>(sc.n_last, sc.bn, 1.0)) / nn;
-    const double fixed = 6000.0;  // prologue and epilogue of a tile
+    const double full = block_cycles<SCH, FORM>(sc.bn, sc.bn, 1.0);
+    const double avg = (full * (nn - 1) + block_cycles<SCH, FORM>(sc.n_last, sc.bn, 1.0)) / nn;
+    const double fixed = 6000.0;  // prologue and epilogue of a tile in the full waves
     const double base = sc.waves * ((sc.waves > 1 ? avg : full) * nkb + fixed);
     for (int f = 1; f == 1 || (f * sc.rest <= pairs && nkb / f >= 2); ++f) {
       sc.parts = f;
       double t = base;
       if (sc.rest > 0) {
-        t += std::ceil((double)nkb / f) * block_cycles<SCH>(sc.bn, sc.bn, (double)(f * sc.rest) / pairs) + fixed;
-        // partial tiles out and back in (L2, about 64 bytes a cycle and SM)
-        if (f > 1) t += 3000.0 + (f + 1) * 8.0 * sc.bn;
+        t += std::ceil((double)nkb / f) * block_cycles<SCH, FORM>(sc.bn, sc.bn, (double)(f * sc.rest) / pairs) +
+             finish_cycles<FORM>(sc.bn, f);
       }
       if (best_t == 0.0 || t < best_t) {
         best = sc;
@@ -1026,29 +1333,29 @@ static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
 
 // One tensor-core application of M to the columns held in the operand pieces bp (rows
 // columns allocated), with epilogue `ep`.
-template <int SCH>
+template <int SCH, int FORM>
 static int apply(const POperand& P, const Pieces& bp, int64_t rows, Epi ep, cudaStream_t s) {
   using T = typename Scheme<SCH>::T;
-  if (ep.k2 <= 0) return CHASE_BSE_OK;
+  if (ep.cols <= 0) return CHASE_BSE_OK;
   static bool attr = false;
   if (!attr) {
-    CB_CUDA(cudaFuncSetAttribute(tc_hop_kernel<SCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    CB_CUDA(cudaFuncSetAttribute(tc_hop_kernel<SCH, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     // the drain warps' share exists only if the kernel was launched with REGS_LAUNCH registers a thread
     cudaFuncAttributes fa;
-    CB_CUDA(cudaFuncGetAttributes(&fa, tc_hop_kernel<SCH>));
+    CB_CUDA(cudaFuncGetAttributes(&fa, tc_hop_kernel<SCH, FORM>));
     if (fa.numRegs != REGS_LAUNCH) return CHASE_BSE_UNSUPPORTED;
     attr = true;
   }
   ep.prow = P.prow;
   ep.L = P.L;
-  const Sched sc = plan<SCH>(ep.n2, ep.k2, (int)(P.kpad / BK), ep.sms / 2);
+  const Sched sc = plan<SCH, FORM>(ep.rows, ep.cols, (int)(P.kpad / BK), ep.sms / 2);
   Maps maps;
   for (int q = 0; q < Scheme<SCH>::NPA; ++q) maps.a[q] = P.map[q];
   for (int q = 0; q < Scheme<SCH>::NPW; ++q)
     CB_TRY(make_map(&maps.b[q], bp.p[q], P.kpad, rows, sc.bn / 2, Piece<T>::BF16));
   const unsigned grid = 2u * (unsigned)(sc.waves > 0 ? sc.pairs : sc.rest * sc.parts);
-  const int64_t tid = timer_begin(0, 16.0 * (double)P.n * (double)P.n * (double)ep.k2, s);
-  tc_hop_kernel<SCH><<<grid, THREADS, SMEM_BYTES, s>>>(maps, ep, sc);
+  const int64_t tid = timer_begin(0, 32.0 * (double)P.n * (double)P.n * (double)(ep.cols / Form<FORM>::COLS), s);
+  tc_hop_kernel<SCH, FORM><<<grid, THREADS, SMEM_BYTES, s>>>(maps, ep, sc);
   timer_end(tid, s);
   count_launch();
   CB_LAUNCH();
@@ -1067,33 +1374,36 @@ static int apply(const POperand& P, const Pieces& bp, int64_t rows, Epi ep, cuda
 // With P2, Q2 (the blocks of H^2 = [[P2, Q2], [conj Q2, conj P2]], row-major n x n) the
 // filter applies H^2 from its blocks, one launch per step (the explicit-H^2 variant, not
 // the paper's method); H itself (A, B) is then used only for the correction source.
-template <int SCH>
+template <int SCH, int FORM>
 static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, int64_t k, const int* degs,
                        double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
                        cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
   using T = typename Scheme<SCH>::T;
+  using F = Form<FORM>;
   constexpr int NPW = Scheme<SCH>::NPW;
+  constexpr bool J = FORM == FORM_J;
   if (k == 0) return CHASE_BSE_OK;
   const int64_t n2 = 2 * n;
   const bool expl = P2 != nullptr && Q2 != nullptr;
   const bool corr = (ritz != nullptr && R != nullptr);
   Workspace ws(s);
   POperand P, PH2;  // [A | B] (H), [P2 | Q2] (H^2)
-  if (!expl || corr) CB_TRY((prepare_p<SCH, 1>(A, B, n, ws, P, s)));
-  if (expl) CB_TRY((prepare_p<SCH, 0>(P2, Q2, n, ws, PH2, s)));
+  if (!expl || corr) CB_TRY((prepare_p<SCH, FORM, 1>(A, B, n, ws, P, s)));
+  if (expl) CB_TRY((prepare_p<SCH, FORM, 0>(P2, Q2, n, ws, PH2, s)));
   const POperand& PK = expl ? PH2 : P;  // the operand of the recurrence (its kpad and pieces layout)
-  const int64_t kpad = PK.kpad;  // the same for both operands (2n padded)
-  const int64_t k2 = 2 * k;      // columns
+  const int64_t kpad = PK.kpad, rows = PK.rows;  // the same for both operands
+  const int64_t nc = F::COLS * k, ns = F::SCALES * k;  // columns, scales
   Pieces Zp{}, Tp{};
   for (int q = 0; q < NPW; ++q) {
     T *zq, *tq;
-    CB_TRY(ws.alloc(&zq, k2 * kpad));
-    CB_TRY(ws.alloc(&tq, k2 * kpad));
+    CB_TRY(ws.alloc(&zq, nc * kpad));
+    CB_TRY(ws.alloc(&tq, nc * kpad));
     Zp.p[q] = zq;
     Tp.p[q] = tq;
-    if (kpad > n2) {  // zero past the entries of a column, as past those of a row of M
-      CB_CUDA(cudaMemset2DAsync(zq + n2, sizeof(T) * kpad, 0, sizeof(T) * (kpad - n2), k2, s));
-      CB_CUDA(cudaMemset2DAsync(tq + n2, sizeof(T) * kpad, 0, sizeof(T) * (kpad - n2), k2, s));
+    const int64_t ke = F::KEL * n;
+    if (kpad > ke) {  // zero past the entries of a column, as past those of an operand row
+      CB_CUDA(cudaMemset2DAsync(zq + ke, sizeof(T) * kpad, 0, sizeof(T) * (kpad - ke), nc, s));
+      CB_CUDA(cudaMemset2DAsync(tq + ke, sizeof(T) * kpad, 0, sizeof(T) * (kpad - ke), nc, s));
     }
   }
   // explicit H^2: the pieces of Z_j alternate between the two sets (j even: Zp)
@@ -1101,8 +1411,8 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
   float *Zb[3], *src = nullptr;
   float* gam;
   int* err;
-  for (int q = 0; q < 3; ++q) CB_TRY(ws.alloc(&Zb[q], n2 * k2));
-  CB_TRY(ws.alloc(&gam, k2));
+  for (int q = 0; q < 3; ++q) CB_TRY(ws.alloc(&Zb[q], 2 * n2 * k));
+  CB_TRY(ws.alloc(&gam, ns));
   auto c2 = [](float* z) { return reinterpret_cast<float2*>(z); };
   CB_TRY(ws.alloc(&err, 1));
   CB_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
@@ -1126,19 +1436,19 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
   const double sigma1 = e / (mu1 * mu1 - c);
   const double tau = 2.0 / sigma1;
   const int maxdeg = degs[0];
-  // per-column maxima and operand exponents, one slot of k2 entries per block:
+  // per-column maxima and operand exponents, one slot of ns entries per block:
   // Z_j (j = 0 .. maxdeg), T_j = H Z_j (j < maxdeg), the residual block R and the
   // correction source r2
   const int64_t nslot = 2 * (int64_t)maxdeg + 3;
   float* amax;
   int* vexp;
-  CB_TRY(ws.alloc(&amax, nslot * k2));
-  CB_TRY(ws.alloc(&vexp, nslot * k2));
-  CB_CUDA(cudaMemsetAsync(amax, 0, sizeof(float) * nslot * k2, s));
-  CB_CUDA(cudaMemsetAsync(vexp, 0, sizeof(int) * nslot * k2, s));
-  auto slotZ = [&](int j) { return (int64_t)j * k2; };
-  auto slotT = [&](int j) { return (int64_t)(maxdeg + 1 + j) * k2; };
-  const int64_t slotR = (int64_t)(2 * maxdeg + 1) * k2, slotS = (int64_t)(2 * maxdeg + 2) * k2;
+  CB_TRY(ws.alloc(&amax, nslot * ns));
+  CB_TRY(ws.alloc(&vexp, nslot * ns));
+  CB_CUDA(cudaMemsetAsync(amax, 0, sizeof(float) * nslot * ns, s));
+  CB_CUDA(cudaMemsetAsync(vexp, 0, sizeof(int) * nslot * ns, s));
+  auto slotZ = [&](int j) { return (int64_t)j * ns; };
+  auto slotT = [&](int j) { return (int64_t)(maxdeg + 1 + j) * ns; };
+  const int64_t slotR = (int64_t)(2 * maxdeg + 1) * ns, slotS = (int64_t)(2 * maxdeg + 2) * ns;
 
   std::vector<double> al(maxdeg), be(maxdeg);  // alpha_j, beta_j of the scaled recurrence
   {
@@ -1168,36 +1478,54 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
       }
     }
   }
-  std::vector<float> gh(k2);
+  std::vector<float> gh(ns);
+  // gamma of the first m vectors to the device, one entry per scaled column
+  auto put_gamma = [&](int64_t m, auto value) -> int {
+    for (int64_t i = 0; i < m; ++i)
+      for (int q = 0; q < F::SCALES; ++q) gh[F::SCALES * i + q] = (float)value(i);
+    CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * F::SCALES * m, cudaMemcpyHostToDevice, s));
+    return CHASE_BSE_OK;
+  };
+  // a block of vectors -> masters and operand pieces, with their maxima and exponents in `slot`
+  auto pack = [&](const cplx* W, float* Z, int64_t slot) -> int {
+    if (J) {
+      col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(W, n, amax + slot, vexp + slot);
+      pack_kernel<T, NPW><<<gsz(kpad / 2 * k), 256, 0, s>>>(W, n, k, c2(Z), Zp, kpad, vexp + slot);
+    } else {
+      col_amax_blocks_kernel<<<(unsigned)k, 256, 0, s>>>(W, n, amax + slot, vexp + slot);
+      pack_blocks_kernel<T, NPW><<<gsz(n * k), 256, 0, s>>>(W, n, k, c2(Z), Zp, kpad, vexp + slot);
+    }
+    count_launch();
+    count_launch();
+    CB_LAUNCH();
+    return CHASE_BSE_OK;
+  };
   int j0 = 0;
   cudaEvent_t e0, e1;
   CB_CUDA(cudaEventCreate(&e0));
   CB_CUDA(cudaEventCreate(&e1));
   CB_CUDA(cudaEventRecord(e0, s));
   if (!corr) {
-    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(Y0, n, amax + slotZ(0), vexp + slotZ(0));
-    count_launch();
-    pack_kernel<T, NPW><<<gsz(kpad / 2 * k), 256, 0, s>>>(Y0, n, k, c2(Zb[0]), Zp, kpad, vexp + slotZ(0));  // Z_0 = W
-    count_launch();
-    CB_LAUNCH();
+    CB_TRY(pack(Y0, Zb[0], slotZ(0)));  // Z_0 = W
   } else {
     // r2 = H R + ritz R on the tensor cores; Z_0 = 0; Z_1 = alpha_0 r2
-    CB_TRY(ws.alloc(&src, n2 * k2));
-    col_amax_kernel<<<(unsigned)k, 256, 0, s>>>(R, n, amax + slotR, vexp + slotR);
-    count_launch();
-    pack_kernel<T, NPW><<<gsz(kpad / 2 * k), 256, 0, s>>>(R, n, k, c2(Zb[2]), Zp, kpad, vexp + slotR);
-    count_launch();
-    for (int64_t i = 0; i < k; ++i) gh[2 * i] = gh[2 * i + 1] = (float)ritz[i];
-    CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * k2, cudaMemcpyHostToDevice, s));
+    CB_TRY(ws.alloc(&src, 2 * n2 * k));
+    CB_TRY(pack(R, Zb[2], slotR));
+    CB_TRY(put_gamma(k, [&](int64_t i) { return ritz[i]; }));
     Epi ep{};
-    ep.mode = 2; ep.n2 = n2; ep.k2 = k2; ep.kpad = kpad; ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam; ep.err = err;
+    ep.mode = 2; ep.n = n; ep.rows = rows; ep.cols = nc; ep.kpad = kpad; ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam; ep.err = err;
     ep.vexp_in = vexp + slotR;
     ep.amax_out = amax + slotS;
     sk(ep);
-    CB_TRY(apply<SCH>(P, Zp, k2, ep, s));
-    CB_CUDA(cudaMemsetAsync(Zb[0], 0, sizeof(float) * n2 * k2, s));
-    scale_pack_kernel<T, NPW><<<gsz(n * k2), 256, 0, s>>>(c2(src), n, k2, (float)al[0], c2(Zb[1]), expl ? Tp : Zp,
-                                                           kpad, amax + slotS, amax + slotZ(1), vexp + slotZ(1));
+    CB_TRY((apply<SCH, FORM>(P, Zp, nc, ep, s)));
+    CB_CUDA(cudaMemsetAsync(Zb[0], 0, sizeof(float) * 2 * n2 * k, s));
+    if (J)
+      scale_pack_kernel<T, NPW><<<gsz(n2 * k), 256, 0, s>>>(c2(src), n, 2 * k, (float)al[0], c2(Zb[1]), expl ? Tp : Zp,
+                                                             kpad, amax + slotS, amax + slotZ(1), vexp + slotZ(1));
+    else
+      scale_pack_blocks_kernel<T, NPW><<<gsz(n * k), 256, 0, s>>>(c2(src), n, k, (float)al[0], c2(Zb[1]),
+                                                                  expl ? Tp : Zp, kpad, amax + slotS, amax + slotZ(1),
+                                                                  vexp + slotZ(1));
     count_launch();
     CB_LAUNCH();
     j0 = 1;
@@ -1211,7 +1539,7 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     int64_t kj = 0;
     while (kj < k && degs[kj] >= j + 1) ++kj;
     Epi ep{};
-    ep.mode = 1; ep.hsign = 1.0f; ep.n2 = n2; ep.k2 = 2 * kj; ep.kpad = kpad; ep.err = err;
+    ep.mode = 1; ep.h2 = 1; ep.n = n; ep.rows = rows; ep.cols = F::COLS * kj; ep.kpad = kpad; ep.err = err;
     sk(ep);
     for (int q = 0; q < NPW; ++q) ep.out[q] = zbuf[(j + 1) % 2]->p[q];
     ep.Znext = Zb[(j + 1) % 3]; ep.Zcur = Zb[j % 3]; ep.Zprev = Zb[(j + 2) % 3];
@@ -1226,13 +1554,12 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     ep.cb = (float)std::fabs(al[j] * c);
     ep.cc = (float)std::fabs(be[j]);
     if (corr) {
-      for (int64_t i = 0; i < kj; ++i) gh[2 * i] = gh[2 * i + 1] = (float)(al[j] * pj[(size_t)j * k + i]);
-      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * 2 * kj, cudaMemcpyHostToDevice, s));
+      CB_TRY(put_gamma(kj, [&](int64_t i) { return al[j] * pj[(size_t)j * k + i]; }));
       ep.src = src;
       ep.gamma = gam;
       ep.amax_d = amax + slotS;
     }
-    CB_TRY(apply<SCH>(PH2, *zbuf[j % 2], k2, ep, s));
+    CB_TRY((apply<SCH, FORM>(PH2, *zbuf[j % 2], nc, ep, s)));
     if (fs) {
       fs->flops += 32.0 * (double)n * (double)n * (double)kj;  // the product with the blocks of H^2
       fs->launches += 1;
@@ -1242,7 +1569,7 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     int64_t kj = 0;
     while (kj < k && degs[kj] >= j + 1) ++kj;
     Epi e1p{};
-    e1p.mode = 0; e1p.n2 = n2; e1p.k2 = 2 * kj; e1p.kpad = P.kpad; e1p.err = err;
+    e1p.mode = 0; e1p.n = n; e1p.rows = rows; e1p.cols = F::COLS * kj; e1p.kpad = kpad; e1p.err = err;
     sk(e1p);
     for (int q = 0; q < NPW; ++q) e1p.out[q] = Tp.p[q];
     e1p.vexp_in = vexp + slotZ(j);
@@ -1250,9 +1577,9 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     e1p.amax_out = amax + slotT(j);
     e1p.amax_a = amax + slotZ(j);
     e1p.ca = 1.0f;
-    CB_TRY(apply<SCH>(P, Zp, k2, e1p, s));  // T = M Z_j
+    CB_TRY((apply<SCH, FORM>(P, Zp, nc, e1p, s)));  // T = H Z_j (J form: M Z_j)
     Epi e2p{};
-    e2p.mode = 1; e2p.hsign = -1.0f; e2p.n2 = n2; e2p.k2 = 2 * kj; e2p.kpad = P.kpad; e2p.err = err;
+    e2p.mode = 1; e2p.n = n; e2p.rows = rows; e2p.cols = F::COLS * kj; e2p.kpad = kpad; e2p.err = err;
     sk(e2p);
     for (int q = 0; q < NPW; ++q) e2p.out[q] = Zp.p[q];
     e2p.Znext = Zb[(j + 1) % 3]; e2p.Zcur = Zb[j % 3]; e2p.Zprev = Zb[(j + 2) % 3];
@@ -1267,13 +1594,12 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     e2p.cb = (float)std::fabs(al[j] * c);
     e2p.cc = (float)std::fabs(be[j]);
     if (corr) {
-      for (int64_t i = 0; i < kj; ++i) gh[2 * i] = gh[2 * i + 1] = (float)(al[j] * pj[(size_t)j * k + i]);
-      CB_CUDA(cudaMemcpyAsync(gam, gh.data(), sizeof(float) * 2 * kj, cudaMemcpyHostToDevice, s));
+      CB_TRY(put_gamma(kj, [&](int64_t i) { return al[j] * pj[(size_t)j * k + i]; }));
       e2p.src = src;
       e2p.gamma = gam;
       e2p.amax_d = amax + slotS;
     }
-    CB_TRY(apply<SCH>(P, Tp, k2, e2p, s));  // Z_{j+1} = alpha (-M T - c Z_j) + beta Z_{j-1} (+ source)
+    CB_TRY((apply<SCH, FORM>(P, Tp, nc, e2p, s)));  // Z_{j+1} = alpha (H T - c Z_j) + beta Z_{j-1} (+ source)
     if (fs) {
       fs->flops += 64.0 * (double)n * (double)n * (double)kj;
       fs->launches += 2;
@@ -1292,8 +1618,9 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
   CB_TRY(ws.alloc(&dcoef, k));
   CB_CUDA(cudaMemcpyAsync(dsel, sel.data(), sizeof(int) * k, cudaMemcpyHostToDevice, s));
   CB_CUDA(cudaMemcpyAsync(dcoef, coef.data(), sizeof(double) * k, cudaMemcpyHostToDevice, s));
-  combine_kernel<<<gsz(n * k), 256, 0, s>>>(out, c2(Zb[0]), c2(Zb[1]), c2(Zb[2]), dsel, corr ? dcoef : nullptr, Y0, n,
-                                           k);
+  const double* dc = corr ? dcoef : nullptr;
+  if (J) combine_kernel<<<gsz(n * k), 256, 0, s>>>(out, c2(Zb[0]), c2(Zb[1]), c2(Zb[2]), dsel, dc, Y0, n, k);
+  else combine_blocks_kernel<<<gsz(n2 * k), 256, 0, s>>>(out, c2(Zb[0]), c2(Zb[1]), c2(Zb[2]), dsel, dc, Y0, n2, k);
   count_launch();
   CB_LAUNCH();
   int herr = 0;
@@ -1322,33 +1649,41 @@ bool mixed_available() {
   return major == 10 && minor == 3 && tc::encode_fn() != nullptr;
 }
 
-static int filter_scheme(int scheme, const cplx* A, const cplx* B, int64_t n, cplx* V, int64_t k, const int* degs,
-                         double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
-                         cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
+// Where both forms are open the J form takes half the operations but, to form the entries of
+// M, four FP64 additions per entry of A and B (1.6e-5 us n^2), and its launches are no shorter
+// where M streams from HBM for few columns.  Measured, J form and blocks: n = 6000, k = 8,
+// degree 4 2.00 and 1.37 ms; 8100, 30, 8 4.91 and 4.60; 16384, 20, 4 14.6 and 10.3; 3001, 10, 10 1.12
+// and 1.13; against 4096, 60, 10 1.96 and 2.29; 16384, 100, 4 15.8 and 18.2; 1301, 6, 12 0.61 and 0.64.
+static bool j_form_faster(int64_t n, int64_t k, const int* degs) {
+  int64_t work = 0;
+  for (int64_t i = 0; i < k; ++i) work += degs[i];
+  return n < 3000 || work >= 300;
+}
+template <int SCH>
+static int filter_form(bool jfixed, const cplx* A, const cplx* B, int64_t n, const cplx* V, int64_t k, const int* degs,
+                       double mu1, double mu_nevex, double muN, cplx* out, const double* ritz, const cplx* R,
+                       cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
+  if (jfixed && j_form_faster(n, k, degs))
+    return tc::filter_impl<SCH, tc::FORM_J>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+  return tc::filter_impl<SCH, tc::FORM_BLOCKS>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+}
+
+int filter_mixed_sorted(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, int64_t k, const int* degs_sorted,
+                        double mu1, double mu_nevex, double muN, cplx* out, int scheme, bool jfixed, const double* ritz,
+                        const cplx* R, cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2) {
   switch (scheme) {
     case SCHEME_BF16X3:
-      return tc::filter_impl<tc::SCH_BF16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return filter_form<tc::SCH_BF16X3>(jfixed, A, B, n, Y0, k, degs_sorted, mu1, mu_nevex, muN, out, ritz, R, s, fs,
+                                         P2, Q2);
     case SCHEME_BF16X6:
-      return tc::filter_impl<tc::SCH_BF16X6>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return filter_form<tc::SCH_BF16X6>(jfixed, A, B, n, Y0, k, degs_sorted, mu1, mu_nevex, muN, out, ritz, R, s, fs,
+                                         P2, Q2);
     case SCHEME_FP16X3:
-      return tc::filter_impl<tc::SCH_FP16X3>(A, B, n, V, k, degs, mu1, mu_nevex, muN, out, ritz, R, s, fs, P2, Q2);
+      return filter_form<tc::SCH_FP16X3>(jfixed, A, B, n, Y0, k, degs_sorted, mu1, mu_nevex, muN, out, ritz, R, s, fs,
+                                         P2, Q2);
     default:
       return CHASE_BSE_BAD_ARG;
   }
-}
-
-int filter_mixed_sorted(const cplx* A, const cplx* B, int64_t n, cplx* Y0, int64_t k, const int* degs_sorted,
-                        double mu1, double mu_nevex, double muN, cplx* out, int scheme, cudaStream_t s,
-                        FilterStats* fs, const cplx* P2, const cplx* Q2) {
-  return filter_scheme(scheme, A, B, n, Y0, k, degs_sorted, mu1, mu_nevex, muN, out, nullptr, nullptr, s, fs, P2,
-                       Q2);
-}
-
-int filter_mixed_correction_sorted(const cplx* A, const cplx* B, int64_t n, cplx* V, int64_t k,
-                                   const int* degs_sorted, const double* ritz_sorted, const cplx* R, double mu1,
-                                   double mu_nevex, double muN, cplx* out, int scheme, cudaStream_t s,
-                                   FilterStats* fs, const cplx* P2, const cplx* Q2) {
-  return filter_scheme(scheme, A, B, n, V, k, degs_sorted, mu1, mu_nevex, muN, out, ritz_sorted, R, s, fs, P2, Q2);
 }
 
 }  // namespace cb

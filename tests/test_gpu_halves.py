@@ -84,3 +84,62 @@ def test_fp64_filter_without_coupling_keeps_a_zero_half(pkg):
     W[:, n:] = 0.0
     got = pkg.filter(A, B, W, [4] * k, 0.9 * float(P.d.min()), 5.0, 1.1 * float(P.d.max()))
     assert not bool(torch.any(got[:, n:] != 0.0)) and bool(torch.all(torch.isfinite(got.abs())))
+
+
+@pytest.fixture(scope="module")
+def tensor_cores(pkg):
+    if not pkg.has_mixed():
+        pytest.fail("tensor-core filter not available on this device")
+    return pkg
+
+
+# The tensor-core filters' gates of a whole vector (tests/test_gpu_mixed.py, test_gpu_h2.py) for each
+# half: FP16x3 keeps 22 bits of an operand entry down to 2^-11 of the largest of its row or vector
+# (16-bit pieces of 11 bits each from 2^13 down to 2^-24), so down to a coupling of 1e-4 (2^-13.3)
+# all but two of them; the BF16 pieces have FP32's exponent range.
+TOL = {"fp16x3": 1e-5, "bf16x6": 1e-5, "bf16x3": 6e-5}
+
+
+@pytest.mark.parametrize("precision", ["fp16x3", "bf16x6", "bf16x3"])
+@pytest.mark.parametrize("beta", [0.3, 1e-3, 1e-4])
+# operand rows n around a tile of 256 rows, columns 4k around 32, 160 and 256, K = 4n around a
+# block of 64; (300, 70): K ranges, (640, 24)
+@pytest.mark.parametrize("n,k,deg", [(31, 1, 3), (47, 8, 4), (129, 33, 4), (255, 9, 3), (256, 40, 3),
+                                     (257, 41, 3), (300, 70, 4), (640, 24, 4)])
+def test_tensor_core_filter_keeps_both_halves(tensor_cores, precision, n, k, deg, beta):
+    P = bi.make_problem(n, seed=n + k, beta=beta)
+    A, B = problem_on_device(P)
+    W = _block(n, k, 4, beta)
+    mus = (0.5 * float(P.d.min()), 0.8 * float(P.d.max()) + 0.1, 1.5 * float(P.d.max()))
+    ref = _filter(A, B, W, deg, *mus)
+    got = tensor_cores.filter(A, B, W.clone(), [deg] * k, *mus, precision=precision)
+    assert max(_errors(got, ref)) <= TOL[precision]
+
+
+@pytest.mark.parametrize("beta", [0.3, 1e-3])
+@pytest.mark.parametrize("n,k", [(64, 9), (300, 70)])
+def test_explicit_square_filter_keeps_both_halves(tensor_cores, n, k, beta):
+    P = bi.make_problem(n, seed=n + k, beta=beta)
+    A, B = problem_on_device(P)
+    W = _block(n, k, 4, beta)
+    mus = (0.5 * float(P.d.min()), 0.8 * float(P.d.max()) + 0.1, 1.5 * float(P.d.max()))
+    ref = _filter(A, B, W, 4, *mus)
+    got = tensor_cores.filter_h2(A, B, W.clone(), [4] * k, *mus)
+    assert max(_errors(got, ref)) <= 5e-5
+
+
+# full waves of CTA pairs and K ranges of the tiles left over, ragged degrees
+@pytest.mark.parametrize("n,k", [(2048, 700), (2050, 645)])
+def test_tensor_core_filter_halves_over_full_waves(tensor_cores, n, k):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn((n, n), generator=g, dtype=torch.complex128, device="cuda")
+    A = (X + X.conj().T) * (0.5 / np.sqrt(n)) + 5.0 * torch.eye(n, dtype=torch.complex128, device="cuda")
+    Y = torch.randn((n, n), generator=g, dtype=torch.complex128, device="cuda")
+    B = (Y + Y.T) * (1e-3 / np.sqrt(n))
+    W = torch.randn((k, 2 * n), generator=g, dtype=torch.complex128, device="cuda")
+    W[:, n:] *= 1e-3
+    degs = np.where(np.arange(k) < 9, 3, 1 + np.arange(k) % 2)
+    got = tensor_cores.filter(A, B, W.clone(), degs, 1.5, 4.0, 8.0, precision="fp16x3")
+    for d in (1, 2, 3):
+        sel = torch.from_numpy(np.flatnonzero(degs == d)).cuda()
+        assert max(_errors(got[sel], _filter(A, B, W[sel], d, 1.5, 4.0, 8.0))) <= 1e-5
