@@ -47,8 +47,7 @@ typedef enum chase_bse_status {
   CHASE_BSE_OOM = -3,            /* workspace allocation failed                       */
   CHASE_BSE_NOT_DEFINITE = -4,   /* Cholesky of Q^* S H Q failed: S H not HPD (in a
                                     solve: and the non-hermitian fallback found fewer
-                                    Ritz values with positive real part than needed, or
-                                    ran in every iteration and no pair converged)     */
+                                    Ritz values with positive real part than needed) */
   CHASE_BSE_QR_FAILED = -5,      /* search space rank-deficient even for Householder  */
   CHASE_BSE_DEVICE_TIMEOUT = -6, /* a bounded device-side wait gave up                */
   CHASE_BSE_UNSUPPORTED = -7,    /* feature needs a device this build cannot run on   */

@@ -1332,10 +1332,6 @@ int solve(const cplx* A, const cplx* B, int64_t n, int64_t nev, int64_t nex, int
     *stats = st;
   }
   if (status != CHASE_BSE_OK) return status;
-  // Q^* S H Q indefinite in every iteration and not one pair from the fallback: S H is not
-  // definite (whether the fallback runs out of positive Ritz values before maxiter depends
-  // on the last bits of its products)
-  if (nout == 0 && o.rr == 0 && it > 0 && st.fallback_rr == it) return CHASE_BSE_NOT_DEFINITE;
   return (nout < nev) ? CHASE_BSE_NOT_CONVERGED : CHASE_BSE_OK;
 }
 
