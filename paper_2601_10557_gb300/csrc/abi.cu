@@ -80,7 +80,7 @@ int chase_bse_gemm_time(int32_t kind, double* total_ms, double* flops, int64_t* 
   return cb::timer_read(kind, total_ms, flops, launches);
 }
 
-int chase_bse_has_mixed(void) { return cb::mixed_available() ? 1 : 0; }
+int chase_bse_has_mixed(void) { return cb::mixed_filter_available() ? 1 : 0; }
 
 void chase_bse_trim_memory(void) { cb::pool_trim(); }
 
@@ -213,7 +213,7 @@ int chase_bse_filter_h2(const void* A, const void* B, int64_t n, void* W, int64_
     return CHASE_BSE_BAD_ARG;
   for (int64_t i = 0; i < k; ++i)
     if (degs[i] < 1) return CHASE_BSE_BAD_ARG;
-  if (!cb::mixed_available()) return CHASE_BSE_UNSUPPORTED;
+  if (!cb::mixed_filter_available()) return CHASE_BSE_UNSUPPORTED;
   CB_GUARD({
     cudaStream_t s = (cudaStream_t)stream;
     cb::Workspace ws(s);

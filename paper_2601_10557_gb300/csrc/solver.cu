@@ -354,7 +354,7 @@ int filter(const cplx* A, const cplx* B, int64_t n, cplx* W, int64_t k, const in
     if (grp == 0) {
       CB_TRY(filter_fp64_sorted(A, B, n, Y0, m, ds.data(), mu1, mu_nevex, muN, out, gws, s, fs, ph, jfixed));
     } else {
-      if (!mixed_available()) return CHASE_BSE_UNSUPPORTED;
+      if (!mixed_filter_available()) return CHASE_BSE_UNSUPPORTED;
       const bool corr = ritz && R;
       cplx* Rs = nullptr;
       std::vector<double> rs(corr ? m : 0);
@@ -1049,7 +1049,7 @@ int solve(const cplx* A, const cplx* B, int64_t n, int64_t nev, int64_t nex, int
   const bool sliced = fp64tc || (mixed && o.fp64_products == 0);
   // FilterScheme codes equal the mixed precision codes (unused when no column is mixed)
   const int scheme = mixed ? o.precision : (int)CHASE_BSE_MIXED_FP16X3;
-  if ((mixed || fp64tc) && !mixed_available()) return CHASE_BSE_UNSUPPORTED;
+  if ((fp64tc && !mixed_available()) || (mixed && !mixed_filter_available())) return CHASE_BSE_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)o.stream;
   const int64_t n2 = 2 * n, nevex = nev + nex;
   {  // inputs with a NaN or an Inf: a defined status, nothing computed

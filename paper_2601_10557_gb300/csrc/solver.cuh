@@ -85,6 +85,8 @@ int gradient(const cplx* V, const double* w, int64_t n, int64_t nev, cplx* gA, c
 int filter_mixed_sorted(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, int64_t k, const int* degs_sorted,
                         double mu1, double mu_nevex, double muN, cplx* out, int scheme, bool jfixed, const double* ritz,
                         const cplx* R, cudaStream_t s, FilterStats* fs, const cplx* P2, const cplx* Q2);
+// Tensor cores and TMA are there (the sliced products); and the filter's kernels can run on them.
 bool mixed_available();
+bool mixed_filter_available();
 
 }  // namespace cb

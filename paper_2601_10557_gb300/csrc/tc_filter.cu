@@ -186,8 +186,13 @@ constexpr int THREADS = 128 + 32 * (DRAIN_WARPS + EPI_WARPS);
 // the MMA issuer and that of the finishing warps give theirs to the drain warps, whose sums
 // take 128.
 constexpr int REGS_LAUNCH = 128, REGS_ROLES = 40, REGS_DRAIN = 184, REGS_EPI = 96;
-static_assert(128 * REGS_ROLES + 32 * DRAIN_WARPS * REGS_DRAIN + 32 * EPI_WARPS * REGS_EPI <= THREADS * REGS_LAUNCH,
-              "register split");
+// The warpgroups draw on what the block was launched with: a kernel compiled to fewer registers a
+// thread than the shares add up to would wait for the rest forever (see mixed_filter_available).
+constexpr bool register_split_fits(int regs) {
+  return 128 * REGS_ROLES + 32 * DRAIN_WARPS * REGS_DRAIN + 32 * EPI_WARPS * REGS_EPI <= THREADS * regs;
+}
+static_assert(register_split_fits(REGS_LAUNCH) && register_split_fits(126) && !register_split_fits(125),
+              "126 registers a thread hold the shares");
 static_assert(SMEM_BYTES <= 232448, "shared memory");
 
 struct Epi {
@@ -1340,10 +1345,6 @@ static int apply(const POperand& P, const Pieces& bp, int64_t rows, Epi ep, cuda
   static bool attr = false;
   if (!attr) {
     CB_CUDA(cudaFuncSetAttribute(tc_hop_kernel<SCH, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    // the drain warps' share exists only if the kernel was launched with REGS_LAUNCH registers a thread
-    cudaFuncAttributes fa;
-    CB_CUDA(cudaFuncGetAttributes(&fa, tc_hop_kernel<SCH, FORM>));
-    if (fa.numRegs != REGS_LAUNCH) return CHASE_BSE_UNSUPPORTED;
     attr = true;
   }
   ep.prow = P.prow;
@@ -1647,6 +1648,22 @@ bool mixed_available() {
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
   return major == 10 && minor == 3 && tc::encode_fn() != nullptr;
+}
+
+template <int SCH, int FORM>
+static bool kernel_fits() {
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, tc::tc_hop_kernel<SCH, FORM>) == cudaSuccess) return tc::register_split_fits(fa.numRegs);
+  cudaGetLastError();
+  return false;
+}
+bool mixed_filter_available() {
+  if (!mixed_available()) return false;
+  // a property of the build
+  static const bool fits = kernel_fits<tc::SCH_BF16X3, tc::FORM_J>() && kernel_fits<tc::SCH_BF16X3, tc::FORM_BLOCKS>() &&
+                           kernel_fits<tc::SCH_BF16X6, tc::FORM_J>() && kernel_fits<tc::SCH_BF16X6, tc::FORM_BLOCKS>() &&
+                           kernel_fits<tc::SCH_FP16X3, tc::FORM_J>() && kernel_fits<tc::SCH_FP16X3, tc::FORM_BLOCKS>();
+  return fits;
 }
 
 // Where both forms are open the J form takes half the operations but, to form the entries of
