@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (lane == 0) mbar_arrive(acce[b]);
     }
     grp0 += ngrp;
-    if (ok && !*abort_sh) {
+    // warp-uniform: another role may abort at this moment, and put_sym shuffles over the whole warp
+    if (ok && __all_sync(0xffffffffu, *abort_sh == 0)) {
       const int64_t row = (int64_t)mt * BM + q * 32 + lane;  // < mp: rows are padded to whole tiles
       const int64_t col = (int64_t)nt * BNS + half * NC;
       if (g.hi) {
