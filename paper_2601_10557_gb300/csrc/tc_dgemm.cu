@@ -242,42 +242,42 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int id = blockIdx.x; ok && id < g.items; id += gridDim.x) {
-    item(id, mt, nt, sp, kb0, nkb);
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int b = grp & 1;
-      const bool first = (kb % CHUNK) == 0;
-      const bool last = (kb % CHUNK) == CHUNK - 1 || kb == nkb - 1;
-      if ((first && grp >= 2 && !mbar_wait(acce[b], (uint32_t)((grp >> 1) - 1) & 1u, abort_sh, g.err, true)) ||
-          !mbar_wait(full[0] + 8 * s, ph, abort_sh, g.err, true)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t st = sbase + s * STAGE_BYTES;
-      const uint32_t buf = tmem + (uint32_t)(b * GCOLS);
-#pragma unroll
-      for (int kk = 0; kk < BK / 16; ++kk) {
-        // sdesc64 is linear in the address here (its 14-bit start field holds address / 16
-        // of a ring below 256 KB and cannot carry): a hoisted base plus constants
-        const uint64_t sd = dbase + (uint64_t)((uint32_t)(st - sbase) >> 4);
-        const uint64_t bd = sd + (uint64_t)((S * A_SLICE + kk * 32) >> 4);
-#pragma unroll
-        for (int t = 0; t < S; ++t) {
-          const uint64_t ad = sd + (uint64_t)((t * A_SLICE + kk * 32) >> 4);
-          const uint32_t acc = (first && kk == 0 && t == 0) ? 0u : 1u;
-          mma_bf16(buf + (uint32_t)(t * BNS), ad, bd, idesc_n((S - t) * BNS), acc);
+      item(id, mt, nt, sp, kb0, nkb);
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int b = grp & 1;
+        const bool first = (kb % CHUNK) == 0;
+        const bool last = (kb % CHUNK) == CHUNK - 1 || kb == nkb - 1;
+        if ((first && grp >= 2 && !mbar_wait(acce[b], (uint32_t)((grp >> 1) - 1) & 1u, abort_sh, g.err, true)) ||
+            !mbar_wait(full[0] + 8 * s, ph, abort_sh, g.err, true)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t st = sbase + s * STAGE_BYTES;
+        const uint32_t buf = tmem + (uint32_t)(b * GCOLS);
+  #pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          // sdesc64 is linear in the address here (its 14-bit start field holds address / 16
+          // of a ring below 256 KB and cannot carry): a hoisted base plus constants
+          const uint64_t sd = dbase + (uint64_t)((uint32_t)(st - sbase) >> 4);
+          const uint64_t bd = sd + (uint64_t)((S * A_SLICE + kk * 32) >> 4);
+  #pragma unroll
+          for (int t = 0; t < S; ++t) {
+            const uint64_t ad = sd + (uint64_t)((t * A_SLICE + kk * 32) >> 4);
+            const uint32_t acc = (first && kk == 0 && t == 0) ? 0u : 1u;
+            mma_bf16(buf + (uint32_t)(t * BNS), ad, bd, idesc_n((S - t) * BNS), acc);
+          }
+        }
+        mma_commit(empty[0] + 8 * s);
+        if (last) {
+          mma_commit(accf[b]);
+          ++grp;
+        }
+        if (++s == ST) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      mma_commit(empty[0] + 8 * s);
-      if (last) {
-        mma_commit(accf[b]);
-        ++grp;
-      }
-      if (++s == ST) {
-        s = 0;
-        ph ^= 1u;
-      }
-    }
     }
     mma_commit(done);
   } else if (warp >= 4) {
@@ -288,77 +288,77 @@ __global__ void __launch_bounds__(THREADS, 1)
     bool ok = true;
     int grp0 = 0;
     for (int id = blockIdx.x; ok && id < g.items; id += gridDim.x) {
-    item(id, mt, nt, sp, kb0, nkb);
-    long long hi[NC], lo[NC];
-#pragma unroll
-    for (int i = 0; i < NC; ++i) {
-      hi[i] = 0;
-      lo[i] = 0;
-    }
-    const int ngrp = (nkb + CHUNK - 1) / CHUNK;
-    for (int grp = grp0; grp < grp0 + ngrp; ++grp) {
-      const int b = grp & 1;
-      const bool w = mbar_wait(accf[b], (uint32_t)(grp >> 1) & 1u, abort_sh, g.err, true);
-      if (!__all_sync(0xffffffffu, w)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t col = tmem + lane_base + (uint32_t)(b * GCOLS + half * NC);
-      uint32_t r0[NC], r1[NC], r2[NC];
-      // group sums g_w are integers below 2^24 (exact in FP32)
-      // hi += (g0 2^8 + g1) 2^16 + g2 2^8 + g3       (each bracket below 2^31)
-      tmem_ld16_nowait(col, r0);
-      tmem_ld16_nowait(col + 32, r1);
-      tmem_wait_ld();
-#pragma unroll
+      item(id, mt, nt, sp, kb0, nkb);
+      long long hi[NC], lo[NC];
+  #pragma unroll
       for (int i = 0; i < NC; ++i) {
-        const int v = __float2int_rn(__uint_as_float(r0[i])) * 256 + __float2int_rn(__uint_as_float(r1[i]));
-        hi[i] += (long long)v * 65536;
+        hi[i] = 0;
+        lo[i] = 0;
       }
-      tmem_ld16_nowait(col + 64, r0);
-      tmem_ld16_nowait(col + 96, r1);
-      tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        const int v = __float2int_rn(__uint_as_float(r0[i])) * 256 + __float2int_rn(__uint_as_float(r1[i]));
-        hi[i] += (long long)v;
-      }
-      // lo += g4 2^16 + g5 2^8 + g6
-      tmem_ld16_nowait(col + 128, r0);
-      tmem_ld16_nowait(col + 160, r1);
-      tmem_ld16_nowait(col + 192, r2);
-      tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        lo[i] += (long long)__float2int_rn(__uint_as_float(r0[i])) * 65536 +
-                 (long long)__float2int_rn(__uint_as_float(r1[i])) * 256 +
-                 (long long)__float2int_rn(__uint_as_float(r2[i]));
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acce[b]);
-    }
-    grp0 += ngrp;
-    // warp-uniform: another role may abort at this moment, and put_sym shuffles over the whole warp
-    if (ok && __all_sync(0xffffffffu, *abort_sh == 0)) {
-      const int64_t row = (int64_t)mt * BM + q * 32 + lane;  // < mp: rows are padded to whole tiles
-      const int64_t col = (int64_t)nt * BNS + half * NC;
-      if (g.hi) {
-        const int64_t base = ((int64_t)sp * g.np + col) * g.mp + row;
-#pragma unroll
-        for (int i = 0; i < NC; ++i) {
-          g.hi[base + (int64_t)i * g.mp] = hi[i];
-          g.lo[base + (int64_t)i * g.mp] = lo[i];
+      const int ngrp = (nkb + CHUNK - 1) / CHUNK;
+      for (int grp = grp0; grp < grp0 + ngrp; ++grp) {
+        const int b = grp & 1;
+        const bool w = mbar_wait(accf[b], (uint32_t)(grp >> 1) & 1u, abort_sh, g.err, true);
+        if (!__all_sync(0xffffffffu, w)) {
+          ok = false;
+          break;
         }
-      } else if (g.sym) {
-        put_sym<NC>(g, row, col, hi, lo);
-      } else if (row < g.M) {
-#pragma unroll
-        for (int i = 0; i < NC; ++i)
-          if (col + i < g.N) put_out(g, row, col + i, hi[i], lo[i]);
+        tc_fence_after();
+        const uint32_t col = tmem + lane_base + (uint32_t)(b * GCOLS + half * NC);
+        uint32_t r0[NC], r1[NC], r2[NC];
+        // group sums g_w are integers below 2^24 (exact in FP32)
+        // hi += (g0 2^8 + g1) 2^16 + g2 2^8 + g3       (each bracket below 2^31)
+        tmem_ld16_nowait(col, r0);
+        tmem_ld16_nowait(col + 32, r1);
+        tmem_wait_ld();
+  #pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          const int v = __float2int_rn(__uint_as_float(r0[i])) * 256 + __float2int_rn(__uint_as_float(r1[i]));
+          hi[i] += (long long)v * 65536;
+        }
+        tmem_ld16_nowait(col + 64, r0);
+        tmem_ld16_nowait(col + 96, r1);
+        tmem_wait_ld();
+  #pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          const int v = __float2int_rn(__uint_as_float(r0[i])) * 256 + __float2int_rn(__uint_as_float(r1[i]));
+          hi[i] += (long long)v;
+        }
+        // lo += g4 2^16 + g5 2^8 + g6
+        tmem_ld16_nowait(col + 128, r0);
+        tmem_ld16_nowait(col + 160, r1);
+        tmem_ld16_nowait(col + 192, r2);
+        tmem_wait_ld();
+  #pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          lo[i] += (long long)__float2int_rn(__uint_as_float(r0[i])) * 65536 +
+                   (long long)__float2int_rn(__uint_as_float(r1[i])) * 256 +
+                   (long long)__float2int_rn(__uint_as_float(r2[i]));
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce[b]);
       }
-    }
+      grp0 += ngrp;
+      // warp-uniform: another role may abort at this moment, and put_sym shuffles over the whole warp
+      if (ok && __all_sync(0xffffffffu, *abort_sh == 0)) {
+        const int64_t row = (int64_t)mt * BM + q * 32 + lane;  // < mp: rows are padded to whole tiles
+        const int64_t col = (int64_t)nt * BNS + half * NC;
+        if (g.hi) {
+          const int64_t base = ((int64_t)sp * g.np + col) * g.mp + row;
+  #pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            g.hi[base + (int64_t)i * g.mp] = hi[i];
+            g.lo[base + (int64_t)i * g.mp] = lo[i];
+          }
+        } else if (g.sym) {
+          put_sym<NC>(g, row, col, hi, lo);
+        } else if (row < g.M) {
+  #pragma unroll
+          for (int i = 0; i < NC; ++i)
+            if (col + i < g.N) put_out(g, row, col + i, hi[i], lo[i]);
+        }
+      }
     }
   }
   tc_fence_before();

@@ -162,7 +162,8 @@ struct Form<FORM_BLOCKS> {
 // cycles at BN = 256 where one CTA per 128 x 128 tile takes 64 KB per 768: shared-memory
 // traffic (operand reads of the MMAs plus the fill) bounds the smaller tile.  Of x0 * y0
 // 16 truncating MMA additions go into a drained sum with two pieces (8 cost 2-8 %), 8 with
-// three, whose 24 bits the truncation of 16 would show (1.9 times the error).  K blocks of 32 in twice the stages lost 10-25 % (64-byte rows).
+// three, whose 24 bits the truncation of 16 would show (1.9 times the error).  K blocks of 32 in
+// twice the stages lost 10-25 % (64-byte rows).
 //
 // Measured on one GB300, FP16x3, time of one launch of a degree's two, before (one CTA per
 // 128 x 128 tile, blocks form) and after, blocks and J form: n = 16384, k = 1300 26.5 -> 23.2 and
@@ -679,7 +680,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   float* my_tiles = ep.part + (size_t)blockIdx.x * (2 * BM * BNMAX);
   // A pair's last tile, for the drain and the finishing warps together: all of them pass the
   // barriers, also after a failed wait.  True where this CTA has the tile's last partial.
-  auto final_tile = [&](bool ok, const Walk& wk, int slot) -> bool {
+  auto final_tile = [&](bool ok, const Walk& wk) -> bool {
     constexpr int N = 32 * (DRAIN_WARPS + EPI_WARPS);
     if (wk.split()) __threadfence();
     asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
@@ -706,104 +707,104 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_ROLES));
-  if (warp == 0 && lane == 0) {
-    int issued = 0, s = 0;
-    uint32_t ph = 0;
-    const uint32_t lead = map_rank(full0, 0);
-    bool ok = true;
-    for (Walk wk(sc, pair); ok && wk.next();) {
-      const int m0 = (2 * wk.mt + (int)rank) * BM, n0 = wk.nt * sc.bn + (int)rank * (wk.cols / 2);
-      for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
-        if (issued >= ST && !mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_sh, ep.err, true)) {
-          ok = false;
-          break;
-        }
-        const uint32_t st = sbase + s * sc.stage_bytes;
-        if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * sc.stage_bytes);
-#pragma unroll
-        for (int q = 0; q < SC::NPA; ++q) tma_load_2d_pair(st + q * A_BYTES, &maps.a[q], kb * BK, m0, lead + 8 * s);
-#pragma unroll
-        for (int q = 0; q < SC::NPW; ++q)
-          tma_load_2d_pair(st + SC::NPA * A_BYTES + q * b_bytes, &maps.b[q], kb * BK, n0, lead + 8 * s);
-        ++issued;
-        if (++s == ST) {
-          s = 0;
-          ph ^= 1u;
+    if (warp == 0 && lane == 0) {
+      int issued = 0, s = 0;
+      uint32_t ph = 0;
+      const uint32_t lead = map_rank(full0, 0);
+      bool ok = true;
+      for (Walk wk(sc, pair); ok && wk.next();) {
+        const int m0 = (2 * wk.mt + (int)rank) * BM, n0 = wk.nt * sc.bn + (int)rank * (wk.cols / 2);
+        for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
+          if (issued >= ST && !mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_sh, ep.err, true)) {
+            ok = false;
+            break;
+          }
+          const uint32_t st = sbase + s * sc.stage_bytes;
+          if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * sc.stage_bytes);
+  #pragma unroll
+          for (int q = 0; q < SC::NPA; ++q) tma_load_2d_pair(st + q * A_BYTES, &maps.a[q], kb * BK, m0, lead + 8 * s);
+  #pragma unroll
+          for (int q = 0; q < SC::NPW; ++q)
+            tma_load_2d_pair(st + SC::NPA * A_BYTES + q * b_bytes, &maps.b[q], kb * BK, n0, lead + 8 * s);
+          ++issued;
+          if (++s == ST) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
       }
-    }
-    *issued_sh = issued;
-  } else if (warp == 1 && lane == 0 && rank == 0) {
-    const uint64_t dbase = sdesc(sbase);
-    int s = 0, b = 0, seg = 0;
-    uint32_t ph = 0, accph = 1;  // the first pass over the buffers does not wait
-    bool ok = true, used = false;
-    for (Walk wk(sc, pair); ok && wk.next(); ++seg) {
-      const uint32_t idesc = make_idesc(wk.cols, Piece<T>::BF16);
-      for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
-        const int i = kb - wk.kb0;
-        const bool first = (i & (FLUSH - 1)) == 0;
-        const bool last = (i & (FLUSH - 1)) == FLUSH - 1 || kb == wk.kb1 - 1;
-        if (!mbar_wait(full0 + 8 * s, ph, abort_sh, ep.err, true)) {
-          ok = false;
-          break;
-        }
-        // sdesc is linear in the address here (its 14-bit start field holds address / 16 of
-        // a 1024-aligned ring below 256 KB and cannot carry): a hoisted base plus constants;
-        // 16 K elements further along a swizzled row is 32 bytes further
-        const uint64_t ad0 = dbase + (uint64_t)((uint32_t)(s * sc.stage_bytes) >> 4);
-        const uint64_t bd0 = ad0 + (uint64_t)((SC::NPA * A_BYTES) >> 4);
-        // x0 * y0 first, so that a finished buffer drains behind the cross products; but a new
-        // buffer's x0 * y0 last, so that the drain has a second block's cross products to hide
-        // behind (except at a tile's start, whose cross products wait for the previous drain)
-        const bool big_last = first && i > 0;
-        auto cross_products = [&]() {
-#pragma unroll
+      *issued_sh = issued;
+    } else if (warp == 1 && lane == 0 && rank == 0) {
+      const uint64_t dbase = sdesc(sbase);
+      int s = 0, b = 0, seg = 0;
+      uint32_t ph = 0, accph = 1;  // the first pass over the buffers does not wait
+      bool ok = true, used = false;
+      for (Walk wk(sc, pair); ok && wk.next(); ++seg) {
+        const uint32_t idesc = make_idesc(wk.cols, Piece<T>::BF16);
+        for (int kb = wk.kb0; kb < wk.kb1; ++kb) {
+          const int i = kb - wk.kb0;
+          const bool first = (i & (FLUSH - 1)) == 0;
+          const bool last = (i & (FLUSH - 1)) == FLUSH - 1 || kb == wk.kb1 - 1;
+          if (!mbar_wait(full0 + 8 * s, ph, abort_sh, ep.err, true)) {
+            ok = false;
+            break;
+          }
+          // sdesc is linear in the address here (its 14-bit start field holds address / 16 of
+          // a 1024-aligned ring below 256 KB and cannot carry): a hoisted base plus constants;
+          // 16 K elements further along a swizzled row is 32 bytes further
+          const uint64_t ad0 = dbase + (uint64_t)((uint32_t)(s * sc.stage_bytes) >> 4);
+          const uint64_t bd0 = ad0 + (uint64_t)((SC::NPA * A_BYTES) >> 4);
+          // x0 * y0 first, so that a finished buffer drains behind the cross products; but a new
+          // buffer's x0 * y0 last, so that the drain has a second block's cross products to hide
+          // behind (except at a tile's start, whose cross products wait for the previous drain)
+          const bool big_last = first && i > 0;
+          auto cross_products = [&]() {
+  #pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+  #pragma unroll
+              for (int pr = 1; pr < SC::NPROD; ++pr)
+                mma_f16_pair(tmem + cross, ad0 + (uint64_t)((SC::pa(pr) * A_BYTES + kk * 32) >> 4),
+                             bd0 + (uint64_t)((SC::pb(pr) * b_bytes + (uint32_t)(kk * 32)) >> 4), idesc,
+                             (i > 0 || kk > 0 || pr > 1) ? 1u : 0u);
+          };
+          tc_fence_after();
+          if (big_last) cross_products();
+          if (first && used) {
+            if (!mbar_wait(acce + 8 * b, accph, abort_sh, ep.err, true)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+  #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-#pragma unroll
-            for (int pr = 1; pr < SC::NPROD; ++pr)
-              mma_f16_pair(tmem + cross, ad0 + (uint64_t)((SC::pa(pr) * A_BYTES + kk * 32) >> 4),
-                           bd0 + (uint64_t)((SC::pb(pr) * b_bytes + (uint32_t)(kk * 32)) >> 4), idesc,
-                           (i > 0 || kk > 0 || pr > 1) ? 1u : 0u);
-        };
-        tc_fence_after();
-        if (big_last) cross_products();
-        if (first && used) {
-          if (!mbar_wait(acce + 8 * b, accph, abort_sh, ep.err, true)) {
-            ok = false;
-            break;
+            mma_f16_pair(tmem + (uint32_t)(b * sc.bn), ad0 + (uint64_t)((kk * 32) >> 4),
+                         bd0 + (uint64_t)((kk * 32) >> 4), idesc, (!first || kk > 0) ? 1u : 0u);
+          if (last) {
+            mma_commit_pair(accf + 8 * b);
+            if (++b == nb) {
+              b = 0;
+              accph ^= 1u;
+              used = true;
+            }
           }
-          tc_fence_after();
-        }
-#pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          mma_f16_pair(tmem + (uint32_t)(b * sc.bn), ad0 + (uint64_t)((kk * 32) >> 4),
-                       bd0 + (uint64_t)((kk * 32) >> 4), idesc, (!first || kk > 0) ? 1u : 0u);
-        if (last) {
-          mma_commit_pair(accf + 8 * b);
-          if (++b == nb) {
-            b = 0;
-            accph ^= 1u;
-            used = true;
+          if (i == 0 && seg > 0) {
+            if (!mbar_wait(crosse, (uint32_t)(seg - 1) & 1u, abort_sh, ep.err, true)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+          if (!big_last) cross_products();
+          mma_commit_pair(empty0 + 8 * s);
+          if (++s == ST) {
+            s = 0;
+            ph ^= 1u;
           }
         }
-        if (i == 0 && seg > 0) {
-          if (!mbar_wait(crosse, (uint32_t)(seg - 1) & 1u, abort_sh, ep.err, true)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-        }
-        if (!big_last) cross_products();
-        mma_commit_pair(empty0 + 8 * s);
-        if (++s == ST) {
-          s = 0;
-          ph ^= 1u;
-        }
+        if (ok) mma_commit_pair(crossf);
       }
-      if (ok) mma_commit_pair(crossf);
     }
-  }
   } else if (warp < 4 + DRAIN_WARPS) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_DRAIN));
     const int dw = warp - 4;
@@ -861,7 +862,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
           if ((c & ~15) < cols) __stcg(mine + c * BM, sum[c]);
       }
       if (wk.final()) {
-        if (final_tile(ok, wk, slot)) finish_final(wk, slot, 1 + (dw >> 2));
+        if (final_tile(ok, wk)) finish_final(wk, slot, 1 + (dw >> 2));
       } else {
         __syncwarp();
         if (lane == 0) mbar_arrive(outf + 8 * slot);
@@ -874,11 +875,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     for (Walk wk(sc, pair); wk.next(); ++seg) {
       const int slot = seg & 1;
       if (wk.final()) {
-        if (final_tile(ok, wk, slot)) finish_final(wk, slot, 0);
+        if (final_tile(ok, wk)) finish_final(wk, slot, 0);
       } else if (ok) {
         const bool w = mbar_wait(outf + 8 * slot, (uint32_t)(seg >> 1) & 1u, abort_sh, ep.err, true);
         ok = __all_sync(0xffffffffu, w);
-        if (ok) finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, 0, 1, my_tiles + (size_t)slot * (BM * BNMAX), 1, 0);
+        const float* tile = my_tiles + (size_t)slot * (BM * BNMAX);
+        if (ok) finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, 0, 1, tile, 1, 0);
         __syncwarp();
         if (lane == 0) mbar_arrive(oute + 8 * slot);
       }
@@ -1514,7 +1516,8 @@ static int filter_impl(const cplx* A, const cplx* B, int64_t n, const cplx* Y0, 
     CB_TRY(pack(R, Zb[2], slotR));
     CB_TRY(put_gamma(k, [&](int64_t i) { return ritz[i]; }));
     Epi ep{};
-    ep.mode = 2; ep.n = n; ep.rows = rows; ep.cols = nc; ep.kpad = kpad; ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam; ep.err = err;
+    ep.mode = 2; ep.n = n; ep.rows = rows; ep.cols = nc; ep.kpad = kpad; ep.err = err;
+    ep.Znext = src; ep.Zcur = Zb[2]; ep.gamma = gam;
     ep.vexp_in = vexp + slotR;
     ep.amax_out = amax + slotS;
     sk(ep);
@@ -1653,16 +1656,20 @@ bool mixed_available() {
 template <int SCH, int FORM>
 static bool kernel_fits() {
   cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, tc::tc_hop_kernel<SCH, FORM>) == cudaSuccess) return tc::register_split_fits(fa.numRegs);
-  cudaGetLastError();
-  return false;
+  if (cudaFuncGetAttributes(&fa, tc::tc_hop_kernel<SCH, FORM>) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return tc::register_split_fits(fa.numRegs);
+}
+template <int SCH>
+static bool scheme_fits() {
+  return kernel_fits<SCH, tc::FORM_J>() && kernel_fits<SCH, tc::FORM_BLOCKS>();
 }
 bool mixed_filter_available() {
   if (!mixed_available()) return false;
   // a property of the build
-  static const bool fits = kernel_fits<tc::SCH_BF16X3, tc::FORM_J>() && kernel_fits<tc::SCH_BF16X3, tc::FORM_BLOCKS>() &&
-                           kernel_fits<tc::SCH_BF16X6, tc::FORM_J>() && kernel_fits<tc::SCH_BF16X6, tc::FORM_BLOCKS>() &&
-                           kernel_fits<tc::SCH_FP16X3, tc::FORM_J>() && kernel_fits<tc::SCH_FP16X3, tc::FORM_BLOCKS>();
+  static const bool fits = scheme_fits<tc::SCH_BF16X3>() && scheme_fits<tc::SCH_BF16X6>() && scheme_fits<tc::SCH_FP16X3>();
   return fits;
 }
 
