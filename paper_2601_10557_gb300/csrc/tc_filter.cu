@@ -1261,10 +1261,11 @@ static int prepare_p(const cplx* A, const cplx* B, int64_t n, Workspace& ws, POp
 // pairs at work: the MMAs (w / 2 each), the shared-memory traffic at 128 bytes a cycle (operand
 // reads and the ring's fill), or 0.027 cycles a byte of a stage, a fit to what a K block was
 // measured to take with all pairs busy (0.8-0.85 us for tiles of 160 and of 192 columns at n = 4096,
-// whose MMAs take 0.5 and 0.6 at the top clock; the same with half of B's loads replaced by
-// multicasts between two pairs and with the accumulators alternating, so the clock under the
-// power cap is the likely cause).  It favours wide tiles: n = 6000, k = 100 225 -> 182 us a
-// launch, n = 8192, k = 300 786 -> 704 us against a choice by the other two terms.
+// whose MMAs take 0.5 and 0.6 at the top clock; the tensor pipe is active in 56-59 % of the cycles
+// and L2 at 29 % of its rate, and replacing half of B's loads by multicasts between two pairs or
+// alternating the accumulators changed nothing, so what the rest is has not been shown).  It
+// favours wide tiles: n = 6000, k = 100 225 -> 182 us a launch in J form, n = 8192, k = 300 786 -> 704 us
+// against a choice by the other two terms.
 // Blocks form: a K block takes no less than 1400 cycles however narrow the tile (n = 1301, tiles of
 // 32 to 160 columns in one K range: 78 to 88 us a launch, 82 blocks).
 template <int SCH, int FORM>
