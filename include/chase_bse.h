@@ -141,6 +141,8 @@ typedef struct chase_bse_stats {
  *            phase-fixed so the largest-magnitude entry of the upper half is real
  *            and positive
  *   stats    host, may be NULL
+ * The lower half y of a pair is off by (conj(A) + lambda)^{-1} times the lower half of its
+ * residual, at most tol rho_hat: relative to |y|, more the weaker the coupling B.
  * Returns OK, NOT_CONVERGED (the first stats->converged entries are valid), or
  * an error; NONFINITE (nothing computed) when A, B, opts->W0 or opts->V0 hold a
  * NaN or an Inf.  Synchronises opts->stream. */
@@ -176,6 +178,9 @@ int chase_bse_filter_h2(const void* A, const void* B, int64_t n, void* W, int64_
  *   precision chase_bse_precision (FP64_TC: the FP64 recurrence with both H
  *            applications of a step as sliced tensor-core GEMMs; the sliced form of
  *            H, 7 * 8 n^2 bytes, is built for the call)
+ * Each half (x or y) of an output vector keeps the precision's accuracy relative to its own
+ * size, however small it is beside the other one (FP16x3: down to 1e-4 of it); with FP64_TC,
+ * relative to the larger one.
  * 0 < mu1 < mu_nevex < muN.  k = 0 is a no-op.  Asynchronous on `stream` except
  * for workspace bookkeeping; the result is ready when the stream reaches it. */
 int chase_bse_filter(const void* A, const void* B, int64_t n, void* W, int64_t k,
