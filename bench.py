@@ -580,8 +580,9 @@ def main():
             fp64["fp64_tc_kind"] = ("measured: one FP64-accurate solve + gradient with every large product a "
                                     "sliced tensor-core GEMM (after one warm-up solve)")
         else:
-            # the plain FP64 solve takes hours here: its filter alone, at the FP64 filter
-            # rate measured on a short call, is a lower bound of its time
+            # the plain FP64 solve takes hours here: its filter alone, at twice the FP64 filter
+            # rate measured on a short call (a solve's filter takes half of a call's operations), is
+            # a lower bound of its time
             kc = 64
             Wf = W0[:kc].clone()
             pkg.filter(A, B, Wf, [1] * kc, 1.0, 2.0, 60.0, precision="fp64")
@@ -594,11 +595,12 @@ def main():
             barrier()
             rate = 64.0 * n * n * kc * 2 / (f0.elapsed_time(f1) / 1e3)
             flops_step = fl / max(args.steps, 1)
-            fp64 = {"time_to_solution_s": flops_step / rate,
+            fp64 = {"time_to_solution_s": flops_step / (2.0 * rate),
                     "kind": "extrapolated lower bound: the mixed solve's filter flops "
-                            f"({flops_step:.3e}) at the FP64 filter rate measured on a degree-2 call over "
-                            f"{kc} columns ({rate / 1e12:.3f} TFLOP/s); QR, Rayleigh-Ritz and the "
-                            "FP64 filter's extra iterations not counted",
+                            f"({flops_step:.3e}) at twice the FP64 filter rate measured on a degree-2 call "
+                            f"over {kc} columns ({rate / 1e12:.3f} TFLOP/s; a solve's filter applies H with "
+                            "half of a call's operations); QR, Rayleigh-Ritz and the FP64 filter's extra "
+                            "iterations not counted",
                     "fp64_filter_tflops": rate / 1e12}
             del Wf
             # the FP64-accurate filter on the tensor cores: a degree-1 call over all columns
