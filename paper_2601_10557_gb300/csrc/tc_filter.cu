@@ -166,12 +166,13 @@ struct Form<FORM_BLOCKS> {
 // twice the stages lost 10-25 % (64-byte rows).
 //
 // Measured on one GB300, FP16x3, time of one launch of a degree's two, before (one CTA per
-// 128 x 128 tile, blocks form) and after, blocks and J form: n = 16384, k = 1300 26.5 -> 23.2 and
+// 128 x 128 tile, blocks form) and after, blocks and J form: n = 16384, k = 1300 26.8 -> 24.0 and
 // 11.5 ms (J form: three products of 16 n^2 k at 1446 TFLOP/s; cuBLAS bf16 1702 sustained); n = 8192,
-// k = 300 1717 -> 1216 and 715 us; n = 4096, k = 260 367 -> 320 and 185 us; n = 3001, k = 83 88 -> 90
-// and 60 us; n = 512, k = 30 29 -> 22 and 20 us.  Whole filters in blocks form: degree 20 at n = 4096
-// 15.1 -> 13.0 ms, degree 8 at n = 16384 431 -> 377 ms.  Errors against 64 bits, of the earlier
-// kernel's: each half in blocks form 0.5 to 1.03 (n = 128 to 16384), the whole vector in J form 0.46
+// k = 300 1707 -> 1218 and 715 us; n = 4096, k = 260 370 -> 315 and 185 us; n = 3001, k = 83 89 -> 85
+// and 60 us; n = 512, k = 30 30 -> 21 and 20 us.  Whole filters in blocks form: degree 20 at n = 4096
+// 15.2 -> 12.5 ms, degree 8 at n = 16384 436 -> 390 ms; of 28 sizes only those below n = 80 are not
+// faster (n = 40, k = 4, degree 28 0.75 -> 0.83 ms, n = 64, k = 6 0.79 -> 0.82).  Errors against 64 bits, of the
+// earlier kernel's: each half in blocks form 0.5 to 1.03 (n = 128 to 16384), the whole vector in J form 0.46
 // to 1.03.
 constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
@@ -185,8 +186,9 @@ constexpr int EPI_WARPS = 4;
 constexpr int THREADS = 128 + 32 * (DRAIN_WARPS + EPI_WARPS);
 // Registers a thread: 128 at launch (65536 over 16 warps); the warpgroup of the producer and
 // the MMA issuer and that of the finishing warps give theirs to the drain warps, whose sums
-// take 128.
-constexpr int REGS_LAUNCH = 128, REGS_ROLES = 40, REGS_DRAIN = 184, REGS_EPI = 96;
+// take 128.  40, 184 and 96 spilled the finishing warps' addresses: blocks form 5-8 % slower (n = 1301,
+// k = 67 42 -> 39 us a launch, n = 3001, k = 83 91 -> 84), the n = 4096 solve 1 %.
+constexpr int REGS_LAUNCH = 128, REGS_ROLES = 48, REGS_DRAIN = 176, REGS_EPI = 104;
 // The warpgroups draw on what the block was launched with: a kernel compiled to fewer registers a
 // thread than the shares add up to would wait for the rest forever (see mixed_filter_available).
 constexpr bool register_split_fits(int regs) {
@@ -250,15 +252,16 @@ __device__ __forceinline__ float vec_bound(const Epi& ep, int64_t v) {
 
 // Work of one launch: 256 x BN output tiles in a grouped raster (group_m row tiles x all
 // column tiles), so that the pairs running at the same time stream the same K blocks of A
-// and B from L2.  Pair c takes the whole tiles w * pairs + c of the full waves, then one of
-// the `parts` equal K ranges of the `rest` tiles that are left (rest * parts <= pairs).  With
-// parts > 1 the CTA that writes a half tile's last partial tile (a counter per half tile) sums
-// them in K order and finishes the tile, so no CTA waits for another and the result does not
-// depend on timing.
+// and B from L2.  Pair c takes the whole tiles w * pairs + c of the full waves; the K blocks of the
+// `rest` tiles that are left, one tile's after the other's, are shared out to `tail` pairs (rest <=
+// tail <= pairs), so a pair holds one K range of a tile or the end of one and the start of the next.
+// Where a tile is cut, the CTA that writes a half tile's last partial tile (a counter per half
+// tile) sums them in K order and finishes the tile, so no CTA waits for another and the result does
+// not depend on timing.
 struct Sched {
   int nkb, num_m, num_n, bn, n_last;  // K blocks; tiles; columns of a tile and of the last one
   int stages, stage_bytes, bufs, dcols, flush;
-  int pairs, waves, rest, parts;      // rest tiles after the full waves
+  int pairs, waves, rest, tail;
   int group_m;
   __device__ void tile_of(int t, int& mt, int& nt) const {
     const int per_group = group_m * num_n;
@@ -268,6 +271,10 @@ struct Sched {
     nt = rem / gm;
     mt = first + rem % gm;
   }
+  // First of the tail's K blocks that pair c holds, and the pair that holds block x (32-bit
+  // products: rest * nkb * tail < 2^31 up to n = 10^6).
+  __device__ int tail_start(int c) const { return (int)((unsigned)(rest * nkb * c) / (unsigned)tail); }
+  __device__ int tail_owner(int x) const { return (int)((unsigned)((x + 1) * tail - 1) / (unsigned)(rest * nkb)); }
 };
 // The segments (tile, K range) of pair c in order; all roles of both CTAs walk the same list.
 struct Walk {
@@ -275,7 +282,13 @@ struct Walk {
   int c, w;
   int mt, nt, cols;  // the current segment's tile and its columns
   int kb0, kb1;
-  __device__ Walk(const Sched& s, int pair) : sc(s), c(pair), w(-1) {}
+  int pos, end;      // the pair's K blocks of the tail not yet walked
+  __device__ Walk(const Sched& s, int pair) : sc(s), c(pair), w(-1), pos(0), end(0) {
+    if (c < sc.tail) {
+      pos = sc.tail_start(c);
+      end = sc.tail_start(c + 1);
+    }
+  }
   __device__ bool next() {
     ++w;
     int t;
@@ -283,11 +296,12 @@ struct Walk {
       t = w * sc.pairs + c;
       kb0 = 0;
       kb1 = sc.nkb;
-    } else if (w == sc.waves && c < sc.rest * sc.parts) {
-      const int r = c / sc.parts, p = c - r * sc.parts;
-      t = w * sc.pairs + r;
-      kb0 = (int)((int64_t)sc.nkb * p / sc.parts);
-      kb1 = (int)((int64_t)sc.nkb * (p + 1) / sc.parts);
+    } else if (pos < end) {
+      const int r = (unsigned)pos / (unsigned)sc.nkb, x = r * sc.nkb;
+      t = sc.waves * sc.pairs + r;
+      kb0 = pos - x;
+      pos = min(x + sc.nkb, end);
+      kb1 = pos - x;
     } else {
       return false;
     }
@@ -295,8 +309,9 @@ struct Walk {
     cols = nt == sc.num_n - 1 ? sc.n_last : sc.bn;
     return true;
   }
-  __device__ bool split() const { return w == sc.waves && sc.parts > 1; }
-  __device__ bool final() const { return w == sc.waves || (w == sc.waves - 1 && c >= sc.rest * sc.parts); }
+  __device__ int tail_tile() const { return (unsigned)(pos - 1) / (unsigned)sc.nkb; }
+  __device__ bool split() const { return w >= sc.waves && sc.tail > sc.rest; }
+  __device__ bool final() const { return pos >= end && w >= sc.waves - 1; }
 };
 
 // Shared-memory matrix descriptor: K-major tile written by TMA with 128-byte rows and
@@ -393,15 +408,21 @@ struct Maps {
   CUtensorMap b[3];
 };
 
-// The end of one half tile: sums its `parts` partial tiles (`stride` floats apart from `tiles`
-// on), undoes the scaling and runs the mode's epilogue for the 32 rows of TMEM lane quarter q and
+// The end of one half tile: sums its partial tiles, undoes the scaling and runs the mode's epilogue for the 32 rows of TMEM lane quarter q and
 // the groups of EB columns first, first + step, ...  It is a chain of L2 latencies, so the scales of
 // four groups are prepared at a time and all loads of a group are in flight together.
 constexpr int EB = 8;
+// The n partial tiles of a half tile in K order: the first, and tile j of the others at
+// rest + j * PART_STRIDE (one pair's two slots in both CTAs further).
+constexpr size_t PART_STRIDE = (size_t)4 * BM * BNMAX;
+struct Partials {
+  const float* first;
+  const float* rest;
+  int n;
+};
 template <int SCH>
 __device__ __forceinline__ void finish_jform(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
-                                            int lane, int first, int step, const float* tiles, int parts,
-                                            size_t stride) {
+                                            int lane, int first, int step, const Partials& pt) {
   using T = typename Scheme<SCH>::T;
   const int row_t = q * 32 + lane;
   const int64_t row = (int64_t)(2 * wk.mt + (int)rank) * BM + row_t;
@@ -436,10 +457,10 @@ __device__ __forceinline__ void finish_jform(const Epi& ep, const Sched& sc, con
       const int64_t vb = v0 + g;
       // loads at clamped rows and columns instead of under a predicate each
       const int64_t oz = vb * ep.rows + min(row, ep.rows - 1);
-      const float* tp = tiles + (size_t)g * BM + row_t;
+      const size_t off = (size_t)g * BM + row_t;
       float x[EB], zc[EB], zp[EB];
 #pragma unroll
-      for (int i = 0; i < EB; ++i) x[i] = __ldcg(tp + i * BM);
+      for (int i = 0; i < EB; ++i) x[i] = __ldcg(pt.first + off + i * BM);
       if (ep.mode != 0) {
 #pragma unroll
         for (int i = 0; i < EB; ++i) zc[i] = ep.Zcur[oz + (i < left ? i : 0) * ep.rows];
@@ -449,15 +470,15 @@ __device__ __forceinline__ void finish_jform(const Epi& ep, const Sched& sc, con
         for (int i = 0; i < EB; ++i) zp[i] = ep.Zprev[oz + (i < left ? i : 0) * ep.rows];
       }
 #pragma unroll 1
-      for (int j = 1; j < parts; j += 3) {
+      for (int j = 1; j < pt.n; j += 3) {
         float y[3][EB];
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(tp + min(j + p, parts - 1) * stride + i * BM);
+          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(pt.rest + off + min(j + p, pt.n - 1) * PART_STRIDE + i * BM);
 #pragma unroll
         for (int p = 0; p < 3; ++p)
-          if (j + p < parts) {
+          if (j + p < pt.n) {
 #pragma unroll
             for (int i = 0; i < EB; ++i) x[i] += y[p][i];
           }
@@ -507,8 +528,7 @@ __device__ __forceinline__ void finish_jform(const Epi& ep, const Sched& sc, con
 // A group of EB columns is two vectors.
 template <int SCH>
 __device__ __forceinline__ void finish_blocks(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
-                                              int lane, int first, int step, const float* tiles, int parts,
-                                              size_t stride) {
+                                              int lane, int first, int step, const Partials& pt) {
   using T = typename Scheme<SCH>::T;
   const int row_t = q * 32 + lane;
   const int64_t row = (int64_t)(2 * wk.mt + (int)rank) * BM + row_t;
@@ -538,13 +558,13 @@ __device__ __forceinline__ void finish_blocks(const Epi& ep, const Sched& sc, co
     for (int t = 0; t < 4; ++t) {
       const int vb = 2 * (g0 + t * step);
       if (vb >= vecs) break;
-      const float* tp = tiles + (size_t)(4 * vb) * BM + row_t;
+      const size_t off = (size_t)(4 * vb) * BM + row_t;
       // masters of the group's two vectors (a missing second one reads the first)
       const int64_t o[2] = {(v0 + vb) * n2 + rc, (v0 + (vb + 1 < vecs ? vb + 1 : vb)) * n2 + rc};
       float x[EB];
       float2 zc[4], zp[4];
 #pragma unroll
-      for (int i = 0; i < EB; ++i) x[i] = __ldcg(tp + i * BM);
+      for (int i = 0; i < EB; ++i) x[i] = __ldcg(pt.first + off + i * BM);
       if (ep.mode != 0) {
         const float2* Z = reinterpret_cast<const float2*>(ep.Zcur);
 #pragma unroll
@@ -556,15 +576,15 @@ __device__ __forceinline__ void finish_blocks(const Epi& ep, const Sched& sc, co
         for (int h = 0; h < 4; ++h) zp[h] = Z[o[h >> 1] + (h & 1) * ep.n];
       }
 #pragma unroll 1
-      for (int j = 1; j < parts; j += 3) {
+      for (int j = 1; j < pt.n; j += 3) {
         float y[3][EB];
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(tp + min(j + p, parts - 1) * stride + i * BM);
+          for (int i = 0; i < EB; ++i) y[p][i] = __ldcg(pt.rest + off + min(j + p, pt.n - 1) * PART_STRIDE + i * BM);
 #pragma unroll
         for (int p = 0; p < 3; ++p)
-          if (j + p < parts) {
+          if (j + p < pt.n) {
 #pragma unroll
             for (int i = 0; i < EB; ++i) x[i] += y[p][i];
           }
@@ -616,10 +636,9 @@ __device__ __forceinline__ void finish_blocks(const Epi& ep, const Sched& sc, co
 }
 template <int SCH, int FORM>
 __device__ __forceinline__ void finish_tile(const Epi& ep, const Sched& sc, const Walk& wk, uint32_t rank, int q,
-                                            int lane, int first, int step, const float* tiles, int parts,
-                                            size_t stride) {
-  if (FORM == FORM_J) finish_jform<SCH>(ep, sc, wk, rank, q, lane, first, step, tiles, parts, stride);
-  else finish_blocks<SCH>(ep, sc, wk, rank, q, lane, first, step, tiles, parts, stride);
+                                            int lane, int first, int step, const Partials& pt) {
+  if (FORM == FORM_J) finish_jform<SCH>(ep, sc, wk, rank, q, lane, first, step, pt);
+  else finish_blocks<SCH>(ep, sc, wk, rank, q, lane, first, step, pt);
 }
 
 template <int SCH, int FORM>
@@ -639,6 +658,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   volatile int* abort_sh = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* issued_sh = reinterpret_cast<int*>(tmem_slot + 2);
   volatile int* last_sh = reinterpret_cast<volatile int*>(tmem_slot + 3);
+  volatile int* last_epi_sh = reinterpret_cast<volatile int*>(tmem_slot + 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int pair = blockIdx.x >> 1;
@@ -678,31 +698,46 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   const uint32_t b_bytes = (uint32_t)(sc.bn / 2) * BK * 2;  // one piece of a stage's B half
 
   float* my_tiles = ep.part + (size_t)blockIdx.x * (2 * BM * BNMAX);
+  // The partial tiles of the tail tile that wk is in: pairs c0 .. c1 hold its K ranges, c0 as its second
+  // segment of the tail where it starts in the tile before, the others as their first.
+  auto partials = [&](const Walk& wk) -> Partials {
+    const int x = wk.tail_tile() * sc.nkb, c0 = sc.tail_owner(x), c1 = sc.tail_owner(x + sc.nkb - 1);
+    const int slot = sc.waves & 1, slot0 = sc.rest * sc.nkb * c0 < x * sc.tail ? slot ^ 1 : slot;  // c0 starts before x
+    const float* at = ep.part + (size_t)(4 * c0 + 2 * (int)rank) * (BM * BNMAX);
+    return Partials{at + (size_t)slot0 * (BM * BNMAX), at + (size_t)slot * (BM * BNMAX), c1 - c0 + 1};
+  };
+  // Whether this CTA has written the last partial tile of its half of wk's tile (its drain warps
+  // have fenced their writes); for N threads, all of which pass the barriers `bar`, `lead` among them.
+  auto count_partial = [&](const Walk& wk, int bar, int N, int lead, volatile int* sh) -> bool {
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(N) : "memory");
+    if (threadIdx.x == lead) {
+      int* cnt = ep.cnt + 2 * wk.tail_tile() + rank;
+      const bool l = atomicAdd(cnt, 1) == partials(wk).n - 1;
+      if (l) *cnt = 0;  // ready for the next launch
+      *sh = l ? 1 : 0;
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(N) : "memory");
+    const bool last = *sh != 0;
+    if (last) __threadfence();
+    return last;
+  };
   // A pair's last tile, for the drain and the finishing warps together: all of them pass the
   // barriers, also after a failed wait.  True where this CTA has the tile's last partial.
   auto final_tile = [&](bool ok, const Walk& wk) -> bool {
     constexpr int N = 32 * (DRAIN_WARPS + EPI_WARPS);
-    if (wk.split()) __threadfence();
-    asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
     bool last = true;
     if (wk.split()) {
-      if (threadIdx.x == 128) {
-        int* cnt = ep.cnt + 2 * (pair / sc.parts) + rank;
-        const bool l = atomicAdd(cnt, 1) == sc.parts - 1;
-        if (l) *cnt = 0;  // ready for the next launch
-        *last_sh = l ? 1 : 0;
-      }
+      __threadfence();
+      last = count_partial(wk, 1, N, 128, last_sh);
+    } else {
       asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
-      last = *last_sh != 0;
-      if (last) __threadfence();
     }
     return last && ok && __all_sync(0xffffffffu, *abort_sh == 0);  // warp-uniform
   };
   auto finish_final = [&](const Walk& wk, int slot, int third) {
-    const bool sp = wk.split();
-    const int p0 = sp ? pair / sc.parts * sc.parts : pair;  // the pair with the tile's first K range
-    const float* t = ep.part + (size_t)(4 * p0 + 2 * (int)rank + slot) * (BM * BNMAX);
-    finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, third, 3, t, sp ? sc.parts : 1, (size_t)4 * BM * BNMAX);
+    const float* mine = my_tiles + (size_t)slot * (BM * BNMAX);
+    const Partials pt = wk.split() ? partials(wk) : Partials{mine, mine, 1};
+    finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, third, 3, pt);
   };
 
   if (warp < 4) {
@@ -864,6 +899,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       if (wk.final()) {
         if (final_tile(ok, wk)) finish_final(wk, slot, 1 + (dw >> 2));
       } else {
+        if (wk.split()) __threadfence();
         __syncwarp();
         if (lane == 0) mbar_arrive(outf + 8 * slot);
       }
@@ -876,14 +912,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       const int slot = seg & 1;
       if (wk.final()) {
         if (final_tile(ok, wk)) finish_final(wk, slot, 0);
-      } else if (ok) {
+        continue;
+      }
+      if (ok) {
         const bool w = mbar_wait(outf + 8 * slot, (uint32_t)(seg >> 1) & 1u, abort_sh, ep.err, true);
         ok = __all_sync(0xffffffffu, w);
-        const float* tile = my_tiles + (size_t)slot * (BM * BNMAX);
-        if (ok) finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, 0, 1, tile, 1, 0);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(oute + 8 * slot);
       }
+      const float* mine = my_tiles + (size_t)slot * (BM * BNMAX);
+      Partials pt{mine, mine, 1};
+      bool last = true;
+      if (wk.split()) {  // the first of a pair's two K ranges of the tail
+        last = count_partial(wk, 2, 32 * EPI_WARPS, 32 * (4 + DRAIN_WARPS), last_epi_sh);
+        pt = partials(wk);
+      }
+      if (ok && last) finish_tile<SCH, FORM>(ep, sc, wk, rank, warp & 3, lane, 0, 1, pt);
+      __syncwarp();
+      if (ok && lane == 0) mbar_arrive(oute + 8 * slot);
     }
   }
   tc_fence_before();
@@ -1279,16 +1323,18 @@ static double block_cycles(int w, int bn, double active) {
 }
 // Cycles to finish a pair's last tile behind its MMAs, summing `parts` partial tiles: three sets of
 // warps take its groups of 8 columns in turn, each a chain of L2 latencies (2 us, and 0.7 us for
-// every three partial tiles more; n = 700 to 1301).  The J form's choices rest on a constant
-// fitted with the rest of its terms.
+// every three partial tiles more; n = 700 to 1301), and a cut tile is counted (n = 74, k = 8 in one
+// K range 0.94, in two 0.98 ms a degree-28 filter).  The J form's choices rest on a constant fitted
+// with the rest of its terms.
 template <int FORM>
 static double finish_cycles(int bn, int parts) {
   if (FORM == FORM_J) return parts > 1 ? 9000.0 + (parts + 1) * 8.0 * bn : 6000.0;
-  return 10000.0 + (double)cdiv(bn, 3 * EB) * (3900.0 + 1350.0 * (double)cdiv(parts - 1, 3));
+  return 10000.0 + (double)cdiv(bn, 3 * EB) * (3900.0 + 1350.0 * (double)cdiv(parts - 1, 3)) +
+         (parts > 1 ? 1500.0 : 0.0);
 }
 // The schedule of a launch with m rows, k2 columns and nkb K blocks: of the column widths
-// (multiples of 32) that ceil(k2 / 256) to 3 more column tiles need, and of the numbers of K
-// ranges to cut the tiles left after the full waves into, the choice of least estimated time.
+// (multiples of 32) that ceil(k2 / 256) to 3 more column tiles need, and of the ways to cut the
+// tiles left after the full waves into K ranges, the choice of least estimated time.
 template <int SCH, int FORM>
 static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
   using SC = Scheme<SCH>;
@@ -1322,19 +1368,26 @@ static Sched plan(int64_t m, int64_t k2, int nkb, int pairs) {
     const double avg = (full * (nn - 1) + block_cycles<SCH, FORM>(sc.n_last, sc.bn, 1.0)) / nn;
     const double fixed = 6000.0;  // prologue and epilogue of a tile in the full waves
     const double base = sc.waves * ((sc.waves > 1 ? avg : full) * nkb + fixed);
-    for (int f = 1; f == 1 || (f * sc.rest <= pairs && nkb / f >= 2); ++f) {
-      sc.parts = f;
-      double t = base;
-      if (sc.rest > 0) {
-        t += std::ceil((double)nkb / f) * block_cycles<SCH, FORM>(sc.bn, sc.bn, (double)(f * sc.rest) / pairs) +
-             finish_cycles<FORM>(sc.bn, f);
-      }
-      if (best_t == 0.0 || t < best_t) {
+    auto consider = [&](int tail, double t) {
+      if (best_t == 0.0 || base + t < best_t) {
         best = sc;
-        best_t = t;
+        best.tail = tail;
+        best_t = base + t;
       }
-      if (sc.rest == 0) break;
-    }
+    };
+    if (sc.rest == 0) consider(0, 0.0);
+    for (int f = 1; sc.rest > 0 && (f == 1 || (f * sc.rest <= pairs && nkb / f >= 2)); ++f)
+      consider(f * sc.rest, std::ceil((double)nkb / f) *
+                                    block_cycles<SCH, FORM>(sc.bn, sc.bn, (double)(f * sc.rest) / pairs) +
+                                finish_cycles<FORM>(sc.bn, f));
+    // blocks form: the tail's K blocks over all pairs, where a pair's range may cross from one tile
+    // into the next (about 2000 cycles more for its second segment).  Equal parts of each tile leave
+    // pairs idle where twice or thrice the tiles just miss their number: n = 4956, k = 79 (40 tiles of 76 pairs)
+    // 278 -> 189 us a launch, n = 8100, k = 30 237 -> 210, n = 16384, k = 20 854 -> 731.
+    const int64_t tail_blocks = (int64_t)sc.rest * nkb;
+    if (FORM == FORM_BLOCKS && tail_blocks >= 4 * (int64_t)pairs)
+      consider(pairs, std::ceil((double)tail_blocks / pairs) * block_cycles<SCH, FORM>(sc.bn, sc.bn, 1.0) +
+                          finish_cycles<FORM>(sc.bn, pairs / sc.rest + 2) + 2000.0);
   }
   return best;
 }
@@ -1357,7 +1410,7 @@ static int apply(const POperand& P, const Pieces& bp, int64_t rows, Epi ep, cuda
   for (int q = 0; q < Scheme<SCH>::NPA; ++q) maps.a[q] = P.map[q];
   for (int q = 0; q < Scheme<SCH>::NPW; ++q)
     CB_TRY(make_map(&maps.b[q], bp.p[q], P.kpad, rows, sc.bn / 2, Piece<T>::BF16));
-  const unsigned grid = 2u * (unsigned)(sc.waves > 0 ? sc.pairs : sc.rest * sc.parts);
+  const unsigned grid = 2u * (unsigned)(sc.waves > 0 ? sc.pairs : sc.tail);
   const int64_t tid = timer_begin(0, 32.0 * (double)P.n * (double)P.n * (double)(ep.cols / Form<FORM>::COLS), s);
   tc_hop_kernel<SCH, FORM><<<grid, THREADS, SMEM_BYTES, s>>>(maps, ep, sc);
   timer_end(tid, s);
@@ -1677,8 +1730,8 @@ bool mixed_filter_available() {
 // Where both forms are open the J form takes half the operations but, to form the entries of
 // M, four FP64 additions per entry of A and B (1.6e-5 us n^2), and its launches are no shorter
 // where M streams from HBM for few columns.  Measured, J form and blocks: n = 6000, k = 8,
-// degree 4 2.00 and 1.37 ms; 8100, 30, 8 4.91 and 4.60; 16384, 20, 4 14.6 and 10.3; 3001, 10, 10 1.12
-// and 1.13; against 4096, 60, 10 1.96 and 2.29; 16384, 100, 4 15.8 and 18.2; 1301, 6, 12 0.61 and 0.64.
+// degree 4 2.00 and 1.35 ms; 8100, 30, 8 4.91 and 4.22; 16384, 20, 4 14.6 and 9.5; 3001, 10, 10 1.12
+// and 1.14; against 4096, 60, 10 1.96 and 2.20; 16384, 100, 4 15.8 and 17.9; 1301, 6, 12 0.61 and 0.64.
 static bool j_form_faster(int64_t n, int64_t k, const int* degs) {
   int64_t work = 0;
   for (int64_t i = 0; i < k; ++i) work += degs[i];

@@ -105,7 +105,7 @@ TOL = {"fp16x3": 1e-5, "bf16x6": 1e-5, "bf16x3": 6e-5}
 # operand rows n around a tile of 256 rows, columns 4k around 32, 160 and 256, K = 4n around a
 # block of 64; (300, 70): K ranges, (640, 24)
 @pytest.mark.parametrize("n,k,deg", [(31, 1, 3), (47, 8, 4), (129, 33, 4), (255, 9, 3), (256, 40, 3),
-                                     (257, 41, 3), (300, 70, 4), (640, 24, 4)])
+                                     (257, 41, 3), (300, 70, 4), (640, 24, 4), (900, 400, 2), (520, 700, 2)])
 def test_tensor_core_filter_keeps_both_halves(tensor_cores, precision, n, k, deg, beta):
     P = bi.make_problem(n, seed=n + k, beta=beta)
     A, B = problem_on_device(P)
@@ -128,8 +128,10 @@ def test_explicit_square_filter_keeps_both_halves(tensor_cores, n, k, beta):
     assert max(_errors(got, ref)) <= 5e-5
 
 
-# full waves of CTA pairs and K ranges of the tiles left over, ragged degrees
-@pytest.mark.parametrize("n,k", [(2048, 700), (2050, 645)])
+# full waves of CTA pairs and K ranges of the tiles left over, ragged degrees; ranges that cross
+# from one tile into the next behind none (1100, 250), (1270, 500), one (2048, 900) and two
+# (2048, 1500) full waves
+@pytest.mark.parametrize("n,k", [(2048, 700), (2050, 645), (1100, 250), (1270, 500), (2048, 900), (2048, 1500)])
 def test_tensor_core_filter_halves_over_full_waves(tensor_cores, n, k):
     g = torch.Generator(device="cuda").manual_seed(n)
     X = torch.randn((n, n), generator=g, dtype=torch.complex128, device="cuda")
@@ -140,6 +142,8 @@ def test_tensor_core_filter_halves_over_full_waves(tensor_cores, n, k):
     W[:, n:] *= 1e-3
     degs = np.where(np.arange(k) < 9, 3, 1 + np.arange(k) % 2)
     got = tensor_cores.filter(A, B, W.clone(), degs, 1.5, 4.0, 8.0, precision="fp16x3")
+    again = tensor_cores.filter(A, B, W.clone(), degs, 1.5, 4.0, 8.0, precision="fp16x3")
+    assert torch.equal(got, again)  # the K ranges are summed in a fixed order
     for d in (1, 2, 3):
         sel = torch.from_numpy(np.flatnonzero(degs == d)).cuda()
         assert max(_errors(got[sel], _filter(A, B, W[sel], d, 1.5, 4.0, 8.0))) <= 1e-5
